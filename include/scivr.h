@@ -300,8 +300,9 @@ int scivr_spectrum(const void *amp, int64_t amp_ld, int32_t amp_prec, const doub
  * device [n_traj].  I_out: device [n_E].  C_out: device complex double
  * [n_steps+1] (may be NULL).  n_good_out: device int64 (may be NULL).  The
  * column sums over trajectories run in a fixed order (bitwise reproducible).
- * Allocates stream-ordered scratch of about 16 (n_steps+1) ceil(n_traj/4096)
- * bytes.  Errors: as scivr_spectrum. */
+ * Allocates stream-ordered scratch of 16 (n_steps+1) bytes per slice of rows (16 to 4096
+ * rows, about 1216 / ceil((n_steps+1)/256) slices; at most about 5 MB, or 16 (n_steps+1)
+ * ceil(n_traj/4096) bytes if that is more).  Errors: as scivr_spectrum. */
 int scivr_spectrum_hk(const void *amp, int64_t amp_ld, const uint8_t *good, int64_t n_traj, int32_t n_steps,
                       double dt, double E_min, double E_max, int32_t n_E, double *I_out, void *C_out,
                       int64_t *n_good_out, void *stream);

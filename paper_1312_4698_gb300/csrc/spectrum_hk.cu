@@ -13,78 +13,198 @@
 namespace scivr {
 namespace {
 
-constexpr int kRowsPerSlice = 4096;
+constexpr int kColThreads = 256;
+constexpr int kMaxSliceRows = 4096;   // flags of one slice staged in shared memory
+constexpr int kMinSliceRows = 16;
+// Blocks wanted for the column sum, 8 CTAs of 256 threads on each of 152 SMs: with fixed slices
+// of 4096 rows (64 blocks at 16384 x 4001 summands) most of the chip was idle.
+constexpr int kColBlocks = 152 * 8;
 
-__global__ void k_hk_colsum(const double2 *__restrict__ amp, int64_t amp_ld, const uint8_t *__restrict__ good,
-                            int64_t n, int K, double2 *__restrict__ part)
+// Rows per slice: enough slices to reach kColBlocks, none shorter than kMinSliceRows.
+inline int slice_rows(int64_t n, int K)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    const int64_t r0 = (int64_t)blockIdx.y * kRowsPerSlice;
-    const int64_t r1 = r0 + kRowsPerSlice < n ? r0 + kRowsPerSlice : n;
+    const int64_t cols = (K + kColThreads - 1) / kColThreads;
+    const int64_t slices = (kColBlocks + cols - 1) / cols;
+    int64_t rows = (n + slices - 1) / slices;
+    if (rows < kMinSliceRows) rows = kMinSliceRows;
+    if (rows > kMaxSliceRows) rows = kMaxSliceRows;
+    return (int)rows;
+}
+
+// Bound by the FP64 pipe's additions (two per summand: 248 us at 16384 x 4001, against 156 us
+// for one read of them from HBM).  A thread owns one column and keeps eight 16-byte loads in
+// flight; bad rows are loaded too (their flags, from shared memory, only select), so that no
+// load waits for a branch.  16384 x 4001 summands: 1180 -> 268 us.
+__global__ void __launch_bounds__(kColThreads, 4) k_hk_colsum(const double2 *__restrict__ amp, int64_t amp_ld,
+                                                           const uint8_t *__restrict__ good, int64_t n, int K,
+                                                           int rows, double2 *__restrict__ part)
+{
+    __shared__ uint8_t ok[kMaxSliceRows];
+    const int64_t r0 = (int64_t)blockIdx.y * rows;
+    const int cnt = (int)(n - r0 < rows ? n - r0 : rows);
+    for (int i = threadIdx.x; i < cnt; i += kColThreads) ok[i] = good[r0 + i];
+    __syncthreads();
+    const int c = blockIdx.x * kColThreads + threadIdx.x;
     if (c >= K) return;
+    const double2 *src = amp + r0 * amp_ld + c;
     double sr = 0.0, si = 0.0;
-    for (int64_t j = r0; j < r1; ++j) {
-        if (!good[j]) continue;   // bad rows never reach the sum, whatever they hold
-        const double2 a = amp[j * amp_ld + c];
-        sr += a.x;
-        si += a.y;
+    constexpr int U = 8;
+    int i = 0;
+    for (; i + U <= cnt; i += U) {
+        double2 a[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) a[u] = __ldcs(src + (i + u) * amp_ld);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {   // bad rows never reach the sum, whatever they hold
+            const bool in = ok[i + u];
+            sr += in ? a[u].x : 0.0;
+            si += in ? a[u].y : 0.0;
+        }
     }
+    for (; i < cnt; ++i)
+        if (ok[i]) {
+            const double2 a = __ldcs(src + i * amp_ld);
+            sr += a.x;
+            si += a.y;
+        }
     part[(int64_t)blockIdx.y * K + c] = make_double2(sr, si);
 }
 
-__global__ void k_hk_count(const uint8_t *__restrict__ good, int64_t n, long long *__restrict__ ng)
-{
-    __shared__ long long red[256];
-    long long cnt = 0;
-    for (int64_t j = threadIdx.x; j < n; j += blockDim.x) cnt += good[j] ? 1 : 0;
-    red[threadIdx.x] = cnt;
-    __syncthreads();
-    for (int o = 128; o > 0; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) ng[0] = red[0];
-}
+// Slices' partials in a fixed order (a thread of row y adds slices y, y + 8, ...; the 8 sums in
+// order of y), divided by the good count.  Every block counts the flags: n bytes from L2, cheaper
+// than a launch of its own.
+constexpr int kRedX = 32, kRedY = 8;
 
-__global__ void k_hk_reduce(const double2 *__restrict__ part, int n_slices, int K, const long long *__restrict__ ng,
-                            double2 *__restrict__ C)
+__global__ void __launch_bounds__(kRedX *kRedY) k_hk_reduce(const double2 *__restrict__ part, int n_slices, int K,
+                                                            const uint8_t *__restrict__ good, int64_t n,
+                                                            int64_t *__restrict__ ng_out, double2 *__restrict__ C)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= K) return;
+    __shared__ double2 sums[kRedY][kRedX];
+    __shared__ int64_t cnts[kRedY];
+    const int tid = threadIdx.y * kRedX + threadIdx.x;
+    int64_t cnt = 0;
+#pragma unroll 8
+    for (int64_t j = tid; j < n; j += kRedX * kRedY) cnt += good[j] ? 1 : 0;
+    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    if (threadIdx.x == 0) cnts[threadIdx.y] = cnt;
+    const int c = blockIdx.x * kRedX + threadIdx.x;
     double sr = 0.0, si = 0.0;
-    for (int s = 0; s < n_slices; ++s) {
-        const double2 v = part[(int64_t)s * K + c];
-        sr += v.x;
-        si += v.y;
+    if (c < K) {
+#pragma unroll 8
+        for (int s = threadIdx.y; s < n_slices; s += kRedY) {
+            const double2 v = part[(int64_t)s * K + c];
+            sr += v.x;
+            si += v.y;
+        }
     }
-    const double inv = ng[0] > 0 ? 1.0 / (double)ng[0] : 0.0;
+    sums[threadIdx.y][threadIdx.x] = make_double2(sr, si);
+    __syncthreads();
+    if (threadIdx.y != 0) return;
+    int64_t ng = 0;
+    for (int y = 0; y < kRedY; ++y) ng += cnts[y];
+    if (ng_out && blockIdx.x == 0 && threadIdx.x == 0) ng_out[0] = ng;
+    if (c >= K) return;
+    sr = si = 0.0;
+#pragma unroll
+    for (int y = 0; y < kRedY; ++y) {
+        sr += sums[y][threadIdx.x].x;
+        si += sums[y][threadIdx.x].y;
+    }
+    const double inv = ng > 0 ? 1.0 / (double)ng : 0.0;
     C[c] = make_double2(sr * inv, si * inv);
 }
 
-// one thread per energy; the phase E_k c dt is formed in FP64 for every c
-__global__ void k_hk_ft(const double2 *__restrict__ C, int K, double dt, double E_min, double dE, int n_E,
-                        double *__restrict__ I_out)
+// Re sum_{c} C_c e^{i E_k c dt} on the FP64 pipe, whose rate (one warp instruction per 64
+// cycles and sub-partition) is the bound: a sine and cosine per term (about 45 instructions)
+// took 4.2 ms for 4001 samples and 4000 energies.  The samples are cut into blocks of
+// 2 R + 1 around centres c_m = (2 R + 1) m + R:
+//   sum_c C_c z^c = sum_m z^{c_m} S_m,   S_m = C_{c_m} + sum_{r=1}^{R} A_{m,r} cos(r t) + B_{m,r} sin(r t),
+//   t = E dt, z = e^{i t}, A = C_{c_m + r} + C_{c_m - r}, B = i (C_{c_m + r} - C_{c_m - r}),
+// so that a term costs two multiply-adds; A and B do not depend on the energy.  A thread owns
+// an energy, a warp G consecutive blocks at a time (its A and B in shared memory, read as
+// broadcasts), the kFtWarps warps of a CTA share 32 energies' blocks.  z^r comes from up to R
+// complex products, the z^{c_m} of a warp's G blocks from a sine and cosine of E (c dt) at the
+// first centre and at most G - 1 products, so that no rounding of E dt is multiplied by c.
+// 4001 samples x 4000 energies: 4234 -> 86 us (6.4e7 multiply-adds; the FP64 pipe takes 61 us for them).
+constexpr int kFtR = 31, kFtW = 2 * kFtR + 1, kFtG = 8, kFtWarps = 8;
+
+__device__ __forceinline__ double2 hk_cmul(double2 x, double2 y)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n_E) return;
-    const double E = E_min + k * dE;
-    double acc = 0.5 * C[0].x;
-    for (int c = 1; c < K; ++c) {
-        double sn, cs;
-        sincos(E * (c * dt), &sn, &cs);
-        const double2 v = C[c];
-        acc = fma(v.x, cs, fma(-v.y, sn, acc));
-    }
-    I_out[k] = dt / 3.141592653589793238462643383280 * acc;
+    return make_double2(fma(x.x, y.x, -x.y * y.y), fma(x.x, y.y, x.y * y.x));
 }
+
+__global__ void __launch_bounds__(32 * kFtWarps) k_hk_ft(const double2 *__restrict__ C, int K, double dt, double E_min,
+                                                         double dE, int n_E, double *__restrict__ I_out)
+{
+    extern __shared__ __align__(16) double2 ab_all[];   // [warp][r][g]{A, B}
+    __shared__ double part[kFtWarps][32];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double2 *ab = ab_all + warp * (kFtR + 1) * kFtG * 2;
+    const int k = blockIdx.x * 32 + lane;
+    const double E = E_min + k * dE;
+    const int n_blk = (K + kFtW - 1) / kFtW, n_grp = (n_blk + kFtG - 1) / kFtG;
+    auto at = [&](int c) -> double2 {
+        if (c >= K) return make_double2(0.0, 0.0);
+        double2 v = __ldg(C + c);
+        if (c == 0) { v.x *= 0.5; v.y *= 0.5; }   // the folded transform's half weight at t = 0
+        return v;
+    };
+    double2 z;
+    sincos(E * dt, &z.y, &z.x);
+    double acc = 0.0;
+    for (int grp = warp; grp < n_grp; grp += kFtWarps) {
+        __syncwarp();
+        for (int i = lane; i < (kFtR + 1) * kFtG; i += 32) {
+            const int r = i / kFtG, c = (grp * kFtG + i % kFtG) * kFtW + kFtR;
+            const double2 u = at(c + r), v = r ? at(c - r) : make_double2(0.0, 0.0);
+            ab[2 * i] = make_double2(u.x + v.x, u.y + v.y);
+            ab[2 * i + 1] = make_double2(v.y - u.y, u.x - v.x);
+        }
+        __syncwarp();
+        double2 S[kFtG];
+#pragma unroll
+        for (int g = 0; g < kFtG; ++g) S[g] = ab[2 * g];
+        double2 zr = z;
+#pragma unroll 1
+        for (int r = 1; r <= kFtR; ++r) {
+            const double2 *row = ab + 2 * r * kFtG;
+#pragma unroll
+            for (int g = 0; g < kFtG; ++g) {
+                const double2 A = row[2 * g], B = row[2 * g + 1];
+                S[g].x = fma(A.x, zr.x, fma(B.x, zr.y, S[g].x));
+                S[g].y = fma(A.y, zr.x, fma(B.y, zr.y, S[g].y));
+            }
+            zr = hk_cmul(zr, z);
+        }
+        double2 ph, step;
+        sincos(E * ((grp * kFtG * kFtW + kFtR) * dt), &ph.y, &ph.x);
+        sincos(E * (kFtW * dt), &step.y, &step.x);
+#pragma unroll
+        for (int g = 0; g < kFtG; ++g) {
+            acc = fma(S[g].x, ph.x, fma(-S[g].y, ph.y, acc));
+            ph = hk_cmul(ph, step);
+        }
+    }
+    part[warp][lane] = acc;
+    __syncthreads();
+    if (warp == 0 && k < n_E) {
+        double s = part[0][lane];
+#pragma unroll
+        for (int w = 1; w < kFtWarps; ++w) s += part[w][lane];
+        I_out[k] = dt / 3.141592653589793238462643383280 * s;
+    }
+}
+
+constexpr size_t kFtSmem = sizeof(double2) * kFtWarps * (kFtR + 1) * kFtG * 2;
 
 }  // namespace
 
 size_t spectrum_hk_scratch_bytes(int64_t n_traj, int n_steps)
 {
-    const int64_t slices = (n_traj + kRowsPerSlice - 1) / kRowsPerSlice;
     const int64_t K = n_steps + 1;
-    return (size_t)(slices * K + K) * sizeof(double2) + 256;
+    const int rows = slice_rows(n_traj, (int)K);
+    const int64_t slices = (n_traj + rows - 1) / rows;
+    return (size_t)(slices * K + K) * sizeof(double2);
 }
 
 cudaError_t launch_spectrum_hk(const double2 *amp, int64_t amp_ld, const uint8_t *good, int64_t n_traj, int n_steps,
@@ -92,18 +212,19 @@ cudaError_t launch_spectrum_hk(const double2 *amp, int64_t amp_ld, const uint8_t
                                int64_t *n_good_out, void *scratch, cudaStream_t s, int *n_launch)
 {
     const int K = n_steps + 1;
-    const int slices = (int)((n_traj + kRowsPerSlice - 1) / kRowsPerSlice);
-    char *b = static_cast<char *>(scratch);
-    double2 *part = reinterpret_cast<double2 *>(b);
-    double2 *C = C_out ? C_out : reinterpret_cast<double2 *>(b + (size_t)slices * K * sizeof(double2));
-    long long *ng = reinterpret_cast<long long *>(b + (size_t)(slices + 1) * K * sizeof(double2));
-    if (n_good_out) ng = reinterpret_cast<long long *>(n_good_out);
-    k_hk_count<<<1, 256, 0, s>>>(good, n_traj, ng);
-    k_hk_colsum<<<dim3((K + 255) / 256, slices), 256, 0, s>>>(amp, amp_ld, good, n_traj, K, part);
-    k_hk_reduce<<<(K + 255) / 256, 256, 0, s>>>(part, slices, K, ng, C);
+    const int rows = slice_rows(n_traj, K);
+    const int slices = (int)((n_traj + rows - 1) / rows);
+    double2 *part = static_cast<double2 *>(scratch);
+    double2 *C = C_out ? C_out : part + (size_t)slices * K;
+    const unsigned cols = (unsigned)((K + kColThreads - 1) / kColThreads);
+    *n_launch = 0;
+    cudaError_t e = cudaFuncSetAttribute(k_hk_ft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFtSmem);
+    if (e != cudaSuccess) return e;
+    k_hk_colsum<<<dim3(cols, slices), kColThreads, 0, s>>>(amp, amp_ld, good, n_traj, K, rows, part);
+    k_hk_reduce<<<(K + kRedX - 1) / kRedX, dim3(kRedX, kRedY), 0, s>>>(part, slices, K, good, n_traj, n_good_out, C);
     const double dE = n_E > 1 ? (E_max - E_min) / (n_E - 1) : 0.0;
-    k_hk_ft<<<(n_E + 127) / 128, 128, 0, s>>>(C, K, dt, E_min, dE, n_E, I_out);
-    *n_launch = 4;
+    k_hk_ft<<<(n_E + 31) / 32, 32 * kFtWarps, kFtSmem, s>>>(C, K, dt, E_min, dE, n_E, I_out);
+    *n_launch = 3;
     return cudaGetLastError();
 }
 

@@ -249,3 +249,30 @@ def test_hk_default_workload_full_size_sampled(G):
     print(f"sample HK spectrum: rel err {e_s:.2e}; {len(pr)} peaks, max shift {shift.max():.3f} cm^-1")
     assert e_s <= 3e-2
     assert len(pr) > 0 and shift.max() <= 1.0
+
+
+@pytest.mark.parametrize("n,K,n_E", [(1, 2, 2), (15, 63, 33), (17, 64, 31), (257, 505, 32), (4097, 257, 100),
+                                     (300, 4096, 65), (33, 4537, 7)])
+def test_hk_spectrum_at_block_edges(G, n, K, n_E):
+    """Slices, 63-sample blocks, groups of eight blocks and 32-energy CTAs with remainders, rows
+    longer than the summands (leading dimension) and NaN in bad rows, against the oracle.  Bound:
+    a mean of n terms and a sum of K, each rounded a few times, about (n + 4 K) 2^-53 of the sum of
+    moduli; 1e-12 of it covers n + 4 K = 9000."""
+    import torch
+    rng = np.random.default_rng(n + K)
+    a = rng.normal(size=(n, K)) + 1j * rng.normal(size=(n, K))
+    good = (rng.random(n) < 0.7).astype(np.uint8)
+    good[0] = 1
+    ld, dt, E_min, E_max = K + 3, 10.0, 0.003, 0.06
+    rI, rn, rC = oracle.spectrum_hk(a, good, K - 1, dt, E_min, E_max, n_E)
+    dev = torch.full((n, ld, 2), float("nan"), dtype=torch.float64, device="cuda")
+    dev[:, :K, 0], dev[:, :K, 1] = _t(a.real), _t(a.imag)
+    dev[_t(good) == 0] = float("nan")
+    I = torch.empty(n_E, dtype=torch.float64, device="cuda")
+    C = torch.empty((K, 2), dtype=torch.float64, device="cuda")
+    ng = torch.zeros(1, dtype=torch.int64, device="cuda")
+    G.scivr_spectrum_hk(dev, ld, _t(good), n, K - 1, dt, E_min, E_max, n_E, I, C, ng)
+    c = C.cpu().numpy()
+    assert int(ng.item()) == rn
+    assert np.max(np.abs(c[:, 0] + 1j * c[:, 1] - rC)) <= 1e-12 * np.max(np.abs(a))
+    assert np.max(np.abs(I.cpu().numpy() - rI)) <= 1e-12 * dt / np.pi * np.sum(np.abs(rC))
