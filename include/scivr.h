@@ -273,11 +273,11 @@ int scivr_propagate(scivr_pes pes, const scivr_prop_params *prm, int64_t n_traj,
  * then sum tiles in FP64: their error is that of the digit count (about
  * 2^-8, 2^-16, 2^-24 relative to the largest terms).  SCIVR_FT_CZT64 evaluates the
  * same sums in FP64 through Bluestein's identity E_k c dt = E_min c dt + w (k^2 + c^2
- * - (k - c)^2)/2 (w = dE dt): a convolution by length-8192 FP64 FFTs per trajectory,
- * about 10 L log2 L flops instead of 8 K n_E, with FP64 rounding; it takes
+ * - (k - c)^2)/2 (w = dE dt): a convolution by FP64 FFTs of L = 1024 .. 8192 points per
+ * trajectory, about 10 L log2 L flops instead of 8 K n_E, with FP64 rounding; it takes
  * n_steps + 1 <= 7169 and n_E <= 12288 (SCIVR_EUNSUPPORTED otherwise; energies beyond
- * 8193 - (n_steps + 1) are transformed in blocks) and allocates about 200 KB plus
- * 8 n_E bytes per SM.  Allocates
+ * L + 1 - (n_steps + 1) are transformed in blocks) and allocates up to about 600 KB plus
+ * 8 n_E bytes for each of its one to four CTAs per SM.  Allocates
  * stream-ordered scratch (cudaMallocAsync): FP64 mode about
  * 16 (n_steps+1) n_E + 8 n_E ceil(n_traj/64) bytes; tensor-core modes about
  * 4 d (n_steps+1) (n_traj + 2 n_E) + 8 n_E ceil(n_traj/128) bytes, d digits.

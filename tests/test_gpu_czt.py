@@ -103,3 +103,32 @@ def test_czt_rejects_shapes_beyond_its_transform(G):
     with pytest.raises(G.ScivrError) as ei:
         G.scivr_spectrum(amp, 7170, w, good, 2, 7169, 10.0, 0.0, 0.1, 100, I, ft_mode=G.SCIVR_FT_CZT64)
     assert ei.value.code == G.SCIVR_EUNSUPPORTED
+
+
+@pytest.mark.parametrize("n,K,n_E", [
+    (3, 25, 1000), (3, 26, 1000), (3, 900, 125),      # K + n_E - 1 = 1024, 1025, 1024
+    (160, 1000, 1049), (5, 1025, 1024),               # 2048 points: K below and above half of them
+    (9, 2049, 2048), (7, 97, 4000), (320, 2048, 2049),  # 4096 points, the last with K = L / 2
+    (11, 3001, 2000),                                 # two blocks of 4096 points
+    (4, 4096, 4097), (4, 4097, 4096),                 # 8192 points, K = L / 2 and above
+    (2, 7169, 12288),                                 # the limits
+])
+def test_czt_at_the_edges_of_its_transform_lengths(G, n, K, n_E):
+    """Every transform length with its upper half empty or not, one and two energy blocks, more
+    trajectories than CTAs, against direct 64-bit sums.  Bound: 2 log2 L butterfly stages of a few
+    roundings each on values that grow with sqrt(L), 1e-12 of the largest intensity."""
+    import torch
+    rng = np.random.default_rng(K + n_E)
+    dt, E_min, E_max = 10.0, 0.004, 0.055
+    amp = (rng.normal(size=(n, K)) + 1j * rng.normal(size=(n, K))) * np.exp(-np.arange(K) / (2.0 * K))
+    w = rng.uniform(0.2, 5.0, n)
+    good = np.ones(n, np.uint8)
+    good[1::5] = 0
+    got, ng = _czt(G, amp, w, good, K - 1, dt, E_min, E_max, n_E)
+    E = _t(np.linspace(E_min, E_max, n_E))
+    ph = torch.arange(K, dtype=torch.float64, device="cuda")[:, None] * dt * E
+    X = _t(amp[good == 1]) @ torch.polar(torch.ones_like(ph), ph)
+    ref = (_t(w[good == 1])[:, None] * X.abs() ** 2).sum(0).cpu().numpy()
+    ref *= dt * dt / (2 * np.pi * (K - 1) * dt * good.sum())
+    assert ng == good.sum()
+    assert np.max(np.abs(got - ref)) <= 1e-12 * np.max(ref)
