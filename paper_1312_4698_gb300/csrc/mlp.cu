@@ -42,7 +42,12 @@ using namespace tc;
 constexpr int HW = 256;                 // hidden width
 constexpr int KT_H = HW / BK;           // k tiles of a 256-wide operand
 constexpr int kMaxF = 9;
-constexpr int TSMEM = BM * HW * 2;      // one 128 x 256 BF16 tile staged in shared memory
+// Row stride of a 128 x 256 BF16 tile staged in shared memory: 33 16-byte vectors, so that 8
+// lanes reading 16 bytes of 8 consecutive rows hit different banks.  With rows of 512 bytes the
+// row copies below were 32-way conflicts and took most of the training step's kernels: 98 us for
+// the hidden activation of 16384 points, 21 us now.
+constexpr int TS = HW + 8;
+constexpr int TSMEM = BM * TS * 2;
 
 __device__ __forceinline__ void silu3(float z, float &f, float &f1, float &f2)
 {
@@ -59,11 +64,13 @@ __device__ __forceinline__ void silu3(float z, float &f, float &f1, float &f2)
 // (row_block n_kt + k_tile) x block bytes); C is FP32 row-major with leading
 // dimension ldc, split z at C + z c_split; rows >= m_valid are not written.
 // grid = (N / 256, M / 128, splits), 128 threads.
-__global__ void __launch_bounds__(128, 1)
+constexpr int GEMM_STAGES = 4;   // 97 KB: two CTAs per SM, one's read-out beside the other's products
+
+__global__ void __launch_bounds__(128, 2)
     k_gemm(const uint8_t *__restrict__ At, const uint8_t *__restrict__ Bt, int n_kt, int kt_split,
            float *__restrict__ C, int64_t ldc, int64_t m_valid, int64_t c_split)
 {
-    constexpr int STAGES = 6;
+    constexpr int STAGES = GEMM_STAGES;
     constexpr int STAGE = TILE_A + TILE_B;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -150,7 +157,7 @@ __global__ void __launch_bounds__(128, 1)
     }
 }
 
-constexpr int GEMM_SMEM = 6 * (TILE_A + TILE_B) + 1024;
+constexpr int GEMM_SMEM = GEMM_STAGES * (TILE_A + TILE_B) + 1024;
 
 // ---------------------------------------------------------------- tiling helpers
 // Byte address of element (r, k) of a tiled operand with RB-row blocks and n_kt k tiles.
@@ -171,14 +178,14 @@ __device__ __forceinline__ void put8(uint8_t *base, int n_kt, int64_t r, int64_t
     *reinterpret_cast<uint4 *>(tile_addr<RB>(base, n_kt, r, k0)) = *reinterpret_cast<const uint4 *>(h);
 }
 
-// A 128 x 256 BF16 tile T (row-major, shared memory) of 128-row block `tile`:
+// A 128 x 256 BF16 tile T (row-major, row stride TS, shared memory) of 128-row block `tile`:
 // rows -> A operand with K = 256 (row = point row, k = hidden index).
 __device__ __forceinline__ void store_rows(const __nv_bfloat16 *T, uint8_t *X, int64_t tile)
 {
     for (int idx = threadIdx.x; idx < BM * (HW / 8); idx += blockDim.x) {
         const int rr = idx % BM, ch = idx / BM;
         *reinterpret_cast<uint4 *>(tile_addr<BM>(X, KT_H, tile * BM + rr, ch * 8)) =
-            *reinterpret_cast<const uint4 *>(T + rr * HW + ch * 8);
+            *reinterpret_cast<const uint4 *>(T + rr * TS + ch * 8);
     }
 }
 
@@ -190,18 +197,23 @@ __device__ __forceinline__ void store_cols(const __nv_bfloat16 *T, uint8_t *XT, 
         const int i = idx % HW, r0 = (idx / HW) * 8;
         __nv_bfloat16 h[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) h[k] = T[(r0 + k) * HW + i];
+        for (int k = 0; k < 8; ++k) h[k] = T[(r0 + k) * TS + i];
         *reinterpret_cast<uint4 *>(tile_addr<RB>(XT, n_kt, i, tile * BM + r0)) = *reinterpret_cast<const uint4 *>(h);
     }
 }
 
-// Weight matrix W [256 out][256 in] (FP32 row-major) -> B tiles of W (forward:
-// rows = out, k = in) or of W^T (reverse: rows = in, k = out).
-__global__ void k_tile_weight(const float *__restrict__ W, int transpose, uint8_t *__restrict__ Bt)
+// Weight matrix W [256 out][256 in] (FP32 row-major) -> B tiles of W (forward: rows = out,
+// k = in) and of W^T (reverse: rows = in, k = out): blockIdx.y = 0..3 is W2, W3, W2^T, W3^T.
+__global__ void k_tile_weights(const float *__restrict__ W2, const float *__restrict__ W3, uint8_t *__restrict__ B0,
+                               uint8_t *__restrict__ B1, uint8_t *__restrict__ B2, uint8_t *__restrict__ B3)
 {
     const int gid = blockIdx.x * blockDim.x + threadIdx.x;   // (row, chunk) over 256 x 32
     if (gid >= HW * (HW / 8)) return;
-    const int r = gid / (HW / 8), k0 = (gid % (HW / 8)) * 8;
+    const bool transpose = blockIdx.y >= 2;
+    const float *W = blockIdx.y % 2 ? W3 : W2;
+    uint8_t *Bt = blockIdx.y == 0 ? B0 : blockIdx.y == 1 ? B1 : blockIdx.y == 2 ? B2 : B3;
+    // consecutive threads: consecutive chunks of a row, or consecutive rows of a column chunk
+    const int r = transpose ? gid % HW : gid / (HW / 8), k0 = 8 * (transpose ? gid / HW : gid % (HW / 8));
     float v[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) v[i] = transpose ? W[(k0 + i) * HW + r] : W[r * HW + k0 + i];
@@ -216,72 +228,99 @@ struct MlpDev {
     const uint8_t *W2t, *W3t, *W2Tt, *W3Tt;               // BF16 B tiles
 };
 
-__device__ __forceinline__ int64_t point_row(const MlpDev &m, int64_t b)
+// ---------------------------------------------------------------- evaluation
+// Eight consecutive FP32 values (32-byte aligned).
+__device__ __forceinline__ void get8(const float *p, float (&v)[8])
 {
-    return (b / m.spt) * BM + (b % m.spt) * m.rows_per_sample;
+    const float4 a = *reinterpret_cast<const float4 *>(p), b = *reinterpret_cast<const float4 *>(p + 4);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+}
+__device__ __forceinline__ void set8(float *p, const float (&v)[8])
+{
+    *reinterpret_cast<float4 *>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4 *>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
 }
 
-// ---------------------------------------------------------------- evaluation
-// Layer 1 (K = F, CUDA cores) for one 128-row tile: writes the layer-2 input
-// rows (a1, and the tangents silu'(z1) W1[:, k] when rows_per_sample = F + 1)
-// as A tiles, and keeps z1 for the reverse pass.  Dynamic shared memory:
-// spt x 256 floats.
-__global__ void k_layer1(MlpDev m, int64_t n, const float *__restrict__ q, uint8_t *__restrict__ X2,
-                         float *__restrict__ Z1)
+// Layer 1 (K = F, CUDA cores), one row per point: writes a1 as A tiles of the layer-2 input and
+// keeps z1 for the reverse pass.  A lane owns a point (its inputs in registers), a warp 32 points
+// and the 8-unit chunks ch = blockIdx.y (mod L1_SPLIT) of its half, whose weights are broadcast
+// reads of shared memory; both outputs leave as whole 16- and 32-byte pieces.  Grid (tiles,
+// L1_SPLIT).  16384 points, F = 9: 107 us with the tile's z1 staged in shared memory (32-way
+// bank conflicts), 17 us now.
+constexpr int L1_SPLIT = 4;
+
+template <int F>
+__global__ void __launch_bounds__(256) k_layer1(MlpDev m, int64_t n, const float *__restrict__ q,
+                                                uint8_t *__restrict__ X2, float *__restrict__ Z1)
 {
-    extern __shared__ float zs[];   // [spt][HW]
-    const int64_t tile = blockIdx.x;
-    const int F = m.F, R = m.rows_per_sample, spt = m.spt;
-    for (int idx = threadIdx.x; idx < spt * HW; idx += blockDim.x) {
-        const int s = idx / HW, o = idx % HW;
-        const int64_t b = tile * spt + s;
-        float z = m.b1[o];
-        if (b < n)
-            for (int i = 0; i < F; ++i) z = fmaf(m.W1[o * F + i], m.s_in[i] * q[b * F + i], z);
-        zs[s * HW + o] = z;
-        if (b < n) Z1[b * HW + o] = z;
-    }
+    __shared__ __align__(16) float ws[F][HW];
+    __shared__ __align__(16) float bs[HW];
+    for (int i = threadIdx.x; i < HW * F; i += 256) ws[i % F][i / F] = m.W1[i];
+    bs[threadIdx.x] = m.b1[threadIdx.x];
     __syncthreads();
-    for (int idx = threadIdx.x; idx < BM * (HW / 8); idx += blockDim.x) {
-        const int rr = idx % BM, ch = idx / BM;
-        const int s = rr / R, k = rr % R;
-        float v[8];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t b = (int64_t)blockIdx.x * BM + (warp & 3) * 32 + lane;
+    float x[F];
+#pragma unroll
+    for (int k = 0; k < F; ++k) x[k] = b < n ? m.s_in[k] * q[b * F + k] : 0.0f;
+    for (int ch = (warp >> 2) * L1_SPLIT + blockIdx.y; ch < HW / 8; ch += 2 * L1_SPLIT) {
+        float z[8], v[8];
+        get8(bs + 8 * ch, z);
+#pragma unroll
+        for (int k = 0; k < F; ++k) {
+            float w[8];
+            get8(&ws[k][8 * ch], w);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) z[i] = fmaf(w[i], x[k], z[i]);
+        }
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const int o = ch * 8 + i;
-            float val = 0.0f;
-            if (s < spt && tile * spt + s < n) {
-                float f, f1, f2;
-                silu3(zs[s * HW + o], f, f1, f2);
-                val = k == 0 ? f : f1 * m.W1[o * F + (k - 1)];
-            }
-            v[i] = val;
+            float f, f1, f2;
+            silu3(z[i], f, f1, f2);
+            v[i] = b < n ? f : 0.0f;
         }
-        put8<BM>(X2, KT_H, tile * BM + rr, ch * 8, v);
+        if (b < n) set8(Z1 + b * HW + 8 * ch, z);
+        put8<BM>(X2, KT_H, b, 8 * ch, v);
     }
 }
 
 // Activation of a hidden layer for one tile: C holds z - b (point rows) and the
-// tangents' dz (tangent rows); writes the next layer's input rows.  With XT
+// tangents' dz (tangent rows, R = 2); writes the next layer's input rows.  With XT
 // set, the tile is also written transposed as a B operand (training).
 // Dynamic shared memory: TSMEM.
-__global__ void k_hidden_act(MlpDev m, int64_t n, const float *__restrict__ Cz, const float *__restrict__ bias,
-                             uint8_t *__restrict__ Xn, uint8_t *__restrict__ XT, int n_kt_rows)
+template <int R>
+__global__ void __launch_bounds__(256) k_hidden_act(MlpDev m, int64_t n, const float *__restrict__ Cz,
+                                                    const float *__restrict__ bias, uint8_t *__restrict__ Xn,
+                                                    uint8_t *__restrict__ XT, int n_kt_rows)
 {
-    extern __shared__ __align__(16) __nv_bfloat16 T[];   // [BM][HW]
+    extern __shared__ __align__(16) __nv_bfloat16 T[];   // [BM][TS]
     const int64_t tile = blockIdx.x;
-    const int R = m.rows_per_sample, spt = m.spt;
-    for (int idx = threadIdx.x; idx < BM * HW; idx += blockDim.x) {
-        const int rr = idx / HW, o = idx % HW;
-        const int s = rr / R, k = rr % R;
-        float val = 0.0f;
-        if (s < spt && tile * spt + s < n) {
-            const int64_t prow = tile * BM + s * R;
-            float f, f1, f2;
-            silu3(Cz[prow * HW + o] + bias[o], f, f1, f2);
-            val = k == 0 ? f : f1 * Cz[(tile * BM + rr) * HW + o];
+    constexpr int SPT = BM / R;
+#pragma unroll 4
+    for (int idx = threadIdx.x; idx < SPT * (HW / 8); idx += 256) {
+        const int s = idx / (HW / 8), ch = idx % (HW / 8);
+        __nv_bfloat16 h[R][8];
+        if (tile * SPT + s < n) {
+            float z[R][8], b8[8];
+#pragma unroll
+            for (int k = 0; k < R; ++k) get8(Cz + (tile * BM + s * R + k) * HW + 8 * ch, z[k]);
+            get8(bias + 8 * ch, b8);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                float f, f1, f2;
+                silu3(z[0][i] + b8[i], f, f1, f2);
+                h[0][i] = __float2bfloat16_rn(f);
+                if (R == 2) h[R - 1][i] = __float2bfloat16_rn(f1 * z[R - 1][i]);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < R; ++k)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) h[k][i] = __float2bfloat16_rn(0.0f);
         }
-        T[idx] = __float2bfloat16_rn(val);
+#pragma unroll
+        for (int k = 0; k < R; ++k)
+            *reinterpret_cast<uint4 *>(T + (s * R + k) * TS + 8 * ch) = *reinterpret_cast<const uint4 *>(h[k]);
     }
     __syncthreads();
     store_rows(T, Xn, tile);
@@ -296,7 +335,7 @@ __global__ void k_output(MlpDev m, int64_t n, const float *__restrict__ C3, floa
     const int64_t b = blockIdx.x;            // one CTA (256 threads) per point
     const int o = threadIdx.x;
     float f = 0.0f, f1 = 0.0f, f2;
-    if (b < n) silu3(C3[point_row(m, b) * HW + o] + m.b3[o], f, f1, f2);
+    if (b < n) silu3(C3[b * HW + o] + m.b3[o], f, f1, f2);
     float part = m.w4[o] * f;
     __shared__ float red[8];
     __shared__ float dv[HW];
@@ -322,22 +361,26 @@ __global__ void k_output(MlpDev m, int64_t n, const float *__restrict__ C3, floa
 __global__ void k_backward_act(MlpDev m, int64_t n, const float *__restrict__ Abar, const float *__restrict__ Cz,
                                const float *__restrict__ bias, uint8_t *__restrict__ Dn)
 {
+    // groups of 8 rows: the rows of a core matrix in consecutive lanes
     const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t n_pad = (n + BM - 1) / BM * BM;
     if (gid >= n_pad * (HW / 8)) return;
-    const int64_t b = gid / (HW / 8);
-    const int ch = (int)(gid % (HW / 8));
+    const int64_t b = gid / (8 * (HW / 8)) * 8 + gid % 8;
+    const int ch = (int)(gid / 8 % (HW / 8));
     float v[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        const int o = ch * 8 + i;
-        float val = 0.0f;
-        if (b < n) {
+    for (int i = 0; i < 8; ++i) v[i] = 0.0f;
+    if (b < n) {
+        float z[8], a[8], b8[8];
+        get8(Cz + b * HW + 8 * ch, z);
+        get8(Abar + b * HW + 8 * ch, a);
+        get8(bias + 8 * ch, b8);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
             float f, f1, f2;
-            silu3(Cz[point_row(m, b) * HW + o] + bias[o], f, f1, f2);
-            val = Abar[b * HW + o] * f1;
+            silu3(z[i] + b8[i], f, f1, f2);
+            v[i] = a[i] * f1;
         }
-        v[i] = val;
     }
     put8<BM>(Dn, KT_H, b, ch * 8, v);
 }
@@ -375,12 +418,18 @@ __global__ void k_grad(MlpDev m, int64_t n, const float *__restrict__ Z1, const 
 // 2 (j mod 64) + 1 (tangent) of the tile.  Per-tile partial sums of the
 // small parameter gradients: [W1 (256 F) | b1 | b2 | b3 | w4 (256 each) | b4].
 constexpr int TR_SPT = BM / 2;
+// Points whose loads a thread of the reverse kernels issues together: one CTA per tile walks its
+// 64 points in order (fixed summation order), so the loads' latency bounds them.  16384 points,
+// F = 9, with a load per iteration -> now: k_tr_out 47 -> 21 us, k_tr_back 73 -> 24 us,
+// k_tr_back1 110 -> 22 us.
+constexpr int TR_U = 8;
 
 __host__ __device__ constexpr int part_len(int F) { return HW * F + 4 * HW + 1; }
 
 // Loss terms, the fixed direction xd = s_in u, and layer 1 of the value and
 // tangent rows.  Dynamic shared memory: TSMEM + 2 TR_SPT kMaxF floats.
-__global__ void k_tr_layer1(MlpDev m, int64_t n, const float *__restrict__ q, const float *__restrict__ V1,
+template <int F>
+__global__ void __launch_bounds__(256) k_tr_layer1(MlpDev m, int64_t n, const float *__restrict__ q, const float *__restrict__ V1,
                             const float *__restrict__ g1, const float *__restrict__ Vref,
                             const float *__restrict__ gref, float alpha, float beta, float inv_n,
                             uint8_t *__restrict__ X2, uint8_t *__restrict__ X2T, int n_kt_rows,
@@ -392,7 +441,6 @@ __global__ void k_tr_layer1(MlpDev m, int64_t n, const float *__restrict__ q, co
     float *xs = reinterpret_cast<float *>(sm + TSMEM);   // [TR_SPT][kMaxF]
     float *xds = xs + TR_SPT * kMaxF;
     const int64_t tile = blockIdx.x;
-    const int F = m.F;
     if (threadIdx.x < TR_SPT) {
         const int s = threadIdx.x;
         const int64_t b = tile * TR_SPT + s;
@@ -419,14 +467,19 @@ __global__ void k_tr_layer1(MlpDev m, int64_t n, const float *__restrict__ q, co
         if ((threadIdx.x & 31) == 0) atomicAdd(loss, lp * inv_n);
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < TR_SPT * HW; idx += blockDim.x) {
-        const int s = idx / HW, o = idx % HW;
+    const int o = threadIdx.x;   // hidden unit
+    float w1[F];
+#pragma unroll
+    for (int k = 0; k < F; ++k) w1[k] = m.W1[o * F + k];
+    const float b1 = m.b1[o];
+#pragma unroll 4
+    for (int s = 0; s < TR_SPT; ++s) {
         const int64_t b = tile * TR_SPT + s;
-        float z = m.b1[o], zd = 0.0f;
+        float z = b1, zd = 0.0f;
+#pragma unroll
         for (int k = 0; k < F; ++k) {
-            const float w = m.W1[o * F + k];
-            z = fmaf(w, xs[s * kMaxF + k], z);
-            zd = fmaf(w, xds[s * kMaxF + k], zd);
+            z = fmaf(w1[k], xs[s * kMaxF + k], z);
+            zd = fmaf(w1[k], xds[s * kMaxF + k], zd);
         }
         float f = 0.0f, f1 = 0.0f, f2;
         if (b < n) {
@@ -434,8 +487,8 @@ __global__ void k_tr_layer1(MlpDev m, int64_t n, const float *__restrict__ q, co
             Zd1[b * HW + o] = zd;
             silu3(z, f, f1, f2);
         }
-        T[(2 * s) * HW + o] = __float2bfloat16_rn(f);
-        T[(2 * s + 1) * HW + o] = __float2bfloat16_rn(f1 * zd);
+        T[(2 * s) * TS + o] = __float2bfloat16_rn(f);
+        T[(2 * s + 1) * TS + o] = __float2bfloat16_rn(f1 * zd);
     }
     __syncthreads();
     store_rows(T, X2, tile);
@@ -453,23 +506,36 @@ __global__ void __launch_bounds__(256) k_tr_out(MlpDev m, int64_t n, const float
     const int o = threadIdx.x;
     const float w4 = m.w4[o], b3 = m.b3[o], at = m.s_out * w4;
     float acc_w4 = 0.0f, acc_b3 = 0.0f, acc_b4 = 0.0f;
-    for (int s = 0; s < TR_SPT; ++s) {
-        const int64_t b = tile * TR_SPT + s;
-        float zb = 0.0f, zdb = 0.0f;
-        if (b < n) {
-            const int64_t r = tile * BM + 2 * s;
-            const float zd = C3[(r + 1) * HW + o];
-            float f, f1, f2;
-            silu3(C3[r * HW + o] + b3, f, f1, f2);
-            const float eb = ebar[b];
-            zb = fmaf(eb * w4, f1, at * f2 * zd);
-            zdb = at * f1;
-            acc_w4 = fmaf(eb, f, fmaf(m.s_out * f1, zd, acc_w4));
-            acc_b3 += zb;
-            acc_b4 += eb;
+    const int cnt = (int)(n - tile * TR_SPT < TR_SPT ? n - tile * TR_SPT : TR_SPT);
+#pragma unroll 1
+    for (int s0 = 0; s0 < TR_SPT; s0 += TR_U) {
+        float zv[TR_U], zdv[TR_U], ev[TR_U];
+#pragma unroll
+        for (int u = 0; u < TR_U; ++u) {
+            const bool in = s0 + u < cnt;
+            const int64_t r = tile * BM + 2 * (s0 + u);
+            zv[u] = in ? C3[r * HW + o] : 0.0f;
+            zdv[u] = in ? C3[(r + 1) * HW + o] : 0.0f;
+            ev[u] = in ? ebar[tile * TR_SPT + s0 + u] : 0.0f;
         }
-        T[(2 * s) * HW + o] = __float2bfloat16_rn(zb);
-        T[(2 * s + 1) * HW + o] = __float2bfloat16_rn(zdb);
+#pragma unroll
+        for (int u = 0; u < TR_U; ++u) {
+            const int s = s0 + u;
+            float zb = 0.0f, zdb = 0.0f;
+            if (s < cnt) {
+                const float zd = zdv[u];
+                float f, f1, f2;
+                silu3(zv[u] + b3, f, f1, f2);
+                const float eb = ev[u];
+                zb = fmaf(eb * w4, f1, at * f2 * zd);
+                zdb = at * f1;
+                acc_w4 = fmaf(eb, f, fmaf(m.s_out * f1, zd, acc_w4));
+                acc_b3 += zb;
+                acc_b4 += eb;
+            }
+            T[(2 * s) * TS + o] = __float2bfloat16_rn(zb);
+            T[(2 * s + 1) * TS + o] = __float2bfloat16_rn(zdb);
+        }
     }
     float *P = part + tile * part_len(m.F);
     const int F = m.F;
@@ -491,21 +557,35 @@ __global__ void __launch_bounds__(256) k_tr_back(MlpDev m, int64_t n, const floa
     const int o = threadIdx.x;
     const float b2 = m.b2[o];
     float acc_b2 = 0.0f;
-    for (int s = 0; s < TR_SPT; ++s) {
-        const int64_t b = tile * TR_SPT + s;
-        float zb = 0.0f, zdb = 0.0f;
-        if (b < n) {
-            const int64_t r = tile * BM + 2 * s;
-            const float zd = C2[(r + 1) * HW + o];
-            float f, f1, f2;
-            silu3(C2[r * HW + o] + b2, f, f1, f2);
-            const float ab = Ab[r * HW + o], adb = Ab[(r + 1) * HW + o];
-            zb = fmaf(ab, f1, adb * f2 * zd);
-            zdb = adb * f1;
-            acc_b2 += zb;
+    const int cnt = (int)(n - tile * TR_SPT < TR_SPT ? n - tile * TR_SPT : TR_SPT);
+#pragma unroll 1
+    for (int s0 = 0; s0 < TR_SPT; s0 += TR_U) {
+        float zv[TR_U], zdv[TR_U], av[TR_U], adv[TR_U];
+#pragma unroll
+        for (int u = 0; u < TR_U; ++u) {
+            const bool in = s0 + u < cnt;
+            const int64_t r = tile * BM + 2 * (s0 + u);
+            zv[u] = in ? C2[r * HW + o] : 0.0f;
+            zdv[u] = in ? C2[(r + 1) * HW + o] : 0.0f;
+            av[u] = in ? Ab[r * HW + o] : 0.0f;
+            adv[u] = in ? Ab[(r + 1) * HW + o] : 0.0f;
         }
-        T[(2 * s) * HW + o] = __float2bfloat16_rn(zb);
-        T[(2 * s + 1) * HW + o] = __float2bfloat16_rn(zdb);
+#pragma unroll
+        for (int u = 0; u < TR_U; ++u) {
+            const int s = s0 + u;
+            float zb = 0.0f, zdb = 0.0f;
+            if (s < cnt) {
+                const float zd = zdv[u];
+                float f, f1, f2;
+                silu3(zv[u] + b2, f, f1, f2);
+                const float ab = av[u], adb = adv[u];
+                zb = fmaf(ab, f1, adb * f2 * zd);
+                zdb = adb * f1;
+                acc_b2 += zb;
+            }
+            T[(2 * s) * TS + o] = __float2bfloat16_rn(zb);
+            T[(2 * s + 1) * TS + o] = __float2bfloat16_rn(zdb);
+        }
     }
     part[tile * part_len(m.F) + HW * m.F + HW + o] = acc_b2;
     __syncthreads();
@@ -525,19 +605,37 @@ __global__ void __launch_bounds__(256) k_tr_back1(MlpDev m, int64_t n, const flo
     float accW[F], acc_b1 = 0.0f;
 #pragma unroll
     for (int k = 0; k < F; ++k) accW[k] = 0.0f;
-    for (int s = 0; s < TR_SPT; ++s) {
-        const int64_t b = tile * TR_SPT + s;
-        if (b >= n) break;
-        const int64_t r = tile * BM + 2 * s;
-        float f, f1, f2;
-        const float zd = Zd1[b * HW + o];
-        silu3(Z1[b * HW + o], f, f1, f2);
-        const float ab = Ab[r * HW + o], adb = Ab[(r + 1) * HW + o];
-        const float zb = fmaf(ab, f1, adb * f2 * zd);
-        const float zdb = adb * f1;
-        acc_b1 += zb;
+    const int cnt = (int)(n - tile * TR_SPT < TR_SPT ? n - tile * TR_SPT : TR_SPT);
+    __shared__ float x0[TR_SPT * F], xd[TR_SPT * F];   // the tile's inputs and directions (broadcast reads)
+    for (int i = o; i < cnt * F; i += HW) {
+        x0[i] = X0[tile * TR_SPT * F + i];
+        xd[i] = Xd0[tile * TR_SPT * F + i];
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int s0 = 0; s0 < cnt; s0 += TR_U) {
+        float zv[TR_U], zdv[TR_U], av[TR_U], adv[TR_U];
 #pragma unroll
-        for (int k = 0; k < F; ++k) accW[k] = fmaf(zb, X0[b * F + k], fmaf(zdb, Xd0[b * F + k], accW[k]));
+        for (int u = 0; u < TR_U; ++u) {
+            const bool in = s0 + u < cnt;
+            const int64_t b = tile * TR_SPT + s0 + u, r = tile * BM + 2 * (s0 + u);
+            zv[u] = in ? Z1[b * HW + o] : 0.0f;
+            zdv[u] = in ? Zd1[b * HW + o] : 0.0f;
+            av[u] = in ? Ab[r * HW + o] : 0.0f;
+            adv[u] = in ? Ab[(r + 1) * HW + o] : 0.0f;
+        }
+#pragma unroll
+        for (int u = 0; u < TR_U; ++u)
+            if (s0 + u < cnt) {
+                float f, f1, f2;
+                silu3(zv[u], f, f1, f2);
+                const float zb = fmaf(av[u], f1, adv[u] * f2 * zdv[u]);
+                const float zdb = adv[u] * f1;
+                acc_b1 += zb;
+#pragma unroll
+                for (int k = 0; k < F; ++k)
+                    accW[k] = fmaf(zb, x0[(s0 + u) * F + k], fmaf(zdb, xd[(s0 + u) * F + k], accW[k]));
+            }
     }
     float *P = part + tile * part_len(F);
 #pragma unroll
@@ -558,6 +656,7 @@ __global__ void k_tr_reduce(int F, int n_tiles, const float *__restrict__ part, 
     float acc = 0.0f;
     if ((p >= oW2 && p < ob2) || (p >= oW3 && p < ob3)) {
         const float *G = p < ob2 ? GW2 + (p - oW2) : GW3 + (p - oW3);
+#pragma unroll 8
         for (int s = 0; s < n_split; ++s) acc += G[(int64_t)s * HW * HW];
     } else {
         int idx;
@@ -566,6 +665,7 @@ __global__ void k_tr_reduce(int F, int n_tiles, const float *__restrict__ part, 
         else if (p < ow4) idx = HW * F + 2 * HW + (int)(p - ob3);     // b3
         else if (p < ob4) idx = HW * F + 3 * HW + (int)(p - ow4);     // w4
         else idx = HW * F + 4 * HW;                                   // b4
+#pragma unroll 16
         for (int t = 0; t < n_tiles; ++t) acc += part[(int64_t)t * PL + idx];
     }
     grad[p] = acc;
@@ -1243,15 +1343,15 @@ cudaError_t set_smem_attributes()
 {
     cudaError_t e = cudaFuncSetAttribute(k_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_layer1, cudaFuncAttributeMaxDynamicSharedMemorySize, BM * HW * 4);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_hidden_act, cudaFuncAttributeMaxDynamicSharedMemorySize, TSMEM);
+        e = cudaFuncSetAttribute(k_hidden_act<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, TSMEM);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_tr_layer1, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 TSMEM + 2 * TR_SPT * kMaxF * 4);
+        e = cudaFuncSetAttribute(k_hidden_act<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, TSMEM);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tr_out, cudaFuncAttributeMaxDynamicSharedMemorySize, TSMEM);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_tr_back, cudaFuncAttributeMaxDynamicSharedMemorySize, TSMEM);
 #define SCIVR_FA(FF) \
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_fused<FF>, cudaFuncAttributeMaxDynamicSharedMemorySize, FU_SMEM);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_mlp_fused<FF>, cudaFuncAttributeMaxDynamicSharedMemorySize, FU_SMEM); \
+    if (e == cudaSuccess)                                                                                               \
+        e = cudaFuncSetAttribute(k_tr_layer1<FF>, cudaFuncAttributeMaxDynamicSharedMemorySize, TSMEM + 2 * TR_SPT * kMaxF * 4);
     SCIVR_FA(1) SCIVR_FA(2) SCIVR_FA(3) SCIVR_FA(4) SCIVR_FA(5) SCIVR_FA(6) SCIVR_FA(7) SCIVR_FA(8) SCIVR_FA(9)
 #undef SCIVR_FA
     return e;
@@ -1276,9 +1376,9 @@ cudaError_t eval_F(const MlpWeightsDev &w, int64_t n, const float *q, float *V, 
     float *C3 = reinterpret_cast<float *>(scr + L.C3), *Ab2 = reinterpret_cast<float *>(scr + L.Ab2);
     float *Ab1 = reinterpret_cast<float *>(scr + L.Ab1);
     const unsigned nt = (unsigned)L.n_tiles;
-    k_layer1<<<nt, 256, (size_t)L.spt * HW * 4, s>>>(m, n, q, X2, Z1);
+    k_layer1<F><<<dim3(nt, L1_SPLIT), 256, 0, s>>>(m, n, q, X2, Z1);
     gemm_rows(X2, m.W2t, C2, L.M_pad, s);
-    k_hidden_act<<<nt, 256, TSMEM, s>>>(m, n, C2, m.b2, X3, nullptr, 0);
+    k_hidden_act<1><<<nt, 256, TSMEM, s>>>(m, n, C2, m.b2, X3, nullptr, 0);
     gemm_rows(X3, m.W3t, C3, L.M_pad, s);
     k_output<<<(unsigned)L.n_pad, 256, 0, s>>>(m, n, C3, V, D3);
     gemm_rows(D3, m.W3Tt, Ab2, L.n_pad, s);
@@ -1324,11 +1424,11 @@ cudaError_t loss_grad_F(const MlpWeightsDev &w, int64_t n, const float *q, const
     uint8_t *X2 = scr + L.X2, *X3 = scr + L.X3, *D3 = scr + L.D3, *D2 = scr + L.D2;
     uint8_t *X2T = scr + L.X2T, *X3T = scr + L.X3T, *D3T = scr + L.D3T, *D2T = scr + L.D2T;
     float *C2 = fp(L.C2), *C3 = fp(L.C3), *Ab2 = fp(L.Ab2), *Ab1 = fp(L.Ab1), *part = fp(L.part);
-    k_tr_layer1<<<nt, 256, TSMEM + 2 * TR_SPT * kMaxF * 4, s>>>(m, n, q, V1, g1, Vref, gref, alpha, beta,
+    k_tr_layer1<F><<<nt, 256, TSMEM + 2 * TR_SPT * kMaxF * 4, s>>>(m, n, q, V1, g1, Vref, gref, alpha, beta,
                                                                1.0f / (float)n, X2, X2T, L.n_kt_rows, fp(L.Z1),
                                                                fp(L.Zd1), fp(L.X0), fp(L.Xd0), fp(L.ebar), loss);
     gemm_rows(X2, m.W2t, C2, L.M_pad, s);
-    k_hidden_act<<<nt, 256, TSMEM, s>>>(m, n, C2, m.b2, X3, X3T, L.n_kt_rows);
+    k_hidden_act<2><<<nt, 256, TSMEM, s>>>(m, n, C2, m.b2, X3, X3T, L.n_kt_rows);
     gemm_rows(X3, m.W3t, C3, L.M_pad, s);
     k_tr_out<<<nt, 256, TSMEM, s>>>(m, n, C3, fp(L.ebar), D3, D3T, L.n_kt_rows, part);
     gemm_rows(D3, m.W3Tt, Ab2, L.M_pad, s);
@@ -1387,10 +1487,7 @@ cudaError_t mlp_loss_grad(const MlpWeightsDev &w, int F, int64_t n, const float 
 cudaError_t mlp_tile_weights(const MlpWeightsDev &w, cudaStream_t s)
 {
     const int n = mlp::HW * (mlp::HW / 8);
-    mlp::k_tile_weight<<<(n + 255) / 256, 256, 0, s>>>(w.W2, 0, w.W2t);
-    mlp::k_tile_weight<<<(n + 255) / 256, 256, 0, s>>>(w.W3, 0, w.W3t);
-    mlp::k_tile_weight<<<(n + 255) / 256, 256, 0, s>>>(w.W2, 1, w.W2Tt);
-    mlp::k_tile_weight<<<(n + 255) / 256, 256, 0, s>>>(w.W3, 1, w.W3Tt);
+    mlp::k_tile_weights<<<dim3((n + 255) / 256, 4), 256, 0, s>>>(w.W2, w.W3, w.W2t, w.W3t, w.W2Tt, w.W3Tt);
     return cudaGetLastError();
 }
 
