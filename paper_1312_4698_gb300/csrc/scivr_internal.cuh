@@ -110,13 +110,11 @@ struct AmpRef {
         }
         return static_cast<const double2 *>(p)[i];
     }
-    __device__ __forceinline__ float re_f(int64_t i) const
+    __device__ __forceinline__ float2 f(int64_t i) const
     {
-        return f32 ? static_cast<const float2 *>(p)[i].x : (float)static_cast<const double2 *>(p)[i].x;
-    }
-    __device__ __forceinline__ float im_f(int64_t i) const
-    {
-        return f32 ? static_cast<const float2 *>(p)[i].y : (float)static_cast<const double2 *>(p)[i].y;
+        if (f32) return static_cast<const float2 *>(p)[i];
+        const double2 v = static_cast<const double2 *>(p)[i];
+        return make_float2((float)v.x, (float)v.y);
     }
 #endif
 };

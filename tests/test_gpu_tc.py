@@ -101,3 +101,21 @@ def test_bounded_wait_reports_timeout_and_context_survives(G):
     gi, _ = gpu_spec(G, amp, w, good, 20, 10.0, 0.0, 0.1, 33, 3)
     assert np.max(np.abs(gi - ri)) <= TOL[3] * np.max(ri)
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("mode", [2, 3])
+@pytest.mark.parametrize("K,n_E", [(2, 3), (7, 9), (8, 127), (119, 128), (120, 129), (125, 136), (130, 8),
+                                   (247, 20), (248, 5), (249, 130), (255, 12), (497, 17)])
+def test_tc_twiddles_at_block_edges(G, mode, K, n_E):
+    """Every offset of the second half's 16-byte chunks, one to three blocks of 248 samples, ragged
+    groups of eight energies.  One unit sample at each end of the series and one inside: |X|^2 then
+    has the three twiddles' moduli and phases; bound TOL, as for random amplitudes."""
+    for at in sorted({0, K // 2, K - 1}):
+        amp = np.zeros((2, K), complex)
+        amp[0, at] = 1.0
+        amp[0, 0] += 0.5j
+        amp[1, max(at - 1, 0)] = 0.25 - 0.5j
+        w, good = np.array([1.0, 2.0]), np.ones(2, np.uint8)
+        ri, _ = oracle.spectrum(amp, w, good, K - 1, 10.0, 0.001, 0.06, n_E)
+        gi, _ = gpu_spec(G, amp, w, good, K - 1, 10.0, 0.001, 0.06, n_E, mode)
+        assert np.max(np.abs(gi - ri)) <= TOL[mode] * np.max(np.abs(ri))
