@@ -317,7 +317,7 @@ int scivr_create_pes(const scivr_pes_desc *d, scivr_pes *out)
     const size_t o_diagf = o_T4f + ((T4f.size() * sizeof(float) + 255) & ~(size_t)255);
     if (e == cudaSuccess) e = cudaMemcpy(b + o_diagf, diagf.data(), diagf.size() * sizeof(float), cudaMemcpyHostToDevice);
     const size_t o_T3p = o_diagf + ((diagf.size() * sizeof(float) + 255) & ~(size_t)255);
-    const size_t o_T4p = o_T3p + ((T3p.size() * sizeof(float) + 255) & ~(size_t)255);
+    const size_t o_T4p = o_T3p + T3p.size() * sizeof(float);   // one array of F + P rows (16-byte rows)
     if (e == cudaSuccess) e = cudaMemcpy(b + o_T3p, T3p.data(), T3p.size() * sizeof(float), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b + o_T4p, T4p.data(), T4p.size() * sizeof(float), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {

@@ -126,7 +126,7 @@ cudaError_t time_candidate(const PropLaunch &L, int warps, int n_sm, float *ms)
 
 cudaError_t choose_warps(const PropLaunch &L, int precision, int n_sm, int *warps)
 {
-    int cand[2];
+    int cand[2] = {0, 0};
     const int nc = batch_warp_candidates(L.args.F, cand);
     if (nc == 0) return cudaErrorInvalidValue;
     const std::string key = tune_key(L.args.F, precision);

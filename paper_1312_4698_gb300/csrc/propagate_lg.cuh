@@ -10,7 +10,8 @@
 //     in registers); lane a < F owns mode a: p_a, q_a (FP64) and the
 //     separable diagonal of the potential.  The Hessian's packed coupling
 //     entries e(a,b) are spread over the group, reading the coupling tensors
-//     staged in shared memory.  det M is Gaussian elimination of M^T across the
+//     staged in shared memory; above F = 13 the warps of a CTA form their
+//     trajectories' Hessians together.  det M is Gaussian elimination of M^T across the
 //     group (pivot column by warp reduction, pivot entries by shuffle).  The
 //     Herman-Kluk matrix A of the step goes to shared memory.
 //   phase 2 (once per chunk, job-parallel): lane j < T*C takes job j =
@@ -287,17 +288,15 @@ constexpr int kDetMEvery = 16;
 
 template <int F, int G, typename Real> __host__ __device__ constexpr int lg_chunk()
 {
-    if constexpr (sizeof(Real) == 4) return G == 32 && F > 16 ? 2 : ((G == 32 && F > 12) || (G == 16 && F > 8) ? 4 : 8);
+    if constexpr (sizeof(Real) == 4) return G == 32 && F > 16 ? 1 : (G == 32 && F > 15 ? 2 : ((G == 32 && F > 12) || (G == 16 && F > 8) ? 4 : 8));
     else return G < 32 ? G : (F > 9 ? 8 : 16);
 }
 
-// Warps per CTA and the launch-bounds CTA count: the wide groups (F > 9) run one CTA per
-// SM on one copy of the coupling tensors, 8 warps up to F = 12 and 4 above (measured:
-// at F = 15 the 8-warp CTA's 216 KB of shared memory leaves too little L1 and runs 16 %
-// slower; at F = 12 8 warps are 5 % faster).
-template <int F, int G> __host__ __device__ constexpr int lg_warps() { return G < 32 ? 4 : (F <= 9 ? 2 : (F <= 12 ? 8 : 4)); }
-// (F > 16: 4 warps, one CTA per SM: 18 KB of per-job prefactor matrices and 9 KB of det M
-// workspace per warp at F = 24)
+// Warps per CTA and the launch-bounds CTA count: above F = 13 one CTA of 8 warps per SM, whose
+// warps form the Hessians of their trajectories together (CoopHessian); F = 10..13 staged tensors
+// and a Hessian per warp, 8 warps up to F = 12 and 2 CTAs of 4 at F = 13 (the shared contraction's
+// barriers cost more than its loads save there: 5.84 against 5.57 ms for 4000 x 100 steps).
+template <int F, int G> __host__ __device__ constexpr int lg_warps() { return G < 32 ? 4 : (F <= 9 ? 2 : (F == 13 ? 4 : 8)); }
 // Two-trajectory mixed warps (F = 6..9) hold the coupling tensors in registers (no
 // shared-memory reads of them, more registers: lg_min_ctas) or read them from shared
 // memory in the same half-split layout (TensorLayout::split).  Measured on the recipe
@@ -401,11 +400,79 @@ struct TensorLayout {
     static constexpr int KH = (((F3E + P + 1) / 2) + 3) & ~3;
     static constexpr int KHS = (KH / 4) % 2 ? KH : KH + 4;
     static constexpr bool split = sizeof(Real) == 4 && STAGED && F >= 6 && F <= 9 && !lg_tensor_regs<F>();
-    static constexpr size_t tensor_elems = !staged ? 0 : (split ? (size_t)2 * P * KHS : (size_t)P * S3 + (size_t)P * S4);
+    // One-trajectory mixed warps above F = 13, and all that do not stage the tensors, contract them
+    // together (CoopHessian): rows of P4
+    // consecutive entries, the F cubic rows first.
+    static constexpr bool coop = sizeof(Real) == 4 && (F > 13 || (F > 9 && !STAGED));
+    static constexpr int P4 = (P + 3) & ~3;
+    static constexpr size_t tensor_elems = !staged ? 0 : (coop ? (size_t)(F + P) * P4 : (split ? (size_t)2 * P * KHS : (size_t)P * S3 + (size_t)P * S4));
     // after the tensors: the Herman-Kluk matrix coefficients acoef[a][b][4] =
     // (1/2) {rg_a/rg_b, rg_b/rg_a, -rg_a rg_b, 1/(rg_a rg_b)}, rg = sqrt(gamma)
     static constexpr size_t bytes = ((sizeof(Real) * (tensor_elems + (size_t)4 * F * F)) + 15) & ~(size_t)15;
 };
+
+// Hessian contraction of the wide mixed groups (F > 13, and all that do not stage the tensors),
+// shared by the warps of a CTA: entry e of trajectory t is sum_k T[k][e] x_t[k] over the cubic rows
+// (x = q) and over the quartic rows (x = q_k q_l).  A lane takes a quad of four entries and TT of
+// the CTA's TRAJ trajectories, so that a 16-byte tensor load feeds 4 TT multiply-adds; alone, a
+// warp's one trajectory used every loaded element once, and the loads bound the kernel (four or
+// eight warps per SM, issue 18-22 %).  Staged tensors (F <= 16): four lanes share a quad, lane s
+// summing the rows k = s mod 4, and the four sums are added as (s0 + s2) + (s1 + s3).  Otherwise the
+// rows stream from L2 through a ring of tiles in shared memory (cp.async), one sum per entry in row
+// order.  Either way each entry's multiply-adds keep the order they have in a single lane's loop,
+// whatever the tile: the results do not depend on TRAJ.  TT is the smallest tile whose items fit one
+// round of the CTA's lanes.  F = 15, 3001 trajectories x 501 steps: 37.0 -> 27.6 ms; F = 24,
+// 2048 x 200: 79.3 -> 45.8 ms.
+template <int F, int WARPS, int TRAJ, bool STAGED>
+struct CoopHessian {
+    static constexpr int P = F * (F + 1) / 2, P4 = (P + 3) & ~3, Q = P4 / 4;
+    static constexpr int SUB = STAGED ? 4 : 1;                      // lanes that share a quad's rows
+    static constexpr int groups(int tt) { return (TRAJ + tt - 1) / tt; }
+    static constexpr bool fits(int tt) { return Q * SUB * groups(tt) <= 32 * WARPS; }
+    static constexpr int TT = fits(1) ? 1 : fits(2) ? 2 : fits(3) ? 3 : fits(4) ? 4 : 8;
+    static_assert(fits(TT), "one round of items");
+    static constexpr int NG = groups(TT);
+    static constexpr int TP = TT == 3 ? 4 : TT;                     // trajectory slots of a group, padded to a vector
+    static constexpr int XW = NG * TP;                              // row length of the contracted vectors
+    static constexpr int ITEMS = Q * SUB * NG;
+    static constexpr int RT = WARPS >= 8 ? 16 : 8, ST = STAGED ? 0 : (WARPS >= 8 ? 3 : 2);   // ring tiles: rows, stages
+    static constexpr size_t x_bytes = (sizeof(float) * (size_t)(F + P) * XW + 15) & ~(size_t)15;
+    static constexpr size_t bytes = x_bytes + sizeof(float) * (size_t)ST * RT * P4;
+    __device__ static __forceinline__ int slot(int traj) { return (traj / TT) * TP + traj % TT; }
+};
+
+__device__ __forceinline__ void cp_async16(float *dst, const float *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+template <int TP>
+__device__ __forceinline__ void load_x(const float *p, float (&x)[TP])
+{
+    if constexpr (TP == 1) x[0] = *p;
+    else if constexpr (TP == 2) { const float2 v = *reinterpret_cast<const float2 *>(p); x[0] = v.x; x[1] = v.y; }
+    else {
+#pragma unroll
+        for (int i = 0; i < TP; i += 4) {
+            const float4 v = *reinterpret_cast<const float4 *>(p + i);
+            x[i] = v.x; x[i + 1] = v.y; x[i + 2] = v.z; x[i + 3] = v.w;
+        }
+    }
+}
+
+template <int TT, int TP>
+__device__ __forceinline__ void coop_fma(const float4 &t, const float (&x)[TP], float (&acc)[TT][4])
+{
+#pragma unroll
+    for (int j = 0; j < TT; ++j) {
+        acc[j][0] = fmaf(t.x, x[j], acc[j][0]);
+        acc[j][1] = fmaf(t.y, x[j], acc[j][1]);
+        acc[j][2] = fmaf(t.z, x[j], acc[j][2]);
+        acc[j][3] = fmaf(t.w, x[j], acc[j][3]);
+    }
+}
 
 template <int F, int G, typename Real>
 struct WarpShared {
@@ -430,8 +497,17 @@ struct WarpShared {
     // prefactor matrix per job, job-major rows of AS entries (AS odd): a lane that walks one
     // row of its job's matrix advances its address by one entry, and lanes of different jobs
     // at the same entry start in different banks
-    static constexpr int AS = ((F * F) % 2) ? F * F : F * F + 1;
+    // (at least the det M workspace of 2F rows of 2F + 1 floats per trajectory)
+    static constexpr int AS0 = sizeof(Real) == 4 ? (T * 2 * F * (2 * F + 1) + 4 * JOBS - 1) / (4 * JOBS) : 0;
+    static constexpr int AS1 = AS0 > F * F ? AS0 : F * F;
+    static constexpr int AS = AS1 % 2 ? AS1 : AS1 + 1;
     typename AEntry<Real>::T A[JOBS][AS];
+    // cubic and quartic parts of the Hessian entries (wide mixed groups): in the storage of the
+    // step's own prefactor matrix, which is written after the step's last kick
+    static constexpr int HP = (P + 3) & ~3;
+    static_assert(F <= 9 || 8 * HP <= 16 * F * F, "the Hessian parts fit a job's matrix");
+    __device__ __forceinline__ float *h3_at(int job) { return reinterpret_cast<float *>(&A[job][0]); }
+    __device__ __forceinline__ float *h4_at(int job) { return h3_at(job) + HP; }
     __device__ __forceinline__ typename AEntry<Real>::T &a_at(int job, int e) { return A[job][e]; }
     Real pj[F][JOBS], qj[F][JOBS];         // state per job, for the overlap (job column swizzled); FP32
                                            // in the mixed path, where the overlap is evaluated in FP32
@@ -442,11 +518,12 @@ struct WarpShared {
     double2 ov0[SCIVR_MAX_CHI][T];          // log of the Herman-Kluk summand's divisor per trajectory
 };
 
-// One CTA's share of a propagation: trajectories (cta * WARPS + warp) * T + t.
+// One CTA's share of a propagation: trajectories (cta * TRAJ_WARPS + warp) * T + t, warp <
+// TRAJ_WARPS; the other warps only share the Hessian contraction (wide mixed groups).
 // Called by the per-molecule kernel (cta = blockIdx.x) and by the batched
 // persistent kernel (cta = the work item's tile).  Stages the molecule's
 // constants itself and leaves shared memory free for the next call.
-template <int F, int G, typename Real, int WARPS, bool STAGED = (F <= 16)>
+template <int F, int G, typename Real, int WARPS, bool STAGED = (F <= 16), int TRAJ_WARPS = WARPS>
 __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsigned char *smem_raw)
 {
     constexpr int N2 = 2 * F;
@@ -463,12 +540,18 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
     using TL = TensorLayout<F, Real, STAGED>;
     constexpr int S3 = TL::S3, S4 = TL::S4;
     Real *sT3 = reinterpret_cast<Real *>(smem_raw);
-    Real *sT4 = sT3 + ((TL::staged && !TL::split) ? P * S3 : 0);
+    Real *sT4 = sT3 + ((TL::staged && !TL::split && !TL::coop) ? P * S3 : 0);
     Real *sTh = sT3;                                  // the half-split layout (TL::split)
     Real *sAc = sT3 + TL::tensor_elems;   // Herman-Kluk matrix coefficients [a][b][4] (16-byte aligned: the tensor block is a vector multiple)
     size_t off = TL::bytes;
     CtaConst<F> &cc = *reinterpret_cast<CtaConst<F> *>(smem_raw + off);
     off += (sizeof(CtaConst<F>) + 15) & ~(size_t)15;
+    // wide mixed groups: the CTA's contracted vectors and the ring of tensor rows
+    constexpr bool kCoop = TL::coop;
+    using CH = CoopHessian<kCoop ? F : 16, kCoop ? WARPS : 8, kCoop ? TRAJ_WARPS : 8, kCoop ? STAGED : true>;
+    float *xall = reinterpret_cast<float *>(smem_raw + off);
+    float *ring = reinterpret_cast<float *>(smem_raw + off + CH::x_bytes);
+    if constexpr (kCoop) off += CH::bytes;
     Sh *wsh_all = reinterpret_cast<Sh *>(smem_raw + off);
 
     const PesDev &pes = L.pes;
@@ -479,7 +562,12 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
         const Real *g3 = nullptr, *g4 = nullptr;
         if constexpr (sizeof(Real) == 4) { g3 = reinterpret_cast<const Real *>(pes.T3f); g4 = reinterpret_cast<const Real *>(pes.T4f); }
         else { g3 = reinterpret_cast<const Real *>(pes.T3); g4 = reinterpret_cast<const Real *>(pes.T4); }
-        if constexpr (TL::split) {
+        if constexpr (kCoop) {
+            const float4 *v3 = reinterpret_cast<const float4 *>(pes.T3p), *v4 = reinterpret_cast<const float4 *>(pes.T4p);
+            float4 *dst = reinterpret_cast<float4 *>(sT3);
+            for (int i = threadIdx.x; i < F * (TL::P4 / 4); i += blockDim.x) dst[i] = v3[i];
+            for (int i = threadIdx.x; i < P * (TL::P4 / 4); i += blockDim.x) dst[F * (TL::P4 / 4) + i] = v4[i];
+        } else if constexpr (TL::split) {
             constexpr int KH = TL::KH, KHS = TL::KHS, F3E = TL::F3E;
             for (int i = threadIdx.x; i < 2 * P * KHS; i += blockDim.x) {
                 const int h = i / (P * KHS), e = (i / KHS) % P, kk = i % KHS, gk = h * KH + kk;
@@ -539,6 +627,121 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
 
     const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31;
     const int t = ln / G, g = ln % G, base = t * G;
+    constexpr int P4 = (P + 3) & ~3;
+    // the CTA's share of one kick's Hessian contraction (CoopHessian): from the trajectories'
+    // vectors in xall to the entries' parts h3, h4 of step c's job
+    auto contract = [&](int c) {
+        if constexpr (kCoop) {
+            const int it = threadIdx.x;
+            const int sub = it % CH::SUB, quad = (it / CH::SUB) % CH::Q, grp = it / (CH::SUB * CH::Q);
+            const bool work = it < CH::ITEMS;
+            constexpr int TT = CH::TT, TP = CH::TP;
+            float a3[TT][4], a4[TT][4];
+#pragma unroll
+            for (int j = 0; j < TT; ++j)
+#pragma unroll
+                for (int c4 = 0; c4 < 4; ++c4) a3[j][c4] = a4[j][c4] = 0.0f;
+            const float *xg = xall + grp * TP;
+            if constexpr (STAGED) {
+                if (work) {
+                    const float4 *trow = reinterpret_cast<const float4 *>(sT3) + quad;
+                    if (use3) {
+#pragma unroll 2
+                        for (int k = sub; k < F; k += 4) {
+                            float x[TP];
+                            load_x<TP>(xg + k * CH::XW, x);
+                            coop_fma<TT, TP>(trow[k * CH::Q], x, a3);
+                        }
+                    }
+                    if (use4) {
+#pragma unroll 4
+                        for (int k = F + sub; k < F + P; k += 4) {
+                            float x[TP];
+                            load_x<TP>(xg + k * CH::XW, x);
+                            coop_fma<TT, TP>(trow[k * CH::Q], x, a4);
+                        }
+                    }
+                }
+                // the four row classes of a quad sit in adjacent lanes
+#pragma unroll
+                for (int j = 0; j < TT; ++j)
+#pragma unroll
+                    for (int c4 = 0; c4 < 4; ++c4) {
+                        a3[j][c4] += __shfl_xor_sync(FULL, a3[j][c4], 2);
+                        a3[j][c4] += __shfl_xor_sync(FULL, a3[j][c4], 1);
+                        a4[j][c4] += __shfl_xor_sync(FULL, a4[j][c4], 2);
+                        a4[j][c4] += __shfl_xor_sync(FULL, a4[j][c4], 1);
+                    }
+            } else {
+                // rows r < n3 of T3p, then the rows of T4p (one array), in tiles of RT rows
+                constexpr int RT = CH::RT, ST = CH::ST;
+                const int n3 = use3 ? F : 0, nr = n3 + (use4 ? P : 0), n_tile = (nr + RT - 1) / RT;
+                const float *xr = xg + (use3 ? 0 : F * CH::XW);
+                const float *src = (use3 ? pes.T3p : pes.T4p) + 4 * threadIdx.x;
+                auto fetch = [&](int tile) {
+                    if (tile < n_tile) {
+                        float *dst = ring + (tile % ST) * (RT * P4) + 4 * threadIdx.x;
+                        const float *from = src + (size_t)tile * (RT * P4);
+                        const int cnt4 = min(RT, nr - tile * RT) * (P4 / 4) - (int)threadIdx.x;
+#pragma unroll
+                        for (int i = 0; i < RT * P4 / 4; i += 32 * WARPS)
+                            if (i < cnt4) cp_async16(dst + 4 * i, from + 4 * i);
+                    }
+                    cp_async_commit();
+                };
+#pragma unroll
+                for (int s = 0; s < ST - 1; ++s) fetch(s);
+                for (int tile = 0; tile < n_tile; ++tile) {
+                    cp_async_wait<ST - 2>();
+                    __syncthreads();   // the tile is in; the one fetched next was read a turn ago
+                    fetch(tile + ST - 1);
+                    if (work) {
+                        const float4 *trow = reinterpret_cast<const float4 *>(ring + (tile % ST) * (RT * P4)) + quad;
+                        const int r0 = tile * RT, r1 = min(r0 + RT, nr);
+                        int r = r0;
+                        for (; r < min(r1, n3); ++r) {
+                            float x[TP];
+                            load_x<TP>(xr + r * CH::XW, x);
+                            coop_fma<TT, TP>(trow[(r - r0) * CH::Q], x, a3);
+                        }
+#pragma unroll 4
+                        for (; r < r1; ++r) {
+                            float x[TP];
+                            load_x<TP>(xr + r * CH::XW, x);
+                            coop_fma<TT, TP>(trow[(r - r0) * CH::Q], x, a4);
+                        }
+                    }
+                }
+                cp_async_wait<0>();
+            }
+            if (work) {
+#pragma unroll
+                for (int j = 0; j < TT; ++j) {
+                    const int tr = grp * TT + j;
+                    if (tr < TRAJ_WARPS && j % CH::SUB == sub) {
+                        *reinterpret_cast<float4 *>(wsh_all[tr].h3_at(c) + 4 * quad) = make_float4(a3[j][0], a3[j][1], a3[j][2], a3[j][3]);
+                        *reinterpret_cast<float4 *>(wsh_all[tr].h4_at(c) + 4 * quad) = make_float4(a4[j][0], a4[j][1], a4[j][2], a4[j][3]);
+                    }
+                }
+            }
+        } else {
+            (void)c;
+        }
+    };
+    if constexpr (TRAJ_WARPS < WARPS) {
+        static_assert(kCoop, "only the shared contraction employs warps without a trajectory");
+        if (warp >= TRAJ_WARPS) {
+            for (int step0 = 0; step0 < A.n_steps; step0 += C)
+                for (int c = 0; c < min(C, A.n_steps - step0); ++c)
+                    for (int kick = 0; kick < 3; ++kick) {
+                        __syncthreads();
+                        contract(c);
+                        __syncthreads();
+                    }
+            __syncthreads();   // the body's last
+            return;
+        }
+    }
     Sh &sh = wsh_all[warp];
     {
         // padding entries of the vector rows are read (multiplied by zero or skipped) but never
@@ -549,7 +752,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
         __syncwarp();
     }
     const int64_t n = L.n_traj;
-    const int64_t j_traj = (cta * WARPS + warp) * T + t;
+    const int64_t j_traj = (cta * TRAJ_WARPS + warp) * T + t;
     const bool active = j_traj < n;
     const int64_t jl = active ? j_traj : n - 1;
 
@@ -616,8 +819,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
             }
         }
     }
-    // above F = 16: four consecutive entries 4 (g + i G) .. + 3 per load, (a, b) packed as a | b << 8
-    constexpr int P4 = (P + 3) & ~3;
+    // tensors not staged: quads of consecutive entries 4 (g + i G) .. + 3, (a, b) packed as a | b << 8
     constexpr int NQ = TL::staged ? 1 : (P4 / 4 + G - 1) / G;
     int eq[TL::staged ? 1 : 4 * NQ];
     if constexpr (!TL::staged) {
@@ -741,6 +943,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                 if (g < F) {
                     sh.qr[t][g] = (Real)coord_f(q);
                     if constexpr (kTreg || kSplit) sh.xs[t][g] = (Real)coord_f(q);
+                    if constexpr (kCoop) xall[g * CH::XW + CH::slot(warp)] = (float)coord_f(q);
                 }
                 __syncwarp();
 #pragma unroll
@@ -750,55 +953,36 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                         const Real v = sh.qr[t][ea[i]] * sh.qr[t][eb[i]];
                         sh.qq[t][e] = v;
                         if constexpr (kTreg || kSplit) sh.xs[t][F3E + e] = v;
+                        if constexpr (kCoop) xall[(F + e) * CH::XW + CH::slot(warp)] = (float)v;
                     }
                 }
                 __syncwarp();
                 Real vpart = Real(0);
-                if constexpr (!TL::staged) {
-                    // entry quads against the tensors in global memory (L2-resident; [k][e] and
-                    // [kl][e] rows padded to P4): one 16-byte load feeds four entries
-                    static_assert(sizeof(Real) == 4, "the global-tensor schedule is the mixed path's");
-                    const float4 *T3v = reinterpret_cast<const float4 *>(pes.T3p);
-                    const float4 *T4v = reinterpret_cast<const float4 *>(pes.T4p);
+                if constexpr (kCoop) {
+                    __syncthreads();   // every warp's x is written; every warp has read its last h3, h4
+                    contract(c);
+                    __syncthreads();
+                    const float *s3 = sh.h3_at(c), *s4 = sh.h4_at(c);
+                    auto entry = [&](int e, int a, int b) {
+                        const float h3 = s3[e], h4 = s4[e];
+                        const float h = h3 + h4;
+                        sh.H[t][a][b] = h;
+                        sh.H[t][b][a] = h;
+                        const float gce = fmaf(0.5f, h3, h4 * (1.0f / 3.0f));
+                        sh.Gc[t][a][b] = gce;
+                        sh.Gc[t][b][a] = gce;
+                        const float vc = fmaf(1.0f / 6.0f, h3, h4 * (1.0f / 12.0f));
+                        vpart = fmaf(a == b ? vc : 2.0f * vc, sh.qq[t][e], vpart);
+                    };
+                    if constexpr (STAGED) {
 #pragma unroll
-                    for (int i = 0; i < NQ; ++i) {
-                        const int q4 = g + i * G;
-                        if (4 * q4 < P) {
-                            float4 h3 = make_float4(0.f, 0.f, 0.f, 0.f), h4 = h3;
-                            if (use3) {
-#pragma unroll 8
-                                for (int k = 0; k < F; ++k) {
-                                    const float4 tv = __ldg(T3v + k * (P4 / 4) + q4);
-                                    const float x = sh.qr[t][k];
-                                    h3.x = fmaf(tv.x, x, h3.x); h3.y = fmaf(tv.y, x, h3.y);
-                                    h3.z = fmaf(tv.z, x, h3.z); h3.w = fmaf(tv.w, x, h3.w);
-                                }
-                            }
-                            if (use4) {
-#pragma unroll 4
-                                for (int kl = 0; kl < P; ++kl) {
-                                    const float4 tv = __ldg(T4v + kl * (P4 / 4) + q4);
-                                    const float x = sh.qq[t][kl];
-                                    h4.x = fmaf(tv.x, x, h4.x); h4.y = fmaf(tv.y, x, h4.y);
-                                    h4.z = fmaf(tv.z, x, h4.z); h4.w = fmaf(tv.w, x, h4.w);
-                                }
-                            }
-                            const float h3j[4] = {h3.x, h3.y, h3.z, h3.w}, h4j[4] = {h4.x, h4.y, h4.z, h4.w};
+                        for (int i = 0; i < EPL; ++i)
+                            if (g + i * G < P) entry(g + i * G, ea[i], eb[i]);
+                    } else {
 #pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const int e = 4 * q4 + j;
-                                if (e < P) {
-                                    const int a = eq[4 * i + j] & 255, b = eq[4 * i + j] >> 8;
-                                    const Real h = h3j[j] + h4j[j];
-                                    sh.H[t][a][b] = h;
-                                    sh.H[t][b][a] = h;
-                                    const Real gce = fma(Real(0.5), h3j[j], h4j[j] * Real(1.0 / 3.0));
-                                    sh.Gc[t][a][b] = gce;
-                                    sh.Gc[t][b][a] = gce;
-                                    const Real vc = fma(Real(1.0 / 6.0), h3j[j], h4j[j] * Real(1.0 / 12.0));
-                                    vpart = fma(a == b ? vc : Real(2) * vc, sh.qq[t][e], vpart);
-                                }
-                            }
+                        for (int i = 0; i < 4 * NQ; ++i) {
+                            const int e = 4 * (g + (i / 4) * G) + i % 4;
+                            if (e < P) entry(e, eq[i] & 255, eq[i] >> 8);
                         }
                     }
                 } else if constexpr (kTreg || kSplit) {
@@ -1456,11 +1640,11 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
     __syncthreads();   // the caller may restage shared memory next
 }
 
-template <int F, int G, typename Real, int WARPS>
+template <int F, int G, typename Real, int WARPS, int TRAJ_WARPS>
 __global__ void __launch_bounds__(32 * WARPS, lg_min_ctas<F, G, Real>()) k_propagate_lg(const PropLaunch L)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    lg_body<F, G, Real, WARPS>(L, blockIdx.x, smem_raw);
+    lg_body<F, G, Real, WARPS, (F <= 16), TRAJ_WARPS>(L, blockIdx.x, smem_raw);
 }
 
 // Batched persistent kernel: CTAs pull (molecule, tile) work items from a
@@ -1513,13 +1697,15 @@ __global__ void __launch_bounds__(128, 1) k_propagate_lg_multi(const PropLaunch 
 
 }  // namespace lg
 
-template <int F, int G, typename Real, int WARPS, bool STAGED = (F <= 16)>
+template <int F, int G, typename Real, int WARPS, bool STAGED = (F <= 16), int TRAJ_WARPS = WARPS>
 size_t lg_smem_bytes()
 {
     using namespace lg;
-    const size_t tensors = TensorLayout<F, Real, STAGED>::bytes;
+    using TL = TensorLayout<F, Real, STAGED>;
     const size_t consts = (sizeof(CtaConst<F>) + 15) & ~(size_t)15;
-    return tensors + consts + WARPS * sizeof(WarpShared<F, G, Real>);
+    size_t coop = 0;
+    if constexpr (TL::coop) coop = CoopHessian<F, WARPS, TRAJ_WARPS, STAGED>::bytes;
+    return TL::bytes + consts + coop + TRAJ_WARPS * sizeof(WarpShared<F, G, Real>);
 }
 
 template <int F, int G, typename Real, int WARPS>
@@ -1545,19 +1731,19 @@ cudaError_t launch_lg_batch(const PropLaunch *items, const int2 *work, int n_wor
     return cudaGetLastError();
 }
 
-template <int F, int G, typename Real, int WARPS>
+template <int F, int G, typename Real, int WARPS, int TRAJ_WARPS = WARPS>
 cudaError_t launch_lg(const PropLaunch &L, cudaStream_t s)
 {
     using namespace lg;
     constexpr int T = 32 / G;
-    const size_t bytes = lg_smem_bytes<F, G, Real, WARPS>();
-    auto kern = k_propagate_lg<F, G, Real, WARPS>;
+    const size_t bytes = lg_smem_bytes<F, G, Real, WARPS, (F <= 16), TRAJ_WARPS>();
+    auto kern = k_propagate_lg<F, G, Real, WARPS, TRAJ_WARPS>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     // the largest shared-memory carveout, so that as many CTAs fit as the registers allow
     e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e != cudaSuccess) return e;
-    const int64_t per_cta = (int64_t)WARPS * T;
+    const int64_t per_cta = (int64_t)TRAJ_WARPS * T;
     const int64_t blocks = (L.n_traj + per_cta - 1) / per_cta;
     kern<<<(unsigned)blocks, 32 * WARPS, bytes, s>>>(L);
     return cudaGetLastError();
@@ -1570,7 +1756,19 @@ template <int F> constexpr int group_lanes() { return 2 * F <= 8 ? 8 : (2 * F <=
 template <int F> cudaError_t launch_group_mixed(const PropLaunch &L, cudaStream_t s)
 {
     constexpr int G = mixed_group_lanes(F);
-    return launch_lg<F, G, float, lg::lg_warps<F, G>()>(L, s);
+    constexpr int W = lg::lg_warps<F, G>();
+    if constexpr (F > 13) {
+        // few trajectories: two or four per CTA, so that they spread over the SMs and the other
+        // warps share their Hessians (F = 24: 50 steps of 64 trajectories take 3.9 ms two to a CTA,
+        // of 600 4.3 ms four to a CTA, of 1216 5.5 ms eight to a CTA)
+        int dev = 0, n_sm = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        if (L.n_traj <= 2 * (int64_t)n_sm) return launch_lg<F, G, float, W, 2>(L, s);
+        if (L.n_traj <= 4 * (int64_t)n_sm) return launch_lg<F, G, float, W, 4>(L, s);
+    }
+    return launch_lg<F, G, float, W>(L, s);
 }
 
 template <int F>
