@@ -156,7 +156,7 @@ __device__ __forceinline__ ff ff_sub_mul_add_mul(ff a, ff x, ff u, ff y, ff v)
 // the exact FMA residual.
 __device__ __forceinline__ ff ff_recip(ff m)
 {
-    const float y0 = 1.0f / m.hi;
+    const float y0 = __frcp_rn(m.hi);
     float r = fmaf(-m.hi, y0, 1.0f);   // 1 - m.hi y0, exact
     r = fmaf(-m.lo, y0, r);
     return ff_norm(y0, y0 * r);
@@ -209,15 +209,13 @@ __device__ __forceinline__ ff coord_add(ff c, float d)
     return ff_norm(s, e + c.lo);
 }
 
-// Complex double-FP32 numbers as packed pairs: hi = (re.hi, im.hi), lo = (re.lo, im.lo).
-// ff2_sub_mul_add_mul(a, x, u, y, v) = a - x u + y v for real double-FP32 x, y: per part
-// the same operations in the same order as ff_sub_mul_add_mul, each instruction doing the
-// real and the imaginary part at once.
+// Complex double-FP32 numbers as packed pairs: hi = (re.hi, im.hi), lo = (re.lo, im.lo); each
+// instruction does the real and the imaginary part at once.  Differences are multiply-adds by
+// -1 (one rounding, the same result), so that no operand has to be negated first.
 struct ff2 { float2 hi, lo; };
 
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.0f, -1.0f), a); }
 
 __device__ __forceinline__ void ff2_two_sum(float2 a, float2 b, float2 &s, float2 &e)
 {
@@ -226,26 +224,40 @@ __device__ __forceinline__ void ff2_two_sum(float2 a, float2 b, float2 &s, float
     e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
 }
 
-__device__ __forceinline__ ff2 ff2_sub_mul_add_mul(ff2 a, ff x, ff2 u, ff y, ff2 v)
+// A row's multiplier l = lr + i li, spread for the packed update: a - l p has the parts
+// a.re - lr p.re + li p.im and a.im - lr p.im - li p.re, i.e. a - x u + y v with u = (p.re, p.im),
+// v = (p.im, p.re), x = (lr, lr) and y = (li, -li).  Held: x, -x, y and -y in the signs the
+// products need.
+struct ElimRow {
+    float2 xh, nxh, xl, y, ny, nyl;
+    __device__ __forceinline__ ElimRow(ff lr, ff li)
+        : xh(make_float2(lr.hi, lr.hi)), nxh(make_float2(-lr.hi, -lr.hi)), xl(make_float2(lr.lo, lr.lo)),
+          y(make_float2(li.hi, -li.hi)), ny(make_float2(-li.hi, li.hi)), nyl(make_float2(-li.lo, li.lo)) {}
+};
+
+// a - l p for entries stored (re.hi, im.hi, re.lo, im.lo): both products exact to their
+// double-FP32 width (d gathers minus their trailing parts: fma(x, u, -x u rounded) and the cross
+// terms), both sums error-free in their leading words, the result normalised.
+__device__ __forceinline__ float4 elim_update(const float4 &a, const ElimRow &l, const float4 &p)
 {
-    const float2 xh = make_float2(x.hi, x.hi), xl = make_float2(x.lo, x.lo);
-    const float2 yh = make_float2(y.hi, y.hi), yl = make_float2(y.lo, y.lo);
-    const float2 p1 = __fmul2_rn(xh, u.hi);
-    float2 e1 = __ffma2_rn(xh, u.hi, neg2(p1));
-    e1 = __ffma2_rn(xh, u.lo, e1);
-    e1 = __ffma2_rn(xl, u.hi, e1);
-    const float2 p2 = __fmul2_rn(yh, v.hi);
-    float2 e2 = __ffma2_rn(yh, v.hi, neg2(p2));
-    e2 = __ffma2_rn(yh, v.lo, e2);
-    e2 = __ffma2_rn(yl, v.hi, e2);
+    const float2 uh = make_float2(p.x, p.y), ul = make_float2(p.z, p.w);
+    const float2 vh = make_float2(p.y, p.x), vl = make_float2(p.w, p.z);
+    const float2 ah = make_float2(a.x, a.y), al = make_float2(a.z, a.w);
+    const float2 p1 = __fmul2_rn(l.nxh, uh);
+    float2 d = __ffma2_rn(l.xh, uh, p1);
+    const float2 p2 = __fmul2_rn(l.y, vh);
+    const float2 d2 = __ffma2_rn(l.ny, vh, p2);
+    d = __ffma2_rn(l.xh, ul, d);
+    d = __ffma2_rn(l.xl, uh, d);
+    d = __ffma2_rn(l.ny, vl, d);
+    d = __ffma2_rn(l.nyl, vh, d);
     float2 s1, t1, s2, t2;
-    ff2_two_sum(a.hi, neg2(p1), s1, t1);
+    ff2_two_sum(ah, p1, s1, t1);
     ff2_two_sum(s1, p2, s2, t2);
-    const float2 lo = add2(add2(sub2(a.lo, e1), e2), add2(t1, t2));
-    ff2 r;
-    r.hi = add2(s2, lo);
-    r.lo = sub2(lo, sub2(r.hi, s2));
-    return r;
+    const float2 lo = add2(sub2(al, add2(d, d2)), add2(t1, t2));
+    const float2 h = add2(s2, lo);
+    const float2 r = sub2(lo, sub2(h, s2));
+    return make_float4(h.x, h.y, r.x, r.y);
 }
 
 // Per-mode and per-reference-state constants, staged in shared memory so that
@@ -422,7 +434,7 @@ struct TensorLayout {
 // order.  Either way each entry's multiply-adds keep the order they have in a single lane's loop,
 // whatever the tile: the results do not depend on TRAJ.  TT is the smallest tile whose items fit one
 // round of the CTA's lanes.  F = 15, 3001 trajectories x 501 steps: 37.0 -> 27.6 ms; F = 24,
-// 2048 x 200: 79.3 -> 45.8 ms.
+// 2048 x 200: 79.3 -> 45.8 ms (with the prefactor elimination's changes 26.0 and 38.4).
 template <int F, int WARPS, int TRAJ, bool STAGED>
 struct CoopHessian {
     static constexpr int P = F * (F + 1) / 2, P4 = (P + 3) & ~3, Q = P4 / 4;
@@ -481,7 +493,12 @@ struct WarpShared {
     static constexpr int JOBS = T * lg_chunk<F, G, Real>();   // jobs per chunk (phases 2-4)
     static constexpr int S3 = TensorLayout<F, Real>::S3;   // q, zero-padded (also the Gc row stride)
     static constexpr int S4 = TensorLayout<F, Real>::S4;   // pair products q_k q_l, zero-padded
-    static constexpr int SH = vec_len<Real>(F);            // row stride of H (rows read by the whole group)
+    // H, read whole by every column lane with 16-byte broadcasts.  Mixed path: rows of an even
+    // length back to back, so that pairs stay aligned and no load is mostly padding (9 instead of 12
+    // loads at F = 6, 23 instead of 27 at F = 9; at F = 10, one trajectory a warp, 0.9 % slower and
+    // not used); FP64: rows of whole vectors.
+    static constexpr int SH = sizeof(Real) == 4 && F != 10 ? (F + 1) & ~1 : vec_len<Real>(F);
+    static constexpr int HV = vec_len<Real>(F * SH);
     alignas(16) Real qr[T][S3];
     alignas(16) Real qq[T][S4];
     // x = (q, zero pad to an even length, pair products, zero pad) in two halves of KH for the
@@ -493,22 +510,33 @@ struct WarpShared {
     static constexpr bool kHalves = (T == 2) && (sizeof(Real) == 4) && F >= 6 && F <= 9;
     alignas(16) Real xs[T][kHalves ? 2 * KH : 4];
     alignas(16) Real Gc[T][F][S3];          // gradient coefficients, full symmetric matrix (row a read by mode lane a)
-    alignas(16) Real H[T][F][SH];
-    // prefactor matrix per job, job-major rows of AS entries (AS odd): a lane that walks one
-    // row of its job's matrix advances its address by one entry, and lanes of different jobs
-    // at the same entry start in different banks
+    alignas(16) Real Hs[T][HV];
+    __device__ __forceinline__ Real &H(int tr, int a, int b) { return Hs[tr][a * SH + b]; }
+    // Prefactor matrix per job.  Mixed path: LPJ = 32 / JOBS lanes of a job read consecutive rows at
+    // the same column with 16-byte accesses, eight lanes (8 / LPJ jobs) to a wavefront.  The row
+    // stride RS and the jobs' bases spread those eight over the eight 16-byte bank groups: an odd
+    // RS for eight rows of one job, bases 4 apart (mod 8) for two jobs of four rows, 2 apart for four
+    // jobs of two rows -- or, at F = 6, where an odd RS would cost a CTA per SM, 0, 5, 4, 1.  (With
+    // F = 24 entries a row all eight fell into one group; with 81 a job two at F = 9.)  FP64 path: a
+    // lane per job, an odd job stride.
+    static constexpr int LPJ = JOBS >= 32 ? 1 : 32 / JOBS;
+    static constexpr bool kMixed = sizeof(Real) == 4;
+    static constexpr int RS = !kMixed || LPJ == 1 || F == 6 ? F : F | 1;
+    static constexpr int up(int n, int r) { return n % 8 == r ? n : up(n + 1, r); }
     // (at least the det M workspace of 2F rows of 2F + 1 floats per trajectory)
-    static constexpr int AS0 = sizeof(Real) == 4 ? (T * 2 * F * (2 * F + 1) + 4 * JOBS - 1) / (4 * JOBS) : 0;
-    static constexpr int AS1 = AS0 > F * F ? AS0 : F * F;
-    static constexpr int AS = AS1 % 2 ? AS1 : AS1 + 1;
-    typename AEntry<Real>::T A[JOBS][AS];
+    static constexpr int AS0 = kMixed ? (T * 2 * F * (2 * F + 1) + 4 * JOBS - 1) / (4 * JOBS) : 0;
+    static constexpr int AS1 = AS0 > F * RS ? AS0 : F * RS;
+    static constexpr int AS = !kMixed || LPJ == 1 || LPJ >= 8 ? AS1 | 1 : (F == 6 ? 38 : up(AS1, LPJ == 4 ? 4 : 2));
+    static_assert(F != 6 || !kMixed || LPJ == 1 || (LPJ == 2 && AS1 <= 37), "the bases of F = 6");
+    typename AEntry<Real>::T A[JOBS * AS];
+    __device__ static __forceinline__ int a_base(int job) { return F == 6 && kMixed && LPJ == 2 ? 38 * job - (job & 1) : AS * job; }
+    __device__ __forceinline__ typename AEntry<Real>::T &a_at(int job, int row, int col) { return A[a_base(job) + row * RS + col]; }
     // cubic and quartic parts of the Hessian entries (wide mixed groups): in the storage of the
     // step's own prefactor matrix, which is written after the step's last kick
     static constexpr int HP = (P + 3) & ~3;
     static_assert(F <= 9 || 8 * HP <= 16 * F * F, "the Hessian parts fit a job's matrix");
-    __device__ __forceinline__ float *h3_at(int job) { return reinterpret_cast<float *>(&A[job][0]); }
+    __device__ __forceinline__ float *h3_at(int job) { return reinterpret_cast<float *>(&A[a_base(job)]); }
     __device__ __forceinline__ float *h4_at(int job) { return h3_at(job) + HP; }
-    __device__ __forceinline__ typename AEntry<Real>::T &a_at(int job, int e) { return A[job][e]; }
     Real pj[F][JOBS], qj[F][JOBS];         // state per job, for the overlap (job column swizzled); FP32
                                            // in the mixed path, where the overlap is evaluated in FP32
     double Sj[JOBS];                        // action per job
@@ -747,7 +775,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
         // padding entries of the vector rows are read (multiplied by zero or skipped) but never
         // written by the step loop: clear the warp's rows once
         Real *z = &sh.qr[0][0];
-        constexpr int nz = (int)((offsetof(Sh, H) + sizeof(Sh::H) - offsetof(Sh, qr)) / sizeof(Real));
+        constexpr int nz = (int)((offsetof(Sh, Hs) + sizeof(Sh::Hs) - offsetof(Sh, qr)) / sizeof(Real));
         for (int i = ln; i < nz; i += 32) z[i] = Real(0);
         __syncwarp();
     }
@@ -966,8 +994,8 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                     auto entry = [&](int e, int a, int b) {
                         const float h3 = s3[e], h4 = s4[e];
                         const float h = h3 + h4;
-                        sh.H[t][a][b] = h;
-                        sh.H[t][b][a] = h;
+                        sh.H(t, a, b) = h;
+                        sh.H(t, b, a) = h;
                         const float gce = fmaf(0.5f, h3, h4 * (1.0f / 3.0f));
                         sh.Gc[t][a][b] = gce;
                         sh.Gc[t][b][a] = gce;
@@ -1057,8 +1085,8 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                         if (e < P) {
                             const int a = ebA[i], b = ebB[i];
                             const float h = h3 + h4;
-                            sh.H[hx][a][b] = h;
-                            sh.H[hx][b][a] = h;
+                            sh.H(hx, a, b) = h;
+                            sh.H(hx, b, a) = h;
                             const float gce = fmaf(0.5f, h3, h4 * (1.0f / 3.0f));
                             sh.Gc[hx][a][b] = gce;
                             sh.Gc[hx][b][a] = gce;
@@ -1077,8 +1105,8 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                         const int a = ea[i], b = eb[i];
                         // coupling part only: the mode lanes add the diagonal term below
                         const Real h = h3 + h4;
-                        sh.H[t][a][b] = h;
-                        sh.H[t][b][a] = h;
+                        sh.H(t, a, b) = h;
+                        sh.H(t, b, a) = h;
                         const Real gce = fma(Real(0.5), h3, h4 * Real(1.0 / 3.0));
                         sh.Gc[t][a][b] = gce;
                         sh.Gc[t][b][a] = gce;
@@ -1105,7 +1133,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                         gd = w2 * sh.qr[t][g];
                         hd = w2;
                     }
-                    sh.H[t][g][g] += hd;
+                    sh.H(t, g, g) += hd;
                     p = coord_kick(p, tk, A.tkick_f[sub], A.tkick_lo[sub], gr + gd);
                     pr = (Real)coord_f(p);
                     vlane += Vd;
@@ -1116,27 +1144,24 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                 if constexpr (kPacked) {
                     // packed pairs of H's row entries against pairs of the column's entries
                     constexpr int SH = Sh::SH;
+                    float2 acc[NCOL];
 #pragma unroll
-                    for (int a = 0; a < F; ++a) {
-                        float2 acc[NCOL];
+                    for (int v0 = 0; v0 < F * SH; v0 += 4) {
+                        const float4 v = *reinterpret_cast<const float4 *>(&sh.Hs[t][v0]);
 #pragma unroll
-                        for (int s = 0; s < NCOL; ++s) acc[s] = make_float2(0.0f, 0.0f);
-#pragma unroll
-                        for (int b0 = 0; b0 < SH; b0 += 4) {
-                            const float4 v = *reinterpret_cast<const float4 *>(&sh.H[t][a][b0]);
-#pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                const int b = b0 + 2 * h;
+                        for (int h = 0; h < 2; ++h) {
+                            const int a = (v0 + 2 * h) / SH, b = (v0 + 2 * h) % SH;
+                            if (a < F && b < F) {
                                 const float2 hv = h ? hi2(v) : lo2(v);
 #pragma unroll
                                 for (int s = 0; s < NCOL; ++s) {
+                                    if (b == 0) acc[s] = make_float2(0.0f, 0.0f);
                                     if (b + 1 < F) acc[s] = ffma2(hv, make_float2(Mq[s][b], Mq[s][b + 1]), acc[s]);
-                                    else if (b < F) acc[s].x = fmaf(hv.x, Mq[s][b], acc[s].x);
+                                    else acc[s].x = fmaf(hv.x, Mq[s][b], acc[s].x);
+                                    if (b + 2 >= F) Mp[s][a] = fmaf(-rtk, acc[s].x + acc[s].y, Mp[s][a]);
                                 }
                             }
                         }
-#pragma unroll
-                        for (int s = 0; s < NCOL; ++s) Mp[s][a] = fmaf(-rtk, acc[s].x + acc[s].y, Mp[s][a]);
                     }
                 } else {
                     using VT = typename V16<Real>::T;
@@ -1148,7 +1173,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                         for (int s = 0; s < NCOL; ++s) acc[s] = Real(0);
 #pragma unroll
                         for (int b0 = 0; b0 < SH; b0 += NV) {
-                            const VT v = *reinterpret_cast<const VT *>(&sh.H[t][a][b0]);
+                            const VT v = *reinterpret_cast<const VT *>(&sh.H(t, a, b0));
 #pragma unroll
                             for (int j = 0; j < NV; ++j)
                                 if (b0 + j < F) {
@@ -1266,9 +1291,9 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                         v.x = fma(k4[0], mqq, k4[1] * Mp[0][a]);
                         v.y = fma(k4[2], Mq[0][a], k4[3] * mpq);
                         if constexpr (sizeof(Real) == 4)
-                            sh.a_at(job, a * F + g) = make_float4(v.x, v.y, 0.0f, 0.0f);
+                            sh.a_at(job, a, g) = make_float4(v.x, v.y, 0.0f, 0.0f);
                         else
-                            sh.a_at(job, a * F + g) = v;
+                            sh.a_at(job, a, g) = v;
                     }
                 }
                 if (g < F) {
@@ -1309,7 +1334,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
             constexpr int LPJ = 32 / JOBS;
             static_assert(LPJ * JOBS == 32, "jobs must tile the warp");
             const int job = ln / LPJ, r = ln % LPJ;
-            auto at = [&](int e) -> float4 & { return sh.a_at(job, e); };
+            auto at = [&](int row, int col) -> float4 & { return sh.a_at(job, row, col); };
             constexpr int PB = F > 16 ? 5 : 4, PPW = 64 / PB;   // bits per field, fields per word
             constexpr unsigned long long PMASK = (1ull << PB) - 1ull;
             unsigned long long perm0 = 0ull, perm1 = 0ull;
@@ -1325,23 +1350,18 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                 if (pos < PPW) perm0 = (perm0 & ~(PMASK << (PB * pos))) | (v << (PB * pos));
                 else perm1 = (perm1 & ~(PMASK << (PB * (pos - PPW)))) | (v << (PB * (pos - PPW)));
             };
-            // det A, the product of the pivots: double-FP32 (re, im) times 2^dexp, renormalised by
-            // an exact power of two after every factor (the FP32 exponent range alone could overflow)
-            ff dr = {1.0f, 0.0f}, di = {0.0f, 0.0f};
-            int dexp = 0;
+            bool odd = false;   // parity of the exchanges
+            // pivot candidate of the next column among this lane's rows: the largest |a_ik|^2
+            // (leading words), taken here for column 0 and from the updates afterwards
+            float best = -1.0f;
+            int bpos = 0;
+            auto candidate = [&](const float4 &v, int pos) {
+                const float m = fmaf(v.x, v.x, v.y * v.y);
+                if (m > best) { best = m; bpos = pos; }
+            };
+            for (int pos = r; pos < F; pos += LPJ) candidate(at(pos, 0), pos);
 #pragma unroll 1
             for (int k = 0; k < F; ++k) {
-                // pivot: the largest |a_ik|^2 (leading words) over the active rows
-                float best = -1.0f;
-                int bpos = k;
-                for (int s0 = k; s0 < F; s0 += LPJ) {
-                    const int pos = s0 + r;
-                    if (pos < F) {
-                        const float4 v = at(prow(pos) * F + k);
-                        const float m = fmaf(v.x, v.x, v.y * v.y);
-                        if (m > best) { best = m; bpos = pos; }
-                    }
-                }
 #pragma unroll
                 for (int o = 1; o < LPJ; o <<= 1) {
                     const float ob = __shfl_xor_sync(FULL, best, o);
@@ -1352,55 +1372,114 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                     const unsigned long long a = (unsigned long long)prow(k), b = (unsigned long long)prow(bpos);
                     pset(k, b);
                     pset(bpos, a);
-                    dr = {-dr.hi, -dr.lo};
-                    di = {-di.hi, -di.lo};
+                    odd = !odd;
                 }
                 const int pr = prow(k);
-                const float4 pk4 = at(pr * F + k);
+                const float4 pk4 = at(pr, k);
                 const ff pre = {pk4.x, pk4.z}, pim = {pk4.y, pk4.w};
-                {
-                    const ff a1 = ff_mul(dr, pre), a2 = ff_mul(di, pim), b1 = ff_mul(dr, pim), b2 = ff_mul(di, pre);
-                    dr = ff_add(a1, {-a2.hi, -a2.lo});
-                    di = ff_add(b1, b2);
-                    const float m = fmaxf(fabsf(dr.hi), fabsf(di.hi));
-                    const int eb = (__float_as_int(m) >> 23) & 255;   // biased exponent of the larger part
-                    if (eb > 0 && eb < 255) {
-                        const float sc = __int_as_float((254 - eb) << 23);   // 2^(127 - eb): the larger part to [1, 2)
-                        dr.hi *= sc; dr.lo *= sc; di.hi *= sc; di.lo *= sc;
-                        dexp += eb - 127;
-                    }
-                }
                 // 1 / pivot = conj(pivot) / |pivot|^2
                 const ff m2 = ff_add(ff_mul(pre, pre), ff_mul(pim, pim));
                 const ff rm = ff_recip(m2);
                 const ff ir = ff_mul(pre, rm);
                 const ff nii = ff_mul(pim, rm);
                 const ff ii = {-nii.hi, -nii.lo};
-                for (int s0 = k + 1; s0 < F; s0 += LPJ) {
-                    const int pos = s0 + r;
-                    if (pos < F) {
-                        const int row = prow(pos);
-                        const float4 aik = at(row * F + k);
-                        const ff ar = {aik.x, aik.z}, ai = {aik.y, aik.w};
-                        // l = a_ik / pivot
-                        const ff zero = {0.0f, 0.0f};
-                        const ff lr = ff_sub_mul_add_mul(zero, ai, ii, ar, ir);                       // ar ir - ai ii
-                        const ff li = ff_sub_mul_add_mul(zero, {-ar.hi, -ar.lo}, ii, ai, ir);         // ar ii + ai ir
+                // The rows below the pivot go to the job's lanes, or, once there are fewer rows than
+                // lanes, 2^sp lanes to a row, which share its columns.  With eight or more lanes to a
+                // job a lane's two rows are updated together, each pivot-row entry read once for both
+                // (with four, 5 % slower at F = 9).
+                const int m = F - 1 - k;
+                int sp = 0;
+                if constexpr (LPJ >= 4) {
+                    if (m > 0) sp = max(0, (31 - __clz(LPJ)) - (32 - __clz(m - 1)));
+                }
+                const int c0 = k + 1 + (r & ((1 << sp) - 1)), cstep = 1 << sp, rstep = LPJ >> sp;
+                const float4 *prow_p = &at(pr, 0);
+                best = -1.0f;
+                bpos = k + 1;
+                auto multiplier = [&](const float4 *row) {
+                    const float4 aik = row[k];
+                    const ff ar = {aik.x, aik.z}, ai = {aik.y, aik.w};
+                    const ff zero = {0.0f, 0.0f};
+                    const ff lr = ff_sub_mul_add_mul(zero, ai, ii, ar, ir);                       // ar ir - ai ii
+                    const ff li = ff_sub_mul_add_mul(zero, {-ar.hi, -ar.lo}, ii, ai, ir);         // ar ii + ai ir
+                    return ElimRow(lr, li);
+                };
+                if constexpr (LPJ >= 8) {
+                    for (int s0 = k + 1; s0 < F; s0 += 2 * rstep) {
+                        const int p0 = s0 + (r >> sp), p1 = p0 + rstep;
+                        if (s0 + rstep < F) {      // some lane has two rows (uniform over the warp)
+                            const bool on = p1 < F;
+                            float4 *r0 = &at(prow(p0), 0), *r1 = on ? &at(prow(p1), 0) : r0;
+                            const ElimRow l0 = multiplier(r0), l1 = multiplier(r1);
+                            for (int cc = c0; cc < F; cc += cstep) {
+                                const float4 pv = prow_p[cc];
+                                const float4 n0 = elim_update(r0[cc], l0, pv), n1 = elim_update(r1[cc], l1, pv);
+                                if (on) r1[cc] = n1;
+                                r0[cc] = n0;
+                                if (cc == k + 1) {
+                                    candidate(n0, p0);
+                                    if (on) candidate(n1, p1);
+                                }
+                            }
+                        } else if (p0 < F) {
+                            float4 *r0 = &at(prow(p0), 0);
+                            const ElimRow l0 = multiplier(r0);
 #pragma unroll 2
-                        for (int cc = k + 1; cc < F; ++cc) {
-                            const float4 pv = at(pr * F + cc);
-                            float4 &dst = at(row * F + cc);
-                            const float4 av = dst;
-                            // a -= l p: re = a.re - lr pr + li pi, im = a.im - lr pi - li pr, i.e.
-                            // a - lr u + li v with u = p and v = (pi, -pr), both parts packed
-                            const ff2 u = {lo2(pv), hi2(pv)};
-                            const ff2 v = {make_float2(pv.y, -pv.x), make_float2(pv.w, -pv.z)};
-                            const ff2 n = ff2_sub_mul_add_mul({lo2(av), hi2(av)}, lr, u, li, v);
-                            dst = make_float4(n.hi.x, n.hi.y, n.lo.x, n.lo.y);
+                            for (int cc = c0; cc < F; cc += cstep) {
+                                const float4 n0 = elim_update(r0[cc], l0, prow_p[cc]);
+                                r0[cc] = n0;
+                                if (cc == k + 1) candidate(n0, p0);
+                            }
+                        }
+                    }
+                } else {
+                    for (int p0 = k + 1 + (r >> sp); p0 < F; p0 += rstep) {
+                        float4 *r0 = &at(prow(p0), 0);
+                        const ElimRow l0 = multiplier(r0);
+#pragma unroll 2
+                        for (int cc = c0; cc < F; cc += cstep) {
+                            const float4 n0 = elim_update(r0[cc], l0, prow_p[cc]);
+                            r0[cc] = n0;
+                            if (cc == k + 1) candidate(n0, p0);
                         }
                     }
                 }
                 if (LPJ > 1) __syncwarp();   // rows updated by the job's other lanes feed the next pivot
+            }
+            // det A, the product of the pivots (left in place): double-FP32 (re, im) times 2^dexp,
+            // renormalised by an exact power of two after every factor (the FP32 exponent range alone
+            // could overflow); each lane multiplies its positions' pivots, then the lanes' products
+            // meet pairwise
+            ff dr = {1.0f, 0.0f}, di = {0.0f, 0.0f};
+            int dexp = 0;
+            auto factor = [&](ff fr, ff fi) {
+                const ff a1 = ff_mul(dr, fr), a2 = ff_mul(di, fi), b1 = ff_mul(dr, fi), b2 = ff_mul(di, fr);
+                dr = ff_add(a1, {-a2.hi, -a2.lo});
+                di = ff_add(b1, b2);
+                const float mx = fmaxf(fabsf(dr.hi), fabsf(di.hi));
+                const int eb = (__float_as_int(mx) >> 23) & 255;   // biased exponent of the larger part
+                if (eb > 0 && eb < 255) {
+                    const float sc = __int_as_float((254 - eb) << 23);   // 2^(127 - eb): the larger part to [1, 2)
+                    dr.hi *= sc; dr.lo *= sc; di.hi *= sc; di.lo *= sc;
+                    dexp += eb - 127;
+                }
+            };
+#pragma unroll 1
+            for (int k = r; k < F; k += LPJ) {
+                const float4 v = at(prow(k), k);
+                factor({v.x, v.z}, {v.y, v.w});
+            }
+#pragma unroll
+            for (int o = 1; o < LPJ; o <<= 1) {
+                const ff fr = {__shfl_xor_sync(FULL, dr.hi, o), __shfl_xor_sync(FULL, dr.lo, o)};
+                const ff fi = {__shfl_xor_sync(FULL, di.hi, o), __shfl_xor_sync(FULL, di.lo, o)};
+                const int fe = __shfl_xor_sync(FULL, dexp, o);
+                factor(fr, fi);
+                dexp += fe;
+            }
+            if (odd) {
+                dr = {-dr.hi, -dr.lo};
+                di = {-di.hi, -di.lo};
             }
             if (r == 0) {
                 const double mr = (double)dr.hi + (double)dr.lo, mi = (double)di.hi + (double)di.lo;
@@ -1418,7 +1497,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
         } else {
             // FP64 path: in-place elimination in FP64, one lane per job, det A as the product of
             // the pivots (no range concern in FP64)
-            auto at = [&](int e) -> R2 & { return sh.a_at(ln, e); };
+            auto at = [&](int e) -> R2 & { return sh.A[ln * Sh::AS + e]; };
             double dr = 1.0, di = 0.0;
 #pragma unroll
             for (int k = 0; k < F; ++k) {
@@ -1475,7 +1554,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
             // loop keeps the code and registers small
             static_assert(kDetMEvery % C == 0, "det M cadence falls on chunk ends");
             if ((step0 + cnt) % kDetMEvery == 0 || step0 + cnt == A.n_steps) {
-                float (*Wm)[N2 + 1] = reinterpret_cast<float (*)[N2 + 1]>(&sh.A[0][0]) + t * N2;
+                float (*Wm)[N2 + 1] = reinterpret_cast<float (*)[N2 + 1]>(&sh.A[0]) + t * N2;
                 static_assert(sizeof(float) * T * N2 * (N2 + 1) <= sizeof(sh.A), "det M workspace");
 #pragma unroll
                     for (int s = 0; s < NCOL; ++s) {
@@ -1759,8 +1838,8 @@ template <int F> cudaError_t launch_group_mixed(const PropLaunch &L, cudaStream_
     constexpr int W = lg::lg_warps<F, G>();
     if constexpr (F > 13) {
         // few trajectories: two or four per CTA, so that they spread over the SMs and the other
-        // warps share their Hessians (F = 24: 50 steps of 64 trajectories take 3.9 ms two to a CTA,
-        // of 600 4.3 ms four to a CTA, of 1216 5.5 ms eight to a CTA)
+        // warps share their Hessians (F = 24: 50 steps of 64 trajectories take 3.6 ms two to a CTA,
+        // of 600 3.9 ms four to a CTA, of 1216 5.0 ms eight to a CTA)
         int dev = 0, n_sm = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
