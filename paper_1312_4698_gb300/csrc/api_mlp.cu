@@ -123,7 +123,7 @@ int scivr_pes_set_mlp(scivr_pes pes, const scivr_mlp_desc *m)
         if (e == cudaSuccess) e = mlp_prepare();
         if (e == cudaSuccess) e = mlp_tile_weights(w, nullptr);
         if (e == cudaSuccess) e = cudaDeviceSynchronize();
-        count_launches(4);
+        count_launches(1);
         if (e != cudaSuccess) {
             cudaFree(blob);
             return cuda_error(e, "scivr_pes_set_mlp: upload");
@@ -187,7 +187,7 @@ int scivr_mlp_set_params(scivr_pes pes, const float *theta, void *stream)
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cudaError_t e = cudaMemcpyAsync(w.theta, theta, (size_t)w.n_params * 4, cudaMemcpyDeviceToDevice, s);
     if (e == cudaSuccess) e = mlp_tile_weights(w, s);
-    count_launches(4);
+    count_launches(1);
     if (e != cudaSuccess) return cuda_error(e, "scivr_mlp_set_params");
     clear_error();
     return SCIVR_OK;
@@ -232,7 +232,7 @@ int scivr_mlp_adamw(scivr_pes pes, const float *grad, float *m1, float *m2, int3
     const double c1 = 1.0 - std::pow(beta1, t), c2 = 1.0 - std::pow(beta2, t);
     cudaError_t e = mlp_adamw(pes->dev.mlp, grad, m1, m2, (float)lr, (float)beta1, (float)beta2, (float)eps,
                               (float)weight_decay, (float)c1, (float)c2, static_cast<cudaStream_t>(stream));
-    count_launches(5);
+    count_launches(2);
     if (e != cudaSuccess) return cuda_error(e, "scivr_mlp_adamw: launch");
     clear_error();
     return SCIVR_OK;

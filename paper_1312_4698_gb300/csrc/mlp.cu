@@ -702,11 +702,20 @@ __global__ void k_adamw(float *__restrict__ theta, const float *__restrict__ gra
 // The four weight products stream BF16 weight tiles (16 KB k-blocks, 3-stage
 // ring, cp.async.bulk); the two Gram products take FP16 operands written by
 // the compute warps (c J rows into the A tile, the F tangent rows of every
-// point packed as the 12 F x 256 B operand).  Warp roles: warps 0-7 compute
-// (tile row r = TMEM lane r is shared by warps r/32 and r/32 + 4, which take
-// the column halves), warp 8 streams weights, warp 9 issues tcgen05.mma.
+// point packed as the 12 F x 256 B operand).  Warp roles: warps 0-15 compute
+// (tile row r = TMEM lane r is shared by warps r/32 + 4 h, h = 0..3, which take
+// the column quarters), warp 16 streams weights, warp 17 issues tcgen05.mma.
+// The CUDA-core epilogues between the products bound a tile; they wait on TMEM, shared memory
+// and MUFU results, so four compute warps a sub-partition hide some of what two could not.  What
+// the reverse pass needs of z2 and z1 is formed beside the products that do not need it,
+// shared-memory rows are read four words at a time, and the sums over hidden units meet by
+// halving exchanges.  65536 points at F = 9: 1174 us with 8 compute warps, 1112 us with 16,
+// 957 us with the rest.
 constexpr int FU_STAGES = 3;
-constexpr int FU_NC = 256;                        // compute threads
+constexpr int FU_NC = 512;                        // compute threads
+constexpr int FU_CQ = FU_NC / BM;                 // threads a row: column quarters
+constexpr int FU_CH = HW / 32 / FU_CQ;            // 32-column chunks of a thread
+constexpr int FU_THREADS = FU_NC + 64;
 constexpr int FU_SPT = 12;                        // points per tile (F <= 9: 12 (F+1) <= 120 rows)
 constexpr int FU_PS = HW + 4;                     // padded row stride of the per-point buffers
 constexpr int FU_BUF = FU_SPT * FU_PS * 4;
@@ -719,10 +728,11 @@ constexpr int FU_O_G = FU_O_B + FU_STAGES * TILE_B;   // Gram B operand, then th
 constexpr int FU_O_P = FU_O_G + KT_H * FU_GBLK;
 constexpr int FU_O_Q = FU_O_P + FU_BUF;
 constexpr int FU_O_ZB = FU_O_Q + FU_BUF;
-constexpr int FU_O_W1 = FU_O_ZB + FU_BUF;             // W1 [256][F]
-constexpr int FU_O_PAR = FU_O_W1 + HW * kMaxF * 4;    // b1, b2, b3, w4 [256] each; s_in [16]; one
-constexpr int FU_O_XQ = FU_O_PAR + (4 * HW + 32) * 4; // x = s_in q [12][F]
-constexpr int FU_O_Y = FU_O_XQ + FU_SPT * kMaxF * 4;  // y per point
+constexpr int FU_O_W1 = FU_O_ZB + FU_BUF;             // W1 transposed [F][FU_PS]
+constexpr int FU_O_PAR = FU_O_W1 + kMaxF * FU_PS * 4; // b1, b2, b3, w4 [256] each; s_in [16]; ones [32]
+constexpr int FU_O_XQ = FU_O_PAR + (4 * HW + 48) * 4; // x = s_in q [12][FU_XS], zero-padded
+constexpr int FU_XS = 12;
+constexpr int FU_O_Y = FU_O_XQ + FU_SPT * FU_XS * 4;  // y per point
 constexpr int FU_SMEM = FU_O_Y + FU_SPT * 4;
 static_assert(FU_SMEM + 1024 <= 227 * 1024, "fused evaluation exceeds shared memory");
 static_assert(BM * FU_SCS * 4 <= KT_H * FU_GBLK, "Gram read-out scratch exceeds its region");
@@ -742,7 +752,8 @@ constexpr uint32_t idesc_f16(int M, int N)
     return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void named_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void named_sync() { asm volatile("bar.sync 1, 512;" ::: "memory"); }
+static_assert(FU_NC == 512, "the named barrier counts the compute threads");
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 {
@@ -787,25 +798,44 @@ __device__ __forceinline__ void put_f32x32(float *dst, const float (&v)[32])
     for (int i = 0; i < 32; i += 4) *reinterpret_cast<float4 *>(dst + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
 }
 
+__device__ __forceinline__ void get_f32x32(const float *src, float (&v)[32])
+{
+#pragma unroll
+    for (int i = 0; i < 32; i += 4) {
+        const float4 a = *reinterpret_cast<const float4 *>(src + i);
+        v[i] = a.x; v[i + 1] = a.y; v[i + 2] = a.z; v[i + 3] = a.w;
+    }
+}
+
+__device__ __forceinline__ void mul_f32x32(const float *p, const float *q, float (&v)[32])
+{
+#pragma unroll
+    for (int i = 0; i < 32; i += 4) {
+        const float4 a = *reinterpret_cast<const float4 *>(p + i), b = *reinterpret_cast<const float4 *>(q + i);
+        v[i] = a.x * b.x; v[i + 1] = a.y * b.y; v[i + 2] = a.z * b.z; v[i + 3] = a.w * b.w;
+    }
+}
+
 template <int F>
-__global__ void __launch_bounds__(320, 1)
+__global__ void __launch_bounds__(FU_THREADS, 1)
     k_mlp_fused(MlpDev m, int64_t n, int n_tiles, const float *__restrict__ q, float *__restrict__ Vout,
                 float *__restrict__ gout, float *__restrict__ Hout)
 {
     using C = FuCfg<F>;
     constexpr int R = C::R, NE = C::NE, NJ = C::NJ, NG = C::NG, SPT = FU_SPT, PS = FU_PS;
+    constexpr int NP = SPT * HW / 2 / FU_NC;   // pairs of hidden units per compute thread
     extern __shared__ __align__(128) uint8_t smem_raw[];
     uint8_t *sm = smem_raw;
     uint8_t *sA = sm + FU_O_A;
     uint8_t *sB = sm + FU_O_B;
     uint8_t *sG = sm + FU_O_G;
     float *sc = reinterpret_cast<float *>(sm + FU_O_G);      // Gram read-out scratch [128][FU_SCS]
-    float *pb = reinterpret_cast<float *>(sm + FU_O_P);      // silu'(z1), silu'(z2), abar2, abar1 -> d1
-    float *qb = reinterpret_cast<float *>(sm + FU_O_Q);      // c3, c2, c1, then the layer-1 Hessian terms
-    float *zb = reinterpret_cast<float *>(sm + FU_O_ZB);     // value-row staging: a1, a2, delta3, delta2
-    float *w1s = reinterpret_cast<float *>(sm + FU_O_W1);
+    float *pb = reinterpret_cast<float *>(sm + FU_O_P);      // silu'(z1), silu'(z2), abar2, abar1
+    float *qb = reinterpret_cast<float *>(sm + FU_O_Q);      // c3, silu''(z2), silu''(z1)
+    float *zb = reinterpret_cast<float *>(sm + FU_O_ZB);     // value rows: a1, a2, delta3; silu'(z2), silu'(z1); sums
+    float *w1t = reinterpret_cast<float *>(sm + FU_O_W1);
     float *b1s = reinterpret_cast<float *>(sm + FU_O_PAR);
-    float *b2s = b1s + HW, *b3s = b2s + HW, *w4s = b3s + HW, *sins = w4s + HW, *one = sins + 16;
+    float *b2s = b1s + HW, *b3s = b2s + HW, *w4s = b3s + HW, *sins = w4s + HW, *ones = sins + 16;
     float *xq = reinterpret_cast<float *>(sm + FU_O_XQ);
     float *ys = reinterpret_cast<float *>(sm + FU_O_Y);
     __shared__ uint64_t full_bar[FU_STAGES], empty_bar[FU_STAGES], a_bar, c_bar;
@@ -819,7 +849,7 @@ __global__ void __launch_bounds__(320, 1)
         abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    for (int i = threadIdx.x; i < HW * F; i += blockDim.x) w1s[i] = m.W1[i];
+    for (int i = threadIdx.x; i < HW * F; i += blockDim.x) w1t[(i % F) * FU_PS + i / F] = m.W1[i];
     for (int i = threadIdx.x; i < HW; i += blockDim.x) {
         b1s[i] = m.b1[i];
         b2s[i] = m.b2[i];
@@ -827,7 +857,8 @@ __global__ void __launch_bounds__(320, 1)
         w4s[i] = m.w4[i];
     }
     if (threadIdx.x < 16) sins[threadIdx.x] = threadIdx.x < F ? m.s_in[threadIdx.x] : 0.0f;
-    if (threadIdx.x == 0) one[0] = 1.0f;
+    if (threadIdx.x < 32) ones[threadIdx.x] = 1.0f;
+    if (threadIdx.x < FU_SPT * FU_XS) xq[threadIdx.x] = 0.0f;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tmem_slot)),
                      "r"(512) : "memory");
@@ -838,7 +869,7 @@ __global__ void __launch_bounds__(320, 1)
     tc_fence_after();
     const uint32_t tmem = tmem_slot;
 
-    if (warp == 8) {
+    if (warp == FU_NC / 32) {
         // ---------------- weight producer: per tile W2, W3 (forward), W3^T, W2^T (reverse)
         if (lane == 0) {
             int kc = 0;
@@ -862,7 +893,7 @@ __global__ void __launch_bounds__(320, 1)
             for (int k = kc - FU_STAGES > 0 ? kc - FU_STAGES : 0; k < kc; ++k)
                 mbar_wait(&full_bar[k % FU_STAGES], (k / FU_STAGES) & 1, kWaitLimitCycles);
         }
-    } else if (warp == 9) {
+    } else if (warp == FU_NC / 32 + 1) {
         // ---------------- MMA issuer: per tile weight, weight, Gram, weight, Gram, weight
         if (lane == 0) {
             constexpr uint32_t idesc_w = idesc_bf16(BM, BN);
@@ -909,13 +940,13 @@ __global__ void __launch_bounds__(320, 1)
         }
     } else {
         // ---------------- compute warps
-        const int c = threadIdx.x;            // 0..255
-        const int hf = warp >> 2;             // column half
+        const int c = threadIdx.x;            // 0..511
+        const int hf = warp >> 2;             // column quarter
         const int qd = warp & 3;              // TMEM lane quadrant
         const int r = qd * 32 + lane;         // tile row = TMEM lane
         const int sr = r / R, kr = r % R;     // point of the row; 0 = value row, k = direction k - 1
         const uint32_t lane_base = tmem + ((uint32_t)(qd * 32) << 16);
-        const uint32_t col_half = hf * 128;
+        const uint32_t col_q = hf * (32 * FU_CH);
         // Gram read-out window of quadrant qq: 64 columns from gwin(qq) cover the blocks of
         // every point with a row in it (checked for F = 1..9)
         auto gwin = [](int qq) { return ((qq * 32) / R * F) / 32 * 32; };
@@ -948,7 +979,7 @@ __global__ void __launch_bounds__(320, 1)
 
             // the read-out of a Gram product (TMEM[256:256+NG)) into hacc, symmetrised
             auto gram_readout = [&]() {
-                if (hf == 0) {   // warp-uniform: the first column half reads, the second waits
+                if (hf == 0) {   // warp-uniform: the first column quarter reads, the others wait
                     float va[32], vb[32];
                     tmem_ld32(lane_base + 256 + gbase, va);
                     tmem_ld32(lane_base + 256 + gbase + 32, vb);
@@ -977,35 +1008,49 @@ __global__ void __launch_bounds__(320, 1)
             if (c < SPT * F) {
                 const int s = c / F, k = c % F;
                 const int64_t b = p0 + s;
-                xq[c] = b < n ? sins[k] * q[b * F + k] : 0.0f;
+                xq[s * FU_XS + k] = b < n ? sins[k] * q[b * F + k] : 0.0f;
             }
             if (c < SPT) ys[c] = *m.b4;
             named_sync();
-#pragma unroll 3
-            for (int idx = c; idx < SPT * HW; idx += FU_NC) {
-                const int s = idx >> 8, o = idx & (HW - 1);
-                float z = b1s[o];
+            // z1 of units o, o + 1 of point s
+            auto layer1 = [&](int s, int o) -> float2 {
+                float x[FU_XS];
 #pragma unroll
-                for (int k = 0; k < F; ++k) z = fmaf(w1s[o * F + k], xq[s * F + k], z);
-                float f, f1, f2;
-                silu3f(z, f, f1, f2);
-                zb[s * PS + o] = f;
-                pb[s * PS + o] = f1;
+                for (int k = 0; k < FU_XS; k += 4) {
+                    const float4 v = *reinterpret_cast<const float4 *>(xq + s * FU_XS + k);
+                    x[k] = v.x; x[k + 1] = v.y; x[k + 2] = v.z; x[k + 3] = v.w;
+                }
+                float2 z = *reinterpret_cast<const float2 *>(b1s + o);
+#pragma unroll
+                for (int k = 0; k < F; ++k) {
+                    const float2 w = *reinterpret_cast<const float2 *>(w1t + k * PS + o);
+                    z.x = fmaf(w.x, x[k], z.x);
+                    z.y = fmaf(w.y, x[k], z.y);
+                }
+                return z;
+            };
+#pragma unroll
+            for (int it = 0; it < NP; ++it) {
+                const int idx = c + it * FU_NC, s = idx >> 7, o = 2 * (idx & 127);
+                const float2 z = layer1(s, o);
+                float2 f, f1;
+                float f2;
+                silu3f(z.x, f.x, f1.x, f2);
+                silu3f(z.y, f.y, f1.y, f2);
+                *reinterpret_cast<float2 *>(zb + s * PS + o) = f;
+                *reinterpret_cast<float2 *>(pb + s * PS + o) = f1;
             }
             named_sync();
             {
                 const float *src = (prim ? zb : pb) + rowp;
-                const float *fac = tang ? w1s + d : one;
-                const int fst = tang ? F : 0;
 #pragma unroll 1
-                for (int j = 0; j < 4; ++j) {
-                    const int ch = hf * 4 + j;
-                    float v[32];
+                for (int j = 0; j < FU_CH; ++j) {
+                    const int ch = hf * FU_CH + j;
+                    float v[32], w[32];
+                    get_f32x32(src + ch * 32, v);
+                    get_f32x32(tang ? w1t + d * PS + ch * 32 : ones, w);
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) {
-                        const int o = ch * 32 + i;
-                        v[i] = sv * src[o] * fac[o * fst];
-                    }
+                    for (int i = 0; i < 32; ++i) v[i] = sv * v[i] * w[i];
                     put_row32<false>(sA, TILE_A, r, ch, v);
                 }
             }
@@ -1014,41 +1059,38 @@ __global__ void __launch_bounds__(320, 1)
             // ---- layer 2: TMEM[0:256) holds z2 - b2 (value rows) and J2 (tangent rows)
             if (!wait_acc()) break;
 #pragma unroll 1
-            for (int j = 0; j < 4; j += 2) {
-                float v[32], u[32];
-                tmem_ld32(lane_base + col_half + j * 32, v);
-                tmem_ld32(lane_base + col_half + (j + 1) * 32, u);
+            for (int j = 0; j < FU_CH; ++j) {
+                float v[32];
+                tmem_ld32(lane_base + col_q + j * 32, v);
                 tmem_wait_ld();
-                if (prim) {
-                    put_f32x32(zb + rowp + (hf * 4 + j) * 32, v);
-                    put_f32x32(zb + rowp + (hf * 4 + j + 1) * 32, u);
-                }
+                if (prim) put_f32x32(zb + rowp + (hf * FU_CH + j) * 32, v);
             }
             named_sync();
-#pragma unroll 3
-            for (int idx = c; idx < SPT * HW; idx += FU_NC) {
-                const int s = idx >> 8, o = idx & (HW - 1);
-                float f, f1, f2;
-                silu3f(zb[s * PS + o] + b2s[o], f, f1, f2);
-                zb[s * PS + o] = f;
-                pb[s * PS + o] = f1;
+#pragma unroll
+            for (int it = 0; it < NP; ++it) {
+                const int idx = c + it * FU_NC, s = idx >> 7, o = 2 * (idx & 127);
+                const float2 z = *reinterpret_cast<const float2 *>(zb + s * PS + o);
+                const float2 b2 = *reinterpret_cast<const float2 *>(b2s + o);
+                float2 f, f1;
+                float f2;
+                silu3f(z.x + b2.x, f.x, f1.x, f2);
+                silu3f(z.y + b2.y, f.y, f1.y, f2);
+                *reinterpret_cast<float2 *>(zb + s * PS + o) = f;
+                *reinterpret_cast<float2 *>(pb + s * PS + o) = f1;
             }
             named_sync();
             {
                 const float *src = (prim ? zb : pb) + rowp;
 #pragma unroll 1
-                for (int j = 0; j < 4; j += 2) {
-                    float v[32], u[32];
-                    tmem_ld32(lane_base + col_half + j * 32, v);
-                    tmem_ld32(lane_base + col_half + (j + 1) * 32, u);
+                for (int j = 0; j < FU_CH; ++j) {
+                    const int ch = hf * FU_CH + j;
+                    float v[32], w[32];
+                    tmem_ld32(lane_base + col_q + j * 32, v);
+                    get_f32x32(src + ch * 32, w);
                     tmem_wait_ld();
-                    const int ch = hf * 4 + j;
 #pragma unroll
-                    for (int i = 0; i < 32; ++i) v[i] = sv * src[ch * 32 + i] * fmaf(pv, 1.0f - v[i], v[i]);
+                    for (int i = 0; i < 32; ++i) v[i] = sv * w[i] * fmaf(pv, 1.0f - v[i], v[i]);
                     put_row32<false>(sA, TILE_A, r, ch, v);
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) u[i] = sv * src[ch * 32 + 32 + i] * fmaf(pv, 1.0f - u[i], u[i]);
-                    put_row32<false>(sA, TILE_A, r, ch + 1, u);
                 }
             }
             release_a();
@@ -1056,26 +1098,25 @@ __global__ void __launch_bounds__(320, 1)
             // ---- layer 3: TMEM[256:512) holds z3 - b3 and J3; V, delta3, c3 and the Gram operands
             if (!wait_acc()) break;
 #pragma unroll 1
-            for (int j = 0; j < 4; j += 2) {
-                float v[32], u[32];
-                tmem_ld32(lane_base + 256 + col_half + j * 32, v);
-                tmem_ld32(lane_base + 256 + col_half + (j + 1) * 32, u);
+            for (int j = 0; j < FU_CH; ++j) {
+                float v[32];
+                tmem_ld32(lane_base + 256 + col_q + j * 32, v);
                 tmem_wait_ld();
-                if (prim) {
-                    put_f32x32(zb + rowp + (hf * 4 + j) * 32, v);
-                    put_f32x32(zb + rowp + (hf * 4 + j + 1) * 32, u);
-                }
+                if (prim) put_f32x32(zb + rowp + (hf * FU_CH + j) * 32, v);
             }
             named_sync();
-#pragma unroll 3
-            for (int idx = c; idx < SPT * HW; idx += FU_NC) {   // the 256 entries of one pass share a point
-                const int s = idx >> 8, o = idx & (HW - 1);
-                float f, f1, f2;
-                silu3f(zb[s * PS + o] + b3s[o], f, f1, f2);
-                const float w4 = w4s[o];
-                zb[s * PS + o] = w4 * f1;        // delta3
-                qb[s * PS + o] = w4 * f2;        // c3
-                float y = w4 * f;
+#pragma unroll
+            for (int it = 0; it < NP; ++it) {   // a warp's 64 units share a point
+                const int idx = c + it * FU_NC, s = idx >> 7, o = 2 * (idx & 127);
+                const float2 z = *reinterpret_cast<const float2 *>(zb + s * PS + o);
+                const float2 b3 = *reinterpret_cast<const float2 *>(b3s + o);
+                const float2 w4 = *reinterpret_cast<const float2 *>(w4s + o);
+                float2 f, f1, f2;
+                silu3f(z.x + b3.x, f.x, f1.x, f2.x);
+                silu3f(z.y + b3.y, f.y, f1.y, f2.y);
+                *reinterpret_cast<float2 *>(zb + s * PS + o) = make_float2(w4.x * f1.x, w4.y * f1.y);   // delta3
+                *reinterpret_cast<float2 *>(qb + s * PS + o) = make_float2(w4.x * f2.x, w4.y * f2.y);   // c3
+                float y = fmaf(w4.x, f.x, w4.y * f.y);
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) y += __shfl_xor_sync(0xffffffffu, y, off);
                 if (lane == 0) atomicAdd(&ys[s], y);
@@ -1083,13 +1124,14 @@ __global__ void __launch_bounds__(320, 1)
             named_sync();
             if (prim && hf == 0) Vout[p0 + sr] = m.s_out * ys[sr];
 #pragma unroll 1
-            for (int j = 0; j < 4; ++j) {                     // Gram operands: c3 J3 (A), J3 (B, tangent rows)
-                const int ch = hf * 4 + j;
+            for (int j = 0; j < FU_CH; ++j) {                     // Gram operands: c3 J3 (A), J3 (B, tangent rows)
+                const int ch = hf * FU_CH + j;
                 float v[32], w[32];
-                tmem_ld32(lane_base + 256 + col_half + j * 32, v);
+                tmem_ld32(lane_base + 256 + col_q + j * 32, v);
+                get_f32x32(qb + rowp + ch * 32, w);
                 tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 32; ++i) w[i] = tv * qb[rowp + ch * 32 + i] * v[i];
+                for (int i = 0; i < 32; ++i) w[i] = tv * w[i] * v[i];
                 put_row32<true>(sA, TILE_A, r, ch, w);
                 if (tang) put_row32<true>(sG, FU_GBLK, gb, ch, v);
             }
@@ -1097,47 +1139,57 @@ __global__ void __launch_bounds__(320, 1)
             if (!wait_acc()) break;                           // Gram product of layer 3 done
             gram_readout();
 #pragma unroll 1
-            for (int j = 0; j < 4; ++j) {                     // delta3 rows
-                const int ch = hf * 4 + j;
+            for (int j = 0; j < FU_CH; ++j) {                     // delta3 rows
+                const int ch = hf * FU_CH + j;
                 float x[32];
+                get_f32x32(zb + rowp + ch * 32, x);
 #pragma unroll
-                for (int i = 0; i < 32; ++i) x[i] = pv * zb[rowp + ch * 32 + i];
+                for (int i = 0; i < 32; ++i) x[i] = pv * x[i];
                 put_row32<false>(sA, TILE_A, r, ch, x);
             }
             release_a();
 
-            // ---- reverse through layer 3: TMEM[256:512) = abar2 (value rows); TMEM[0:256) = z2 - b2, J2
+            // ---- reverse through layer 3: TMEM[256:512) = abar2 (value rows); TMEM[0:256) = z2 - b2, J2.
+            // Beside the product: silu'(z2) into zb, silu''(z2) into qb
+            named_sync();                                     // delta3 has been read
+#pragma unroll 1
+            for (int j = 0; j < FU_CH; ++j) {
+                float u[32];
+                tmem_ld32(lane_base + col_q + j * 32, u);
+                tmem_wait_ld();
+                if (prim) put_f32x32(zb + rowp + (hf * FU_CH + j) * 32, u);
+            }
+            named_sync();
+#pragma unroll
+            for (int it = 0; it < NP; ++it) {
+                const int idx = c + it * FU_NC, s = idx >> 7, o = 2 * (idx & 127);
+                const float2 z = *reinterpret_cast<const float2 *>(zb + s * PS + o);
+                const float2 b2 = *reinterpret_cast<const float2 *>(b2s + o);
+                float f;
+                float2 f1, f2;
+                silu3f(z.x + b2.x, f, f1.x, f2.x);
+                silu3f(z.y + b2.y, f, f1.y, f2.y);
+                *reinterpret_cast<float2 *>(zb + s * PS + o) = f1;
+                *reinterpret_cast<float2 *>(qb + s * PS + o) = f2;
+            }
             if (!wait_acc()) break;
 #pragma unroll 1
-            for (int j = 0; j < 4; ++j) {
-                float v[32], u[32];
-                tmem_ld32(lane_base + 256 + col_half + j * 32, v);
-                tmem_ld32(lane_base + col_half + j * 32, u);
+            for (int j = 0; j < FU_CH; ++j) {
+                float v[32];
+                tmem_ld32(lane_base + 256 + col_q + j * 32, v);
                 tmem_wait_ld();
-                if (prim) {
-                    put_f32x32(pb + rowp + (hf * 4 + j) * 32, v);
-                    put_f32x32(zb + rowp + (hf * 4 + j) * 32, u);
-                }
-            }
-            named_sync();
-#pragma unroll 3
-            for (int idx = c; idx < SPT * HW; idx += FU_NC) {
-                const int s = idx >> 8, o = idx & (HW - 1);
-                float f, f1, f2;
-                silu3f(zb[s * PS + o] + b2s[o], f, f1, f2);
-                const float ab = pb[s * PS + o];
-                zb[s * PS + o] = ab * f1;        // delta2 = abar2 silu'(z2)
-                qb[s * PS + o] = ab * f2;        // c2 = abar2 silu''(z2)
+                if (prim) put_f32x32(pb + rowp + (hf * FU_CH + j) * 32, v);
             }
             named_sync();
 #pragma unroll 1
-            for (int j = 0; j < 4; ++j) {                     // Gram operands: c2 J2 (A), J2 (B)
-                const int ch = hf * 4 + j;
+            for (int j = 0; j < FU_CH; ++j) {                     // Gram operands: c2 J2 (A), J2 (B), c2 = abar2 silu''(z2)
+                const int ch = hf * FU_CH + j;
                 float v[32], w[32];
-                tmem_ld32(lane_base + col_half + j * 32, v);
+                tmem_ld32(lane_base + col_q + j * 32, v);
+                mul_f32x32(pb + rowp + ch * 32, qb + rowp + ch * 32, w);
                 tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 32; ++i) w[i] = tv * qb[rowp + ch * 32 + i] * v[i];
+                for (int i = 0; i < 32; ++i) w[i] = tv * w[i] * v[i];
                 put_row32<true>(sA, TILE_A, r, ch, w);
                 if (tang) put_row32<true>(sG, FU_GBLK, gb, ch, v);
             }
@@ -1145,86 +1197,90 @@ __global__ void __launch_bounds__(320, 1)
             if (!wait_acc()) break;                           // Gram product of layer 2 done
             gram_readout();
 #pragma unroll 1
-            for (int j = 0; j < 4; ++j) {                     // delta2 rows
-                const int ch = hf * 4 + j;
+            for (int j = 0; j < FU_CH; ++j) {                     // delta2 rows, delta2 = abar2 silu'(z2)
+                const int ch = hf * FU_CH + j;
                 float x[32];
+                mul_f32x32(pb + rowp + ch * 32, zb + rowp + ch * 32, x);
 #pragma unroll
-                for (int i = 0; i < 32; ++i) x[i] = pv * zb[rowp + ch * 32 + i];
+                for (int i = 0; i < 32; ++i) x[i] = pv * x[i];
                 put_row32<false>(sA, TILE_A, r, ch, x);
             }
             release_a();
 
-            // ---- reverse through layer 2: TMEM[256:512) = abar1; grad V and the layer-1 term
+            // ---- reverse through layer 2: TMEM[256:512) = abar1; grad V and the layer-1 term.
+            // Beside the product: silu'(z1) into zb, silu''(z1) into qb
+            named_sync();                                     // delta2 and c2 have been read
+#pragma unroll
+            for (int it = 0; it < NP; ++it) {
+                const int idx = c + it * FU_NC, s = idx >> 7, o = 2 * (idx & 127);
+                const float2 z = layer1(s, o);
+                float f;
+                float2 f1, f2;
+                silu3f(z.x, f, f1.x, f2.x);
+                silu3f(z.y, f, f1.y, f2.y);
+                *reinterpret_cast<float2 *>(zb + s * PS + o) = f1;
+                *reinterpret_cast<float2 *>(qb + s * PS + o) = f2;
+            }
             if (!wait_acc()) break;
 #pragma unroll 1
-            for (int j = 0; j < 4; j += 2) {
-                float v[32], u[32];
-                tmem_ld32(lane_base + 256 + col_half + j * 32, v);
-                tmem_ld32(lane_base + 256 + col_half + (j + 1) * 32, u);
+            for (int j = 0; j < FU_CH; ++j) {
+                float v[32];
+                tmem_ld32(lane_base + 256 + col_q + j * 32, v);
                 tmem_wait_ld();
-                if (prim) {
-                    put_f32x32(pb + rowp + (hf * 4 + j) * 32, v);
-                    put_f32x32(pb + rowp + (hf * 4 + j + 1) * 32, u);
-                }
+                if (prim) put_f32x32(pb + rowp + (hf * FU_CH + j) * 32, v);
             }
             tc_fence_before();
             named_sync();
-#pragma unroll 3
-            for (int idx = c; idx < SPT * HW; idx += FU_NC) {
-                const int s = idx >> 8, o = idx & (HW - 1);
-                float z = b1s[o];
+            // grad V = W1^T d1 and H1 = W1^T diag(c1) W1, d1 = abar1 silu'(z1), c1 = abar1 silu''(z1): warp
+            // s sums point s, a lane 8 hidden units; the lanes' sums are added by halving exchanges (a
+            // lane keeps one half of its values and sends the other), the last two levels in full
+            if (warp < SPT) {
+                const int s = warp;
+                constexpr int NV = (F + NE + 7) / 8 * 8;
+                float a[NV];
 #pragma unroll
-                for (int k = 0; k < F; ++k) z = fmaf(w1s[o * F + k], xq[s * F + k], z);
-                float f, f1, f2;
-                silu3f(z, f, f1, f2);
-                const float ab = pb[s * PS + o];
-                pb[s * PS + o] = ab * f1;        // d1 = abar1 silu'(z1)
-                qb[s * PS + o] = ab * f2;        // c1 = abar1 silu''(z1)
-            }
-            named_sync();
-            // grad V and H1 = W1^T diag(c1) W1: thread (point s, slice sl) sums 16 hidden units,
-            // then the 16 slices of a point (adjacent lanes) are added by shuffles
-            if (c < SPT * 16) {
-                const int s = c >> 4, sl = c & 15;
-                float ga[F], ha[NE];
-#pragma unroll
-                for (int k = 0; k < F; ++k) ga[k] = 0.0f;
-#pragma unroll
-                for (int e = 0; e < NE; ++e) ha[e] = 0.0f;
+                for (int i = 0; i < NV; ++i) a[i] = 0.0f;
 #pragma unroll 1
-                for (int oo = 0; oo < 16; ++oo) {
-                    const int o = sl * 16 + ((oo + sl) & 15);   // staggered start: fewer bank conflicts
-                    const float d1 = pb[s * PS + o], c1 = qb[s * PS + o];
+                for (int oo = 0; oo < HW / 32; ++oo) {
+                    const int o = oo * 32 + lane;
+                    const float ab = pb[s * PS + o], d1 = ab * zb[s * PS + o], c1 = ab * qb[s * PS + o];
                     float wk[F];
 #pragma unroll
-                    for (int k = 0; k < F; ++k) wk[k] = w1s[o * F + k];
-                    int e = 0;
+                    for (int k = 0; k < F; ++k) wk[k] = w1t[k * PS + o];
+                    int e = F;
 #pragma unroll
                     for (int k1 = 0; k1 < F; ++k1) {
-                        ga[k1] = fmaf(d1, wk[k1], ga[k1]);
+                        a[k1] = fmaf(d1, wk[k1], a[k1]);
                         const float cw = c1 * wk[k1];
 #pragma unroll
-                        for (int k2 = k1; k2 < F; ++k2, ++e) ha[e] = fmaf(cw, wk[k2], ha[e]);
+                        for (int k2 = k1; k2 < F; ++k2, ++e) a[e] = fmaf(cw, wk[k2], a[e]);
                     }
                 }
+                int base = 0;
 #pragma unroll
-                for (int off = 1; off < 16; off <<= 1) {
+                for (int lev = 0; lev < 3; ++lev) {
+                    const int half = NV >> (lev + 1), bit = 16 >> lev;
+                    const bool up = lane & bit;
 #pragma unroll
-                    for (int k = 0; k < F; ++k) ga[k] += __shfl_xor_sync(0xffffffffu, ga[k], off);
-#pragma unroll
-                    for (int e = 0; e < NE; ++e) ha[e] += __shfl_xor_sync(0xffffffffu, ha[e], off);
+                    for (int i = 0; i < half; ++i) {
+                        const float give = up ? a[i] : a[half + i], keep = up ? a[half + i] : a[i];
+                        a[i] = keep + __shfl_xor_sync(0xffffffffu, give, bit);
+                    }
+                    base += up ? half : 0;
                 }
-                const int64_t b = p0 + s;
-                if (sl == 0 && b < n) {
 #pragma unroll
-                    for (int k = 0; k < F; ++k) gout[b * F + k] = m.s_out * sins[k] * ga[k];
+                for (int i = 0; i < NV / 8; ++i) {
+                    a[i] += __shfl_xor_sync(0xffffffffu, a[i], 2);
+                    a[i] += __shfl_xor_sync(0xffffffffu, a[i], 1);
                 }
-                if (sl == 0) {
+                __syncwarp();   // the point's rows have been read
+                if ((lane & 3) == 0) {
 #pragma unroll
-                    for (int e = 0; e < NE; ++e) zb[s * PS + e] = ha[e];
+                    for (int i = 0; i < NV / 8; ++i) zb[s * PS + base + i] = a[i];
                 }
             }
             named_sync();
+            if (c < SPT * F && p0 + c / F < n) gout[p0 * F + c] = m.s_out * sins[c % F] * zb[c / F * PS + c % F];
             if (tang && hf == 0) {
                 const int64_t b = p0 + sr;
 #pragma unroll
@@ -1234,7 +1290,7 @@ __global__ void __launch_bounds__(320, 1)
                     if ((F % 2 == 0) && j == F / 2 && d >= F / 2) continue;   // pair already taken
                     const int lo = d < k ? d : k, hi = d < k ? k : d;
                     const int e = lo * F - lo * (lo - 1) / 2 + (hi - lo);
-                    const float h = m.s_out * sins[d] * sins[k] * (hacc[j] + zb[rowp + e]);
+                    const float h = m.s_out * sins[d] * sins[k] * (hacc[j] + zb[rowp + F + e]);
                     Hout[(b * F + d) * F + k] = h;
                     Hout[(b * F + k) * F + d] = h;
                 }
@@ -1401,7 +1457,7 @@ cudaError_t eval_fused_F(const MlpWeightsDev &w, int64_t n, const float *q, floa
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int grid = (int)(n_tiles < n_sm ? n_tiles : n_sm);
-    k_mlp_fused<F><<<grid, 320, FU_SMEM, s>>>(m, n, (int)n_tiles, q, V, g, H);
+    k_mlp_fused<F><<<grid, FU_THREADS, FU_SMEM, s>>>(m, n, (int)n_tiles, q, V, g, H);
     *n_launch = 1;
     return cudaGetLastError();
 }
