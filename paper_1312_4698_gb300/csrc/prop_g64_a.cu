@@ -1,0 +1,11 @@
+// Instantiations of the FP64 lane-group propagation kernel (split for parallel builds).
+#include "propagate_g64.cuh"
+
+namespace scivr {
+
+template cudaError_t launch_group_fp64<1>(const PropLaunch &, cudaStream_t);
+template cudaError_t launch_group_fp64<2>(const PropLaunch &, cudaStream_t);
+template cudaError_t launch_group_fp64<3>(const PropLaunch &, cudaStream_t);
+template cudaError_t launch_group_fp64<4>(const PropLaunch &, cudaStream_t);
+
+}  // namespace scivr

@@ -4,7 +4,6 @@
 namespace scivr {
 
 template cudaError_t launch_group_mixed<9>(const PropLaunch &, cudaStream_t);
-template cudaError_t launch_group_fp64<9>(const PropLaunch &, cudaStream_t);
 
 template cudaError_t launch_group_batch_mixed_F<9>(int, const PropLaunch *, const int2 *, int, int *, int, cudaStream_t);
 

@@ -38,20 +38,19 @@ constexpr int kMaxThreadF = 9;   // thread-per-trajectory FP64 kernel
 constexpr int kMaxGroupF = 9;    // FP64 lane-group kernel
 constexpr int kMaxMixedF = 24;   // mixed lane-group kernel (one trajectory per warp above F = 9, two columns per lane above F = 16)
 
-// Schedule choice when the caller leaves it to the library: the lane-group
-// kernel keeps every SM busy with few trajectories (it launches G lanes per
-// trajectory); the thread kernel wins in FP64 once there are enough
-// trajectories to fill the GPU with one warp per SM sub-partition.  The FP64
-// crossover was measured on GB300 (400 steps of the F = 3, 6, 9 workloads): the
-// thread kernel's time is flat up to ~16k trajectories while the lane-group
-// time grows linearly, and they meet near 6k (F <= 3), 8.5k (F = 4..6) and 5k
-// (F >= 7) trajectories.
+// Schedule choice when the caller leaves it to the library: the lane groups, but in FP64 at F <= 2
+// beyond the numbers of trajectories where the thread kernel passes them.  Measured on GB300, us
+// per step, groups / thread: F = 1: 6.5 / 10.2 at 8192 trajectories, 11.5 / 11.4 at 19456,
+// 38.7 / 37.3 at 65536; F = 2: 15.8 / 24.0, 31.0 / 26.6, 107 / 91; F = 3: 23.8 / 47.5, 48.5 / 51.7,
+// 163 / 194; F = 6: 118 / 253, 235 / 282, 820 / 981; F = 9: 458 / 998, 801 / 1102 at 16384.  The
+// lines are where the groups' rounds of four warps per SM (9728 trajectories a round at F = 1, 4864
+// at F = 2) add up to the thread kernel's one flat round.
 int choose(int F, int precision, int64_t n_traj)
 {
     if (precision == SCIVR_MIXED) return SCIVR_KERNEL_GROUP;
     if (F > kMaxGroupF) return SCIVR_KERNEL_THREAD;
-    const int64_t crossover = F <= 3 ? 6144 : F <= 6 ? 8192 : 5120;
-    return n_traj >= crossover ? SCIVR_KERNEL_THREAD : SCIVR_KERNEL_GROUP;
+    if (F > 2) return SCIVR_KERNEL_GROUP;
+    return n_traj > (F == 1 ? 9728 : 14592) ? SCIVR_KERNEL_THREAD : SCIVR_KERNEL_GROUP;
 }
 
 }  // namespace

@@ -1,37 +1,32 @@
-// Lane-group propagation kernel (Sec. III.A / III.B of arXiv:1312.4698).
+// Mixed-precision lane-group propagation kernel (Sec. III.A / III.B of arXiv:1312.4698); the
+// FP64 lane groups are in propagate_g64.cuh.
 //
-// A group of G lanes (G = 8, 16 or 32, 2F <= G) owns one trajectory; a warp
-// holds T = 32/G trajectories.  Steps are processed in chunks of C (C = G, or
-// 16 / 8 steps for the one-trajectory-per-warp groups at F = 9 / F > 9), and
-// work is split by what parallelises:
+// A group of G lanes (mixed_group_lanes) owns one trajectory; a warp holds T = 32/G
+// trajectories.  Steps are processed in chunks of C (lg_chunk), and work is split by
+// what parallelises:
 //
-//   phase 1 (per step, group-parallel, arithmetic type Real):
-//     lane g < 2F owns column g of the monodromy matrix M (its p- and q-rows
-//     in registers); lane a < F owns mode a: p_a, q_a (FP64) and the
+//   phase 1 (per step, group-parallel):
+//     lane g owns columns g, g + G < 2F of the monodromy matrix M (their p- and q-rows
+//     in registers); lane a < F owns mode a: p_a, q_a and the
 //     separable diagonal of the potential.  The Hessian's packed coupling
 //     entries e(a,b) are spread over the group, reading the coupling tensors
 //     staged in shared memory; above F = 13 the warps of a CTA form their
-//     trajectories' Hessians together.  det M is Gaussian elimination of M^T across the
-//     group (pivot column by warp reduction, pivot entries by shuffle).  The
-//     Herman-Kluk matrix A of the step goes to shared memory.
-//   phase 2 (once per chunk, job-parallel): lane j < T*C takes job j =
-//     (trajectory j / C, step j % C) and computes det A and its argument by an
-//     LU in place in shared memory (FP64 path in FP64; mixed path in FP32, the
-//     entries being FP32 already).
+//     trajectories' Hessians together.  The Herman-Kluk matrix A of the step goes to
+//     shared memory.
+//   phase 2 (once per chunk): 32 / (T C) lanes take a job (trajectory, step) and compute det A
+//     and its argument by an LU in place in shared memory; every kDetMEvery steps det M by
+//     Gaussian elimination of M^T across the group.
 //   phase 3: the continuous phase, a segmented prefix sum over each group.
 //   phase 4 (job-parallel): overlap <chi|p q>, action, phase and the amplitude;
 //     each group writes C consecutive samples of its row.
 //
-// Real = float is the mixed-precision path: monodromy, potential, det M, A,
-// the elimination that gives det A, the overlap and each step's action
-// increment in FP32; positions, momenta, the accumulated action and the
-// continuous phase in FP64; the amplitude's phase is reduced modulo 2 pi in FP64
-// and its sine, cosine and magnitude are evaluated in FP32.  Real = double is the
-// same schedule in FP64 throughout.
+// Real = float: monodromy, potential, det M, A, the overlap and each step's action
+// increment; positions, momenta, the accumulated action and the elimination that gives det A
+// in double-FP32; the continuous phase in FP64; the amplitude's phase is reduced modulo 2 pi
+// in FP64 and its sine, cosine and magnitude are evaluated in FP32.
 //
 // On GB300 a warp-wide FP64 instruction holds a sub-partition's FP64 pipe for
-// about 64 cycles, so in the mixed path phase 1 keeps FP64 to the state updates
-// (one FMA per drift and per kick in the mode lanes) and one FP64 add per step.
+// about 64 cycles, so phase 1 keeps off it altogether.
 #pragma once
 
 #include <math_constants.h>
@@ -55,46 +50,15 @@ __host__ __device__ constexpr int pidx(int a, int b)
 
 template <typename Real> __device__ __forceinline__ Real rexp(Real x);
 template <> __device__ __forceinline__ float rexp<float>(float x) { return expf(x); }
-template <> __device__ __forceinline__ double rexp<double>(double x) { return exp(x); }
-
-// 1/x in FP64 from the FP32 reciprocal refined by two Newton steps
-// (e_{k+1} = e_k^2: 2^-23 -> 2^-46 -> below FP64 rounding); FP64 division
-// outside the FP32 exponent range.
-__device__ __forceinline__ double recip64(double x)
-{
-    const double ax = fabs(x);
-    if (!(ax > 1e-30 && ax < 1e30)) return 1.0 / x;
-    double r = (double)__frcp_rn((float)x);
-    r = r * fma(-x, r, 2.0);
-    r = r * fma(-x, r, 2.0);
-    return r;
-}
-
-
-// Compile-time loop: f(std::integral_constant<int, k>) for k = 0..N-1, every index a
-// constant (the unroller would leave long loops rolled, indexing register arrays).
-template <typename Fn, int... Ks>
-__device__ __forceinline__ void static_for_impl(Fn &&f, std::integer_sequence<int, Ks...>)
-{
-    (f(std::integral_constant<int, Ks>{}), ...);
-}
-template <int N, typename Fn>
-__device__ __forceinline__ void static_for(Fn &&f)
-{
-    static_for_impl(f, std::make_integer_sequence<int, N>{});
-}
 
 template <typename Real> struct Vec2;
 template <> struct Vec2<float> { using T = float2; };
-template <> struct Vec2<double> { using T = double2; };
 
-// Storage of one entry of the Herman-Kluk matrix A during its elimination: FP64
-// path a double2 (re, im); mixed path a double-FP32 complex (re.hi, im.hi, re.lo,
-// im.lo) -- the entries are formed in FP32 and eliminated to FP64-class accuracy, the
-// real and imaginary words side by side for packed FP32 arithmetic.
+// Storage of one entry of the Herman-Kluk matrix A during its elimination: a double-FP32
+// complex (re.hi, im.hi, re.lo, im.lo) -- the entries are formed in FP32 and eliminated to
+// FP64-class accuracy, the real and imaginary words side by side for packed FP32 arithmetic.
 template <typename Real> struct AEntry;
 template <> struct AEntry<float> { using T = float4; };
-template <> struct AEntry<double> { using T = double2; };
 
 // ---- double-FP32 arithmetic (hi + lo, |lo| <= ulp(hi)/2): error-free sum and
 // product of two floats (Knuth's TwoSum, the FMA form of Dekker's TwoProduct) and
@@ -162,25 +126,19 @@ __device__ __forceinline__ ff ff_recip(ff m)
     return ff_norm(y0, y0 * r);
 }
 
-// Positions, momenta and the action: FP64 in the FP64 path, double-FP32 pairs in the
-// mixed path (FP64-class accuracy, about 2^-46 relative per operation, on the FP32 pipe:
-// on this GPU an FP64 instruction or conversion costs the FP64 pipe ~70 times the issue
-// of an FP32 one).  coord_axpy: c + t x; coord_kick: c - t g for an FP32 force g; t is
-// given as FP64 (td) and as FP32 leading and trailing words (th, tl).
-__device__ __forceinline__ void coord_set(double &c, double x) { c = x; }
+// Positions, momenta and the action: double-FP32 pairs (FP64-class accuracy, about 2^-46
+// relative per operation, on the FP32 pipe: on this GPU an FP64 instruction or conversion costs
+// the FP64 pipe ~70 times the issue of an FP32 one).  coord_axpy: c + t x; coord_kick: c - t g
+// for an FP32 force g; t is given as FP32 leading and trailing words (th, tl).
 __device__ __forceinline__ void coord_set(ff &c, double x)
 {
     c.hi = (float)x;
     c.lo = (float)(x - (double)c.hi);
 }
-__device__ __forceinline__ double coord_get(double c) { return c; }
 __device__ __forceinline__ double coord_get(ff c) { return (double)c.hi + (double)c.lo; }
-__device__ __forceinline__ double coord_f(double c) { return c; }
 __device__ __forceinline__ float coord_f(ff c) { return c.hi; }
-__device__ __forceinline__ bool coord_finite(double c) { return isfinite(c); }
 __device__ __forceinline__ bool coord_finite(ff c) { return isfinite(c.hi) && isfinite(c.lo); }
-__device__ __forceinline__ double coord_axpy(double c, double td, float, float, double x) { return fma(td, x, c); }
-__device__ __forceinline__ ff coord_axpy(ff c, double, float th, float tl, ff x)
+__device__ __forceinline__ ff coord_axpy(ff c, float th, float tl, ff x)
 {
     const float p = th * x.hi;
     float e = fmaf(th, x.hi, -p);   // th x.hi - p, exact
@@ -190,8 +148,7 @@ __device__ __forceinline__ ff coord_axpy(ff c, double, float th, float tl, ff x)
     ff_two_sum(c.hi, p, s, e2);
     return ff_norm(s, e2 + (c.lo + e));
 }
-__device__ __forceinline__ double coord_kick(double c, double td, float, float, double g) { return fma(-td, g, c); }
-__device__ __forceinline__ ff coord_kick(ff c, double, float th, float tl, float g)
+__device__ __forceinline__ ff coord_kick(ff c, float th, float tl, float g)
 {
     const float p = -th * g;
     float e = fmaf(-th, g, -p);
@@ -201,7 +158,6 @@ __device__ __forceinline__ ff coord_kick(ff c, double, float th, float tl, float
     return ff_norm(s, e2 + (c.lo + e));
 }
 // the action increment (FP32 partial sums) joins the running action
-__device__ __forceinline__ double coord_add(double c, double d) { return c + d; }
 __device__ __forceinline__ ff coord_add(ff c, float d)
 {
     float s, e;
@@ -266,16 +222,10 @@ template <int F>
 struct CtaConst {
     double qw[F], pw[F];
     double p_eq[SCIVR_MAX_CHI][F], q_eq[SCIVR_MAX_CHI][F];
-    float Df[F], af[F], w2f[F];            // diagonal parameters in FP32
-    double Dd[F], ad[F], w2d[F];           // and in FP64
+    float Df[F], af[F], w2f[F];            // diagonal parameters
     float qwf[F], pwf[F];                  // overlap constants in FP32 (mixed path's overlap)
     float p_eqf[SCIVR_MAX_CHI][F], q_eqf[SCIVR_MAX_CHI][F];
 };
-
-// Real-typed views of the staged constants.
-template <typename Real, int F> __device__ __forceinline__ Real c_D(const CtaConst<F> &c, int i) { if constexpr (sizeof(Real) == 4) return c.Df[i]; else return c.Dd[i]; }
-template <typename Real, int F> __device__ __forceinline__ Real c_a(const CtaConst<F> &c, int i) { if constexpr (sizeof(Real) == 4) return c.af[i]; else return c.ad[i]; }
-template <typename Real, int F> __device__ __forceinline__ Real c_w2(const CtaConst<F> &c, int i) { if constexpr (sizeof(Real) == 4) return c.w2f[i]; else return c.w2d[i]; }
 
 // Column of job j in row r of the per-job arrays: the F mode lanes of a group
 // store one job into F different rows, which a plain [row][job] layout puts
@@ -284,13 +234,9 @@ template <typename Real, int F> __device__ __forceinline__ Real c_w2(const CtaCo
 template <int JOBS>
 __device__ __forceinline__ int jswz(int r, int j) { return j ^ (r & (JOBS >= 16 ? 15 : JOBS - 1)); }
 
-// Steps per chunk of a lane group.  Phases 2-4 work on T * C jobs (trajectory, step)
-// per warp.  FP64 path: one lane per job; groups of 8 and 16 lanes fill all 32 lanes,
-// the one-trajectory-per-warp groups take 16 jobs (F = 9) or 8 (F > 9).  Mixed path:
-// the double-FP32 elimination keeps two FP32 words per real entry, so chunks are
-// shorter (8 steps; 4 above F = 12) and 32 / (T * C) lanes share a job's elimination
-// by rows; the per-job prefactor matrices then take the same shared memory as one
-// FP32 word per entry at the FP64 path's chunk length.
+// Steps per chunk of a lane group.  Phases 2-4 work on T * C jobs (trajectory, step) per warp.
+// The double-FP32 elimination keeps two FP32 words per real entry, so chunks are short (8 steps; 4
+// above F = 12) and 32 / (T * C) lanes share a job's elimination by rows.
 // Mixed path: steps between stability tests (a multiple of every mixed chunk length).
 // The flag is sticky and a bad trajectory is dropped whole, so a coarser test differs
 // from the per-step one only for a deviation that crosses the threshold and falls back
@@ -300,8 +246,7 @@ constexpr int kDetMEvery = 16;
 
 template <int F, int G, typename Real> __host__ __device__ constexpr int lg_chunk()
 {
-    if constexpr (sizeof(Real) == 4) return G == 32 && F > 16 ? 1 : (G == 32 && F > 15 ? 2 : ((G == 32 && F > 12) || (G == 16 && F > 8) ? 4 : 8));
-    else return G < 32 ? G : (F > 9 ? 8 : 16);
+    return G == 32 && F > 16 ? 1 : (G == 32 && F > 15 ? 2 : ((G == 32 && F > 12) || (G == 16 && F > 8) ? 4 : 8));
 }
 
 // Warps per CTA and the launch-bounds CTA count: above F = 13 one CTA of 8 warps per SM, whose
@@ -320,14 +265,13 @@ template <int F> __host__ __device__ constexpr bool lg_tensor_regs() { return F 
 template <int F, int G, typename Real> __host__ __device__ constexpr int lg_min_ctas()
 {
     // register-held tensors: two CTAs per SM at F = 8, 9 (up to 255 registers), three at F = 6, 7
-    if constexpr (sizeof(Real) == 4 && G == 16 && F >= 6 && lg_tensor_regs<F>()) return F >= 8 ? 2 : 3;
+    if constexpr (G == 16 && F >= 6 && lg_tensor_regs<F>()) return F >= 8 ? 2 : 3;
     return F > 9 ? 1 : (sizeof(Real) == 4 && 2 * F > G ? 3 : 4);
 }
 
 // 16-byte vectors of Real for shared-memory loads.
 template <typename Real> struct V16;
 template <> struct V16<float> { using T = float4; static constexpr int N = 4; };
-template <> struct V16<double> { using T = double2; static constexpr int N = 2; };
 
 template <typename Real>
 __device__ __forceinline__ Real vcomp(const typename V16<Real>::T &v, int j)
@@ -517,8 +461,7 @@ struct WarpShared {
     // stride RS and the jobs' bases spread those eight over the eight 16-byte bank groups: an odd
     // RS for eight rows of one job, bases 4 apart (mod 8) for two jobs of four rows, 2 apart for four
     // jobs of two rows -- or, at F = 6, where an odd RS would cost a CTA per SM, 0, 5, 4, 1.  (With
-    // F = 24 entries a row all eight fell into one group; with 81 a job two at F = 9.)  FP64 path: a
-    // lane per job, an odd job stride.
+    // F = 24 entries a row all eight fell into one group; with 81 a job two at F = 9.)
     static constexpr int LPJ = JOBS >= 32 ? 1 : 32 / JOBS;
     static constexpr bool kMixed = sizeof(Real) == 4;
     static constexpr int RS = !kMixed || LPJ == 1 || F == 6 ? F : F | 1;
@@ -624,9 +567,6 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
             cc.pw[a] = A.pw[a];
             cc.qwf[a] = (float)A.qw[a];
             cc.pwf[a] = (float)A.pw[a];
-            cc.Dd[a] = pes.D[a];
-            cc.ad[a] = pes.a[a];
-            cc.w2d[a] = pes.omega[a] * pes.omega[a];
             cc.Df[a] = pes.D_f[a];
             cc.af[a] = pes.a_f[a];
             cc.w2f[a] = pes.omega_f[a] * pes.omega_f[a];
@@ -862,25 +802,18 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
 
     // mode state (lane g < F)
     const int mode = g < F ? g : 0;
-    using Coord = std::conditional_t<sizeof(Real) == 4, ff, double>;
+    using Coord = ff;
     Coord p, q;
     coord_set(p, L.p0[mode * n + jl]);
     coord_set(q, L.q0[mode * n + jl]);
     Real pr = (Real)coord_get(p);   // the momentum as seen by the Real-precision bulk
     Coord S;                        // accumulated action (lane 0 of the group holds the total)
     coord_set(S, 0.0);
-    // per-job action in the job table: FP64, or the double-FP32 pair in the same 8 bytes
-    auto sj_put = [&](int j, Coord v) {
-        if constexpr (sizeof(Real) == 4) reinterpret_cast<float2 *>(sh.Sj)[j] = make_float2(v.hi, v.lo);
-        else sh.Sj[j] = v;
-    };
+    // per-job action in the job table: the double-FP32 pair in the 8 bytes of a double
+    auto sj_put = [&](int j, Coord v) { reinterpret_cast<float2 *>(sh.Sj)[j] = make_float2(v.hi, v.lo); };
     auto sj_get = [&](int j) -> double {
-        if constexpr (sizeof(Real) == 4) {
-            const float2 v = reinterpret_cast<const float2 *>(sh.Sj)[j];
-            return (double)v.x + (double)v.y;
-        } else {
-            return sh.Sj[j];
-        }
+        const float2 v = reinterpret_cast<const float2 *>(sh.Sj)[j];
+        return (double)v.x + (double)v.y;
     };
     // column state: slot s of lane g holds column c = g + s G of M = d(p,q)/d(p0,q0) (c < 2F;
     // a slot past 2F holds a zero column)
@@ -937,10 +870,9 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
             for (int sub = 0; sub < 4; ++sub) {
                 // drift: q += tau p, S += tau p.p/2, M_q += tau M_p
                 {
-                    Real rt;
-                    if constexpr (sizeof(Real) == 4) rt = A.tdrift_f[sub]; else rt = A.tdrift[sub];
+                    const Real rt = A.tdrift_f[sub];
                     if (g < F) {
-                        q = coord_axpy(q, A.tdrift[sub], A.tdrift_f[sub], A.tdrift_lo[sub], p);
+                        q = coord_axpy(q, A.tdrift_f[sub], A.tdrift_lo[sub], p);
                         dS = fma(rt * Real(0.5) * pr, pr, dS);
                     }
                     if constexpr (kPacked) {
@@ -964,9 +896,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                 }
                 if (sub == 3) break;
                 // kick: potential at q
-                const double tk = A.tkick[sub];
-                Real rtk;
-                if constexpr (sizeof(Real) == 4) rtk = A.tkick_f[sub]; else rtk = tk;
+                const Real rtk = A.tkick_f[sub];
                 __syncwarp();   // previous kick's readers of qr/H are done
                 if (g < F) {
                     sh.qr[t][g] = (Real)coord_f(q);
@@ -1121,20 +1051,20 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                     const Real gr = dot16<Real, S3>(sh.Gc[t][g], sh.qr[t]);
                     Real Vd, gd, hd;   // the separable diagonal: value, gradient, Hessian
                     if (pes.diag_kind == SCIVR_DIAG_MORSE) {
-                        const Real Dm = c_D<Real>(cc, g), am = c_a<Real>(cc, g);
+                        const Real Dm = cc.Df[g], am = cc.af[g];
                         const Real u = rexp<Real>(-am * sh.qr[t][g]);
                         const Real omu = Real(1) - u;
                         Vd = Dm * omu * omu;
                         gd = Real(2) * Dm * am * u * omu;
                         hd = Real(2) * Dm * am * am * u * (Real(2) * u - Real(1));
                     } else {
-                        const Real w2 = c_w2<Real>(cc, g);
+                        const Real w2 = cc.w2f[g];
                         Vd = Real(0.5) * w2 * sh.qr[t][g] * sh.qr[t][g];
                         gd = w2 * sh.qr[t][g];
                         hd = w2;
                     }
                     sh.H(t, g, g) += hd;
-                    p = coord_kick(p, tk, A.tkick_f[sub], A.tkick_lo[sub], gr + gd);
+                    p = coord_kick(p, A.tkick_f[sub], A.tkick_lo[sub], gr + gd);
                     pr = (Real)coord_f(p);
                     vlane += Vd;
                 }
@@ -1185,84 +1115,6 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                         for (int s = 0; s < NCOL; ++s) Mp[s][a] = fma(-rtk, acc[s], Mp[s][a]);
                     }
                 }
-            }
-            // ---- stability: det M = det M^T by Gaussian elimination of M^T with partial pivoting ----
-            // Column c of M (lane c % G, slot c / G) is row c of M^T.  Stage k picks, among the rows
-            // not used yet, the one with the largest |M[k][c]| (an arg-max over the group by warp
-            // reduction, ties to the higher row), and every other unused row subtracts its multiple
-            // of the pivot row's entries below k.  Rows are marked used instead of being moved; the
-            // sign of det is the parity of the order in which they were picked, counted as
-            // inversions on the bitmask of unused rows.
-            // Cadence: the FP64 path tests every step (flags equal to the oracle's bit for bit);
-            // the mixed path tests every kDetMEvery steps, after phase 2 (below).  The FP32
-            // threshold (537) sits far above the rounding noise, where a deviation that has
-            // grown past it keeps growing (Sec. III.A: chaotic trajectories are the ones removed).
-            if constexpr (sizeof(Real) == 8) {
-                Real W[NCOL][N2];
-#pragma unroll
-                for (int s = 0; s < NCOL; ++s)
-#pragma unroll
-                    for (int a = 0; a < F; ++a) { W[s][a] = Mp[s][a]; W[s][F + a] = Mq[s][a]; }
-                Real det = Real(1);
-                unsigned long long unused = N2 == 64 ? ~0ull : (1ull << N2) - 1ull;
-                unsigned parity = 0u;
-                static_for<N2>([&](auto kc) {
-                    constexpr int k = decltype(kc)::value;
-                    // non-negative floats order like their bit patterns; the low 6 bits carry row + 1
-                    // (so a used or idle slot's key 0 never wins), at the cost of 6 mantissa bits of
-                    // the comparison
-                    unsigned key = 0u;
-#pragma unroll
-                    for (int s = 0; s < NCOL; ++s) {
-                        const int col = g + s * G;
-                        if (col < N2 && ((unused >> col) & 1ull)) {
-                            float mag;
-                            if constexpr (sizeof(Real) == 4) mag = fabsf(W[s][k]); else mag = (float)fabs(W[s][k]);
-                            const unsigned kk = (__float_as_uint(mag) & ~63u) | (unsigned)(col + 1);
-                            key = kk > key ? kk : key;
-                        }
-                    }
-                    // one full-warp integer max per group (the other groups' lanes contribute 0)
-                    unsigned kmax = 0u;
-#pragma unroll
-                    for (int tt = 0; tt < T; ++tt) {
-                        const unsigned r = __reduce_max_sync(FULL, t == tt ? key : 0u);
-                        kmax = (t == tt) ? r : kmax;
-                    }
-                    const int pc = (int)(kmax & 63u) - 1;          // pivot row of M^T
-                    const int pl = base + pc % G, ps = pc / G;     // its lane and slot
-                    auto sel = [&](int i) -> Real { if constexpr (NCOL == 1) return W[0][i]; else return ps ? W[1][i] : W[0][i]; };
-                    const Real pk = __shfl_sync(FULL, sel(k), pl);
-                    // FP32: the hardware reciprocal (det M only feeds the stability test, whose FP32
-                    // tolerance is far above its ulp-level error); FP64: exact division
-                    Real inv;
-                    if constexpr (sizeof(Real) == 4) inv = __fdividef(1.0f, pk); else inv = Real(1) / pk;
-                    parity ^= (unsigned)__popcll(unused & ((1ull << pc) - 1ull)) & 1u;
-                    unused &= ~(1ull << pc);
-                    det *= pk;
-                    Real l[NCOL];
-                    bool elim[NCOL];
-#pragma unroll
-                    for (int s = 0; s < NCOL; ++s) {
-                        const int col = g + s * G;
-                        elim[s] = col < N2 && ((unused >> col) & 1ull);
-                        l[s] = W[s][k] * inv;
-                    }
-#pragma unroll
-                    for (int i = k + 1; i < N2; ++i) {
-                        const Real wp = __shfl_sync(FULL, sel(i), pl);
-#pragma unroll
-                        for (int s = 0; s < NCOL; ++s)
-                            if (elim[s]) W[s][i] = fma(-l[s], wp, W[s][i]);
-                    }
-                });
-                if (parity) det = -det;
-                const Real dev = isfinite(det) ? fabs(fma(det, det, Real(-1))) : Real(CUDART_INF);
-                stab = dev > stab ? dev : stab;
-                Real tolr;
-                if constexpr (sizeof(Real) == 4) tolr = A.stab_tol_f; else tolr = A.stab_tol;
-                if (dev > tolr) good = false;
-                if (c == cnt - 1) detM_last = (double)det;
             }
             // ---- Herman-Kluk matrix column b = g (needs column F + b) ----
             {
@@ -1492,59 +1344,6 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                 argA = sh.argj[jb];
                 detA = sh.detAj[jb];
             }
-        } else if (ln >= JOBS) {
-            // no job for this lane (wide groups): the in-place elimination must not touch a job's storage
-        } else {
-            // FP64 path: in-place elimination in FP64, one lane per job, det A as the product of
-            // the pivots (no range concern in FP64)
-            auto at = [&](int e) -> R2 & { return sh.A[ln * Sh::AS + e]; };
-            double dr = 1.0, di = 0.0;
-#pragma unroll
-            for (int k = 0; k < F; ++k) {
-                int piv = k;
-                double best;
-                {
-                    const R2 v = at(k * F + k);
-                    best = v.x * v.x + v.y * v.y;
-                }
-#pragma unroll
-                for (int i = k + 1; i < F; ++i) {
-                    const R2 v = at(i * F + k);
-                    const double m = v.x * v.x + v.y * v.y;
-                    if (m > best) { best = m; piv = i; }
-                }
-                R2 prow[F];
-#pragma unroll
-                for (int cc = k; cc < F; ++cc) prow[cc] = at(piv * F + cc);
-                if (piv != k) {
-#pragma unroll
-                    for (int cc = k; cc < F; ++cc) at(piv * F + cc) = at(k * F + cc);
-                    dr = -dr;
-                    di = -di;
-                }
-                const double kr = prow[k].x, ki = prow[k].y;
-                const double nr = fma(dr, kr, -di * ki), ni = fma(dr, ki, di * kr);
-                dr = nr;
-                di = ni;
-                const double rr = recip64(fma(kr, kr, ki * ki));
-                const double ir = kr * rr, ii = -ki * rr;
-#pragma unroll
-                for (int i = k + 1; i < F; ++i) {
-                    const R2 aik = at(i * F + k);
-                    const double lr = fma(aik.x, ir, -aik.y * ii);
-                    const double li = fma(aik.x, ii, aik.y * ir);
-#pragma unroll
-                    for (int cc = k + 1; cc < F; ++cc) {
-                        R2 a = at(i * F + cc);
-                        a.x = fma(-lr, prow[cc].x, fma(li, prow[cc].y, a.x));
-                        a.y = fma(-lr, prow[cc].y, fma(-li, prow[cc].x, a.y));
-                        at(i * F + cc) = a;
-                    }
-                }
-            }
-            detA = make_double2(dr, di);
-            argA = atan2(di, dr);
-            if (A.amplitude == SCIVR_AMP_HK) sh.lnA[ln] = 0.5 * log(hypot(dr, di));
         }
         if constexpr (sizeof(Real) == 4) {
             // det M every kDetMEvery steps and at the last step (at a chunk end: M is unchanged
@@ -1661,26 +1460,6 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                     const int64_t ia = x * L.chi_stride + jl * L.amp_ld + step0 + jc + 1;
                     if (L.amp_f32) reinterpret_cast<float2 *>(L.amp)[ia] = make_float2(mag * cf, mag * sf);
                     else L.amp[ia] = make_double2((double)(mag * cf), (double)(mag * sf));
-                } else {
-                    double re = 0.0, im = 0.0;
-#pragma unroll
-                    for (int a = 0; a < F; ++a) {
-                        const double pa = sh.pj[a][jswz<JOBS>(a, jb)], qa = sh.qj[a][jswz<JOBS>(a, jb)];
-                        const double dq = cc.q_eq[x][a] - qa, dp = cc.p_eq[x][a] - pa;
-                        re = fma(-cc.qw[a] * dq, dq, re);
-                        re = fma(-cc.pw[a] * dp, dp, re);
-                        im = fma(0.5 * (cc.p_eq[x][a] + pa), dq, im);
-                    }
-                    double ph = im + S + 0.5 * theta;
-                    if (A.amplitude == SCIVR_AMP_HK) {
-                        const double2 o = sh.ov0[x][t];
-                        re = re - o.x + sh.lnA[jb];
-                        ph -= o.y;
-                    }
-                    double sn, cs;
-                    sincos(ph, &sn, &cs);
-                    const double mag = exp(re);
-                    amp_store(L, x * L.chi_stride + jl * L.amp_ld + step0 + jc + 1, mag * cs, mag * sn);
                 }
             }
         }
@@ -1830,7 +1609,6 @@ cudaError_t launch_lg(const PropLaunch &L, cudaStream_t s)
 
 // Launchers instantiated by the prop_lg_*.cu units: lanes per trajectory by F
 // (2F columns must fit), warps per CTA, and the batch variants the tuner may pick.
-template <int F> constexpr int group_lanes() { return 2 * F <= 8 ? 8 : (2 * F <= 16 ? 16 : 32); }
 
 template <int F> cudaError_t launch_group_mixed(const PropLaunch &L, cudaStream_t s)
 {
@@ -1898,11 +1676,6 @@ struct MultiLaunch {
         return cudaGetLastError();
     }
 };
-
-template <int F> cudaError_t launch_group_fp64(const PropLaunch &L, cudaStream_t s)
-{
-    return launch_lg<F, group_lanes<F>(), double, group_lanes<F>() == 32 ? 2 : 4>(L, s);
-}
 
 
 }  // namespace scivr
