@@ -35,6 +35,7 @@
 #include <utility>
 #include <type_traits>
 
+#include "fp64_ops.cuh"
 #include "scivr_internal.cuh"
 
 namespace scivr {
@@ -378,7 +379,7 @@ struct TensorLayout {
 // order.  Either way each entry's multiply-adds keep the order they have in a single lane's loop,
 // whatever the tile: the results do not depend on TRAJ.  TT is the smallest tile whose items fit one
 // round of the CTA's lanes.  F = 15, 3001 trajectories x 501 steps: 37.0 -> 27.6 ms; F = 24,
-// 2048 x 200: 79.3 -> 45.8 ms (with the prefactor elimination's changes 26.0 and 38.4).
+// 2048 x 200: 79.3 -> 45.8 ms (with the later changes to the prefactor 24.9 and 37.2).
 template <int F, int WARPS, int TRAJ, bool STAGED>
 struct CoopHessian {
     static constexpr int P = F * (F + 1) / 2, P4 = (P + 3) & ~3, Q = P4 / 4;
@@ -813,7 +814,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
     auto sj_put = [&](int j, Coord v) { reinterpret_cast<float2 *>(sh.Sj)[j] = make_float2(v.hi, v.lo); };
     auto sj_get = [&](int j) -> double {
         const float2 v = reinterpret_cast<const float2 *>(sh.Sj)[j];
-        return (double)v.x + (double)v.y;
+        return widen(v.x) + widen(v.y);
     };
     // column state: slot s of lane g holds column c = g + s G of M = d(p,q)/d(p0,q0) (c < 2F;
     // a slot past 2F holds a zero column)
@@ -1334,9 +1335,11 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                 di = {-di.hi, -di.lo};
             }
             if (r == 0) {
-                const double mr = (double)dr.hi + (double)dr.lo, mi = (double)di.hi + (double)di.lo;
-                sh.argj[job] = atan2(mi, mr);   // the power of two does not change the argument
-                sh.detAj[job] = make_double2(ldexp(mr, dexp), ldexp(mi, dexp));
+                const double mr = widen(dr.hi) + widen(dr.lo), mi = widen(di.hi) + widen(di.lo);
+                // (the power of two does not change the argument; with atan2 and conversions the FP64 pipe was
+                // busy 21 % of the time: F = 9, 65536 x 1000: 166.0 -> 161.1 ms, F = 15, 3001 x 501: 26.0 -> 24.9)
+                sh.argj[job] = arg_normal(mr, mi, dr.hi, di.hi);
+                if (step0 + cnt == A.n_steps) sh.detAj[job] = make_double2(ldexp(mr, dexp), ldexp(mi, dexp));
                 if (A.amplitude == SCIVR_AMP_HK) sh.lnA[job] = 0.5 * (log(hypot(mr, mi)) + dexp * 0.69314718055994530942);
             }
             __syncwarp();
@@ -1417,7 +1420,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
         d = fma(-kTwoPi, rint(d * kInvTwoPi), d);
         double inc = jvalid ? d - A.ref_step : 0.0;
 #pragma unroll
-        for (int o = 1; o < G; o <<= 1) {
+        for (int o = 1; o < C; o <<= 1) {
             const double v = __shfl_up_sync(FULL, inc, o, G);
             if (g >= o) inc += v;
         }
@@ -1427,7 +1430,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
         arg_last = __shfl_sync(FULL, arg, lastlane);
         detA_last.x = __shfl_sync(FULL, detA.x, lastlane);
         detA_last.y = __shfl_sync(FULL, detA.y, lastlane);
-        if (!isfinite(theta_last)) good = false;
+        if (!finite_bits(theta_last)) good = false;
         // ---------------- phase 4: amplitudes (job-parallel) ----------------
         if (jvalid && active) {
             const double S = sj_get(jb);
@@ -1445,7 +1448,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                         rf = fmaf(-cc.pwf[a] * dp, dp, rf);
                         imf = fmaf(0.5f * (cc.p_eqf[x][a] + pa), dq, imf);
                     }
-                    double ph = fma(0.5, theta, (double)imf + S);
+                    double ph = fma(0.5, theta, widen(imf) + S);
                     if (A.amplitude == SCIVR_AMP_HK) {
                         // Herman-Kluk summand: |det A|^{1/2} and the division by the initial
                         // overlap times the sampling weight
@@ -1463,7 +1466,10 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                 }
             }
         }
-        if (!isfinite(sj_get(t * C + cnt - 1))) good = false;
+        {
+            const float2 v = reinterpret_cast<const float2 *>(sh.Sj)[t * C + cnt - 1];
+            if (!(isfinite(v.x) && isfinite(v.y))) good = false;
+        }
         __syncwarp();
     }
 
