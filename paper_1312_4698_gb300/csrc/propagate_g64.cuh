@@ -18,6 +18,8 @@
 // with the factor -tau of their kick, V and its gradient from the rows of H q and H3 q,
 // reciprocals in three multiply-adds from the hardware's approximation, exponentials from a
 // 64-entry table, pivots and thresholds compared as integers, det M's pivots multiplied pairwise.
+// Against the groups of 8 to 32 lanes without these, us per step: F = 6, 4096 trajectories: 103 -> 59;
+// F = 3, 96: 17.0 -> 9.7 (7.2 with a recording warp).
 #pragma once
 
 #include <math_constants.h>
@@ -51,12 +53,15 @@ struct Geo {
     static constexpr int S3 = row_len(F), S4 = row_len(P), SH = even(F), HT = row_len(F * SH);
     static constexpr int AS = (F * F) | 1;
 
-    // FP64 instructions of a warp per step, counted from the code below: the measure by which the
-    // group size is chosen.
+    // FP64 instructions of a warp per step, counted from the code below: the trajectory and its
+    // monodromy, and the records (determinants, phase, amplitude).  The measure by which the group
+    // size is chosen.
     static constexpr int kStepInstr =
-        4 * (NC * F + 3 * NM) + 3 * (NE * (1 + F + P) + NM * (2 * F + 28) + NC * F * F) +
+        4 * (NC * F + 3 * NM) + 3 * (NE * (1 + F + P) + NM * (2 * F + 28) + NC * F * F) + ilog2(G);
+    static constexpr int kRecordInstr =
         NC * (N2 * (N2 - 1) / 2) + N2 * (3 + NC) + NC + ilog2(G) + 4 * NM * F + 6 +
         (4 * (F * (F * F - 1)) / 3 + 11 * F + 4 * F * (F - 1) / 2 + 9 * F + 110) / C;
+    static constexpr int MAIL = NC * N2 + 2 * NM + 1;   // state of a step that its records need, per lane
 };
 
 // Constants of a CTA, staged once: the coupling tensors and diagonal parameters times -tau of each
@@ -87,6 +92,17 @@ struct WarpShared {
     double2 ov0[SCIVR_MAX_CHI][E::T];         // log of the Herman-Kluk summand's divisor
 };
 
+// A step's state on its way from the warp that propagates to the warp that records (two slots;
+// a lane's values go to the same lane).
+template <int F, int G>
+struct Mail {
+    double v[2][Geo<F, G>::MAIL][32];
+};
+
+// Named barriers of 64 threads: a pair of warps.
+__device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+__device__ __forceinline__ void pair_arrive(int id) { asm volatile("bar.arrive %0, 64;" ::"r"(id) : "memory"); }
+
 // Column of job j in row r of the per-job arrays: a group's lanes store one job into different rows.
 template <int JOBS>
 __device__ __forceinline__ int swz(int r, int j) { return j ^ (r & (JOBS >= 16 ? 15 : JOBS - 1)); }
@@ -112,7 +128,10 @@ __device__ __forceinline__ double slot(const double (&w)[N], int s)
     return v;
 }
 
-template <int F, int G>
+// HELP: a second warp, on another sub-partition, makes the records (a quarter to a third of the
+// instructions), for launches that leave half of the sub-partitions without a warp.  F = 3, 96
+// trajectories x 400 steps, the whole FP64 run: 3.68 -> 2.93 ms.
+template <int F, int G, bool HELP>
 __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropLaunch L)
 {
     using E = Geo<F, G>;
@@ -163,8 +182,13 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropL
 
     const int warp = threadIdx.x >> 5, ln = threadIdx.x & 31;
     const int t = ln / G, g = ln % G, base = t * G;
-    Sh &sh = reinterpret_cast<Sh *>(smem_raw + cta_bytes)[warp];
-    {
+    const int n_set = HELP ? blockDim.x >> 6 : blockDim.x >> 5;   // sets of T trajectories in the CTA
+    const int set = HELP ? warp % n_set : warp;
+    const bool advances = !HELP || warp < n_set, records = !HELP || warp >= n_set;
+    Sh &sh = reinterpret_cast<Sh *>(smem_raw + cta_bytes)[set];
+    Mail<F, G> &mail = reinterpret_cast<Mail<F, G> *>(smem_raw + cta_bytes + n_set * sizeof(Sh))[HELP ? set : 0];
+    const int bar_full = 1 + 4 * set, bar_free = bar_full + 2;    // + slot
+    if (advances) {
         // the rows' padding is multiplied by zero but never written: clear it once
         double *z = &sh.q[0][0];
         constexpr int nz = (int)(offsetof(Sh, A) / sizeof(double));
@@ -172,7 +196,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropL
         __syncwarp();
     }
     const int64_t n = L.n_traj;
-    const int64_t j_traj = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * T + t;
+    const int64_t j_traj = ((int64_t)blockIdx.x * n_set + set) * T + t;
     const bool active = j_traj < n;
     const int64_t jl = active ? j_traj : n - 1;
 
@@ -208,7 +232,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropL
     double2 detA_last = make_double2(1.0, 0.0);
 
     // amplitude at c = 0 (M = I, S = 0, theta = 0): lane 0 of each group
-    if (g == 0 && active) {
+    if (records && g == 0 && active) {
         double re00 = 0.0;
         for (int x = 0; x < A.n_chi; ++x) {
             double re = 0.0, im = 0.0;
@@ -240,7 +264,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropL
         for (int c = 0; c < cnt; ++c) {
             double dS = 0.0;   // this lane's share of the step's action increment
 #pragma unroll 1
-            for (int sub = 0; sub < 4; ++sub) {
+            for (int sub = advances ? 0 : 4; sub < 4; ++sub) {
                 // drift: q += tau p, S += tau p.p / 2, M_q += tau M_p
                 const double td = A.tdrift[sub], th = 0.5 * td;
 #pragma unroll
@@ -370,6 +394,37 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropL
                         }
                     }
             }
+#pragma unroll
+            for (int o = G / 2; o > 0; o >>= 1) dS += __shfl_xor_sync(FULL, dS, o);
+            S += dS;
+            if constexpr (HELP) {
+                const int step = step0 + c, sl = step & 1;
+                auto pass = [&](auto &&move) {
+                    int k = 0;
+#pragma unroll
+                    for (int s = 0; s < NC; ++s)
+#pragma unroll
+                        for (int a = 0; a < F; ++a) {
+                            move(Mp[s][a], mail.v[sl][k++][ln]);
+                            move(Mq[s][a], mail.v[sl][k++][ln]);
+                        }
+#pragma unroll
+                    for (int s = 0; s < NM; ++s) {
+                        move(p[s], mail.v[sl][k++][ln]);
+                        move(q[s], mail.v[sl][k++][ln]);
+                    }
+                    move(S, mail.v[sl][k][ln]);
+                };
+                if (advances) {
+                    if (step >= 2) pair_sync(bar_free + sl);
+                    pass([](double &x, double &m) { m = x; });
+                    pair_arrive(bar_full + sl);
+                    continue;
+                }
+                pair_sync(bar_full + sl);
+                pass([](double &x, double &m) { x = m; });
+                if (step + 2 < A.n_steps) pair_arrive(bar_free + sl);
+            }
             // ---- stability: det M = det M^T by Gaussian elimination of M^T with partial pivoting ----
             // Column c of M is row c of M^T, held by lane c % G in slot c / G.  Stage k picks the unused
             // row of the largest |entry k| (keys: the leading bits of the magnitude, then the row), and
@@ -465,11 +520,9 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropL
                     sh.qj[b][swz<JOBS>(b, job)] = q[s];
                 }
             }
-#pragma unroll
-            for (int o = G / 2; o > 0; o >>= 1) dS += __shfl_xor_sync(FULL, dS, o);
-            S += dS;
             if (g == 0) sh.Sj[job] = S;
         }
+        if (!records) continue;
         {
             // non-finite state persists, so testing once per chunk marks the same trajectories
             bool fin = true;
@@ -573,7 +626,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropL
         __syncwarp();
     }
 
-    if (!active) return;
+    if (!active || !records) return;
     if (g == 0) L.good[jl] = good ? 1 : 0;
     const FinalDev &fo = L.fin;
 #pragma unroll
@@ -604,45 +657,51 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropL
     }
 }
 
-// Warps per CTA: up to four, fewer where fewer spread over all SMs.
-template <int F, int G>
+// Sets of T trajectories per CTA: up to four warps, fewer where fewer spread over all SMs.
+template <int F, int G, bool HELP>
 cudaError_t launch(const PropLaunch &L, int n_sm, cudaStream_t s)
 {
     using E = Geo<F, G>;
-    const int64_t warps = (L.n_traj + E::T - 1) / E::T;
-    const int W = warps >= (int64_t)kMaxWarps * n_sm ? kMaxWarps : (int)((warps + n_sm - 1) / n_sm);
+    constexpr int most = HELP ? kMaxWarps / 2 : kMaxWarps;
+    const int64_t sets = (L.n_traj + E::T - 1) / E::T;
+    const int W = sets >= (int64_t)most * n_sm ? most : (int)((sets + n_sm - 1) / n_sm);
     constexpr size_t cta_bytes = (sizeof(CtaShared<F>) + 15) & ~(size_t)15;
-    static_assert(sizeof(WarpShared<F, G>) % 16 == 0, "the warps' shared blocks stay aligned");
-    static_assert(cta_bytes + kMaxWarps * sizeof(WarpShared<F, G>) <= 227 * 1024, "four warps fit an SM");
-    auto kern = k_propagate_g64<F, G>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)(cta_bytes + kMaxWarps * sizeof(WarpShared<F, G>)));
+    constexpr size_t set_bytes = sizeof(WarpShared<F, G>) + (HELP ? sizeof(Mail<F, G>) : 0);
+    static_assert(sizeof(WarpShared<F, G>) % 16 == 0 && sizeof(Mail<F, G>) % 16 == 0, "the sets' shared blocks stay aligned");
+    static_assert(cta_bytes + most * set_bytes <= 227 * 1024, "four warps fit an SM");
+    auto kern = k_propagate_g64<F, G, HELP>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(cta_bytes + most * set_bytes));
     if (e != cudaSuccess) return e;
-    kern<<<(unsigned)((warps + W - 1) / W), 32 * W, cta_bytes + W * sizeof(WarpShared<F, G>), s>>>(L);
+    kern<<<(unsigned)((sets + W - 1) / W), (HELP ? 64 : 32) * W, cta_bytes + W * set_bytes, s>>>(L);
     return cudaGetLastError();
 }
 
 // The narrowest group a lane's registers allow (its columns and their copy for det M).
 constexpr int min_lanes(int F) { return F <= 1 ? 2 : F <= 6 ? 4 : 8; }
+// The widest that still saves instructions where a warp records.
+constexpr int max_lanes(int F) { return F <= 1 ? 2 : F == 2 ? 4 : F == 3 ? 8 : F <= 5 ? 16 : 32; }
 
 }  // namespace g64
 
 // Group size: the fewest FP64 instructions over the rounds of four warps per SM that the
-// trajectories take.
+// trajectories take; with a recording warp where two per SM suffice.
 template <int F, int G = g64::min_lanes(F)>
-void choose_g64_lanes(int64_t n_traj, int n_sm, double &best, int &lanes)
+void choose_g64_lanes(int64_t n_traj, int n_sm, double &best, int &lanes, bool &help)
 {
+    using E = g64::Geo<F, G>;
     const int64_t warps = (n_traj * G + 31) / 32, slots = (int64_t)g64::kMaxWarps * n_sm;
-    const double cost = (double)((warps + slots - 1) / slots) * g64::Geo<F, G>::kStepInstr;
-    if (lanes == 0 || cost < best) { best = cost; lanes = G; }
-    if constexpr (G < 32) choose_g64_lanes<F, 2 * G>(n_traj, n_sm, best, lanes);
+    const bool h = 2 * warps <= slots;
+    const int instr = !h ? E::kStepInstr + E::kRecordInstr : E::kStepInstr > E::kRecordInstr ? E::kStepInstr : E::kRecordInstr;
+    const double cost = (double)((warps + slots - 1) / slots) * instr;
+    if (lanes == 0 || cost < best) { best = cost; lanes = G; help = h; }
+    if constexpr (G < g64::max_lanes(F)) choose_g64_lanes<F, 2 * G>(n_traj, n_sm, best, lanes, help);
 }
 
 template <int F, int G = g64::min_lanes(F)>
-cudaError_t launch_g64_lanes(const PropLaunch &L, int lanes, int n_sm, cudaStream_t s)
+cudaError_t launch_g64_lanes(const PropLaunch &L, int lanes, bool help, int n_sm, cudaStream_t s)
 {
-    if (lanes == G) return g64::launch<F, G>(L, n_sm, s);
-    if constexpr (G < 32) return launch_g64_lanes<F, 2 * G>(L, lanes, n_sm, s);
+    if (lanes == G) return help ? g64::launch<F, G, true>(L, n_sm, s) : g64::launch<F, G, false>(L, n_sm, s);
+    if constexpr (G < g64::max_lanes(F)) return launch_g64_lanes<F, 2 * G>(L, lanes, help, n_sm, s);
     return cudaErrorInvalidValue;
 }
 
@@ -654,8 +713,9 @@ template <int F> cudaError_t launch_group_fp64(const PropLaunch &L, cudaStream_t
     if (e != cudaSuccess) return e;
     double cost = 0.0;
     int lanes = 0;
-    choose_g64_lanes<F>(L.n_traj, n_sm, cost, lanes);
-    return launch_g64_lanes<F>(L, lanes, n_sm, s);
+    bool help = false;
+    choose_g64_lanes<F>(L.n_traj, n_sm, cost, lanes, help);
+    return launch_g64_lanes<F>(L, lanes, help, n_sm, s);
 }
 
 }  // namespace scivr
