@@ -31,10 +31,69 @@ inline int slice_rows(int64_t n, int K)
     return (int)rows;
 }
 
-// Bound by the FP64 pipe's additions (two per summand: 248 us at 16384 x 4001, against 156 us
-// for one read of them from HBM).  A thread owns one column and keeps eight 16-byte loads in
-// flight; bad rows are loaded too (their flags, from shared memory, only select), so that no
-// load waits for a branch.  16384 x 4001 summands: 1180 -> 268 us.
+// A column's running sum as a 64-bit integer in units of 2^(top + kHead - 1085), for summands whose
+// biased exponent is at most top; 2^kHead summands cannot overflow it, so it is flushed into FP64
+// that often.  top = -1: no window.
+constexpr int kHead = 6;
+
+struct FixedSum {
+    int top = -1;
+    long long re = 0, im = 0;
+    double2 out = make_double2(0.0, 0.0);   // what has left the integers, and summands beyond any window
+
+    __device__ __forceinline__ long long fixed(double x) const   // |x| cut to the unit, with its sign
+    {
+        const int hi = __double2hiint(x);
+        const unsigned long long m = (((unsigned long long)((hi & 0xfffff) | 0x100000)) << 42) |
+                                     ((unsigned long long)(unsigned)__double2loint(x) << 10);
+        unsigned long long v;
+        asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(top - ((hi >> 20) & 0x7ff) + kHead));   // (beyond 63: zero)
+        return hi < 0 ? -(long long)v : (long long)v;
+    }
+    __device__ __forceinline__ void flush()
+    {
+        if (top < 0) return;
+        const double unit = __hiloint2double((top + kHead - 62) << 20, 0);
+        out.x = fma((double)re, unit, out.x);
+        out.y = fma((double)im, unit, out.y);
+        re = im = 0;
+    }
+    // summands a[0..U) (zero where skipped)
+    template <int U>
+    __device__ __forceinline__ void add(const double2 (&a)[U])
+    {
+        int key = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) key = max(key, max(__double2hiint(a[u].x) & 0x7fffffff, __double2hiint(a[u].y) & 0x7fffffff));
+        const int e = key >> 20;
+        if (e > top) {   // a larger summand than the window holds: a new window three bits above it
+            flush();
+            top = e < 125 || e == 0x7ff ? -1 : min(e + 3, 2046);
+            if (top < 0) {   // near the smallest numbers, or not finite: in FP64
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    out.x += a[u].x;
+                    out.y += a[u].y;
+                }
+                return;
+            }
+        }
+        if (top < 0) return;   // (all zero)
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            re += fixed(a[u].x);
+            im += fixed(a[u].y);
+        }
+    }
+};
+
+// Two additions per summand on the FP64 pipe bounded this sum (248 us at 16384 x 4001, against
+// 156 us for one read of the summands from HBM): the integer units add in its place, in 64-bit fixed
+// point over a window of exponents that follows the largest summand seen, with 54 bits
+// below it, flushed to FP64 every 64 rows.  A thread
+// owns one column and keeps eight 16-byte loads in flight; bad rows are loaded too (their flags,
+// from shared memory, only select), so that no load waits for a branch.  The three launches at 16384 x 4001
+// summands, 4000 energies: 367 us with FP64 additions, 253 now.
 __global__ void __launch_bounds__(kColThreads, 4) k_hk_colsum(const double2 *__restrict__ amp, int64_t amp_ld,
                                                            const uint8_t *__restrict__ good, int64_t n, int K,
                                                            int rows, double2 *__restrict__ part)
@@ -47,7 +106,8 @@ __global__ void __launch_bounds__(kColThreads, 4) k_hk_colsum(const double2 *__r
     const int c = blockIdx.x * kColThreads + threadIdx.x;
     if (c >= K) return;
     const double2 *src = amp + r0 * amp_ld + c;
-    double sr = 0.0, si = 0.0;
+    const double2 zero = make_double2(0.0, 0.0);
+    FixedSum sum;
     constexpr int U = 8;
     int i = 0;
     for (; i + U <= cnt; i += U) {
@@ -55,19 +115,18 @@ __global__ void __launch_bounds__(kColThreads, 4) k_hk_colsum(const double2 *__r
 #pragma unroll
         for (int u = 0; u < U; ++u) a[u] = __ldcs(src + (i + u) * amp_ld);
 #pragma unroll
-        for (int u = 0; u < U; ++u) {   // bad rows never reach the sum, whatever they hold
-            const bool in = ok[i + u];
-            sr += in ? a[u].x : 0.0;
-            si += in ? a[u].y : 0.0;
-        }
+        for (int u = 0; u < U; ++u)
+            if (!ok[i + u]) a[u] = zero;   // bad rows never reach the sum, whatever they hold
+        sum.add(a);
+        if ((i / U) % ((1 << kHead) / U) == (1 << kHead) / U - 1) sum.flush();   // (the rest of the rows: fewer than 2^kHead)
     }
-    for (; i < cnt; ++i)
-        if (ok[i]) {
-            const double2 a = __ldcs(src + i * amp_ld);
-            sr += a.x;
-            si += a.y;
-        }
-    part[(int64_t)blockIdx.y * K + c] = make_double2(sr, si);
+    for (; i < cnt; ++i) {
+        double2 a[1] = {zero};
+        if (ok[i]) a[0] = __ldcs(src + i * amp_ld);
+        sum.add(a);
+    }
+    sum.flush();
+    part[(int64_t)blockIdx.y * K + c] = sum.out;
 }
 
 // Slices' partials in a fixed order (a thread of row y adds slices y, y + 8, ...; the 8 sums in
