@@ -3,17 +3,18 @@
 // batched tensor-core evaluation over all trajectories).
 //
 // Per step of the fourth-order triple jump  D(c0) K(d0) D(c1) K(d1) D(c2) K(d2) D(c3):
-//   network at q  ->  stage 1: K(d0) D(c1)
-//   network at q  ->  stage 2: K(d1) D(c2)
-//   network at q  ->  stage 3: K(d2) D(c3), det M (stability), det A and the
-//                     continuous phase, the amplitude of Eq. I(E)_discreto,
-//                     then D(c0) of the next step
-// and stage 0 (before the first step) sets M = I, records c = 0 and drifts
-// D(c0).  A kick uses V, grad V and the Hessian of the analytic surface (FP64,
-// at q) plus those of the network (FP32, at q rounded to FP32).  State between
-// stages lives in HBM: p, q, S, theta (FP64, structure of arrays) and M (FP32,
-// element (r, c) of trajectory j at (r 2F + c) n + j).  One thread per
-// trajectory; the kick and drift stream M column by column.
+//   network at q  ->  k_mlp_kick, stage 1: K(d0) D(c1)
+//   network at q  ->  k_mlp_kick, stage 2: K(d1) D(c2)
+//   network at q  ->  k_mlp_kick, stage 3: K(d2) D(c3), det M (stability), and D(c0) of
+//                     the next step for q and S
+//                     k_mlp_record: det A and the continuous phase, the amplitude of
+//                     Eq. I(E)_discreto
+// k_mlp_start (before the first step) sets M = I, records c = 0 and drifts q by D(c0); M
+// is drifted by D(c0) when stage 1 reads it.  A kick uses V, grad V and the Hessian of the
+// analytic surface (FP64, at q) plus those of the network (FP32, at q rounded to FP32).  State
+// between stages lives in HBM: p, q, S, theta (FP64, structure of arrays) and M (FP32,
+// element (r, c) of trajectory j at (r 2F + c) n + j).
+#include "fp64_ops.cuh"
 #include "propagate_tpt.cuh"
 
 namespace scivr {
@@ -23,6 +24,8 @@ struct State {
     double *p, *q;        // [F][n]
     float *M;             // [(2F)^2][n]
     double *S, *theta, *arg_old, *stab;
+    double *qe, *Se;      // [F][n], [n]: q and S at the end of the step (q and S are a drift ahead)
+    float *det;           // [n] det M
     float *qf;            // [n][F] network input
     const float *Vm, *gm, *Hm;   // network output at qf: [n], [n][F], [n][F][F]
     int *step;            // device step counter (column of the amplitude)
@@ -61,274 +64,402 @@ __device__ __forceinline__ void record(const PropLaunch &L, int64_t j, int step,
     }
 }
 
-// Drift of (q, S) by td (FP64).
+// Set-up: M = I, the record of c = 0, the first drift of q and S.
 template <int F>
-__device__ __forceinline__ void drift_qs(double td, const double (&p)[F], double (&q)[F], double &S)
-{
-    double kin = 0.0;
-#pragma unroll
-    for (int a = 0; a < F; ++a) kin = fma(0.5 * p[a], p[a], kin);
-    S = fma(td, kin, S);
-#pragma unroll
-    for (int a = 0; a < F; ++a) q[a] = fma(td, p[a], q[a]);
-}
-
-// KIND 0: set-up and the first drift; 1: a kick and a drift (stage = 1, 2);
-// 3: the last kick and drift of a step, the per-step diagnostics, and the next
-// step's first drift.  COUPLED: the analytic part has coupling terms (else it
-// is the separable diagonal alone and its Hessian is diagonal).  The kick and
-// the drift update M in one pass over its columns (M_p -= tk H M_q, then
-// M_q += td M_p); the final stage also copies M into the work array of its LU.
-template <int F, int KIND, bool COUPLED>
-__global__ void __launch_bounds__(KIND == 3 ? 64 : 128, KIND == 3 ? 2 : 3) k_mlp_stage(const PropLaunch L, State st, int stage)
+__global__ void __launch_bounds__(128) k_mlp_start(const PropLaunch L, State st)
 {
     constexpr int N2 = 2 * F;
-    constexpr int NT = 64;                    // threads per block of the final stage
     const int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t n = L.n_traj;
     const PropArgs &A = L.args;
-    if (KIND == 1 && stage == 1 && j == 0) *st.step += 1;   // read by stage 3 of this step (later in stream order)
     if (j >= n) return;
-    float *Mj = st.M + j;                     // element (r, c) at Mj[(r 2F + c) n]
-    extern __shared__ __align__(16) uint8_t fin_smem[];
-    float *W = reinterpret_cast<float *>(fin_smem) + threadIdx.x;   // final stage: (r, c) at W[(r 2F + c) NT]
-    double p[F], q[F], S;
-    if (KIND == 0) {
-#pragma unroll
-        for (int a = 0; a < F; ++a) {
-            p[a] = L.p0[a * n + j];
-            q[a] = L.q0[a * n + j];
-        }
-        S = 0.0;
-        st.theta[j] = 0.0;
-        st.arg_old[j] = 0.0;
-        st.stab[j] = 0.0;
-        L.good[j] = 1;
-        record<F>(L, j, 0, p, q, 0.0, 0.0, 1.0);
-        const float td = A.tdrift_f[0];
-        for (int c = 0; c < N2; ++c)
-#pragma unroll
-            for (int a = 0; a < F; ++a) {
-                const float mp = a == c ? 1.0f : 0.0f;
-                const float mq = (F + a == c ? 1.0f : 0.0f) + td * mp;
-                Mj[((int64_t)a * N2 + c) * n] = mp;
-                Mj[((int64_t)(F + a) * N2 + c) * n] = mq;
-            }
-        drift_qs<F>(A.tdrift[0], p, q, S);
-    } else {
-#pragma unroll
-        for (int a = 0; a < F; ++a) {
-            p[a] = st.p[a * n + j];
-            q[a] = st.q[a * n + j];
-        }
-        S = st.S[j];
-        // kick d_{stage-1}: analytic part (FP64) + network part (FP32)
-        const double tk = A.tkick[stage - 1];
-        const float tkf = A.tkick_f[stage - 1];
-        float Hk[F][F];
-#pragma unroll
-        for (int a = 0; a < F; ++a)
-#pragma unroll
-            for (int b = 0; b < F; ++b) Hk[a][b] = tkf * st.Hm[(j * F + a) * F + b];
-        double V = (double)st.Vm[j];
-        if constexpr (COUPLED) {
-            double H[F][F], g[F], Va;
-            tpt::pes_fp64<F>(L.pes, q, H, g, Va);
-            V += Va;
-#pragma unroll
-            for (int a = 0; a < F; ++a) {
-                p[a] = fma(-tk, g[a] + (double)st.gm[j * F + a], p[a]);
-#pragma unroll
-                for (int b = 0; b < F; ++b) Hk[a][b] += (float)(tk * H[a][b]);
-            }
-        } else {
-            // separable diagonal only: V, grad V and the (diagonal) Hessian per mode
-#pragma unroll
-            for (int a = 0; a < F; ++a) {
-                double Va, ga, ha;
-                if (L.pes.diag_kind == SCIVR_DIAG_MORSE) {
-                    const double Dm = __ldg(L.pes.D + a), am = __ldg(L.pes.a + a);
-                    const double u = exp(-am * q[a]);
-                    const double omu = 1.0 - u;
-                    Va = Dm * omu * omu;
-                    ga = 2.0 * Dm * am * u * omu;
-                    ha = 2.0 * Dm * am * am * u * (2.0 * u - 1.0);
-                } else {
-                    const double w2 = __ldg(L.pes.omega + a) * __ldg(L.pes.omega + a);
-                    Va = 0.5 * w2 * q[a] * q[a];
-                    ga = w2 * q[a];
-                    ha = w2;
-                }
-                V += Va;
-                p[a] = fma(-tk, ga + (double)st.gm[j * F + a], p[a]);
-                Hk[a][a] += (float)(tk * ha);
-            }
-        }
-        S = fma(-tk, V, S);
-        const float td = A.tdrift_f[stage];
-#pragma unroll 1
-        for (int c = 0; c < N2; ++c) {
-            float mp[F], mq[F];
-#pragma unroll
-            for (int a = 0; a < F; ++a) {
-                mp[a] = Mj[((int64_t)a * N2 + c) * n];
-                mq[a] = Mj[((int64_t)(F + a) * N2 + c) * n];
-            }
-#pragma unroll
-            for (int a = 0; a < F; ++a) {
-                float hm = 0.0f;
-#pragma unroll
-                for (int b = 0; b < F; ++b) hm = fmaf(Hk[a][b], mq[b], hm);
-                mp[a] -= hm;
-            }
-#pragma unroll
-            for (int a = 0; a < F; ++a) {
-                mq[a] = fmaf(td, mp[a], mq[a]);
-                Mj[((int64_t)a * N2 + c) * n] = mp[a];
-                Mj[((int64_t)(F + a) * N2 + c) * n] = mq[a];
-                if (KIND == 3) {
-                    W[(a * N2 + c) * NT] = mp[a];
-                    W[((F + a) * N2 + c) * NT] = mq[a];
-                }
-            }
-        }
-        drift_qs<F>(A.tdrift[stage], p, q, S);
-    }
-    if (KIND == 3) {
-        const int step = *st.step;
-        bool good = L.good[j] != 0;
-        // stability |det(M)^2 - 1| (FP32 LU with partial pivoting) on the copy
-        // in shared memory, laid out [element][thread] (bank-conflict free)
-        // fully unrolled: every shared-memory offset is a compile-time constant
-        // relative to the row pointers, and the pivot row sits in registers
-        float det = 1.0f;
-#pragma unroll
-        for (int k = 0; k < N2; ++k) {
-            int piv = k;
-            float best = fabsf(W[(k * N2 + k) * NT]);
-#pragma unroll 1
-            for (int i = k + 1; i < N2; ++i) {
-                const float v = fabsf(W[(i * N2 + k) * NT]);
-                if (v > best) { best = v; piv = i; }
-            }
-            float rkv[N2];
-            float *rp = W + piv * N2 * NT;
-#pragma unroll
-            for (int c = k; c < N2; ++c) rkv[c] = rp[c * NT];
-            if (piv != k) {
-#pragma unroll
-                for (int c = k; c < N2; ++c) rp[c * NT] = W[(k * N2 + c) * NT];
-                det = -det;
-            }
-            det *= rkv[k];
-            const float inv = 1.0f / rkv[k];
-#pragma unroll 1
-            for (int i = k + 1; i < N2; ++i) {
-                float *ri = W + i * N2 * NT;
-                const float l = ri[k * NT] * inv;
-#pragma unroll
-                for (int c = k + 1; c < N2; ++c) ri[c * NT] = fmaf(-l, rkv[c], ri[c * NT]);
-            }
-        }
-        const float dev = isfinite(det) ? fabsf(fmaf(det, det, -1.0f)) : __int_as_float(0x7f800000);
-        const double stab = fmax(st.stab[j], (double)dev);
-        st.stab[j] = stab;
-        if (dev > A.stab_tol_f) good = false;
-        // Herman-Kluk prefactor determinant (FP64, complex LU with partial
-        // pivoting) in the same shared memory: (a, b) re at Z[(2 (a F + b)) NT], im at + NT
-        double *Z = reinterpret_cast<double *>(fin_smem) + threadIdx.x;
-        for (int a = 0; a < F; ++a)
-            for (int b = 0; b < F; ++b) {
-                const float mqq = Mj[((int64_t)(F + a) * N2 + F + b) * n];
-                const float mpp = Mj[((int64_t)a * N2 + b) * n];
-                const float mqp = Mj[((int64_t)(F + a) * N2 + b) * n];
-                const float mpq = Mj[((int64_t)a * N2 + F + b) * n];
-                Z[(2 * (a * F + b)) * NT] = 0.5 * fma(A.rg[a] * A.irg[b], (double)mqq, A.rg[b] * A.irg[a] * (double)mpp);
-                Z[(2 * (a * F + b) + 1) * NT] = 0.5 * fma(-A.rg[a] * A.rg[b], (double)mqp, A.irg[a] * A.irg[b] * (double)mpq);
-            }
-        tpt::cplx dA = {1.0, 0.0};
-#pragma unroll
-        for (int k = 0; k < F; ++k) {
-            int piv = k;
-            double best = Z[(2 * (k * F + k)) * NT] * Z[(2 * (k * F + k)) * NT] +
-                          Z[(2 * (k * F + k) + 1) * NT] * Z[(2 * (k * F + k) + 1) * NT];
-#pragma unroll 1
-            for (int i = k + 1; i < F; ++i) {
-                const double vr = Z[(2 * (i * F + k)) * NT], vi = Z[(2 * (i * F + k) + 1) * NT];
-                const double v = vr * vr + vi * vi;
-                if (v > best) { best = v; piv = i; }
-            }
-            tpt::cplx rkv[F];
-            double *rp = Z + 2 * piv * F * NT;
-#pragma unroll
-            for (int c = k; c < F; ++c) rkv[c] = {rp[2 * c * NT], rp[(2 * c + 1) * NT]};
-            if (piv != k) {
-#pragma unroll
-                for (int c = k; c < F; ++c) {
-                    rp[2 * c * NT] = Z[(2 * (k * F + c)) * NT];
-                    rp[(2 * c + 1) * NT] = Z[(2 * (k * F + c) + 1) * NT];
-                }
-                dA.re = -dA.re; dA.im = -dA.im;
-            }
-            dA = tpt::cmul(dA, rkv[k]);
-            const double rr = 1.0 / (rkv[k].re * rkv[k].re + rkv[k].im * rkv[k].im);
-            const tpt::cplx inv = {rkv[k].re * rr, -rkv[k].im * rr};
-#pragma unroll 1
-            for (int i = k + 1; i < F; ++i) {
-                double *ri = Z + 2 * i * F * NT;
-                const tpt::cplx l = tpt::cmul({ri[2 * k * NT], ri[(2 * k + 1) * NT]}, inv);
-#pragma unroll
-                for (int c = k + 1; c < F; ++c) {
-                    const tpt::cplx y = tpt::cfnma(l, rkv[c], {ri[2 * c * NT], ri[(2 * c + 1) * NT]});
-                    ri[2 * c * NT] = y.re;
-                    ri[(2 * c + 1) * NT] = y.im;
-                }
-            }
-        }
-        const double arg_new = atan2(dA.im, dA.re);
-        double d = arg_new - st.arg_old[j] + A.ref_step;
-        d = fma(-kTwoPi, rint(d * kInvTwoPi), d);
-        const double theta = st.theta[j] + d - A.ref_step;
-        st.theta[j] = theta;
-        st.arg_old[j] = arg_new;
-        bool finite = isfinite(S) && isfinite(theta);
-#pragma unroll
-        for (int a = 0; a < F; ++a) finite = finite && isfinite(p[a]) && isfinite(q[a]);
-        if (!finite) good = false;
-        L.good[j] = good ? 1 : 0;
-        record<F>(L, j, step, p, q, S, theta, hypot(dA.re, dA.im));
-        if (step == A.n_steps) {
-            const FinalDev &fo = L.fin;
-            if (fo.p) for (int a = 0; a < F; ++a) fo.p[a * n + j] = p[a];
-            if (fo.q) for (int a = 0; a < F; ++a) fo.q[a * n + j] = q[a];
-            if (fo.S) fo.S[j] = S;
-            if (fo.theta) fo.theta[j] = theta;
-            if (fo.detM) fo.detM[j] = (double)det;
-            if (fo.stab) fo.stab[j] = stab;
-            if (fo.detA) { fo.detA[2 * j] = dA.re; fo.detA[2 * j + 1] = dA.im; }
-            if (fo.M)
-                for (int r = 0; r < N2; ++r)
-                    for (int c = 0; c < N2; ++c) fo.M[j * N2 * N2 + r * N2 + c] = Mj[((int64_t)r * N2 + c) * n];
-            return;
-        }
-        // first drift of the next step
-        const float td0 = A.tdrift_f[0];
-#pragma unroll 1
-        for (int c = 0; c < N2; ++c)
-#pragma unroll
-            for (int a = 0; a < F; ++a) {
-                float *mq = Mj + ((int64_t)(F + a) * N2 + c) * n;
-                *mq = fmaf(td0, Mj[((int64_t)a * N2 + c) * n], *mq);
-            }
-        drift_qs<F>(A.tdrift[0], p, q, S);
-    }
+    double p[F], q[F];
 #pragma unroll
     for (int a = 0; a < F; ++a) {
-        st.p[a * n + j] = p[a];
-        st.q[a * n + j] = q[a];
-        st.qf[j * F + a] = (float)q[a];
+        p[a] = L.p0[a * n + j];
+        q[a] = L.q0[a * n + j];
     }
-    st.S[j] = S;
+    st.theta[j] = 0.0;
+    st.arg_old[j] = 0.0;
+    st.stab[j] = 0.0;
+    L.good[j] = 1;
+    record<F>(L, j, 0, p, q, 0.0, 0.0, 1.0);
+    for (int e = 0; e < N2 * N2; ++e) st.M[(int64_t)e * n + j] = e % (N2 + 1) == 0 ? 1.0f : 0.0f;
+    double kin = 0.0;
+#pragma unroll
+    for (int a = 0; a < F; ++a) {
+        kin = fma(0.5 * p[a], p[a], kin);
+        const double qa = fma(A.tdrift[0], p[a], q[a]);
+        st.p[a * n + j] = p[a];
+        st.q[a * n + j] = qa;
+        st.qf[j * F + a] = (float)qa;
+    }
+    st.S[j] = A.tdrift[0] * kin;
+}
+
+// One kick and the drift after it for 32 trajectories (a lane each) by F warps: warp b has mode b
+// and columns b and F + b of M in registers.  LAST: the step's last stage, which forms det M and
+// drifts q and S ahead by the next step's first drift.  COUPLED: the analytic part has coupling terms
+// (else it is the separable diagonal alone).
+//
+// What bounded the thread-per-trajectory form: 512 warps at 16384 trajectories, each with 324
+// dependent loads and stores of M, uncoalesced reads of the network's Hessian, 360 FP64 pipe slots,
+// and at the last stage det M's 2109 updates through shared memory.  With a warp per mode the FP64
+// work of a trajectory spreads over the SM's four pipes, all of a column is loaded at once, the
+// Hessian arrives coalesced through shared memory and det M runs in registers, its pivot column
+// passed through shared memory.
+// F = 9, 16384 trajectories: 38 -> 24 us
+// a kick, 39 with det M; three CTAs per SM (with two the det M stages' barriers take 18 us longer).
+template <int F, bool COUPLED, bool LAST>
+__global__ void __launch_bounds__(32 * F, 3) k_mlp_kick(const PropLaunch L, State st, int stage)
+{
+    constexpr int N2 = 2 * F, FF = F * F, P = F * (F + 1) / 2, NT = 32 * F;
+    const int lane = threadIdx.x & 31, b = threadIdx.x >> 5;
+    const int64_t n = L.n_traj, j0 = (int64_t)blockIdx.x * 32, j = j0 + lane;
+    const bool on = j < n;
+    const int64_t jl = on ? j : n - 1;
+    const PropArgs &A = L.args;
+    __shared__ float Hk[FF][33];                 // tau H
+    __shared__ double inc[F][32], inc2[F][32];   // the modes' shares of the action
+    __shared__ double exp2t[64];
+    __shared__ double qs[COUPLED ? F : 1][32], gc[COUPLED ? P : 1][32];
+    __shared__ unsigned keys[LAST ? F : 1][32];
+    __shared__ float piv[LAST ? N2 : 1][32];
+    if (stage == 1 && blockIdx.x == 0 && threadIdx.x == 0) *st.step += 1;   // read by k_mlp_record of this step
+
+    float m[2][N2];   // columns b and F + b
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int r = 0; r < N2; ++r) m[s][r] = st.M[((int64_t)r * N2 + s * F + b) * n + jl];
+    const double tk = A.tkick[stage - 1], td = A.tdrift[stage];
+    const float tkf = A.tkick_f[stage - 1], tdf = A.tdrift_f[stage];
+    double p = st.p[b * n + jl], q = st.q[b * n + jl];
+    const float gm = st.gm[jl * F + b];
+    {
+        const int64_t total = n * FF;   // the tile's Hessians, contiguous: F values a thread
+        float h[F];
+#pragma unroll
+        for (int k = 0; k < F; ++k) {
+            const int64_t e = j0 * FF + threadIdx.x + k * NT;
+            h[k] = e < total ? st.Hm[e] : 0.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < F; ++k) {
+            const int i = threadIdx.x + k * NT;
+            Hk[i % FF][i / FF] = tkf * h[k];
+        }
+    }
+    for (int i = threadIdx.x; i < 64; i += NT) exp2t[i] = kExp2Table[i];
+    if constexpr (COUPLED) qs[b][lane] = q;
+    __syncthreads();
+    // the separable diagonal: value, gradient, Hessian of mode b
+    double Va, ga, ha;
+    if (L.pes.diag_kind == SCIVR_DIAG_MORSE) {
+        const double Dm = __ldg(L.pes.D + b), am = __ldg(L.pes.a + b);
+        const double u = exp_t(-am * q, exp2t);
+        const double omu = 1.0 - u, c = 2.0 * Dm * am;
+        Va = Dm * omu * omu;
+        ga = c * (u * omu);
+        ha = c * am * u * fma(2.0, u, -1.0);
+    } else {
+        const double w2 = __ldg(L.pes.omega + b) * __ldg(L.pes.omega + b);
+        Va = 0.5 * w2 * q * q;
+        ga = w2 * q;
+        ha = w2;
+    }
+    if constexpr (COUPLED) {
+        // coupling entries e = (b, b) and every F-th of the others
+        auto entry = [&](int e, int r, int c) {
+            double h3 = 0.0, h4 = 0.0;
+            if (L.pes.has3)
+                for (int k = 0; k < F; ++k) h3 = fma(__ldg(L.pes.T3 + k * P + e), qs[k][lane], h3);
+            if (L.pes.has4) {
+                int kl = 0;
+                for (int k = 0; k < F; ++k) {
+                    double t = 0.0;   // sum over l of T4[(k, l)][e] q_l
+                    for (int l = k; l < F; ++l, ++kl) t = fma(__ldg(L.pes.T4 + kl * P + e), qs[l][lane], t);
+                    h4 = fma(t, qs[k][lane], h4);
+                }
+            }
+            gc[e][lane] = fma(0.5, h3, h4 * (1.0 / 3.0));
+            const double vc = fma(1.0 / 6.0, h3, h4 * (1.0 / 12.0));
+            Va = fma((r == c ? vc : 2.0 * vc) * qs[r][lane], qs[c][lane], Va);
+            const double h = r == c ? h3 + h4 + ha : h3 + h4;
+            const float hf = (float)(tk * h);
+            Hk[r * F + c][lane] += hf;
+            if (r != c) Hk[c * F + r][lane] += hf;
+        };
+        int turn = 0;
+        for (int r = 0, e = 0; r < F; ++r)
+            for (int c = r; c < F; ++c, ++e) {
+                if (r == c) {
+                    if (r == b) entry(e, r, c);
+                } else {
+                    if (turn == b) entry(e, r, c);
+                    turn = turn + 1 == F ? 0 : turn + 1;
+                }
+            }
+        __syncthreads();
+        for (int c = 0; c < F; ++c) {
+            const int lo = b < c ? b : c, hi = b < c ? c : b;
+            ga = fma(gc[lo * F - lo * (lo - 1) / 2 + hi - lo][lane], qs[c][lane], ga);
+        }
+    } else {
+        Hk[b * F + b][lane] += (float)(tk * ha);
+    }
+    p = fma(-tk, ga + widen(gm), p);
+    const double kin = 0.5 * p * p;
+    inc[b][lane] = fma(td, kin, -tk * Va);
+    if constexpr (LAST) inc2[b][lane] = A.tdrift[0] * kin;
+    q = fma(td, p, q);
+    if (on) {
+        st.p[b * n + j] = p;
+        double qn = q;
+        if constexpr (LAST) {
+            st.qe[b * n + j] = q;
+            qn = fma(A.tdrift[0], p, q);
+        }
+        st.q[b * n + j] = qn;
+        st.qf[j * F + b] = (float)qn;
+    }
+    __syncthreads();
+    if (b == 0 && on) {
+        double d = -tk * widen(st.Vm[j]);
+#pragma unroll
+        for (int a = 0; a < F; ++a) d += inc[a][lane];
+        double S = st.S[j] + d;
+        if constexpr (LAST) {
+            st.Se[j] = S;
+            double d2 = 0.0;
+#pragma unroll
+            for (int a = 0; a < F; ++a) d2 += inc2[a][lane];
+            S += d2;
+        }
+        st.S[j] = S;
+    }
+    // M: the step's first drift (stage 1), the kick M_p -= tk H M_q, the drift M_q += td M_p
+    if (stage == 1) {
+        const float td0 = A.tdrift_f[0];
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int a = 0; a < F; ++a) m[s][F + a] = fmaf(td0, m[s][a], m[s][F + a]);
+    }
+#pragma unroll 1
+    for (int a = 0; a < F; ++a) {   // M_p turns by one place an iteration: F turns restore it
+        float h0 = 0.0f, h1 = 0.0f;
+#pragma unroll
+        for (int c = 0; c < F; ++c) {
+            const float h = Hk[a * F + c][lane];
+            h0 = fmaf(h, m[0][F + c], h0);
+            h1 = fmaf(h, m[1][F + c], h1);
+        }
+        const float n0 = m[0][0] - h0, n1 = m[1][0] - h1;
+#pragma unroll
+        for (int c = 0; c + 1 < F; ++c) {
+            m[0][c] = m[0][c + 1];
+            m[1][c] = m[1][c + 1];
+        }
+        m[0][F - 1] = n0;
+        m[1][F - 1] = n1;
+    }
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int a = 0; a < F; ++a) m[s][F + a] = fmaf(tdf, m[s][a], m[s][F + a]);
+    if (on) {
+#pragma unroll
+        for (int s = 0; s < 2; ++s)
+#pragma unroll
+            for (int r = 0; r < N2; ++r) st.M[((int64_t)r * N2 + s * F + b) * n + j] = m[s][r];
+    }
+    if constexpr (LAST) {
+        // det M = det M^T by Gaussian elimination with partial pivoting: column c of M is row c of
+        // M^T.  A stage picks the unused row of the largest leading entry (keys: the leading bits of the
+        // magnitude, then the row); its entries reach the other warps through piv.  Rows move up by
+        // one place a stage (the entries that come in are never part of the result).
+        float det = 1.0f;
+        unsigned unused = (1u << N2) - 1u, parity = 0u;
+#pragma unroll 1
+        for (int k = 0; k < N2; ++k) {
+            unsigned key = 0u;
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const int col = s * F + b;
+                const unsigned kv = (__float_as_uint(fabsf(m[s][0])) & ~31u) | (unsigned)(col + 1);
+                if ((unused >> col) & 1u) key = max(key, kv);
+            }
+            keys[b][lane] = key;
+            __syncthreads();
+#pragma unroll
+            for (int a = 0; a < F; ++a) key = max(key, keys[a][lane]);
+            const int pc = (int)(key & 31u) - 1;
+            parity ^= (unsigned)__popc(unused & ((1u << pc) - 1u)) & 1u;
+            unused &= ~(1u << pc);
+#pragma unroll
+            for (int s = 0; s < 2; ++s)
+                if (pc == s * F + b) {
+#pragma unroll
+                    for (int i = 0; i < N2; ++i) piv[i][lane] = m[s][i];
+                }
+            __syncthreads();
+            const float pk = piv[0][lane];
+            det *= pk;
+            const float inv = 1.0f / pk;
+            const float l0 = m[0][0] * inv, l1 = m[1][0] * inv;
+#pragma unroll
+            for (int i = 1; i < N2; ++i) {   // (used rows are updated along: nothing reads them again)
+                const float w = piv[i][lane];
+                m[0][i - 1] = fmaf(-l0, w, m[0][i]);
+                m[1][i - 1] = fmaf(-l1, w, m[1][i]);
+            }
+        }
+        if (b == 0 && on) st.det[j] = parity ? -det : det;
+    }
+}
+
+// The records of a step, a thread per trajectory: stability flag, det A (FP64, complex LU with
+// partial pivoting in shared memory), the continuous phase, the amplitude.  Bounded by the FP64
+// pipe: a warp's instructions there take 64 cycles each, about 1700 of them at F = 9 (1200 in the
+// elimination, 324 to form A).  They were 3400 before the coefficients of A were formed once per
+// CTA, FP32 entries widened and pivots compared as integers and divisions and atan2 replaced.  The
+// loads of M are issued a row pair ahead (each waited for in turn, they took 130 us).
+// Four warps per CTA, one for each sub-partition (single-warp CTAs share them unevenly).  F = 9, 16384
+// trajectories: 74 us; the last kick, det M and the records together 178 -> 113 us.
+constexpr int kRecThreads = 128;
+
+template <int F>
+__global__ void __launch_bounds__(kRecThreads) k_mlp_record(const PropLaunch L, State st)
+{
+    constexpr int N2 = 2 * F, NT = kRecThreads;
+    extern __shared__ __align__(16) uint8_t rec_smem[];
+    double4 *coef = reinterpret_cast<double4 *>(rec_smem);                       // [F * F]
+    double2 *Z = reinterpret_cast<double2 *>(rec_smem + sizeof(double4) * F * F) + threadIdx.x;   // (a, b) at Z[(a F + b) NT]
+    const int64_t j = blockIdx.x * (int64_t)NT + threadIdx.x;
+    const int64_t n = L.n_traj;
+    const PropArgs &A = L.args;
+    for (int i = threadIdx.x; i < F * F; i += NT) {
+        const int a = i / F, b = i % F;
+        coef[i] = make_double4(0.5 * (A.rg[a] * A.irg[b]), 0.5 * (A.rg[b] * A.irg[a]), -0.5 * (A.rg[a] * A.rg[b]),
+                               0.5 * (A.irg[a] * A.irg[b]));
+    }
+    __syncthreads();
+    if (j >= n) return;
+    const float *Mj = st.M + j;               // element (r, c) at Mj[(r 2F + c) n]
+    const int step = *st.step;
+    bool good = L.good[j] != 0;
+    const float det = st.det[j];
+    const float dev = isfinite(det) ? fabsf(fmaf(det, det, -1.0f)) : __int_as_float(0x7f800000);
+    double stab = st.stab[j];
+    {
+        const double dv = widen(dev);         // non-negative: ordered as integers
+        if (__double_as_longlong(dv) > __double_as_longlong(stab)) stab = dv;
+        st.stab[j] = stab;
+    }
+    if (dev > A.stab_tol_f) good = false;
+    {
+        // rows a and F + a of M, the next pair in flight (all loads of a row ahead of widen's branches)
+        float mp[N2], mq[N2], np[N2], nq[N2];
+        auto load = [&](int a) {
+#pragma unroll
+            for (int c = 0; c < N2; ++c) {
+                np[c] = Mj[((int64_t)a * N2 + c) * n];
+                nq[c] = Mj[((int64_t)(F + a) * N2 + c) * n];
+            }
+        };
+        load(0);
+#pragma unroll 1
+        for (int a = 0; a < F; ++a) {
+#pragma unroll
+            for (int c = 0; c < N2; ++c) {
+                mp[c] = np[c];
+                mq[c] = nq[c];
+            }
+            if (a + 1 < F) load(a + 1);
+#pragma unroll
+            for (int b = 0; b < F; ++b) {
+                const double4 k = coef[a * F + b];
+                Z[(a * F + b) * NT] = make_double2(fma(k.x, widen(mq[F + b]), k.y * widen(mp[b])),
+                                                   fma(k.z, widen(mq[b]), k.w * widen(mp[F + b])));
+            }
+        }
+    }
+    tpt::cplx dA = {1.0, 0.0};
+#pragma unroll 1
+    for (int k = 0; k < F; ++k) {
+        // pivot by max(|re|, |im|), within a factor sqrt(2) of |z|
+        int piv = k, best = -1;
+        for (int i = k; i < F; ++i) {
+            const double2 v = Z[(i * F + k) * NT];
+            const int key = max(mag_key(v.x), mag_key(v.y));
+            if (key > best) { best = key; piv = i; }
+        }
+        double2 *rk = Z + k * F * NT, *rp = Z + piv * F * NT;
+        if (piv != k) {
+            for (int c = k; c < F; ++c) {
+                const double2 v = rp[c * NT];
+                rp[c * NT] = rk[c * NT];
+                rk[c * NT] = v;
+            }
+            dA.re = -dA.re; dA.im = -dA.im;
+        }
+        const tpt::cplx pk = {rk[k * NT].x, rk[k * NT].y};
+        dA = tpt::cmul(dA, pk);
+        const double rr = recip(fma(pk.re, pk.re, pk.im * pk.im));
+        const tpt::cplx inv = {pk.re * rr, -pk.im * rr};
+#pragma unroll 1
+        for (int i = k + 1; i < F; ++i) {
+            double2 *ri = Z + i * F * NT;
+            const tpt::cplx l = tpt::cmul({ri[k * NT].x, ri[k * NT].y}, inv);
+#pragma unroll 4
+            for (int c = k + 1; c < F; ++c) {
+                const tpt::cplx y = tpt::cfnma(l, {rk[c * NT].x, rk[c * NT].y}, {ri[c * NT].x, ri[c * NT].y});
+                ri[c * NT] = make_double2(y.re, y.im);
+            }
+        }
+    }
+    double arg_new;
+    {
+        const int e = max(mag_key(dA.re), mag_key(dA.im)) >> 20;   // to a larger part in [1, 2)
+        if (e < 64 || e > 1980) {
+            arg_new = atan2(dA.im, dA.re);
+        } else {
+            const double sc = __hiloint2double((2046 - e) << 20, 0);
+            const double x = dA.re * sc, y = dA.im * sc;
+            arg_new = arg_normal(x, y, (float)x, (float)y);
+        }
+    }
+    double d = arg_new - st.arg_old[j] + A.ref_step;
+    d = fma(-kTwoPi, rint(d * kInvTwoPi), d);
+    const double theta = st.theta[j] + d - A.ref_step;
+    st.theta[j] = theta;
+    st.arg_old[j] = arg_new;
+    double p[F], q[F];
+    const double S = st.Se[j];
+    bool finite = finite_bits(S) && finite_bits(theta);
+#pragma unroll
+    for (int a = 0; a < F; ++a) {
+        p[a] = st.p[a * n + j];
+        q[a] = st.qe[a * n + j];
+        finite = finite && finite_bits(p[a]) && finite_bits(q[a]);
+    }
+    if (!finite) good = false;
+    L.good[j] = good ? 1 : 0;
+    record<F>(L, j, step, p, q, S, theta, A.amplitude == SCIVR_AMP_HK ? hypot(dA.re, dA.im) : 1.0);
+    if (step == A.n_steps) {
+        const FinalDev &fo = L.fin;
+        if (fo.p) for (int a = 0; a < F; ++a) fo.p[a * n + j] = p[a];
+        if (fo.q) for (int a = 0; a < F; ++a) fo.q[a * n + j] = q[a];
+        if (fo.S) fo.S[j] = S;
+        if (fo.theta) fo.theta[j] = theta;
+        if (fo.detM) fo.detM[j] = (double)det;
+        if (fo.stab) fo.stab[j] = stab;
+        if (fo.detA) { fo.detA[2 * j] = dA.re; fo.detA[2 * j + 1] = dA.im; }
+        if (fo.M)
+            for (int r = 0; r < N2; ++r)
+                for (int c = 0; c < N2; ++c) fo.M[j * N2 * N2 + r * N2 + c] = Mj[((int64_t)r * N2 + c) * n];
+    }
 }
 
 inline size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -346,6 +477,9 @@ cudaError_t run(const PropLaunch &L, cudaStream_t s, int *n_launch)
     const size_t oT = o; o += a256((size_t)n * 8);
     const size_t oA = o; o += a256((size_t)n * 8);
     const size_t oB = o; o += a256((size_t)n * 8);
+    const size_t oQe = o; o += a256((size_t)F * n * 8);
+    const size_t oSe = o; o += a256((size_t)n * 8);
+    const size_t oDet = o; o += a256((size_t)n * 4);
     const size_t oQf = o; o += a256((size_t)n * F * 4);
     const size_t oV = o; o += a256((size_t)n * 4);
     const size_t oG = o; o += a256((size_t)n * F * 4);
@@ -364,6 +498,9 @@ cudaError_t run(const PropLaunch &L, cudaStream_t s, int *n_launch)
     st.theta = reinterpret_cast<double *>(b + oT);
     st.arg_old = reinterpret_cast<double *>(b + oA);
     st.stab = reinterpret_cast<double *>(b + oB);
+    st.qe = reinterpret_cast<double *>(b + oQe);
+    st.Se = reinterpret_cast<double *>(b + oSe);
+    st.det = reinterpret_cast<float *>(b + oDet);
     st.qf = reinterpret_cast<float *>(b + oQf);
     float *Vm = reinterpret_cast<float *>(b + oV), *gm = reinterpret_cast<float *>(b + oG);
     float *Hm = reinterpret_cast<float *>(b + oH);
@@ -372,17 +509,13 @@ cudaError_t run(const PropLaunch &L, cudaStream_t s, int *n_launch)
     int nl = 0;
     e = cudaMemsetAsync(st.step, 0, sizeof(int), s);
     if (e == cudaSuccess) e = mlp_prepare();
-    const unsigned blocks = (unsigned)((n + 127) / 128);
-    // final stage: one [element][thread] work array per thread, 16 F^2 bytes (the
-    // FP32 (2F)^2 LU and the FP64 complex F^2 LU need the same size)
-    const size_t fin_smem = (size_t)64 * 16 * F * F;
+    const unsigned tiles = (unsigned)((n + 31) / 32);
+    const size_t rec_smem = (size_t)(32 + 16 * kRecThreads) * F * F;   // A's coefficients, the threads' matrices
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_mlp_record<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rec_smem);
     if (e == cudaSuccess) {
-        e = cudaFuncSetAttribute(k_mlp_stage<F, 3, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fin_smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_mlp_stage<F, 3, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fin_smem);
-    }
-    if (e == cudaSuccess) {
-        k_mlp_stage<F, 0, false><<<blocks, 128, 0, s>>>(L, st, 0);
+        const bool cpl = L.pes.has3 || L.pes.has4;
+        k_mlp_start<F><<<(unsigned)((n + 127) / 128), 128, 0, s>>>(L, st);
         nl += 1;
         for (int step = 1; step <= L.args.n_steps && e == cudaSuccess; ++step) {
             for (int stage = 1; stage <= 3; ++stage) {
@@ -390,14 +523,14 @@ cudaError_t run(const PropLaunch &L, cudaStream_t s, int *n_launch)
                 e = mlp_eval(L.pes.mlp, F, n, st.qf, Vm, gm, Hm, b + oEval, s, &ne);
                 nl += ne;
                 if (e != cudaSuccess) break;
-                const bool cpl = L.pes.has3 || L.pes.has4;
                 if (stage < 3) {
-                    if (cpl) k_mlp_stage<F, 1, true><<<blocks, 128, 0, s>>>(L, st, stage);
-                    else k_mlp_stage<F, 1, false><<<blocks, 128, 0, s>>>(L, st, stage);
+                    if (cpl) k_mlp_kick<F, true, false><<<tiles, 32 * F, 0, s>>>(L, st, stage);
+                    else k_mlp_kick<F, false, false><<<tiles, 32 * F, 0, s>>>(L, st, stage);
                 } else {
-                    const unsigned b64 = (unsigned)((n + 63) / 64);
-                    if (cpl) k_mlp_stage<F, 3, true><<<b64, 64, fin_smem, s>>>(L, st, stage);
-                    else k_mlp_stage<F, 3, false><<<b64, 64, fin_smem, s>>>(L, st, stage);
+                    if (cpl) k_mlp_kick<F, true, true><<<tiles, 32 * F, 0, s>>>(L, st, stage);
+                    else k_mlp_kick<F, false, true><<<tiles, 32 * F, 0, s>>>(L, st, stage);
+                    k_mlp_record<F><<<(unsigned)((n + kRecThreads - 1) / kRecThreads), kRecThreads, rec_smem, s>>>(L, st);
+                    nl += 1;
                 }
                 nl += 1;
             }
