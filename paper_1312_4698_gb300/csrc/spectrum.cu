@@ -25,6 +25,7 @@ namespace {
 
 constexpr int B = 16, BLOCK = 2 * B + 1;         // samples on each side of a block's centre
 constexpr int WARPS = 4, COLS = 32;              // a CTA: 32 energies (a lane's own), four warps of rows
+constexpr int kMaxGridY = 65535;                 // energy tiles beyond it go to the grid's z
 
 __global__ void k_count_good(const uint8_t *__restrict__ good, int64_t n, int64_t *__restrict__ out,
                              int64_t *__restrict__ out2)
@@ -78,7 +79,9 @@ __global__ void __launch_bounds__(32 * WARPS) k_ft_fp64(const AmpRef amp, int64_
     __shared__ double red[WARPS][COLS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t row0 = (int64_t)blockIdx.x * ROWS;
-    const int col = blockIdx.y * COLS + lane;
+    const int tile = blockIdx.z * kMaxGridY + blockIdx.y;   // of energies
+    if ((int64_t)tile * COLS >= n_E) return;
+    const int col = tile * COLS + lane;
     const bool on = col < n_E;
     const int colc = on ? col : n_E - 1;
 
@@ -171,7 +174,7 @@ inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 // size; with 8, 608 tiles of 32 x 32 are where an uneven last round costs at most a fifth).
 int fp64_rows(int64_t n_traj, int n_E)
 {
-    const int64_t tiles = ((n_traj + 8 * WARPS - 1) / (8 * WARPS)) * ((n_E + COLS - 1) / COLS);
+    const int64_t tiles = ((n_traj + 8 * WARPS - 1) / (8 * WARPS)) * (((int64_t)n_E + COLS - 1) / COLS);
     return tiles >= 4 * 152 ? 8 : 2;
 }
 
@@ -210,7 +213,8 @@ cudaError_t launch_spectrum_fp64(AmpRef amp, int64_t amp_ld, const double *w,
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     k_twiddles<<<(unsigned)((n_tab + 255) / 256), 256, 0, s>>>(tab, n_blocks, n_E, E_min, dE, dt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    const dim3 grid((unsigned)n_mt, (unsigned)((n_E + COLS - 1) / COLS));
+    const unsigned tiles = (unsigned)(((int64_t)n_E + COLS - 1) / COLS);
+    const dim3 grid((unsigned)n_mt, tiles < kMaxGridY ? tiles : kMaxGridY, (tiles + kMaxGridY - 1) / kMaxGridY);
     if (fp64_rows(n_traj, n_E) == 8)
         k_ft_fp64<8><<<grid, 32 * WARPS, 0, s>>>(amp, amp_ld, tab, w, good, n_traj, K, n_blocks, n_E, part);
     else

@@ -46,6 +46,8 @@ def _surface(F, kind):
     *[(F, n, 37, "full", 0) for F in range(1, 10) for n in (1, 609, 1217, 2437)],
     (1, 4867, 5, "full", 0), (3, 4867, 37, "full", 1), (6, 4867, 1, "full", 0), (9, 2437, 3, "full", 1),
     (6, 609, 33, "full", 1), (9, 17, 31, "full", 1),
+    # a second warp makes the records: one and two sets of trajectories per CTA, 1, 2 and 3 steps in its two slots
+    (6, 150, 1, "full", 0), (6, 303, 2, "full", 0), (6, 305, 3, "full", 1), (9, 300, 33, "full", 0), (5, 305, 18, "full", 0),
     *[(6, 1217, 9, kind, 0) for kind in ("diagonal", "cubic", "quartic", "harmonic")],
 ])
 def test_group_sizes_agree_with_the_thread_schedule(F, n, steps, kind, amplitude):
