@@ -67,13 +67,19 @@ __device__ __forceinline__ double recip(double x)
 __device__ __forceinline__ int mag_key(double x) { return __double2hiint(x) & 0x7fffffff; }
 __device__ __forceinline__ bool finite_bits(double x) { return mag_key(x) < 0x7ff00000; }
 
-// An FP32 value as FP64 by its bits (denormals by conversion).
-__device__ __forceinline__ double widen(float x)
+// An FP32 value as FP64 by its bits; denormals become zero.
+__device__ __forceinline__ double widen_normal(float x)
 {
     const int b = __float_as_int(x), e = b & 0x7f800000, s = b & 0x80000000;
-    if (e == 0) return (b & 0x7fffffff) ? (double)x : __hiloint2double(s, 0);
     const int hi = ((b & 0x7fffffff) >> 3) + (e == 0x7f800000 ? 0x70000000 : 0x38000000);
-    return __hiloint2double(hi | s, b << 29);
+    return __hiloint2double(e ? hi | s : s, e ? b << 29 : 0);
+}
+
+// The same with denormals, by conversion (a branch: loads behind it do not move ahead of it).
+__device__ __forceinline__ double widen(float x)
+{
+    if ((unsigned)((__float_as_int(x) & 0x7fffffff) - 1) < 0x7fffffu) return (double)x;
+    return widen_normal(x);
 }
 
 __device__ const double2 kAngleTable[33] = {   // (cos, sin)(k pi / 64)

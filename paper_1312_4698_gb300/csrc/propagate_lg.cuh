@@ -810,11 +810,12 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
     Real pr = (Real)coord_get(p);   // the momentum as seen by the Real-precision bulk
     Coord S;                        // accumulated action (lane 0 of the group holds the total)
     coord_set(S, 0.0);
-    // per-job action in the job table: the double-FP32 pair in the 8 bytes of a double
+    // per-job action in the job table: the double-FP32 pair in the 8 bytes of a double (a phase: what a
+    // denormal word adds is nothing)
     auto sj_put = [&](int j, Coord v) { reinterpret_cast<float2 *>(sh.Sj)[j] = make_float2(v.hi, v.lo); };
     auto sj_get = [&](int j) -> double {
         const float2 v = reinterpret_cast<const float2 *>(sh.Sj)[j];
-        return widen(v.x) + widen(v.y);
+        return widen_normal(v.x) + widen_normal(v.y);
     };
     // column state: slot s of lane g holds column c = g + s G of M = d(p,q)/d(p0,q0) (c < 2F;
     // a slot past 2F holds a zero column)
@@ -910,8 +911,8 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                     const int e = g + i * G;
                     if (e < P) {
                         const Real v = sh.qr[t][ea[i]] * sh.qr[t][eb[i]];
-                        sh.qq[t][e] = v;
                         if constexpr (kTreg || kSplit) sh.xs[t][F3E + e] = v;
+                        else sh.qq[t][e] = v;
                         if constexpr (kCoop) xall[(F + e) * CH::XW + CH::slot(warp)] = (float)v;
                     }
                 }
@@ -1022,7 +1023,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                             sh.Gc[hx][a][b] = gce;
                             sh.Gc[hx][b][a] = gce;
                             const float vc = fmaf(1.0f / 6.0f, h3, h4 * (1.0f / 12.0f));
-                            vp = fmaf(a == b ? vc : 2.0f * vc, sh.qq[hx][e], vp);
+                            vp = fmaf(a == b ? vc : 2.0f * vc, sh.xs[hx][F3E + e], vp);
                         }
                     }
                     vpart = vp;   // lane ln belongs to group hx = t
@@ -1335,7 +1336,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                 di = {-di.hi, -di.lo};
             }
             if (r == 0) {
-                const double mr = widen(dr.hi) + widen(dr.lo), mi = widen(di.hi) + widen(di.lo);
+                const double mr = widen_normal(dr.hi) + widen_normal(dr.lo), mi = widen_normal(di.hi) + widen_normal(di.lo);
                 // (the power of two does not change the argument; with atan2 and conversions the FP64 pipe was
                 // busy 21 % of the time: F = 9, 65536 x 1000: 166.0 -> 161.1 ms, F = 15, 3001 x 501: 26.0 -> 24.9)
                 sh.argj[job] = arg_normal(mr, mi, dr.hi, di.hi);
@@ -1448,7 +1449,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                         rf = fmaf(-cc.pwf[a] * dp, dp, rf);
                         imf = fmaf(0.5f * (cc.p_eqf[x][a] + pa), dq, imf);
                     }
-                    double ph = fma(0.5, theta, widen(imf) + S);
+                    double ph = fma(0.5, theta, widen_normal(imf) + S);
                     if (A.amplitude == SCIVR_AMP_HK) {
                         // Herman-Kluk summand: |det A|^{1/2} and the division by the initial
                         // overlap times the sampling weight

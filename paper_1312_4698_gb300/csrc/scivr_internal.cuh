@@ -162,9 +162,9 @@ cudaError_t mlp_eval(const MlpWeightsDev &w, int F, int64_t n, const float *q, f
 cudaError_t mlp_loss_grad(const MlpWeightsDev &w, int F, int64_t n, const float *q, const float *Vref,
                           const float *gref, float alpha, float beta, float *grad, float *loss, void *scratch,
                           cudaStream_t s, int *n_launch);
-cudaError_t mlp_tile_weights(const MlpWeightsDev &w, cudaStream_t s);   // 4 launches
+cudaError_t mlp_tile_weights(const MlpWeightsDev &w, cudaStream_t s);   // 1 launch
 cudaError_t mlp_adamw(const MlpWeightsDev &w, const float *grad, float *m1, float *m2, float lr, float beta1,
-                      float beta2, float eps, float wd, float c1, float c2, cudaStream_t s);   // 5 launches
+                      float beta2, float eps, float wd, float c1, float c2, cudaStream_t s);   // 2 launches
 // Split-step propagation on a potential with a learned residual (pes.mlp.H != 0).
 cudaError_t launch_propagate_mlp(const PropLaunch &L, cudaStream_t s, int *n_launch);
 cudaError_t launch_pes_eval(const PesDev &pes, int64_t n, const double *q, int terms, double *V, double *g,
