@@ -31,69 +31,95 @@ inline int slice_rows(int64_t n, int K)
     return (int)rows;
 }
 
-// A column's running sum as a 64-bit integer in units of 2^(top + kHead - 1085), for summands whose
-// biased exponent is at most top; 2^kHead summands cannot overflow it, so it is flushed into FP64
-// that often.  top = -1: no window.
-constexpr int kHead = 6;
+// Sum of one column's real or imaginary parts as a 128-bit integer in units of 2^(top - 1023 - kLead):
+// a summand with the window's largest biased exponent, top, has its leading bit at kLead = 126 - kHead,
+// so that 2^kHead summands, all rows of a slice, cannot overflow it, and one up to 2^62 times smaller
+// keeps all of its bits (a smaller one is cut at the unit).  The window opens kRoom binades above the first
+// summand and moves on when a larger one arrives; the integer is then rounded, once and correctly,
+// into FP64, as it is at the end.  So a slice's sum carries one rounding where FP64 additions carry
+// one for every row, and a part keeps its own precision however large the other part is.
+// top = -1: no window.
+constexpr int kHead = 12, kLead = 126 - kHead, kRoom = 8;
+static_assert(kMaxSliceRows <= 1 << kHead, "a slice's rows fit the integer");
 
-struct FixedSum {
+struct WideSum {
     int top = -1;
-    long long re = 0, im = 0;
-    double2 out = make_double2(0.0, 0.0);   // what has left the integers, and summands beyond any window
+    unsigned neg = 0;                     // negative summands: each has been added as its complement, one unit low
+    unsigned long long lo = 0, hi = 0;
+    double out = 0.0;                     // what has left the integer, and summands beyond any window
 
-    __device__ __forceinline__ long long fixed(double x) const   // |x| cut to the unit, with its sign
+    __device__ __forceinline__ void put(double x)
     {
-        const int hi = __double2hiint(x);
-        const unsigned long long m = (((unsigned long long)((hi & 0xfffff) | 0x100000)) << 42) |
-                                     ((unsigned long long)(unsigned)__double2loint(x) << 10);
-        unsigned long long v;
-        asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"(top - ((hi >> 20) & 0x7ff) + kHead));   // (beyond 63: zero)
-        return hi < 0 ? -(long long)v : (long long)v;
+        const int h = __double2hiint(x);
+        const unsigned l = (unsigned)__double2loint(x);
+        // the mantissa with its leading bit at 63, then moved down 128 bits' worth (shifts past the width give zero)
+        const unsigned long long m = ((unsigned long long)(__funnelshift_l(l, (unsigned)h, 11) | 0x80000000u) << 32) | (l << 11);
+        const int s = top - ((h >> 20) & 0x7ff) + (127 - kLead);
+        unsigned long long vh, v1, v2;
+        asm("shr.u64 %0, %1, %2;" : "=l"(vh) : "l"(m), "r"(s));
+        asm("shl.b64 %0, %1, %2;" : "=l"(v1) : "l"(m), "r"(64 - s));
+        asm("shr.u64 %0, %1, %2;" : "=l"(v2) : "l"(m), "r"(s - 64));
+        const unsigned long long sign = (long long)(h >> 31);
+        const unsigned long long vl = (v1 | v2) ^ sign;
+        vh ^= sign;
+        neg += (unsigned)h >> 31;
+        asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;" : "+l"(lo), "+l"(hi) : "l"(vl), "l"(vh));
     }
     __device__ __forceinline__ void flush()
     {
         if (top < 0) return;
-        const double unit = __hiloint2double((top + kHead - 62) << 20, 0);
-        out.x = fma((double)re, unit, out.x);
-        out.y = fma((double)im, unit, out.y);
-        re = im = 0;
+        lo += neg;
+        hi += lo < neg ? 1 : 0;
+        const bool minus = (long long)hi < 0;
+        if (minus) {
+            lo = 0 - lo;
+            hi = ~hi + (lo == 0 ? 1 : 0);
+        }
+        int down = 0;                     // binades by which the leading bit is below 127
+        if (hi == 0) {
+            hi = lo;
+            lo = 0;
+            down = 64;
+        }
+        if (hi != 0) {
+            const int z = __clzll(hi);
+            if (z > 0) hi = (hi << z) | (lo >> (64 - z));
+            lo <<= z;
+            down += z;
+            const double v = __ull2double_rn(hi | (lo != 0 ? 1 : 0));   // (a bit below the 53 stands for all of them)
+            const double unit = __hiloint2double((top - kLead + 64 - down) << 20, 0);
+            out = fma(minus ? -v : v, unit, out);
+        }
+        lo = hi = 0;
+        neg = 0;
     }
-    // summands a[0..U) (zero where skipped)
+    // the summands x[0..U) (zero where skipped)
     template <int U>
-    __device__ __forceinline__ void add(const double2 (&a)[U])
+    __device__ __forceinline__ void add(const double (&x)[U])
     {
         int key = 0;
 #pragma unroll
-        for (int u = 0; u < U; ++u) key = max(key, max(__double2hiint(a[u].x) & 0x7fffffff, __double2hiint(a[u].y) & 0x7fffffff));
+        for (int u = 0; u < U; ++u) key = max(key, __double2hiint(x[u]) & 0x7fffffff);
         const int e = key >> 20;
-        if (e > top) {   // a larger summand than the window holds: a new window three bits above it
+        if (e > top) {
             flush();
-            top = e < 125 || e == 0x7ff ? -1 : min(e + 3, 2046);
+            top = e < 200 || e == 0x7ff ? -1 : min(e + kRoom, 2046);
             if (top < 0) {   // near the smallest numbers, or not finite: in FP64
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    out.x += a[u].x;
-                    out.y += a[u].y;
-                }
+                for (int u = 0; u < U; ++u) out += x[u];
                 return;
             }
         }
-        if (top < 0) return;   // (all zero)
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            re += fixed(a[u].x);
-            im += fixed(a[u].y);
-        }
+        for (int u = 0; u < U; ++u) put(x[u]);
     }
 };
 
-// Two additions per summand on the FP64 pipe bounded this sum (248 us at 16384 x 4001, against
-// 156 us for one read of the summands from HBM): the integer units add in its place, in 64-bit fixed
-// point over a window of exponents that follows the largest summand seen, with 54 bits
-// below it, flushed to FP64 every 64 rows.  A thread
-// owns one column and keeps eight 16-byte loads in flight; bad rows are loaded too (their flags,
-// from shared memory, only select), so that no load waits for a branch.  The three launches at 16384 x 4001
-// summands, 4000 energies: 367 us with FP64 additions, 253 now.
+// Two additions per summand on the FP64 pipe bounded this sum (248 us at 16384 x 4001, against 156 us for
+// one read of the summands from HBM), so the integer units
+// add in its place (WideSum).  A thread owns one column and keeps eight 16-byte loads in flight; bad
+// rows are loaded too (their flags, from shared memory, only select), so that no load waits for a
+// branch.  The three launches at 16384 x 4001 summands, 4000 energies: 373 us with FP64 additions, 300 now.
 __global__ void __launch_bounds__(kColThreads, 4) k_hk_colsum(const double2 *__restrict__ amp, int64_t amp_ld,
                                                            const uint8_t *__restrict__ good, int64_t n, int K,
                                                            int rows, double2 *__restrict__ part)
@@ -106,27 +132,37 @@ __global__ void __launch_bounds__(kColThreads, 4) k_hk_colsum(const double2 *__r
     const int c = blockIdx.x * kColThreads + threadIdx.x;
     if (c >= K) return;
     const double2 *src = amp + r0 * amp_ld + c;
-    const double2 zero = make_double2(0.0, 0.0);
-    FixedSum sum;
+    WideSum re, im;
     constexpr int U = 8;
     int i = 0;
     for (; i + U <= cnt; i += U) {
         double2 a[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) a[u] = __ldcs(src + (i + u) * amp_ld);
+        double x[U], y[U];
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-            if (!ok[i + u]) a[u] = zero;   // bad rows never reach the sum, whatever they hold
-        sum.add(a);
-        if ((i / U) % ((1 << kHead) / U) == (1 << kHead) / U - 1) sum.flush();   // (the rest of the rows: fewer than 2^kHead)
+        for (int u = 0; u < U; ++u) {
+            const bool take = ok[i + u];   // bad rows never reach the sum, whatever they hold
+            x[u] = take ? a[u].x : 0.0;
+            y[u] = take ? a[u].y : 0.0;
+        }
+        re.add(x);
+        im.add(y);
     }
+#pragma unroll 1
     for (; i < cnt; ++i) {
-        double2 a[1] = {zero};
-        if (ok[i]) a[0] = __ldcs(src + i * amp_ld);
-        sum.add(a);
+        double x[1] = {0.0}, y[1] = {0.0};
+        if (ok[i]) {
+            const double2 a = __ldcs(src + i * amp_ld);
+            x[0] = a.x;
+            y[0] = a.y;
+        }
+        re.add(x);
+        im.add(y);
     }
-    sum.flush();
-    part[(int64_t)blockIdx.y * K + c] = sum.out;
+    re.flush();
+    im.flush();
+    part[(int64_t)blockIdx.y * K + c] = make_double2(re.out, im.out);
 }
 
 // Slices' partials in a fixed order (a thread of row y adds slices y, y + 8, ...; the 8 sums in
