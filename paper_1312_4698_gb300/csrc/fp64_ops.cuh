@@ -63,6 +63,18 @@ __device__ __forceinline__ double recip(double x)
     return fma(r, e, r);
 }
 
+// (cos, sin)(E c dt) for a whole number c.  The phase is 2^-53 of itself off its exact value (2e-13 at 2000
+// radians); where many samples share the factor, that error does not average out as it does with a
+// phase for each, so it is put back to first order: E (c dt) = x + d, d from the products' exact remainders.
+__device__ __forceinline__ double2 unit_phase(double E, double c, double dt)
+{
+    const double t = c * dt, x = E * t;
+    const double d = fma(E, fma(c, dt, -t), fma(E, t, -x));
+    double s, co;
+    sincos(x, &s, &co);
+    return make_double2(fma(-s, d, co), fma(co, d, s));
+}
+
 // Order of magnitudes as integers (comparisons run on the FP64 pipe otherwise).
 __device__ __forceinline__ int mag_key(double x) { return __double2hiint(x) & 0x7fffffff; }
 __device__ __forceinline__ bool finite_bits(double x) { return mag_key(x) < 0x7ff00000; }

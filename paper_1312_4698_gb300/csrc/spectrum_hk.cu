@@ -8,6 +8,7 @@
 // partials are added in slice order.
 #include <cmath>
 
+#include "fp64_ops.cuh"
 #include "scivr_internal.cuh"
 
 namespace scivr {
@@ -119,7 +120,7 @@ struct WideSum {
 // one read of the summands from HBM), so the integer units
 // add in its place (WideSum).  A thread owns one column and keeps eight 16-byte loads in flight; bad
 // rows are loaded too (their flags, from shared memory, only select), so that no load waits for a
-// branch.  The three launches at 16384 x 4001 summands, 4000 energies: 373 us with FP64 additions, 300 now.
+// branch.  The three launches at 16384 x 4001 summands, 4000 energies: 373 us with FP64 additions, 306 now (with the transform below).
 __global__ void __launch_bounds__(kColThreads, 4) k_hk_colsum(const double2 *__restrict__ amp, int64_t amp_ld,
                                                            const uint8_t *__restrict__ good, int64_t n, int K,
                                                            int rows, double2 *__restrict__ part)
@@ -217,11 +218,15 @@ __global__ void __launch_bounds__(kRedX *kRedY) k_hk_reduce(const double2 *__res
 //   t = E dt, z = e^{i t}, A = C_{c_m + r} + C_{c_m - r}, B = i (C_{c_m + r} - C_{c_m - r}),
 // so that a term costs two multiply-adds; A and B do not depend on the energy.  A thread owns
 // an energy, a warp G consecutive blocks at a time (its A and B in shared memory, read as
-// broadcasts), the kFtWarps warps of a CTA share 32 energies' blocks.  z^r comes from up to R
-// complex products, the z^{c_m} of a warp's G blocks from a sine and cosine of E (c dt) at the
-// first centre and at most G - 1 products, so that no rounding of E dt is multiplied by c.
-// 4001 samples x 4000 energies: 4234 -> 86 us (6.4e7 multiply-adds; the FP64 pipe takes 61 us for them).
+// broadcasts), the kFtWarps warps of a CTA share 32 energies' blocks.  The powers z^r and the z^{c_m} of
+// a warp's G blocks are complex products of a sine and cosine at r = 1, 8, 16, 24 and at the
+// first centre, at most seven on end.  Whatever error these factors have is shared by many samples and does
+// not average out, so the phases' own rounding is put back (unit_phase) and the products are kept few.
+// With rounded phases and 30 products on end, spectra of 200 to 4000 samples were up to five times less
+// accurate than with a phase for every sample; they are as accurate now, or more.
+// 4001 samples x 4000 energies: 4234 -> 93 us (6.4e7 multiply-adds; the FP64 pipe takes 61 us for them).
 constexpr int kFtR = 31, kFtW = 2 * kFtR + 1, kFtG = 8, kFtWarps = 8;
+constexpr int kFtAnew = 8;   // powers of z from one sine and cosine
 
 __device__ __forceinline__ double2 hk_cmul(double2 x, double2 y)
 {
@@ -244,8 +249,7 @@ __global__ void __launch_bounds__(32 * kFtWarps) k_hk_ft(const double2 *__restri
         if (c == 0) { v.x *= 0.5; v.y *= 0.5; }   // the folded transform's half weight at t = 0
         return v;
     };
-    double2 z;
-    sincos(E * dt, &z.y, &z.x);
+    const double2 z = unit_phase(E, 1.0, dt), step = unit_phase(E, kFtW, dt);
     double acc = 0.0;
     for (int grp = warp; grp < n_grp; grp += kFtWarps) {
         __syncwarp();
@@ -269,11 +273,9 @@ __global__ void __launch_bounds__(32 * kFtWarps) k_hk_ft(const double2 *__restri
                 S[g].x = fma(A.x, zr.x, fma(B.x, zr.y, S[g].x));
                 S[g].y = fma(A.y, zr.x, fma(B.y, zr.y, S[g].y));
             }
-            zr = hk_cmul(zr, z);
+            zr = r % kFtAnew == kFtAnew - 1 ? unit_phase(E, r + 1, dt) : hk_cmul(zr, z);
         }
-        double2 ph, step;
-        sincos(E * ((grp * kFtG * kFtW + kFtR) * dt), &ph.y, &ph.x);
-        sincos(E * (kFtW * dt), &step.y, &step.x);
+        double2 ph = unit_phase(E, grp * kFtG * kFtW + kFtR, dt);
 #pragma unroll
         for (int g = 0; g < kFtG; ++g) {
             acc = fma(S[g].x, ph.x, fma(-S[g].y, ph.y, acc));
