@@ -226,19 +226,27 @@ __global__ void __launch_bounds__(256) k_czt_tables(CztTables tb, int log2L, int
 
 // V = FFT(v), one of kVParts blocks of the transform's fourth stage per CTA: the residue of
 // v modulo z^(L/16) - rho (15 multiply-adds a point instead of the first four stages), then the
-// remaining stages on L / 16 points.  One CTA for the whole transform took 190 us.
+// remaining stages on L / 16 points.  One CTA for the whole transform took 190 us.  The powers of rho are
+// each rounded once: Horner's rule multiplies rho's rounding by up to 15, and V, which every trajectory
+// shares, came out 3 to 8 times less accurate than by the stages.
 __global__ void __launch_bounds__(256) k_czt_kernel_fft(CztTables tb, int log2L)
 {
-    __shared__ double2 x[(1 << kLog2Max) / kVParts];
+    __shared__ double2 x[(1 << kLog2Max) / kVParts], rho[kVParts];
     const int L = 1 << log2L, n = L / kVParts, part = blockIdx.x;
-    double s, c;
-    sincospi(-2.0 * (double)__brev((unsigned)part) * 0x1p-32, &s, &c);
-    const double2 rho = make_double2(c, s);
+    if (threadIdx.x < kVParts) {
+        // rho = exp(-2 pi i r / 16), r the bits of part from the other end
+        const int r = (int)(__brev((unsigned)part) >> 28) * (int)threadIdx.x % kVParts;
+        double s, c;
+        sincospi(-2.0 * r / kVParts, &s, &c);
+        rho[threadIdx.x] = make_double2(c, s);
+    }
+    __syncthreads();
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
-        double2 y = tb.v[k + (kVParts - 1) * n];
-        for (int j = kVParts - 2; j >= 0; --j) {
-            const double2 u = tb.v[k + j * n];
-            y = make_double2(fma(-rho.y, y.y, fma(rho.x, y.x, u.x)), fma(rho.y, y.x, fma(rho.x, y.y, u.y)));
+        double2 y = tb.v[k];
+#pragma unroll
+        for (int j = 1; j < kVParts; ++j) {
+            const double2 u = tb.v[k + j * n], w = rho[j];
+            y = make_double2(fma(-w.y, u.y, fma(w.x, u.x, y.x)), fma(w.y, u.x, fma(w.x, u.y, y.y)));
         }
         x[k] = y;
     }
