@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(32 * F, 3) k_mlp_kick(const PropLaunch L, Stat
     const PropArgs &A = L.args;
     __shared__ float Hk[FF][33];                 // tau H
     __shared__ double inc[F][32], inc2[F][32];   // the modes' shares of the action
-    __shared__ double exp2t[64];
+    __shared__ double2 exp2t[64];
     __shared__ double qs[COUPLED ? F : 1][32], gc[COUPLED ? P : 1][32];
     __shared__ unsigned keys[LAST ? F : 1][32];
     __shared__ float piv[LAST ? N2 : 1][32];

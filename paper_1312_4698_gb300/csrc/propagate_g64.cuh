@@ -76,7 +76,7 @@ struct CtaShared {
     double na[F];                             // -a
     double qw[F], pw[F];
     double p_eq[SCIVR_MAX_CHI][F], q_eq[SCIVR_MAX_CHI][F];
-    double exp2t[64];
+    alignas(16) double2 exp2t[64];
 };
 
 template <int F, int G>
