@@ -416,7 +416,11 @@ template <int LOGL>
 cudaError_t launch_czt(const CztLayout &Y, AmpRef amp, int64_t amp_ld, const double *w, const uint8_t *good,
                        int64_t n_traj, int n_E, const CztTables &tb, cudaStream_t s)
 {
-    const cudaError_t e = cudaFuncSetAttribute(k_czt<LOGL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Y.smem);
+    // the largest size any grid needs: the limit is the kernel's, shared by all host threads, and one
+    // set to this call's size could be lowered by another thread before the launch
+    constexpr size_t most = sizeof(double2) * ((size_t)1 << LOGL) + sizeof(double) * kCztMaxEnergies;
+    static_assert(most <= 227 * 1024, "the vector and the sums fit an SM's shared memory");
+    const cudaError_t e = cudaFuncSetAttribute(k_czt<LOGL>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (e != cudaSuccess) return e;
     k_czt<LOGL><<<Y.n_cta, (1 << LOGL) / 16, Y.smem, s>>>(amp, amp_ld, w, good, n_traj, Y.K, n_E, Y.n_blk, Y.nb, tb);
     return cudaGetLastError();
