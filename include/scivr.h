@@ -276,11 +276,12 @@ int scivr_propagate(scivr_pes pes, const scivr_prop_params *prm, int64_t n_traj,
  * - (k - c)^2)/2 (w = dE dt): a convolution by FP64 FFTs of L = 1024 .. 8192 points per
  * trajectory, about 10 L log2 L flops instead of 8 K n_E, with FP64 rounding; it takes
  * n_steps + 1 <= 7169 and n_E <= 12288 (SCIVR_EUNSUPPORTED otherwise; energies beyond
- * L + 1 - (n_steps + 1) are transformed in blocks) and allocates up to about 600 KB plus
- * 8 n_E bytes for each of its one to four CTAs per SM.  Allocates
+ * L + 1 - (n_steps + 1) are transformed in blocks).  Allocates
  * stream-ordered scratch (cudaMallocAsync): FP64 mode about
- * 16 (n_steps+1) n_E + 8 n_E ceil(n_traj/64) bytes; tensor-core modes about
- * 4 d (n_steps+1) (n_traj + 2 n_E) + 8 n_E ceil(n_traj/128) bytes, d digits.
+ * 16 n_E (16 + ceil((n_steps+1)/33)) + 8 n_E ceil(n_traj/32) bytes (ceil(n_traj/8) where
+ * ceil(n_traj/32) ceil(n_E/32) < 608); tensor-core modes about
+ * 4 d (n_steps+1) (n_traj + 2 n_E) + 8 n_E ceil(n_traj/128) bytes, d digits; SCIVR_FT_CZT64 about
+ * 48 L + 16 (n_steps+1) ceil(n_E/(L - n_steps)) + 8 n_E C bytes, C = one to four CTAs per SM.
  * Errors: SCIVR_EINVAL (NULL pointers, n_traj < 1, n_steps < 1, n_E < 2,
  * E_max <= E_min, dt <= 0, amp_ld < n_steps + 1), SCIVR_EUNSUPPORTED
  * (amp_prec or ft_mode not built), SCIVR_ENOMEM.  A tensor-core wait that
