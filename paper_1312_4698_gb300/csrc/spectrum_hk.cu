@@ -227,14 +227,20 @@ __global__ void __launch_bounds__(kRedX *kRedY) k_hk_reduce(const double2 *__res
 // 4001 samples x 4000 energies: 4234 -> 93 us (6.4e7 multiply-adds; the FP64 pipe takes 61 us for them).
 constexpr int kFtR = 31, kFtW = 2 * kFtR + 1, kFtG = 8, kFtWarps = 8;
 constexpr int kFtAnew = 8;   // powers of z from one sine and cosine
+// Few samples take a sine and cosine per term, shared out over the CTA's warps.  Blocks take 50 us
+// whatever one warp's hold (up to 504 samples); terms 0.3 us a sample while each CTA has an SM to itself, and
+// with more CTAs the instructions count, 50 a term against 1500 for the blocks.  The three launches,
+// blocks / terms: 400 energies, 2 samples 61 / 9 us, 128 samples 62 / 48; 4900 energies, 64 samples
+// 66 / 48; 30000 energies, 64 samples 184 / 149.
+inline int few_samples(int n_E) { return n_E <= 32 * 152 ? 128 : 80; }
 
 __device__ __forceinline__ double2 hk_cmul(double2 x, double2 y)
 {
     return make_double2(fma(x.x, y.x, -x.y * y.y), fma(x.x, y.y, x.y * y.x));
 }
 
-__global__ void __launch_bounds__(32 * kFtWarps) k_hk_ft(const double2 *__restrict__ C, int K, double dt, double E_min,
-                                                         double dE, int n_E, double *__restrict__ I_out)
+__global__ void __launch_bounds__(32 * kFtWarps) k_hk_ft(const double2 *__restrict__ C, int K, int few, double dt,
+                                                         double E_min, double dE, int n_E, double *__restrict__ I_out)
 {
     extern __shared__ __align__(16) double2 ab_all[];   // [warp][r][g]{A, B}
     __shared__ double part[kFtWarps][32];
@@ -249,37 +255,44 @@ __global__ void __launch_bounds__(32 * kFtWarps) k_hk_ft(const double2 *__restri
         if (c == 0) { v.x *= 0.5; v.y *= 0.5; }   // the folded transform's half weight at t = 0
         return v;
     };
-    const double2 z = unit_phase(E, 1.0, dt), step = unit_phase(E, kFtW, dt);
     double acc = 0.0;
-    for (int grp = warp; grp < n_grp; grp += kFtWarps) {
-        __syncwarp();
-        for (int i = lane; i < (kFtR + 1) * kFtG; i += 32) {
-            const int r = i / kFtG, c = (grp * kFtG + i % kFtG) * kFtW + kFtR;
-            const double2 u = at(c + r), v = r ? at(c - r) : make_double2(0.0, 0.0);
-            ab[2 * i] = make_double2(u.x + v.x, u.y + v.y);
-            ab[2 * i + 1] = make_double2(v.y - u.y, u.x - v.x);
+    if (K <= few) {
+        for (int c = warp; c < K; c += kFtWarps) {
+            const double2 v = at(c), ph = unit_phase(E, c, dt);
+            acc = fma(v.x, ph.x, fma(-v.y, ph.y, acc));
         }
-        __syncwarp();
-        double2 S[kFtG];
+    } else {
+        const double2 z = unit_phase(E, 1.0, dt), step = unit_phase(E, kFtW, dt);
+        for (int grp = warp; grp < n_grp; grp += kFtWarps) {
+            __syncwarp();
+            for (int i = lane; i < (kFtR + 1) * kFtG; i += 32) {
+                const int r = i / kFtG, c = (grp * kFtG + i % kFtG) * kFtW + kFtR;
+                const double2 u = at(c + r), v = r ? at(c - r) : make_double2(0.0, 0.0);
+                ab[2 * i] = make_double2(u.x + v.x, u.y + v.y);
+                ab[2 * i + 1] = make_double2(v.y - u.y, u.x - v.x);
+            }
+            __syncwarp();
+            double2 S[kFtG];
 #pragma unroll
-        for (int g = 0; g < kFtG; ++g) S[g] = ab[2 * g];
-        double2 zr = z;
+            for (int g = 0; g < kFtG; ++g) S[g] = ab[2 * g];
+            double2 zr = z;
 #pragma unroll 1
-        for (int r = 1; r <= kFtR; ++r) {
-            const double2 *row = ab + 2 * r * kFtG;
+            for (int r = 1; r <= kFtR; ++r) {
+                const double2 *row = ab + 2 * r * kFtG;
+#pragma unroll
+                for (int g = 0; g < kFtG; ++g) {
+                    const double2 A = row[2 * g], B = row[2 * g + 1];
+                    S[g].x = fma(A.x, zr.x, fma(B.x, zr.y, S[g].x));
+                    S[g].y = fma(A.y, zr.x, fma(B.y, zr.y, S[g].y));
+                }
+                zr = r % kFtAnew == kFtAnew - 1 ? unit_phase(E, r + 1, dt) : hk_cmul(zr, z);
+            }
+            double2 ph = unit_phase(E, grp * kFtG * kFtW + kFtR, dt);
 #pragma unroll
             for (int g = 0; g < kFtG; ++g) {
-                const double2 A = row[2 * g], B = row[2 * g + 1];
-                S[g].x = fma(A.x, zr.x, fma(B.x, zr.y, S[g].x));
-                S[g].y = fma(A.y, zr.x, fma(B.y, zr.y, S[g].y));
+                acc = fma(S[g].x, ph.x, fma(-S[g].y, ph.y, acc));
+                ph = hk_cmul(ph, step);
             }
-            zr = r % kFtAnew == kFtAnew - 1 ? unit_phase(E, r + 1, dt) : hk_cmul(zr, z);
-        }
-        double2 ph = unit_phase(E, grp * kFtG * kFtW + kFtR, dt);
-#pragma unroll
-        for (int g = 0; g < kFtG; ++g) {
-            acc = fma(S[g].x, ph.x, fma(-S[g].y, ph.y, acc));
-            ph = hk_cmul(ph, step);
         }
     }
     part[warp][lane] = acc;
@@ -320,7 +333,7 @@ cudaError_t launch_spectrum_hk(const double2 *amp, int64_t amp_ld, const uint8_t
     k_hk_colsum<<<dim3(cols, slices), kColThreads, 0, s>>>(amp, amp_ld, good, n_traj, K, rows, part);
     k_hk_reduce<<<(K + kRedX - 1) / kRedX, dim3(kRedX, kRedY), 0, s>>>(part, slices, K, good, n_traj, n_good_out, C);
     const double dE = n_E > 1 ? (E_max - E_min) / (n_E - 1) : 0.0;
-    k_hk_ft<<<(n_E + 31) / 32, 32 * kFtWarps, kFtSmem, s>>>(C, K, dt, E_min, dE, n_E, I_out);
+    k_hk_ft<<<(n_E + 31) / 32, 32 * kFtWarps, kFtSmem, s>>>(C, K, few_samples(n_E), dt, E_min, dE, n_E, I_out);
     *n_launch = 3;
     return cudaGetLastError();
 }
