@@ -20,7 +20,7 @@
 //   phase 4 (job-parallel): overlap <chi|p q>, action, phase and the amplitude;
 //     each group writes C consecutive samples of its row.
 //
-// Real = float: monodromy, potential, det M, A, the overlap and each step's action
+// FP32: monodromy, potential, det M, A, the overlap and each step's action
 // increment; positions, momenta, the accumulated action and the elimination that gives det A
 // in double-FP32; the continuous phase in FP64; the amplitude's phase is reduced modulo 2 pi
 // in FP64 and its sine, cosine and magnitude are evaluated in FP32.
@@ -49,17 +49,10 @@ __host__ __device__ constexpr int pidx(int a, int b)
     return a * F - a * (a - 1) / 2 + (b - a);
 }
 
-template <typename Real> __device__ __forceinline__ Real rexp(Real x);
-template <> __device__ __forceinline__ float rexp<float>(float x) { return expf(x); }
-
-template <typename Real> struct Vec2;
-template <> struct Vec2<float> { using T = float2; };
-
 // Storage of one entry of the Herman-Kluk matrix A during its elimination: a double-FP32
 // complex (re.hi, im.hi, re.lo, im.lo) -- the entries are formed in FP32 and eliminated to
 // FP64-class accuracy, the real and imaginary words side by side for packed FP32 arithmetic.
-template <typename Real> struct AEntry;
-template <> struct AEntry<float> { using T = float4; };
+using AEntry = float4;
 
 // ---- double-FP32 arithmetic (hi + lo, |lo| <= ulp(hi)/2): error-free sum and
 // product of two floats (Knuth's TwoSum, the FMA form of Dekker's TwoProduct) and
@@ -237,7 +230,7 @@ __device__ __forceinline__ int jswz(int r, int j) { return j ^ (r & (JOBS >= 16 
 
 // Steps per chunk of a lane group.  Phases 2-4 work on T * C jobs (trajectory, step) per warp.
 // The double-FP32 elimination keeps two FP32 words per real entry, so chunks are short (8 steps; 4
-// above F = 12) and 32 / (T * C) lanes share a job's elimination by rows.
+// at F = 9 and 13..15, 2 at 16, 1 above) and 32 / (T * C) lanes share a job's elimination by rows.
 // Mixed path: steps between stability tests (a multiple of every mixed chunk length).
 // The flag is sticky and a bad trajectory is dropped whole, so a coarser test differs
 // from the per-step one only for a deviation that crosses the threshold and falls back
@@ -245,7 +238,7 @@ __device__ __forceinline__ int jswz(int r, int j) { return j ^ (r & (JOBS >= 16 
 // 16-step cadences equal the per-step ones).
 constexpr int kDetMEvery = 16;
 
-template <int F, int G, typename Real> __host__ __device__ constexpr int lg_chunk()
+template <int F, int G> __host__ __device__ constexpr int lg_chunk()
 {
     return G == 32 && F > 16 ? 1 : (G == 32 && F > 15 ? 2 : ((G == 32 && F > 12) || (G == 16 && F > 8) ? 4 : 8));
 }
@@ -263,88 +256,50 @@ template <int F, int G> __host__ __device__ constexpr int lg_warps() { return G 
 // CTAs per SM against three) and at F = 9 (12 %, three against two).
 template <int F> __host__ __device__ constexpr bool lg_tensor_regs() { return F == 7 || F == 8; }
 
-template <int F, int G, typename Real> __host__ __device__ constexpr int lg_min_ctas()
+template <int F, int G> __host__ __device__ constexpr int lg_min_ctas()
 {
     // register-held tensors: two CTAs per SM at F = 8, 9 (up to 255 registers), three at F = 6, 7
     if constexpr (G == 16 && F >= 6 && lg_tensor_regs<F>()) return F >= 8 ? 2 : 3;
-    return F > 9 ? 1 : (sizeof(Real) == 4 && 2 * F > G ? 3 : 4);
-}
-
-// 16-byte vectors of Real for shared-memory loads.
-template <typename Real> struct V16;
-template <> struct V16<float> { using T = float4; static constexpr int N = 4; };
-
-template <typename Real>
-__device__ __forceinline__ Real vcomp(const typename V16<Real>::T &v, int j)
-{
-    if constexpr (V16<Real>::N == 4) return j == 0 ? v.x : j == 1 ? v.y : j == 2 ? v.z : v.w;
-    else return j == 0 ? v.x : v.y;
+    return F > 9 ? 1 : (2 * F > G ? 3 : 4);
 }
 
 // Length of a row padded to whole 16-byte vectors.
-template <typename Real>
-__host__ __device__ constexpr int vec_len(int n)
-{
-    return (n + V16<Real>::N - 1) / V16<Real>::N * V16<Real>::N;
-}
+__host__ __device__ constexpr int vec_len(int n) { return (n + 3) / 4 * 4; }
 
 // Row stride for rows that different lanes read with 16-byte loads at the same
 // time: whole vectors, an odd number of them, so that the 8 lanes served by one
 // shared-memory wavefront start in 8 different groups of 4 banks.
-template <typename Real>
-__host__ __device__ constexpr int row_stride(int n)
-{
-    return (vec_len<Real>(n) / V16<Real>::N) % 2 == 0 ? vec_len<Real>(n) + V16<Real>::N : vec_len<Real>(n);
-}
+__host__ __device__ constexpr int row_stride(int n) { return vec_len(n) / 4 % 2 == 0 ? vec_len(n) + 4 : vec_len(n); }
 
 // Packed FP32 multiply-add on register pairs (one instruction, two lanes of work).
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 lo2(const float4 &v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(const float4 &v) { return make_float2(v.z, v.w); }
 
-// sum_{i < S} a[i] b[i] over 16-byte aligned shared rows (S a multiple of the
-// vector length) with one partial sum per vector lane (FP32: packed pairs).
-template <typename Real, int S>
-__device__ __forceinline__ Real dot16(const Real *a, const Real *b)
+// sum_{i < S} a[i] b[i] over 16-byte aligned shared rows (S a multiple of four) in packed pairs.
+template <int S>
+__device__ __forceinline__ float dot16(const float *a, const float *b)
 {
-    using VT = typename V16<Real>::T;
-    constexpr int N = V16<Real>::N;
-    static_assert(S % N == 0, "padded length");
-    if constexpr (sizeof(Real) == 4) {
-        float2 a0 = make_float2(0.0f, 0.0f), a1 = a0;
+    static_assert(S % 4 == 0, "padded length");
+    float2 a0 = make_float2(0.0f, 0.0f), a1 = a0;
 #pragma unroll
-        for (int i = 0; i < S; i += 4) {
-            const float4 x = *reinterpret_cast<const float4 *>(a + i);
-            const float4 y = *reinterpret_cast<const float4 *>(b + i);
-            a0 = ffma2(lo2(x), lo2(y), a0);
-            a1 = ffma2(hi2(x), hi2(y), a1);
-        }
-        return (a0.x + a1.x) + (a0.y + a1.y);
+    for (int i = 0; i < S; i += 4) {
+        const float4 x = *reinterpret_cast<const float4 *>(a + i);
+        const float4 y = *reinterpret_cast<const float4 *>(b + i);
+        a0 = ffma2(lo2(x), lo2(y), a0);
+        a1 = ffma2(hi2(x), hi2(y), a1);
     }
-    Real acc[N];
-#pragma unroll
-    for (int j = 0; j < N; ++j) acc[j] = Real(0);
-#pragma unroll
-    for (int i = 0; i < S; i += N) {
-        const VT x = *reinterpret_cast<const VT *>(a + i);
-        const VT y = *reinterpret_cast<const VT *>(b + i);
-#pragma unroll
-        for (int j = 0; j < N; ++j) acc[j] = fma(vcomp<Real>(x, j), vcomp<Real>(y, j), acc[j]);
-    }
-    Real r = acc[0];
-#pragma unroll
-    for (int j = 1; j < N; ++j) r += acc[j];
-    return r;
+    return (a0.x + a1.x) + (a0.y + a1.y);
 }
 
 // Coupling tensors staged per CTA, transposed so that one potential entry e
 // reads one contiguous row: sT3[e][k] (k < F, stride S3), sT4[e][kl] (kl < P,
 // stride S4), zero-padded.
-template <int F, typename Real, bool STAGED = (F <= 16)>
+template <int F, bool STAGED = (F <= 16)>
 struct TensorLayout {
     static constexpr int P = F * (F + 1) / 2;
-    static constexpr int S3 = vec_len<Real>(F);   // short rows: fewer loads outweigh a 2-way conflict
-    static constexpr int S4 = row_stride<Real>(P);
+    static constexpr int S3 = vec_len(F);   // short rows: fewer loads outweigh a 2-way conflict
+    static constexpr int S4 = row_stride(P);
     // Above F = 16 the quartic tensor (P^2 entries, 360 KB at F = 24) does not fit shared
     // memory: both tensors are read from global memory (L2) and only the coefficients are staged.
     static constexpr bool staged = STAGED;
@@ -356,16 +311,16 @@ struct TensorLayout {
     static constexpr int F3E = (F + 1) & ~1;
     static constexpr int KH = (((F3E + P + 1) / 2) + 3) & ~3;
     static constexpr int KHS = (KH / 4) % 2 ? KH : KH + 4;
-    static constexpr bool split = sizeof(Real) == 4 && STAGED && F >= 6 && F <= 9 && !lg_tensor_regs<F>();
+    static constexpr bool split = STAGED && F >= 6 && F <= 9 && !lg_tensor_regs<F>();
     // One-trajectory mixed warps above F = 13, and all that do not stage the tensors, contract them
     // together (CoopHessian): rows of P4
     // consecutive entries, the F cubic rows first.
-    static constexpr bool coop = sizeof(Real) == 4 && (F > 13 || (F > 9 && !STAGED));
+    static constexpr bool coop = F > 13 || (F > 9 && !STAGED);
     static constexpr int P4 = (P + 3) & ~3;
     static constexpr size_t tensor_elems = !staged ? 0 : (coop ? (size_t)(F + P) * P4 : (split ? (size_t)2 * P * KHS : (size_t)P * S3 + (size_t)P * S4));
     // after the tensors: the Herman-Kluk matrix coefficients acoef[a][b][4] =
     // (1/2) {rg_a/rg_b, rg_b/rg_a, -rg_a rg_b, 1/(rg_a rg_b)}, rg = sqrt(gamma)
-    static constexpr size_t bytes = ((sizeof(Real) * (tensor_elems + (size_t)4 * F * F)) + 15) & ~(size_t)15;
+    static constexpr size_t bytes = ((sizeof(float) * (tensor_elems + (size_t)4 * F * F)) + 15) & ~(size_t)15;
 };
 
 // Hessian contraction of the wide mixed groups (F > 13, and all that do not stage the tensors),
@@ -431,57 +386,56 @@ __device__ __forceinline__ void coop_fma(const float4 &t, const float (&x)[TP], 
     }
 }
 
-template <int F, int G, typename Real>
+template <int F, int G>
 struct WarpShared {
     static constexpr int P = F * (F + 1) / 2;
     static constexpr int T = 32 / G;
-    static constexpr int JOBS = T * lg_chunk<F, G, Real>();   // jobs per chunk (phases 2-4)
-    static constexpr int S3 = TensorLayout<F, Real>::S3;   // q, zero-padded (also the Gc row stride)
-    static constexpr int S4 = TensorLayout<F, Real>::S4;   // pair products q_k q_l, zero-padded
-    // H, read whole by every column lane with 16-byte broadcasts.  Mixed path: rows of an even
+    static constexpr int JOBS = T * lg_chunk<F, G>();   // jobs per chunk (phases 2-4)
+    static constexpr int S3 = TensorLayout<F>::S3;   // q, zero-padded (also the Gc row stride)
+    static constexpr int S4 = TensorLayout<F>::S4;   // pair products q_k q_l, zero-padded
+    // H, read whole by every column lane with 16-byte broadcasts: rows of an even
     // length back to back, so that pairs stay aligned and no load is mostly padding (9 instead of 12
     // loads at F = 6, 23 instead of 27 at F = 9; at F = 10, one trajectory a warp, 0.9 % slower and
-    // not used); FP64: rows of whole vectors.
-    static constexpr int SH = sizeof(Real) == 4 && F != 10 ? (F + 1) & ~1 : vec_len<Real>(F);
-    static constexpr int HV = vec_len<Real>(F * SH);
-    alignas(16) Real qr[T][S3];
-    alignas(16) Real qq[T][S4];
+    // not used: rows of whole vectors there).
+    static constexpr int SH = F != 10 ? (F + 1) & ~1 : vec_len(F);
+    static constexpr int HV = vec_len(F * SH);
+    alignas(16) float qr[T][S3];
+    alignas(16) float qq[T][S4];
     // x = (q, zero pad to an even length, pair products, zero pad) in two halves of KH for the
     // half-split Hessian of two-trajectory warps (see TensorLayout and lg_body)
-    static constexpr int F3E = TensorLayout<F, Real>::F3E;
-    static constexpr int KH = TensorLayout<F, Real>::KH;
+    static constexpr int F3E = TensorLayout<F>::F3E;
+    static constexpr int KH = TensorLayout<F>::KH;
     // only two-trajectory mixed warps use it: elsewhere a stub, so that the shared memory
     // left to L1 (the wide groups read their tensors through it) does not shrink
-    static constexpr bool kHalves = (T == 2) && (sizeof(Real) == 4) && F >= 6 && F <= 9;
-    alignas(16) Real xs[T][kHalves ? 2 * KH : 4];
-    alignas(16) Real Gc[T][F][S3];          // gradient coefficients, full symmetric matrix (row a read by mode lane a)
-    alignas(16) Real Hs[T][HV];
-    __device__ __forceinline__ Real &H(int tr, int a, int b) { return Hs[tr][a * SH + b]; }
-    // Prefactor matrix per job.  Mixed path: LPJ = 32 / JOBS lanes of a job read consecutive rows at
+    static constexpr bool kHalves = T == 2 && F >= 6 && F <= 9;
+    alignas(16) float xs[T][kHalves ? 2 * KH : 4];
+    alignas(16) float Gc[T][F][S3];          // gradient coefficients, full symmetric matrix (row a read by mode lane a)
+    alignas(16) float Hs[T][HV];
+    __device__ __forceinline__ float &H(int tr, int a, int b) { return Hs[tr][a * SH + b]; }
+    // Prefactor matrix per job.  LPJ = 32 / JOBS lanes of a job read consecutive rows at
     // the same column with 16-byte accesses, eight lanes (8 / LPJ jobs) to a wavefront.  The row
     // stride RS and the jobs' bases spread those eight over the eight 16-byte bank groups: an odd
     // RS for eight rows of one job, bases 4 apart (mod 8) for two jobs of four rows, 2 apart for four
     // jobs of two rows -- or, at F = 6, where an odd RS would cost a CTA per SM, 0, 5, 4, 1.  (With
     // F = 24 entries a row all eight fell into one group; with 81 a job two at F = 9.)
     static constexpr int LPJ = JOBS >= 32 ? 1 : 32 / JOBS;
-    static constexpr bool kMixed = sizeof(Real) == 4;
-    static constexpr int RS = !kMixed || LPJ == 1 || F == 6 ? F : F | 1;
+    static constexpr int RS = LPJ == 1 || F == 6 ? F : F | 1;
     static constexpr int up(int n, int r) { return n % 8 == r ? n : up(n + 1, r); }
     // (at least the det M workspace of 2F rows of 2F + 1 floats per trajectory)
-    static constexpr int AS0 = kMixed ? (T * 2 * F * (2 * F + 1) + 4 * JOBS - 1) / (4 * JOBS) : 0;
+    static constexpr int AS0 = (T * 2 * F * (2 * F + 1) + 4 * JOBS - 1) / (4 * JOBS);
     static constexpr int AS1 = AS0 > F * RS ? AS0 : F * RS;
-    static constexpr int AS = !kMixed || LPJ == 1 || LPJ >= 8 ? AS1 | 1 : (F == 6 ? 38 : up(AS1, LPJ == 4 ? 4 : 2));
-    static_assert(F != 6 || !kMixed || LPJ == 1 || (LPJ == 2 && AS1 <= 37), "the bases of F = 6");
-    typename AEntry<Real>::T A[JOBS * AS];
-    __device__ static __forceinline__ int a_base(int job) { return F == 6 && kMixed && LPJ == 2 ? 38 * job - (job & 1) : AS * job; }
-    __device__ __forceinline__ typename AEntry<Real>::T &a_at(int job, int row, int col) { return A[a_base(job) + row * RS + col]; }
+    static constexpr int AS = LPJ == 1 || LPJ >= 8 ? AS1 | 1 : (F == 6 ? 38 : up(AS1, LPJ == 4 ? 4 : 2));
+    static_assert(F != 6 || LPJ == 1 || (LPJ == 2 && AS1 <= 37), "the bases of F = 6");
+    AEntry A[JOBS * AS];
+    __device__ static __forceinline__ int a_base(int job) { return F == 6 && LPJ == 2 ? 38 * job - (job & 1) : AS * job; }
+    __device__ __forceinline__ AEntry &a_at(int job, int row, int col) { return A[a_base(job) + row * RS + col]; }
     // cubic and quartic parts of the Hessian entries (wide mixed groups): in the storage of the
     // step's own prefactor matrix, which is written after the step's last kick
     static constexpr int HP = (P + 3) & ~3;
     static_assert(F <= 9 || 8 * HP <= 16 * F * F, "the Hessian parts fit a job's matrix");
     __device__ __forceinline__ float *h3_at(int job) { return reinterpret_cast<float *>(&A[a_base(job)]); }
     __device__ __forceinline__ float *h4_at(int job) { return h3_at(job) + HP; }
-    Real pj[F][JOBS], qj[F][JOBS];         // state per job, for the overlap (job column swizzled); FP32
+    float pj[F][JOBS], qj[F][JOBS];         // state per job, for the overlap (job column swizzled); FP32
                                            // in the mixed path, where the overlap is evaluated in FP32
     double Sj[JOBS];                        // action per job
     double lnA[JOBS];                       // log |det A|^{1/2} per job (Herman-Kluk summand only)
@@ -495,26 +449,25 @@ struct WarpShared {
 // Called by the per-molecule kernel (cta = blockIdx.x) and by the batched
 // persistent kernel (cta = the work item's tile).  Stages the molecule's
 // constants itself and leaves shared memory free for the next call.
-template <int F, int G, typename Real, int WARPS, bool STAGED = (F <= 16), int TRAJ_WARPS = WARPS>
+template <int F, int G, int WARPS, bool STAGED = (F <= 16), int TRAJ_WARPS = WARPS>
 __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsigned char *smem_raw)
 {
     constexpr int N2 = 2 * F;
     constexpr int P = F * (F + 1) / 2;
     constexpr int T = 32 / G;
-    constexpr int C = lg_chunk<F, G, Real>();  // steps per chunk
+    constexpr int C = lg_chunk<F, G>();  // steps per chunk
     constexpr int JOBS = T * C;                // jobs per chunk: job t * C + c is trajectory t's step c
     constexpr int EPL = (P + G - 1) / G;       // packed Hessian entries per lane
     constexpr int NCOL = (N2 + G - 1) / G;     // monodromy columns per lane: column c sits in lane c % G, slot c / G
     static_assert(F <= G && NCOL <= 2, "a group holds every mode and at most two columns per lane");
-    using Sh = WarpShared<F, G, Real>;
-    using R2 = typename Vec2<Real>::T;
+    using Sh = WarpShared<F, G>;
 
-    using TL = TensorLayout<F, Real, STAGED>;
+    using TL = TensorLayout<F, STAGED>;
     constexpr int S3 = TL::S3, S4 = TL::S4;
-    Real *sT3 = reinterpret_cast<Real *>(smem_raw);
-    Real *sT4 = sT3 + ((TL::staged && !TL::split && !TL::coop) ? P * S3 : 0);
-    Real *sTh = sT3;                                  // the half-split layout (TL::split)
-    Real *sAc = sT3 + TL::tensor_elems;   // Herman-Kluk matrix coefficients [a][b][4] (16-byte aligned: the tensor block is a vector multiple)
+    float *sT3 = reinterpret_cast<float *>(smem_raw);
+    float *sT4 = sT3 + ((TL::staged && !TL::split && !TL::coop) ? P * S3 : 0);
+    float *sTh = sT3;                                  // the half-split layout (TL::split)
+    float *sAc = sT3 + TL::tensor_elems;   // Herman-Kluk matrix coefficients [a][b][4] (16-byte aligned: the tensor block is a vector multiple)
     size_t off = TL::bytes;
     CtaConst<F> &cc = *reinterpret_cast<CtaConst<F> *>(smem_raw + off);
     off += (sizeof(CtaConst<F>) + 15) & ~(size_t)15;
@@ -531,9 +484,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
     const bool use3 = pes.has3, use4 = pes.has4;
     // stage the coupling tensors once per CTA
     if constexpr (TL::staged) {
-        const Real *g3 = nullptr, *g4 = nullptr;
-        if constexpr (sizeof(Real) == 4) { g3 = reinterpret_cast<const Real *>(pes.T3f); g4 = reinterpret_cast<const Real *>(pes.T4f); }
-        else { g3 = reinterpret_cast<const Real *>(pes.T3); g4 = reinterpret_cast<const Real *>(pes.T4); }
+        const float *g3 = pes.T3f, *g4 = pes.T4f;
         if constexpr (kCoop) {
             const float4 *v3 = reinterpret_cast<const float4 *>(pes.T3p), *v4 = reinterpret_cast<const float4 *>(pes.T4p);
             float4 *dst = reinterpret_cast<float4 *>(sT3);
@@ -543,21 +494,21 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
             constexpr int KH = TL::KH, KHS = TL::KHS, F3E = TL::F3E;
             for (int i = threadIdx.x; i < 2 * P * KHS; i += blockDim.x) {
                 const int h = i / (P * KHS), e = (i / KHS) % P, kk = i % KHS, gk = h * KH + kk;
-                Real v = Real(0);
+                float v = 0.0f;
                 if (kk < KH) {
-                    if (gk < F) v = use3 ? g3[gk * P + e] : Real(0);
-                    else if (gk >= F3E && gk - F3E < P) v = use4 ? g4[(gk - F3E) * P + e] : Real(0);
+                    if (gk < F) v = use3 ? g3[gk * P + e] : 0.0f;
+                    else if (gk >= F3E && gk - F3E < P) v = use4 ? g4[(gk - F3E) * P + e] : 0.0f;
                 }
                 sTh[i] = v;
             }
         } else {
             for (int i = threadIdx.x; i < P * S3; i += blockDim.x) {
                 const int e = i / S3, k = i % S3;
-                sT3[i] = (use3 && k < F) ? g3[k * P + e] : Real(0);
+                sT3[i] = (use3 && k < F) ? g3[k * P + e] : 0.0f;
             }
             for (int i = threadIdx.x; i < P * S4; i += blockDim.x) {
                 const int e = i / S4, kl = i % S4;
-                sT4[i] = (use4 && kl < P) ? g4[kl * P + e] : Real(0);
+                sT4[i] = (use4 && kl < P) ? g4[kl * P + e] : 0.0f;
             }
         }
     }
@@ -575,12 +526,12 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
         // (rolled: thread 0 alone, and unrolling F^2 iterations starves the step loop of registers)
         for (int a = 0; a < F; ++a)
             for (int b = 0; b < F; ++b) {
-                const Real rga = (Real)A.rg[a], irga = (Real)A.irg[a], rgb = (Real)A.rg[b], irgb = (Real)A.irg[b];
-                Real *k = sAc + 4 * (a * F + b);
-                k[0] = Real(0.5) * (rga * irgb);
-                k[1] = Real(0.5) * (rgb * irga);
-                k[2] = Real(-0.5) * (rga * rgb);
-                k[3] = Real(0.5) * (irga * irgb);
+                const float rga = (float)A.rg[a], irga = (float)A.irg[a], rgb = (float)A.rg[b], irgb = (float)A.irg[b];
+                float *k = sAc + 4 * (a * F + b);
+                k[0] = 0.5f * (rga * irgb);
+                k[1] = 0.5f * (rgb * irga);
+                k[2] = -0.5f * (rga * rgb);
+                k[3] = 0.5f * (irga * irgb);
             }
 #pragma unroll
         for (int x = 0; x < SCIVR_MAX_CHI; ++x)
@@ -715,9 +666,9 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
     {
         // padding entries of the vector rows are read (multiplied by zero or skipped) but never
         // written by the step loop: clear the warp's rows once
-        Real *z = &sh.qr[0][0];
-        constexpr int nz = (int)((offsetof(Sh, Hs) + sizeof(Sh::Hs) - offsetof(Sh, qr)) / sizeof(Real));
-        for (int i = ln; i < nz; i += 32) z[i] = Real(0);
+        float *z = &sh.qr[0][0];
+        constexpr int nz = (int)((offsetof(Sh, Hs) + sizeof(Sh::Hs) - offsetof(Sh, qr)) / sizeof(float));
+        for (int i = ln; i < nz; i += 32) z[i] = 0.0f;
         __syncwarp();
     }
     const int64_t n = L.n_traj;
@@ -741,14 +692,12 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
     // jx + 16 i (jx = ln % 16, i < EPH), and multiplies them by both trajectories' halves of
     // x (read as warp-broadcast 16-byte loads).  Lanes ln and ln ^ 16 then exchange partial
     // sums so that each ends with whole entries of its own trajectory.
-    constexpr bool kPair = (T == 2) && (sizeof(Real) == 4) && TL::staged && (P <= 64) && (P > 16);
+    constexpr bool kPair = (T == 2) && TL::staged && (P <= 64) && (P > 16);
     constexpr bool kTreg = kPair && lg_tensor_regs<F>();
     // or the same cut with the tensor rows read from shared memory (TL::split)
     constexpr bool kSplit = kPair && !kTreg && TL::split;
     static_assert(kPair == (kTreg || kSplit), "two-trajectory warps take one of the two half-split schedules");
     static_assert(!kPair || Sh::kHalves, "the half-split schedules need the halves of x");
-    // packed FP32 pairs in the monodromy drift and kick
-    constexpr bool kPacked = sizeof(Real) == 4;
     constexpr int F3E = Sh::F3E, KH = Sh::KH, KHS = TL::KHS;
     constexpr int EPH = (kTreg || kSplit) ? (P + 15) / 16 : 1;
     const int hx = ln >> 4, jx = ln & 15;
@@ -807,7 +756,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
     Coord p, q;
     coord_set(p, L.p0[mode * n + jl]);
     coord_set(q, L.q0[mode * n + jl]);
-    Real pr = (Real)coord_get(p);   // the momentum as seen by the Real-precision bulk
+    float pr = (float)coord_get(p);   // the momentum as seen by the FP32 bulk
     Coord S;                        // accumulated action (lane 0 of the group holds the total)
     coord_set(S, 0.0);
     // per-job action in the job table: the double-FP32 pair in the 8 bytes of a double (a phase: what a
@@ -819,18 +768,18 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
     };
     // column state: slot s of lane g holds column c = g + s G of M = d(p,q)/d(p0,q0) (c < 2F;
     // a slot past 2F holds a zero column)
-    Real Mp[NCOL][F], Mq[NCOL][F];
+    float Mp[NCOL][F], Mq[NCOL][F];
 #pragma unroll
     for (int s = 0; s < NCOL; ++s) {
         const int col = g + s * G;
 #pragma unroll
         for (int a = 0; a < F; ++a) {
-            Mp[s][a] = (col < F && a == col) ? Real(1) : Real(0);
-            Mq[s][a] = (col >= F && col < N2 && a == col - F) ? Real(1) : Real(0);
+            Mp[s][a] = (col < F && a == col) ? 1.0f : 0.0f;
+            Mq[s][a] = (col >= F && col < N2 && a == col - F) ? 1.0f : 0.0f;
         }
     }
     bool good = true;
-    Real stab = Real(0);
+    float stab = 0.0f;
     double detM_last = 1.0;
     double theta_last = 0.0, arg_last = 0.0;
     double2 detA_last = make_double2(1.0, 0.0);   // det A of the last step
@@ -867,42 +816,35 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
         const int cnt = min(C, A.n_steps - step0);
         // ---------------- phase 1: cnt steps, group-parallel ----------------
         for (int c = 0; c < cnt; ++c) {
-            Real dS = Real(0);   // this lane's share of the step's action increment
+            float dS = 0.0f;   // this lane's share of the step's action increment
 #pragma unroll 1
             for (int sub = 0; sub < 4; ++sub) {
                 // drift: q += tau p, S += tau p.p/2, M_q += tau M_p
                 {
-                    const Real rt = A.tdrift_f[sub];
+                    const float rt = A.tdrift_f[sub];
                     if (g < F) {
                         q = coord_axpy(q, A.tdrift_f[sub], A.tdrift_lo[sub], p);
-                        dS = fma(rt * Real(0.5) * pr, pr, dS);
+                        dS = fma(rt * 0.5f * pr, pr, dS);
                     }
-                    if constexpr (kPacked) {
-                        const float2 rt2 = make_float2(rt, rt);
+                    const float2 rt2 = make_float2(rt, rt);
 #pragma unroll
-                        for (int s = 0; s < NCOL; ++s) {
+                    for (int s = 0; s < NCOL; ++s) {
 #pragma unroll
-                            for (int a = 0; a + 1 < F; a += 2) {
-                                const float2 r = ffma2(rt2, make_float2(Mp[s][a], Mp[s][a + 1]), make_float2(Mq[s][a], Mq[s][a + 1]));
-                                Mq[s][a] = r.x;
-                                Mq[s][a + 1] = r.y;
-                            }
-                            if constexpr (F % 2) Mq[s][F - 1] = fmaf(rt, Mp[s][F - 1], Mq[s][F - 1]);
+                        for (int a = 0; a + 1 < F; a += 2) {
+                            const float2 r = ffma2(rt2, make_float2(Mp[s][a], Mp[s][a + 1]), make_float2(Mq[s][a], Mq[s][a + 1]));
+                            Mq[s][a] = r.x;
+                            Mq[s][a + 1] = r.y;
                         }
-                    } else {
-#pragma unroll
-                        for (int s = 0; s < NCOL; ++s)
-#pragma unroll
-                            for (int a = 0; a < F; ++a) Mq[s][a] = fma(rt, Mp[s][a], Mq[s][a]);
+                        if constexpr (F % 2) Mq[s][F - 1] = fmaf(rt, Mp[s][F - 1], Mq[s][F - 1]);
                     }
                 }
                 if (sub == 3) break;
                 // kick: potential at q
-                const Real rtk = A.tkick_f[sub];
+                const float rtk = A.tkick_f[sub];
                 __syncwarp();   // previous kick's readers of qr/H are done
                 if (g < F) {
-                    sh.qr[t][g] = (Real)coord_f(q);
-                    if constexpr (kTreg || kSplit) sh.xs[t][g] = (Real)coord_f(q);
+                    sh.qr[t][g] = (float)coord_f(q);
+                    if constexpr (kTreg || kSplit) sh.xs[t][g] = (float)coord_f(q);
                     if constexpr (kCoop) xall[g * CH::XW + CH::slot(warp)] = (float)coord_f(q);
                 }
                 __syncwarp();
@@ -910,14 +852,14 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                 for (int i = 0; i < EPL; ++i) {
                     const int e = g + i * G;
                     if (e < P) {
-                        const Real v = sh.qr[t][ea[i]] * sh.qr[t][eb[i]];
+                        const float v = sh.qr[t][ea[i]] * sh.qr[t][eb[i]];
                         if constexpr (kTreg || kSplit) sh.xs[t][F3E + e] = v;
                         else sh.qq[t][e] = v;
                         if constexpr (kCoop) xall[(F + e) * CH::XW + CH::slot(warp)] = (float)v;
                     }
                 }
                 __syncwarp();
-                Real vpart = Real(0);
+                float vpart = 0.0f;
                 if constexpr (kCoop) {
                     __syncthreads();   // every warp's x is written; every warp has read its last h3, h4
                     contract(c);
@@ -1032,48 +974,48 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                 for (int i = 0; i < EPL; ++i) {
                     const int e = g + i * G;
                     if (e < P) {
-                        const Real h3 = use3 ? dot16<Real, S3>(sT3 + e * S3, sh.qr[t]) : Real(0);
-                        const Real h4 = use4 ? dot16<Real, S4>(sT4 + e * S4, sh.qq[t]) : Real(0);
+                        const float h3 = use3 ? dot16<S3>(sT3 + e * S3, sh.qr[t]) : 0.0f;
+                        const float h4 = use4 ? dot16<S4>(sT4 + e * S4, sh.qq[t]) : 0.0f;
                         const int a = ea[i], b = eb[i];
                         // coupling part only: the mode lanes add the diagonal term below
-                        const Real h = h3 + h4;
+                        const float h = h3 + h4;
                         sh.H(t, a, b) = h;
                         sh.H(t, b, a) = h;
-                        const Real gce = fma(Real(0.5), h3, h4 * Real(1.0 / 3.0));
+                        const float gce = fma(0.5f, h3, h4 * (1.0f / 3.0f));
                         sh.Gc[t][a][b] = gce;
                         sh.Gc[t][b][a] = gce;
-                        const Real vc = fma(Real(1.0 / 6.0), h3, h4 * Real(1.0 / 12.0));
-                        vpart = fma(a == b ? vc : Real(2) * vc, sh.qq[t][e], vpart);
+                        const float vc = fma((1.0f / 6.0f), h3, h4 * (1.0f / 12.0f));
+                        vpart = fma(a == b ? vc : 2.0f * vc, sh.qq[t][e], vpart);
                     }
                 }
                 __syncwarp();
                 // gradient, p and action (mode lanes)
-                Real vlane = vpart;
+                float vlane = vpart;
                 if (g < F) {
-                    const Real gr = dot16<Real, S3>(sh.Gc[t][g], sh.qr[t]);
-                    Real Vd, gd, hd;   // the separable diagonal: value, gradient, Hessian
+                    const float gr = dot16<S3>(sh.Gc[t][g], sh.qr[t]);
+                    float Vd, gd, hd;   // the separable diagonal: value, gradient, Hessian
                     if (pes.diag_kind == SCIVR_DIAG_MORSE) {
-                        const Real Dm = cc.Df[g], am = cc.af[g];
-                        const Real u = rexp<Real>(-am * sh.qr[t][g]);
-                        const Real omu = Real(1) - u;
+                        const float Dm = cc.Df[g], am = cc.af[g];
+                        const float u = expf(-am * sh.qr[t][g]);
+                        const float omu = 1.0f - u;
                         Vd = Dm * omu * omu;
-                        gd = Real(2) * Dm * am * u * omu;
-                        hd = Real(2) * Dm * am * am * u * (Real(2) * u - Real(1));
+                        gd = 2.0f * Dm * am * u * omu;
+                        hd = 2.0f * Dm * am * am * u * (2.0f * u - 1.0f);
                     } else {
-                        const Real w2 = cc.w2f[g];
-                        Vd = Real(0.5) * w2 * sh.qr[t][g] * sh.qr[t][g];
+                        const float w2 = cc.w2f[g];
+                        Vd = 0.5f * w2 * sh.qr[t][g] * sh.qr[t][g];
                         gd = w2 * sh.qr[t][g];
                         hd = w2;
                     }
                     sh.H(t, g, g) += hd;
                     p = coord_kick(p, A.tkick_f[sub], A.tkick_lo[sub], gr + gd);
-                    pr = (Real)coord_f(p);
+                    pr = (float)coord_f(p);
                     vlane += Vd;
                 }
                 __syncwarp();   // H complete before the monodromy kick reads it
                 dS = fma(-rtk, vlane, dS);
                 // monodromy kick: M_p -= tau H M_q (column lanes; rows of H by 16-byte broadcast loads)
-                if constexpr (kPacked) {
+                {
                     // packed pairs of H's row entries against pairs of the column's entries
                     constexpr int SH = Sh::SH;
                     float2 acc[NCOL];
@@ -1095,27 +1037,6 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                             }
                         }
                     }
-                } else {
-                    using VT = typename V16<Real>::T;
-                    constexpr int NV = V16<Real>::N, SH = Sh::SH;
-#pragma unroll
-                    for (int a = 0; a < F; ++a) {
-                        Real acc[NCOL];
-#pragma unroll
-                        for (int s = 0; s < NCOL; ++s) acc[s] = Real(0);
-#pragma unroll
-                        for (int b0 = 0; b0 < SH; b0 += NV) {
-                            const VT v = *reinterpret_cast<const VT *>(&sh.H(t, a, b0));
-#pragma unroll
-                            for (int j = 0; j < NV; ++j)
-                                if (b0 + j < F) {
-#pragma unroll
-                                    for (int s = 0; s < NCOL; ++s) acc[s] = fma(vcomp<Real>(v, j), Mq[s][b0 + j], acc[s]);
-                                }
-                        }
-#pragma unroll
-                        for (int s = 0; s < NCOL; ++s) Mp[s][a] = fma(-rtk, acc[s], Mp[s][a]);
-                    }
                 }
             }
             // ---- Herman-Kluk matrix column b = g (needs column F + b) ----
@@ -1126,35 +1047,21 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                 const int job = t * C + c;
 #pragma unroll
                 for (int a = 0; a < F; ++a) {
-                    Real sp, sq;
+                    float sp, sq;
                     if constexpr (NCOL == 1) { sp = Mp[0][a]; sq = Mq[0][a]; }
                     else { sp = g >= F ? Mp[0][a] : Mp[1][a]; sq = g >= F ? Mq[0][a] : Mq[1][a]; }
-                    const Real mpq = __shfl_sync(FULL, sp, src);
-                    const Real mqq = __shfl_sync(FULL, sq, src);
+                    const float mpq = __shfl_sync(FULL, sp, src);
+                    const float mqq = __shfl_sync(FULL, sq, src);
                     if (g < F) {
-                        using VT = typename V16<Real>::T;
-                        constexpr int NV = V16<Real>::N;
-                        Real k4[4];
-#pragma unroll
-                        for (int j0 = 0; j0 < 4; j0 += NV) {
-                            const VT kv = *reinterpret_cast<const VT *>(sAc + 4 * (a * F + g) + j0);
-#pragma unroll
-                            for (int j = 0; j < NV; ++j) k4[j0 + j] = vcomp<Real>(kv, j);
-                        }
-                        R2 v;
-                        v.x = fma(k4[0], mqq, k4[1] * Mp[0][a]);
-                        v.y = fma(k4[2], Mq[0][a], k4[3] * mpq);
-                        if constexpr (sizeof(Real) == 4)
-                            sh.a_at(job, a, g) = make_float4(v.x, v.y, 0.0f, 0.0f);
-                        else
-                            sh.a_at(job, a, g) = v;
+                        const float4 k4 = *reinterpret_cast<const float4 *>(sAc + 4 * (a * F + g));
+                        sh.a_at(job, a, g) = make_float4(fma(k4.x, mqq, k4.y * Mp[0][a]), fma(k4.z, Mq[0][a], k4.w * mpq), 0.0f, 0.0f);
                     }
                 }
                 if (g < F) {
                     sh.pj[g][jswz<JOBS>(g, job)] = pr;   // p did not change since the last kick set pr
-                    sh.qj[g][jswz<JOBS>(g, job)] = (Real)coord_f(q);
+                    sh.qj[g][jswz<JOBS>(g, job)] = (float)coord_f(q);
                 }
-                // the step's action increment, summed over the group, joins the FP64 action
+                // the step's action increment, summed over the group, joins the running action
 #pragma unroll
                 for (int o = G / 2; o > 0; o >>= 1) dS += __shfl_xor_sync(FULL, dS, o, G);
                 if (g == 0) {
@@ -1176,14 +1083,14 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
         const bool jvalid = jc < cnt;
         double argA = 0.0;                // arg det A of this lane's job (principal value)
         double2 detA = make_double2(1.0, 0.0);
-        if constexpr (sizeof(Real) == 4) {
-            // Mixed path: the entries of A are FP32 (formed from the FP32 monodromy) and the
+        {
+            // The entries of A are FP32 (formed from the FP32 monodromy) and the
             // elimination runs in double-FP32 on the FP32 pipe, so det A carries FP64-class
             // accuracy for those entries.  LPJ lanes share a job: the rows still to be
             // eliminated are dealt out over them through a permutation (a 4-bit field per row
             // up to F = 16, 5 bits above, in two 64-bit words; positions k.. are the active
             // rows), the pivot is an arg-max of
-            // |a_ik|^2 over the job's lanes, and det A is the product of the pivots in FP64,
+            // |a_ik|^2 over the job's lanes, and det A is the product of the pivots,
             // its sign flipped per exchange of the permutation.
             constexpr int LPJ = 32 / JOBS;
             static_assert(LPJ * JOBS == 32, "jobs must tile the warp");
@@ -1349,7 +1256,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                 detA = sh.detAj[jb];
             }
         }
-        if constexpr (sizeof(Real) == 4) {
+        {
             // det M every kDetMEvery steps and at the last step (at a chunk end: M is unchanged
             // since): rows of M^T in the job matrices' storage, free once det A is done
             // (2F (2F + 1) words per trajectory fit in its 4 F^2 C words), row stride 2F + 1 so
@@ -1436,7 +1343,7 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
         if (jvalid && active) {
             const double S = sj_get(jb);
             for (int x = 0; x < A.n_chi; ++x) {
-                if constexpr (sizeof(Real) == 4) {
+                {
                     // the overlap's exponent and phase are O(1)-O(10) in size: FP32 from the FP32
                     // state copies; the action and the continuous phase join in FP64, and the
                     // total phase is reduced modulo 2 pi in FP64 before FP32 sine and cosine
@@ -1505,18 +1412,18 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
     __syncthreads();   // the caller may restage shared memory next
 }
 
-template <int F, int G, typename Real, int WARPS, int TRAJ_WARPS>
-__global__ void __launch_bounds__(32 * WARPS, lg_min_ctas<F, G, Real>()) k_propagate_lg(const PropLaunch L)
+template <int F, int G, int WARPS, int TRAJ_WARPS>
+__global__ void __launch_bounds__(32 * WARPS, lg_min_ctas<F, G>()) k_propagate_lg(const PropLaunch L)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    lg_body<F, G, Real, WARPS, (F <= 16), TRAJ_WARPS>(L, blockIdx.x, smem_raw);
+    lg_body<F, G, WARPS, (F <= 16), TRAJ_WARPS>(L, blockIdx.x, smem_raw);
 }
 
 // Batched persistent kernel: CTAs pull (molecule, tile) work items from a
 // list sorted by decreasing cost until it is exhausted.  items: device array
 // of per-molecule launches (all of this F); work: (item, tile) pairs.
-template <int F, int G, typename Real, int WARPS>
-__global__ void __launch_bounds__(32 * WARPS, lg_min_ctas<F, G, Real>()) k_propagate_lg_batch(const PropLaunch *__restrict__ items,
+template <int F, int G, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, lg_min_ctas<F, G>()) k_propagate_lg_batch(const PropLaunch *__restrict__ items,
                                                                        const int2 *__restrict__ work,
                                                                        int n_work, int *__restrict__ counter)
 {
@@ -1529,7 +1436,7 @@ __global__ void __launch_bounds__(32 * WARPS, lg_min_ctas<F, G, Real>()) k_propa
         __syncthreads();
         if (w >= n_work) break;
         const int2 it = work[w];
-        lg_body<F, G, Real, WARPS>(items[it.x], it.y, smem_raw);
+        lg_body<F, G, WARPS>(items[it.x], it.y, smem_raw);
     }
 }
 
@@ -1552,7 +1459,7 @@ __global__ void __launch_bounds__(128, 1) k_propagate_lg_multi(const PropLaunch 
         if (w >= n_work) break;
         const int2 it = work[w];
         const int F = items[it.x].args.F;
-        const bool ran = ((F == Fs ? (lg_body<Fs, mixed_group_lanes(Fs), float, 4, (Fs <= 9)>(items[it.x], it.y, smem_raw),
+        const bool ran = ((F == Fs ? (lg_body<Fs, mixed_group_lanes(Fs), 4, (Fs <= 9)>(items[it.x], it.y, smem_raw),
                                       true)
                                    : false) ||
                           ...);
@@ -1562,24 +1469,24 @@ __global__ void __launch_bounds__(128, 1) k_propagate_lg_multi(const PropLaunch 
 
 }  // namespace lg
 
-template <int F, int G, typename Real, int WARPS, bool STAGED = (F <= 16), int TRAJ_WARPS = WARPS>
+template <int F, int G, int WARPS, bool STAGED = (F <= 16), int TRAJ_WARPS = WARPS>
 size_t lg_smem_bytes()
 {
     using namespace lg;
-    using TL = TensorLayout<F, Real, STAGED>;
+    using TL = TensorLayout<F, STAGED>;
     const size_t consts = (sizeof(CtaConst<F>) + 15) & ~(size_t)15;
     size_t coop = 0;
     if constexpr (TL::coop) coop = CoopHessian<F, WARPS, TRAJ_WARPS, STAGED>::bytes;
-    return TL::bytes + consts + coop + TRAJ_WARPS * sizeof(WarpShared<F, G, Real>);
+    return TL::bytes + consts + coop + TRAJ_WARPS * sizeof(WarpShared<F, G>);
 }
 
-template <int F, int G, typename Real, int WARPS>
+template <int F, int G, int WARPS>
 cudaError_t launch_lg_batch(const PropLaunch *items, const int2 *work, int n_work, int *counter, int n_sm,
                             cudaStream_t s)
 {
     using namespace lg;
-    const size_t bytes = lg_smem_bytes<F, G, Real, WARPS>();
-    auto kern = k_propagate_lg_batch<F, G, Real, WARPS>;
+    const size_t bytes = lg_smem_bytes<F, G, WARPS>();
+    auto kern = k_propagate_lg_batch<F, G, WARPS>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     // the largest shared-memory carveout, so that as many CTAs fit as the registers allow
@@ -1596,13 +1503,13 @@ cudaError_t launch_lg_batch(const PropLaunch *items, const int2 *work, int n_wor
     return cudaGetLastError();
 }
 
-template <int F, int G, typename Real, int WARPS, int TRAJ_WARPS = WARPS>
+template <int F, int G, int WARPS, int TRAJ_WARPS = WARPS>
 cudaError_t launch_lg(const PropLaunch &L, cudaStream_t s)
 {
     using namespace lg;
     constexpr int T = 32 / G;
-    const size_t bytes = lg_smem_bytes<F, G, Real, WARPS, (F <= 16), TRAJ_WARPS>();
-    auto kern = k_propagate_lg<F, G, Real, WARPS, TRAJ_WARPS>;
+    const size_t bytes = lg_smem_bytes<F, G, WARPS, (F <= 16), TRAJ_WARPS>();
+    auto kern = k_propagate_lg<F, G, WARPS, TRAJ_WARPS>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     // the largest shared-memory carveout, so that as many CTAs fit as the registers allow
@@ -1629,10 +1536,10 @@ template <int F> cudaError_t launch_group_mixed(const PropLaunch &L, cudaStream_
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        if (L.n_traj <= 2 * (int64_t)n_sm) return launch_lg<F, G, float, W, 2>(L, s);
-        if (L.n_traj <= 4 * (int64_t)n_sm) return launch_lg<F, G, float, W, 4>(L, s);
+        if (L.n_traj <= 2 * (int64_t)n_sm) return launch_lg<F, G, W, 2>(L, s);
+        if (L.n_traj <= 4 * (int64_t)n_sm) return launch_lg<F, G, W, 4>(L, s);
     }
-    return launch_lg<F, G, float, W>(L, s);
+    return launch_lg<F, G, W>(L, s);
 }
 
 template <int F>
@@ -1642,13 +1549,13 @@ cudaError_t launch_group_batch_mixed_F(int warps, const PropLaunch *items, const
     constexpr int G = mixed_group_lanes(F);
     if constexpr (G == 32 && F > 9) {
         constexpr int W = lg::lg_warps<F, G>();
-        if (warps == W) return launch_lg_batch<F, G, float, W>(items, work, n_work, counter, n_sm, s);
+        if (warps == W) return launch_lg_batch<F, G, W>(items, work, n_work, counter, n_sm, s);
     } else if constexpr (G == 32) {
-        if (warps == 1) return launch_lg_batch<F, G, float, 1>(items, work, n_work, counter, n_sm, s);
-        if (warps == 2) return launch_lg_batch<F, G, float, 2>(items, work, n_work, counter, n_sm, s);
+        if (warps == 1) return launch_lg_batch<F, G, 1>(items, work, n_work, counter, n_sm, s);
+        if (warps == 2) return launch_lg_batch<F, G, 2>(items, work, n_work, counter, n_sm, s);
     } else {
-        if (warps == 2) return launch_lg_batch<F, G, float, 2>(items, work, n_work, counter, n_sm, s);
-        if (warps == 4) return launch_lg_batch<F, G, float, 4>(items, work, n_work, counter, n_sm, s);
+        if (warps == 2) return launch_lg_batch<F, G, 2>(items, work, n_work, counter, n_sm, s);
+        if (warps == 4) return launch_lg_batch<F, G, 4>(items, work, n_work, counter, n_sm, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -1660,7 +1567,7 @@ struct MultiLaunch {
     static size_t smem_bytes()
     {
         size_t m = 0;
-        ((m = std::max(m, lg_smem_bytes<Fs, mixed_group_lanes(Fs), float, 4, (Fs <= 9)>())), ...);
+        ((m = std::max(m, lg_smem_bytes<Fs, mixed_group_lanes(Fs), 4, (Fs <= 9)>())), ...);
         return m;
     }
     static cudaError_t launch(const PropLaunch *items, const int2 *work, int n_work, int *counter, int n_sm,
