@@ -1,7 +1,7 @@
 // Batched runs (scivr_batch_*): many molecules with different F, trajectory
 // counts and step counts.  Trajectories of all molecules are independent
 // (Sec. III.B of arXiv:1312.4698), so the plan groups molecules by
-// (F, precision) and runs each mixed-precision group as one persistent
+// (F, precision; at F = 14..23 those without quartic terms apart) and runs each mixed-precision group as one persistent
 // lane-group launch whose CTAs pull (molecule, tile) work items, the
 // longest first.  FP64 molecules are launched one by one.  Each molecule's
 // spectra follow.  The launch sequence allocates nothing and never
@@ -19,6 +19,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "scivr_internal.cuh"
@@ -39,7 +40,10 @@ struct Group {
 std::mutex g_tune_mu;
 std::map<std::string, int> g_tuned;
 
-std::string tune_key(int F, int precision)
+// A molecule of the kernels for surfaces without quartic terms.
+bool cubic_class(const PropLaunch &L) { return !L.pes.has4 && cubic_schedule(L.args.F); }
+
+std::string tune_key(int F, int precision, bool cubic)
 {
     int dev = 0;
     cudaGetDevice(&dev);
@@ -48,7 +52,7 @@ std::string tune_key(int F, int precision)
     std::string name = p.name;
     for (char &c : name)
         if (c == ' ') c = '_';
-    return "F" + std::to_string(F) + ":prec" + std::to_string(precision) + ":" + name;
+    return "F" + std::to_string(F) + (cubic ? "c" : "") + ":prec" + std::to_string(precision) + ":" + name;
 }
 
 void load_tune_file()
@@ -127,9 +131,9 @@ cudaError_t time_candidate(const PropLaunch &L, int warps, int n_sm, float *ms)
 cudaError_t choose_warps(const PropLaunch &L, int precision, int n_sm, int *warps)
 {
     int cand[2] = {0, 0};
-    const int nc = batch_warp_candidates(L.args.F, cand);
+    const int nc = batch_warp_candidates(L.args.F, L.pes.has4, cand);
     if (nc == 0) return cudaErrorInvalidValue;
-    const std::string key = tune_key(L.args.F, precision);
+    const std::string key = tune_key(L.args.F, precision, cubic_class(L));
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         if (g_tuned.empty()) load_tune_file();
@@ -197,13 +201,13 @@ cudaError_t one_launch_is_faster(const std::vector<PropLaunch> &recs, const std:
         amp_bytes += ((sizeof(double2) * (size_t)L.args.n_chi * L.chi_stride + (size_t)L.n_traj) + 255) & ~(size_t)255;
     }
     // per-class work lists of the probe
-    std::map<int, std::vector<int>> cls;
-    for (int k = 0; k < (int)P.size(); ++k) cls[P[k].args.F].push_back(k);
+    std::map<std::pair<int, int>, std::vector<int>> cls;   // by F and warps per CTA
+    for (int k = 0; k < (int)P.size(); ++k) cls[{P[k].args.F, warps_of_rec[k]}].push_back(k);
     std::vector<int2> mw = multi_work(P);
     size_t bytes = amp_bytes + sizeof(PropLaunch) * P.size() + sizeof(int2) * (mw.size() + 16) * 2 + 4096 +
                    256 * cls.size();
     for (auto &c : cls) {
-        const int per_tile = warps_of_rec[c.second[0]] * (32 / mixed_group_lanes(c.first));
+        const int per_tile = c.first.second * (32 / mixed_group_lanes(c.first.first));
         size_t n = 0;
         for (int k : c.second) n += (P[k].n_traj + per_tile - 1) / per_tile;
         bytes += sizeof(int2) * n + sizeof(PropLaunch) * c.second.size() + 512;
@@ -232,8 +236,8 @@ cudaError_t one_launch_is_faster(const std::vector<PropLaunch> &recs, const std:
     for (auto &c : cls) {
         std::vector<PropLaunch> rr;
         for (int k : c.second) rr.push_back(P[k]);
-        const int warps = warps_of_rec[c.second[0]];
-        const int per_tile = warps * (32 / mixed_group_lanes(c.first));
+        const int warps = c.first.second;
+        const int per_tile = warps * (32 / mixed_group_lanes(c.first.first));
         std::vector<int2> w;
         for (int k = 0; k < (int)rr.size(); ++k)
             for (int t = 0; t < (int)((rr[k].n_traj + per_tile - 1) / per_tile); ++t) w.push_back(make_int2(k, t));
@@ -242,7 +246,7 @@ cudaError_t one_launch_is_faster(const std::vector<PropLaunch> &recs, const std:
         cp.work = static_cast<int2 *>(put(w.data(), sizeof(int2) * w.size()));
         cp.n_work = (int)w.size();
         cp.warps = warps;
-        cp.F = c.first;
+        cp.F = c.first.first;
         cps.push_back(cp);
     }
     int *counters = reinterpret_cast<int *>(b);   // one per class + one for the one launch
@@ -339,18 +343,19 @@ int scivr_batch_create(const scivr_batch_item *items, int32_t n_items, int32_t f
         scratch = std::max(scratch, sb);
     }
     // groups
-    std::map<int, int> gidx;
+    std::map<std::pair<int, bool>, int> gidx;
     for (int i = 0; i < n_items; ++i) {
         const PropLaunch &L = B->launches[i];
         if (L.args.precision != SCIVR_MIXED) { B->fp64_items.push_back(i); continue; }
-        auto f = gidx.find(L.args.F);
+        const std::pair<int, bool> cls{L.args.F, cubic_class(L)};
+        auto f = gidx.find(cls);
         if (f == gidx.end()) {
-            gidx[L.args.F] = (int)B->groups.size();
+            gidx[cls] = (int)B->groups.size();
             Group g;
             g.F = L.args.F;
             g.precision = SCIVR_MIXED;
             B->groups.push_back(g);
-            f = gidx.find(L.args.F);
+            f = gidx.find(cls);
         }
         B->groups[f->second].members.push_back(i);
     }

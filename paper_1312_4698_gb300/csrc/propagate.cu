@@ -10,9 +10,10 @@ template <int F>
 cudaError_t launch_group_batch_mixed_F(int warps, const PropLaunch *items, const int2 *work, int n_work,
                                       int *counter, int n_sm, cudaStream_t s);
 
-int batch_warp_candidates(int F, int *out)
+int batch_warp_candidates(int F, bool has4, int *out)
 {
     if (F < 1 || F > 24) return 0;
+    if (!has4 && cubic_schedule(F)) { out[0] = 4; return 1; }
     if (F > 9) { out[0] = F == 13 ? 4 : 8; return 1; }   // wide groups: one shape each (lg_warps)
     if (mixed_group_lanes(F) == 32) { out[0] = 1; out[1] = 2; }
     else { out[0] = 2; out[1] = 4; }

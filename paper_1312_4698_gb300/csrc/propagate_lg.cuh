@@ -231,6 +231,7 @@ __device__ __forceinline__ int jswz(int r, int j) { return j ^ (r & (JOBS >= 16 
 // Steps per chunk of a lane group.  Phases 2-4 work on T * C jobs (trajectory, step) per warp.
 // The double-FP32 elimination keeps two FP32 words per real entry, so chunks are short (8 steps; 4
 // at F = 9 and 13..15, 2 at 16, 1 above) and 32 / (T * C) lanes share a job's elimination by rows.
+// CUBIC: the kernels for surfaces without quartic terms (cubic_schedule).
 // Mixed path: steps between stability tests (a multiple of every mixed chunk length).
 // The flag is sticky and a bad trajectory is dropped whole, so a coarser test differs
 // from the per-step one only for a deviation that crosses the threshold and falls back
@@ -238,8 +239,9 @@ __device__ __forceinline__ int jswz(int r, int j) { return j ^ (r & (JOBS >= 16 
 // 16-step cadences equal the per-step ones).
 constexpr int kDetMEvery = 16;
 
-template <int F, int G> __host__ __device__ constexpr int lg_chunk()
+template <int F, int G, bool CUBIC = false> __host__ __device__ constexpr int lg_chunk()
 {
+    if (CUBIC) return F > 16 ? 2 : 4;
     return G == 32 && F > 16 ? 1 : (G == 32 && F > 15 ? 2 : ((G == 32 && F > 12) || (G == 16 && F > 8) ? 4 : 8));
 }
 
@@ -295,7 +297,7 @@ __device__ __forceinline__ float dot16(const float *a, const float *b)
 // Coupling tensors staged per CTA, transposed so that one potential entry e
 // reads one contiguous row: sT3[e][k] (k < F, stride S3), sT4[e][kl] (kl < P,
 // stride S4), zero-padded.
-template <int F, bool STAGED = (F <= 16)>
+template <int F, bool STAGED = (F <= 16), bool CUBIC = false>
 struct TensorLayout {
     static constexpr int P = F * (F + 1) / 2;
     static constexpr int S3 = vec_len(F);   // short rows: fewer loads outweigh a 2-way conflict
@@ -315,7 +317,7 @@ struct TensorLayout {
     // One-trajectory mixed warps above F = 13, and all that do not stage the tensors, contract them
     // together (CoopHessian): rows of P4
     // consecutive entries, the F cubic rows first.
-    static constexpr bool coop = F > 13 || (F > 9 && !STAGED);
+    static constexpr bool coop = !CUBIC && (F > 13 || (F > 9 && !STAGED));
     static constexpr int P4 = (P + 3) & ~3;
     static constexpr size_t tensor_elems = !staged ? 0 : (coop ? (size_t)(F + P) * P4 : (split ? (size_t)2 * P * KHS : (size_t)P * S3 + (size_t)P * S4));
     // after the tensors: the Herman-Kluk matrix coefficients acoef[a][b][4] =
@@ -386,11 +388,11 @@ __device__ __forceinline__ void coop_fma(const float4 &t, const float (&x)[TP], 
     }
 }
 
-template <int F, int G>
+template <int F, int G, bool CUBIC = false>
 struct WarpShared {
     static constexpr int P = F * (F + 1) / 2;
     static constexpr int T = 32 / G;
-    static constexpr int JOBS = T * lg_chunk<F, G>();   // jobs per chunk (phases 2-4)
+    static constexpr int JOBS = T * lg_chunk<F, G, CUBIC>();   // jobs per chunk (phases 2-4)
     static constexpr int S3 = TensorLayout<F>::S3;   // q, zero-padded (also the Gc row stride)
     static constexpr int S4 = TensorLayout<F>::S4;   // pair products q_k q_l, zero-padded
     // H, read whole by every column lane with 16-byte broadcasts: rows of an even
@@ -449,20 +451,20 @@ struct WarpShared {
 // Called by the per-molecule kernel (cta = blockIdx.x) and by the batched
 // persistent kernel (cta = the work item's tile).  Stages the molecule's
 // constants itself and leaves shared memory free for the next call.
-template <int F, int G, int WARPS, bool STAGED = (F <= 16), int TRAJ_WARPS = WARPS>
+template <int F, int G, int WARPS, bool STAGED = (F <= 16), int TRAJ_WARPS = WARPS, bool CUBIC = false>
 __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsigned char *smem_raw)
 {
     constexpr int N2 = 2 * F;
     constexpr int P = F * (F + 1) / 2;
     constexpr int T = 32 / G;
-    constexpr int C = lg_chunk<F, G>();  // steps per chunk
+    constexpr int C = lg_chunk<F, G, CUBIC>();  // steps per chunk
     constexpr int JOBS = T * C;                // jobs per chunk: job t * C + c is trajectory t's step c
     constexpr int EPL = (P + G - 1) / G;       // packed Hessian entries per lane
     constexpr int NCOL = (N2 + G - 1) / G;     // monodromy columns per lane: column c sits in lane c % G, slot c / G
     static_assert(F <= G && NCOL <= 2, "a group holds every mode and at most two columns per lane");
-    using Sh = WarpShared<F, G>;
+    using Sh = WarpShared<F, G, CUBIC>;
 
-    using TL = TensorLayout<F, STAGED>;
+    using TL = TensorLayout<F, STAGED, CUBIC>;
     constexpr int S3 = TL::S3, S4 = TL::S4;
     float *sT3 = reinterpret_cast<float *>(smem_raw);
     float *sT4 = sT3 + ((TL::staged && !TL::split && !TL::coop) ? P * S3 : 0);
@@ -885,6 +887,39 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                         for (int i = 0; i < 4 * NQ; ++i) {
                             const int e = 4 * (g + (i / 4) * G) + i % 4;
                             if (e < P) entry(e, eq[i] & 255, eq[i] >> 8);
+                        }
+                    }
+                } else if constexpr (CUBIC) {
+                    // a lane's quads of entries against the cubic rows in L2, 4 F multiply-adds each
+                    const float4 *T3v = reinterpret_cast<const float4 *>(pes.T3p);
+#pragma unroll
+                    for (int i = 0; i < NQ; ++i) {
+                        const int q4 = g + i * G;
+                        if (4 * q4 < P) {
+                            float4 h = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                            if (use3) {
+#pragma unroll 8
+                                for (int k = 0; k < F; ++k) {
+                                    const float4 tv = __ldg(T3v + k * (P4 / 4) + q4);
+                                    const float x = sh.qr[t][k];
+                                    h.x = fmaf(tv.x, x, h.x); h.y = fmaf(tv.y, x, h.y);
+                                    h.z = fmaf(tv.z, x, h.z); h.w = fmaf(tv.w, x, h.w);
+                                }
+                            }
+                            const float hj[4] = {h.x, h.y, h.z, h.w};
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const int e = 4 * q4 + j;
+                                if (e < P) {
+                                    const int a = eq[4 * i + j] & 255, b = eq[4 * i + j] >> 8;
+                                    sh.H(t, a, b) = hj[j];
+                                    sh.H(t, b, a) = hj[j];
+                                    sh.Gc[t][a][b] = 0.5f * hj[j];
+                                    sh.Gc[t][b][a] = 0.5f * hj[j];
+                                    const float vc = (1.0f / 6.0f) * hj[j];
+                                    vpart = fmaf(a == b ? vc : 2.0f * vc, sh.qq[t][e], vpart);
+                                }
+                            }
                         }
                     }
                 } else if constexpr (kTreg || kSplit) {
@@ -1412,17 +1447,17 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
     __syncthreads();   // the caller may restage shared memory next
 }
 
-template <int F, int G, int WARPS, int TRAJ_WARPS>
+template <int F, int G, int WARPS, int TRAJ_WARPS, bool CUBIC>
 __global__ void __launch_bounds__(32 * WARPS, lg_min_ctas<F, G>()) k_propagate_lg(const PropLaunch L)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    lg_body<F, G, WARPS, (F <= 16), TRAJ_WARPS>(L, blockIdx.x, smem_raw);
+    lg_body<F, G, WARPS, (F <= 16 && !CUBIC), TRAJ_WARPS, CUBIC>(L, blockIdx.x, smem_raw);
 }
 
 // Batched persistent kernel: CTAs pull (molecule, tile) work items from a
 // list sorted by decreasing cost until it is exhausted.  items: device array
 // of per-molecule launches (all of this F); work: (item, tile) pairs.
-template <int F, int G, int WARPS>
+template <int F, int G, int WARPS, bool CUBIC>
 __global__ void __launch_bounds__(32 * WARPS, lg_min_ctas<F, G>()) k_propagate_lg_batch(const PropLaunch *__restrict__ items,
                                                                        const int2 *__restrict__ work,
                                                                        int n_work, int *__restrict__ counter)
@@ -1436,7 +1471,7 @@ __global__ void __launch_bounds__(32 * WARPS, lg_min_ctas<F, G>()) k_propagate_l
         __syncthreads();
         if (w >= n_work) break;
         const int2 it = work[w];
-        lg_body<F, G, WARPS>(items[it.x], it.y, smem_raw);
+        lg_body<F, G, WARPS, (F <= 16 && !CUBIC), WARPS, CUBIC>(items[it.x], it.y, smem_raw);
     }
 }
 
@@ -1469,24 +1504,24 @@ __global__ void __launch_bounds__(128, 1) k_propagate_lg_multi(const PropLaunch 
 
 }  // namespace lg
 
-template <int F, int G, int WARPS, bool STAGED = (F <= 16), int TRAJ_WARPS = WARPS>
+template <int F, int G, int WARPS, bool STAGED = (F <= 16), int TRAJ_WARPS = WARPS, bool CUBIC = false>
 size_t lg_smem_bytes()
 {
     using namespace lg;
-    using TL = TensorLayout<F, STAGED>;
+    using TL = TensorLayout<F, STAGED, CUBIC>;
     const size_t consts = (sizeof(CtaConst<F>) + 15) & ~(size_t)15;
     size_t coop = 0;
     if constexpr (TL::coop) coop = CoopHessian<F, WARPS, TRAJ_WARPS, STAGED>::bytes;
-    return TL::bytes + consts + coop + TRAJ_WARPS * sizeof(WarpShared<F, G>);
+    return TL::bytes + consts + coop + TRAJ_WARPS * sizeof(WarpShared<F, G, CUBIC>);
 }
 
-template <int F, int G, int WARPS>
+template <int F, int G, int WARPS, bool CUBIC = false>
 cudaError_t launch_lg_batch(const PropLaunch *items, const int2 *work, int n_work, int *counter, int n_sm,
                             cudaStream_t s)
 {
     using namespace lg;
-    const size_t bytes = lg_smem_bytes<F, G, WARPS>();
-    auto kern = k_propagate_lg_batch<F, G, WARPS>;
+    const size_t bytes = lg_smem_bytes<F, G, WARPS, (F <= 16 && !CUBIC), WARPS, CUBIC>();
+    auto kern = k_propagate_lg_batch<F, G, WARPS, CUBIC>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     // the largest shared-memory carveout, so that as many CTAs fit as the registers allow
@@ -1503,13 +1538,13 @@ cudaError_t launch_lg_batch(const PropLaunch *items, const int2 *work, int n_wor
     return cudaGetLastError();
 }
 
-template <int F, int G, int WARPS, int TRAJ_WARPS = WARPS>
+template <int F, int G, int WARPS, int TRAJ_WARPS = WARPS, bool CUBIC = false>
 cudaError_t launch_lg(const PropLaunch &L, cudaStream_t s)
 {
     using namespace lg;
     constexpr int T = 32 / G;
-    const size_t bytes = lg_smem_bytes<F, G, WARPS, (F <= 16), TRAJ_WARPS>();
-    auto kern = k_propagate_lg<F, G, WARPS, TRAJ_WARPS>;
+    const size_t bytes = lg_smem_bytes<F, G, WARPS, (F <= 16 && !CUBIC), TRAJ_WARPS, CUBIC>();
+    auto kern = k_propagate_lg<F, G, WARPS, TRAJ_WARPS, CUBIC>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     // the largest shared-memory carveout, so that as many CTAs fit as the registers allow
@@ -1528,6 +1563,9 @@ template <int F> cudaError_t launch_group_mixed(const PropLaunch &L, cudaStream_
 {
     constexpr int G = mixed_group_lanes(F);
     constexpr int W = lg::lg_warps<F, G>();
+    if constexpr (cubic_schedule(F)) {
+        if (!L.pes.has4) return launch_lg<F, G, 4, 4, true>(L, s);
+    }
     if constexpr (F > 13) {
         // few trajectories: two or four per CTA, so that they spread over the SMs and the other
         // warps share their Hessians (F = 24: 50 steps of 64 trajectories take 3.6 ms two to a CTA,
@@ -1550,6 +1588,10 @@ cudaError_t launch_group_batch_mixed_F(int warps, const PropLaunch *items, const
     if constexpr (G == 32 && F > 9) {
         constexpr int W = lg::lg_warps<F, G>();
         if (warps == W) return launch_lg_batch<F, G, W>(items, work, n_work, counter, n_sm, s);
+        if constexpr (cubic_schedule(F)) {
+            static_assert(W != 4, "four warps mark the class without quartic terms");
+            if (warps == 4) return launch_lg_batch<F, G, 4, true>(items, work, n_work, counter, n_sm, s);
+        }
     } else if constexpr (G == 32) {
         if (warps == 1) return launch_lg_batch<F, G, 1>(items, work, n_work, counter, n_sm, s);
         if (warps == 2) return launch_lg_batch<F, G, 2>(items, work, n_work, counter, n_sm, s);

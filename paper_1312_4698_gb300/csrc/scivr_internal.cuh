@@ -186,7 +186,7 @@ int cuda_error(cudaError_t e, const char *where);
 // batch_warp_candidates(F).
 cudaError_t launch_group_batch_mixed(int F, int warps, const PropLaunch *items, const int2 *work, int n_work,
                                      int *counter, int n_sm, cudaStream_t s);
-int batch_warp_candidates(int F, int *out);   // returns the count (<= 2)
+int batch_warp_candidates(int F, bool has4, int *out);   // returns the count (<= 2)
 // One persistent launch for molecules of several F (the batch recipe's classes).
 bool multi_launch_holds(int F);
 int multi_launch_tile(int F);                  // trajectories per work item
@@ -197,6 +197,15 @@ cudaError_t launch_group_batch_multi(const PropLaunch *items, const int2 *work, 
 // most two monodromy columns per lane -- 8 lanes up to F = 4, 16 up to F = 9 (at F = 9
 // two lanes hold a second column, so a warp carries two trajectories), 32 above.
 __host__ __device__ constexpr int mixed_group_lanes(int F) { return 2 * F <= 8 ? 8 : (F <= 9 ? 16 : 32); }
+
+// Mixed propagation of a surface without quartic terms at these F: four warps a CTA, each with its own
+// trajectory, cubic rows from L2, two steps a chunk above F = 16.  The Hessian that the other kernels
+// have a CTA's warps form together is small then, and its barriers and the one-step chunks that leave
+// room for its tensor rows cost more than it saves.  64 steps of 4096 uncoupled oscillators, shared / own:
+// F = 14 3.04 / 2.21 ms, 16 4.89 / 2.68, 17 7.19 / 4.48, 20 9.48 / 5.89, 23 12.57 / 8.62, with cubic
+// couplings 3.20 / 2.35, 5.06 / 2.97, 7.79 / 4.81, 10.28 / 6.26, 13.44 / 10.26; below, the kernels are that
+// already; at F = 24 the two-step chunks' matrices leave an SM too few warps: 13.27 / 13.83 and 14.20 / 17.37.
+__host__ __device__ constexpr bool cubic_schedule(int F) { return F > 13 && F < 24; }
 
 // log <chi_x|p0_j, q0_j> (Eq. coherent_state with unit-norm states).
 template <int F>
