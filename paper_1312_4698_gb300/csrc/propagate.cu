@@ -45,13 +45,18 @@ constexpr int kMaxMixedF = 24;   // mixed lane-group kernel (one trajectory per 
 // 38.7 / 37.3 at 65536; F = 2: 15.8 / 24.0, 31.0 / 26.6, 107 / 91; F = 3: 23.8 / 47.5, 48.5 / 51.7,
 // 163 / 194; F = 6: 118 / 253, 235 / 282, 820 / 981; F = 9: 458 / 998, 801 / 1102 at 16384.  The
 // lines are where the groups' rounds of four warps per SM (9728 trajectories a round at F = 1, 4864
-// at F = 2) add up to the thread kernel's one flat round.
-int choose(int F, int precision, int64_t n_traj)
+// at F = 2) add up to the thread kernel's one flat round.  Without couplings that round is also the
+// shorter one at F = 3 and 5 while the groups take four (30 steps of 16384: 1.26 / 1.20 and 3.15 / 3.00 ms;
+// of 12000 0.93 / 1.20 and 2.53 / 3.01, of 24000 1.52 / 1.69 and 4.02 / 4.21).
+int choose(const PropLaunch &L)
 {
-    if (precision == SCIVR_MIXED) return SCIVR_KERNEL_GROUP;
+    const int F = L.args.F;
+    const int64_t n = L.n_traj;
+    if (L.args.precision == SCIVR_MIXED) return SCIVR_KERNEL_GROUP;
     if (F > kMaxGroupF) return SCIVR_KERNEL_THREAD;
+    if ((F == 3 || F == 5) && !L.pes.has3 && !L.pes.has4 && n > 14592 && n <= 19456) return SCIVR_KERNEL_THREAD;
     if (F > 2) return SCIVR_KERNEL_GROUP;
-    return n_traj > (F == 1 ? 9728 : 14592) ? SCIVR_KERNEL_THREAD : SCIVR_KERNEL_GROUP;
+    return n > (F == 1 ? 9728 : 14592) ? SCIVR_KERNEL_THREAD : SCIVR_KERNEL_GROUP;
 }
 
 }  // namespace
@@ -74,8 +79,7 @@ bool propagate_supported(int F, int precision, int kernel)
 cudaError_t launch_propagate(const PropLaunch &L, cudaStream_t s, int *n_launch)
 {
     *n_launch = 1;
-    const int kern = L.args.kernel == SCIVR_KERNEL_AUTO ? choose(L.args.F, L.args.precision, L.n_traj)
-                                                          : L.args.kernel;
+    const int kern = L.args.kernel == SCIVR_KERNEL_AUTO ? choose(L) : L.args.kernel;
     if (L.args.precision == SCIVR_MIXED) {
         switch (L.args.F) {
             SCIVR_CASES(launch_group_mixed, L)
