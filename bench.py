@@ -389,7 +389,7 @@ def batch_arm(args):
                    "schedule": ("one persistent launch over all F classes" if plan.one_launch()
                                 else "one persistent launch per F class") + " (chosen by a timed probe of the plan)"},
         "spectra_per_s": world * len(mols) / (ms * 1e-3),
-        "roofline": {"kernel": "k_propagate_lg_batch<float> (scivr_batch_launch)", "bound": "alu",
+        "roofline": {"kernel": "k_propagate_lg_batch (scivr_batch_launch)", "bound": "alu",
                      "achieved": achieved, "peak": eff_peak, "unit": "TFLOP/s", "frac": achieved / eff_peak,
                      "traffic": None, "peak_source": f"two-pipe bound summed over molecules (FP32 bulk at "
                                                      f"{probe['fp32']:.1f} + FP64-kept at {probe['fp64']:.3f} "
@@ -1017,7 +1017,7 @@ def main(argv=None):
                       (kept * n * w8.n_steps) / (fp64_peak * 1e12)
             eff_peak = pr_flops / t_bound / 1e12
             tr = TRAFFIC.get(("k_propagate_lg_mixed", args.workload, "f32" if amp_f32 else "f64"))
-            roof = {"kernel": "k_propagate_lg<float> (scivr_propagate, mixed)", "bound": "alu",
+            roof = {"kernel": "k_propagate_lg (scivr_propagate, mixed)", "bound": "alu",
                     "achieved": pr_tf, "peak": eff_peak, "unit": "TFLOP/s", "frac": pr_tf / eff_peak,
                     "traffic": tr * n * w8.n_steps if (tr is not None and full) else None,
                     "peak_source": (f"two-pipe bound: FP32 bulk {bulk:.0f} flop/step at {fp32_peak:.1f} "

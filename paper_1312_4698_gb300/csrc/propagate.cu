@@ -41,9 +41,9 @@ constexpr int kMaxMixedF = 24;   // mixed lane-group kernel (one trajectory per 
 
 // Schedule choice when the caller leaves it to the library: the lane groups, but in FP64 at F <= 2
 // beyond the numbers of trajectories where the thread kernel passes them.  Measured on GB300, us
-// per step, groups / thread: F = 1: 6.5 / 10.2 at 8192 trajectories, 11.5 / 11.4 at 19456,
-// 38.7 / 37.3 at 65536; F = 2: 15.8 / 24.0, 31.0 / 26.6, 107 / 91; F = 3: 23.8 / 47.5, 48.5 / 51.7,
-// 163 / 194; F = 6: 118 / 253, 235 / 282, 820 / 981; F = 9: 458 / 998, 801 / 1102 at 16384.  The
+// per step, groups / thread: F = 1: 6.3 / 9.8 at 8192 trajectories, 11.4 / 11.0 at 19456,
+// 39.8 / 36.8 at 65536; F = 2: 15.7 / 23.5, 31.3 / 26.1, 109 / 90; F = 3: 26.6 / 49.8, 51.8 / 54.3,
+// 169 / 199; F = 6: 117 / 252, 236 / 297, 821 / 1005; F = 9: 458 / 1005, 803 / 1106 at 16384.  The
 // lines are where the groups' rounds of four warps per SM (9728 trajectories a round at F = 1, 4864
 // at F = 2) add up to the thread kernel's one flat round.  Without couplings that round is also the
 // shorter one at F = 3 and 5 while the groups take four (30 steps of 16384: 1.26 / 1.20 and 3.15 / 3.00 ms;

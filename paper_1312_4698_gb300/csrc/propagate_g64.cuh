@@ -19,7 +19,7 @@
 // reciprocals in three multiply-adds from the hardware's approximation, exponentials from a
 // 64-entry table, pivots and thresholds compared as integers, det M's pivots multiplied pairwise.
 // Against the groups of 8 to 32 lanes without these, us per step: F = 6, 4096 trajectories: 103 -> 59;
-// F = 3, 96: 17.0 -> 9.7 (7.2 with a recording warp).
+// F = 3, 96: 17.0 -> 9.7 (6.6 with a recording warp).
 #pragma once
 
 #include <math_constants.h>
@@ -130,7 +130,7 @@ __device__ __forceinline__ double slot(const double (&w)[N], int s)
 
 // HELP: a second warp, on another sub-partition, makes the records (a quarter to a third of the
 // instructions), for launches that leave half of the sub-partitions without a warp.  F = 3, 96
-// trajectories x 400 steps, the whole FP64 run: 3.68 -> 2.93 ms.
+// trajectories x 400 steps, the whole FP64 run: 3.68 -> 2.93 ms (2.72 with the later Fourier step).
 template <int F, int G, bool HELP>
 __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropLaunch L)
 {

@@ -1,7 +1,7 @@
 // Plain Herman-Kluk SC-IVR spectrum (Eq. I(E)_SCIVR of arXiv:1312.4698) from
 // the per-trajectory Herman-Kluk summands that scivr_propagate records with
 // SCIVR_AMP_HK: the survival amplitude C(c dt) is their mean over the good
-// trajectories (a column sum of the amplitude matrix, HBM-bound: one read of
+// trajectories (a column sum of the amplitude matrix, one read of
 // 16 n K bytes), then I(E_k) = (dt/pi) Re[C(0)/2 + sum_{c>=1} C(c dt) e^{i E_k c dt}].
 // Column sums are deterministic: each block sums a fixed slice of rows for
 // 256 consecutive columns (coalesced along the time axis), and the slices'
@@ -120,7 +120,8 @@ struct WideSum {
 // one read of the summands from HBM), so the integer units
 // add in its place (WideSum).  A thread owns one column and keeps eight 16-byte loads in flight; bad
 // rows are loaded too (their flags, from shared memory, only select), so that no load waits for a
-// branch.  The three launches at 16384 x 4001 summands, 4000 energies: 373 us with FP64 additions, 306 now (with the transform below).
+// branch.  The three launches at 16384 x 4001 summands, 4000 energies: 373 us with FP64 additions, 310 now (with the transform below); the integer units are 80 % busy,
+// HBM at 63 % of the copy rate.
 __global__ void __launch_bounds__(kColThreads, 4) k_hk_colsum(const double2 *__restrict__ amp, int64_t amp_ld,
                                                            const uint8_t *__restrict__ good, int64_t n, int K,
                                                            int rows, double2 *__restrict__ part)
@@ -224,7 +225,7 @@ __global__ void __launch_bounds__(kRedX *kRedY) k_hk_reduce(const double2 *__res
 // not average out, so the phases' own rounding is put back (unit_phase) and the products are kept few.
 // With rounded phases and 30 products on end, spectra of 200 to 4000 samples were up to five times less
 // accurate than with a phase for every sample; they are as accurate now, or more.
-// 4001 samples x 4000 energies: 4234 -> 93 us (6.4e7 multiply-adds; the FP64 pipe takes 61 us for them).
+// 4001 samples x 4000 energies: 4234 -> 97 us (6.4e7 multiply-adds; the FP64 pipe takes 61 us for them).
 constexpr int kFtR = 31, kFtW = 2 * kFtR + 1, kFtG = 8, kFtWarps = 8;
 constexpr int kFtAnew = 8;   // powers of z from one sine and cosine
 // Few samples take a sine and cosine per term, shared out over the CTA's warps.  Blocks take 50 us
