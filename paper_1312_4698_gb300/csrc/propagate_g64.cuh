@@ -600,6 +600,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropL
         // ---------------- amplitudes ----------------
         if (jvalid && active) {
             const double Sc = sh.Sj[jb];
+            const double lnA = A.amplitude == SCIVR_AMP_HK ? 0.5 * log(hypot(detA.x, detA.y)) : 0.0;   // the same for every state
             for (int x = 0; x < A.n_chi; ++x) {
                 double re = 0.0, im = 0.0;
 #pragma unroll
@@ -613,7 +614,7 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropL
                 double ph = im + Sc + 0.5 * theta;
                 if (A.amplitude == SCIVR_AMP_HK) {
                     const double2 o = sh.ov0[x][t];
-                    re = re - o.x + 0.5 * log(hypot(detA.x, detA.y));
+                    re = re - o.x + lnA;
                     ph -= o.y;
                 }
                 double sn, cs_;
