@@ -231,31 +231,35 @@ __global__ void __launch_bounds__(32 * kMaxWarps, 1) k_propagate_g64(const PropL
     double stab = 0.0, detM_last = 1.0, theta_last = 0.0, arg_last = 0.0;
     double2 detA_last = make_double2(1.0, 0.0);
 
-    // amplitude at c = 0 (M = I, S = 0, theta = 0): lane 0 of each group
-    if (records && g == 0 && active) {
+    // amplitude at c = 0 (M = I, S = 0, theta = 0): a group's lanes take the reference states in turn
+    if (records) {
         double re00 = 0.0;
-        for (int x = 0; x < A.n_chi; ++x) {
+        for (int x0 = 0; x0 < A.n_chi; x0 += G) {
+            const int x = x0 + g, xc = x < A.n_chi ? x : 0;
             double re = 0.0, im = 0.0;
             for (int a = 0; a < F; ++a) {
                 const double pa = L.p0[a * n + jl], qa = L.q0[a * n + jl];
-                const double dq = cs.q_eq[x][a] - qa, dp = cs.p_eq[x][a] - pa;
+                const double dq = cs.q_eq[xc][a] - qa, dp = cs.p_eq[xc][a] - pa;
                 re = fma(-cs.qw[a] * dq, dq, re);
                 re = fma(-cs.pw[a] * dp, dp, re);
-                im = fma(0.5 * (cs.p_eq[x][a] + pa), dq, im);
+                im = fma(0.5 * (cs.p_eq[xc][a] + pa), dq, im);
             }
-            if (x == 0) re00 = re;
+            if (x0 == 0) re00 = __shfl_sync(FULL, re, base);
             // the Herman-Kluk summand divides by the initial overlap times the importance weight
             // of the sampling density, the first reference state's (chi_log_overlap0); at t = 0 it
             // is |<chi_x|p0 q0>|^2 / |<chi_0|p0 q0>|^2
             const double rdiv = x == 0 ? re : 2.0 * re00 - re;
-            sh.ov0[x][t] = make_double2(rdiv, im);
-            double sn, cs_;
-            sincos(im, &sn, &cs_);
-            const double mag = exp(re);
-            const int64_t ia = x * L.chi_stride + jl * L.amp_ld;
-            if (A.amplitude == SCIVR_AMP_HK) amp_store(L, ia, x == 0 ? 1.0 : exp(re - rdiv), 0.0);
-            else amp_store(L, ia, mag * cs_, mag * sn);
+            if (x < A.n_chi && active) {
+                sh.ov0[x][t] = make_double2(rdiv, im);
+                double sn, cs_;
+                sincos(im, &sn, &cs_);
+                const double mag = exp(re);
+                const int64_t ia = x * L.chi_stride + jl * L.amp_ld;
+                if (A.amplitude == SCIVR_AMP_HK) amp_store(L, ia, x == 0 ? 1.0 : exp(re - rdiv), 0.0);
+                else amp_store(L, ia, mag * cs_, mag * sn);
+            }
         }
+        __syncwarp();
     }
 
     const int jc = g, jb = t * C + jc;   // this lane's job of a chunk: step jc of its trajectory
