@@ -45,16 +45,21 @@ constexpr int kMaxMixedF = 24;   // mixed lane-group kernel (one trajectory per 
 // 39.8 / 36.8 at 65536; F = 2: 15.7 / 23.5, 31.3 / 26.1, 109 / 90; F = 3: 26.6 / 49.8, 51.8 / 54.3,
 // 169 / 199; F = 6: 117 / 252, 236 / 297, 821 / 1005; F = 9: 458 / 1005, 803 / 1106 at 16384.  The
 // lines are where the groups' rounds of four warps per SM (9728 trajectories a round at F = 1, 4864
-// at F = 2) add up to the thread kernel's one flat round.  Without couplings that round is also the
-// shorter one at F = 3 and 5 while the groups take four (30 steps of 16384: 1.26 / 1.20 and 3.15 / 3.00 ms;
-// of 12000 0.93 / 1.20 and 2.53 / 3.01, of 24000 1.52 / 1.69 and 4.02 / 4.21).
+// at F = 2) add up to the thread kernel's one flat round.  That round is also the shorter one while the
+// groups take four at F = 3 without couplings or with both kinds (64 steps of 16384: 2.59 / 2.52 and
+// 3.44 / 3.29 ms; cubic alone 3.14 / 3.31, quartic alone 3.29 / 3.30) and at F = 5 without (6.62 / 6.37; with
+// both 9.51 / 10.47).  And a chunk's records cost the groups as much for one step as for a chunk: one
+// step of 16384 takes them 1.0 to 1.5 times as long at F = 3..9, two steps 1.0 to 1.2 times up to F = 7.
 int choose(const PropLaunch &L)
 {
     const int F = L.args.F;
     const int64_t n = L.n_traj;
     if (L.args.precision == SCIVR_MIXED) return SCIVR_KERNEL_GROUP;
     if (F > kMaxGroupF) return SCIVR_KERNEL_THREAD;
-    if ((F == 3 || F == 5) && !L.pes.has3 && !L.pes.has4 && n > 14592 && n <= 19456) return SCIVR_KERNEL_THREAD;
+    const bool has3 = L.pes.has3, has4 = L.pes.has4;
+    if (n > 14592 && n <= 19456 && ((F == 3 && has3 == has4) || (F == 5 && !has3 && !has4))) return SCIVR_KERNEL_THREAD;
+    if (L.args.n_steps == 1 && n > (F <= 7 ? 9728 : 14592)) return SCIVR_KERNEL_THREAD;
+    if (L.args.n_steps == 2 && n > 14592 && F <= 7) return SCIVR_KERNEL_THREAD;
     if (F > 2) return SCIVR_KERNEL_GROUP;
     return n > (F == 1 ? 9728 : 14592) ? SCIVR_KERNEL_THREAD : SCIVR_KERNEL_GROUP;
 }
