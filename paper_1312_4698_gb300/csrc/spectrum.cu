@@ -20,6 +20,7 @@
 // epilogue and only one partial row per row tile reaches global memory.
 #include "fp64_ops.cuh"
 #include "scivr_internal.cuh"
+#include "spectrum_reduce.cuh"
 
 namespace scivr {
 namespace {
@@ -157,18 +158,6 @@ __global__ void __launch_bounds__(32 * WARPS) k_ft_fp64(const AmpRef amp, int64_
     }
 }
 
-__global__ void k_reduce_parts(const double *__restrict__ part, int n_mt, int n_E,
-                               const int64_t *__restrict__ n_good, double scale,
-                               double *__restrict__ I_out)
-{
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n_E) return;
-    double s = 0.0;
-    for (int m = 0; m < n_mt; ++m) s += part[(int64_t)m * n_E + k];
-    const int64_t ng = n_good[0];
-    I_out[k] = ng > 0 ? s * (scale / (double)ng) : 0.0;
-}
-
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Rows per lane: 8 once such tiles fill the 152 SMs four times over, else 2 (tiles a quarter the
@@ -221,9 +210,8 @@ cudaError_t launch_spectrum_fp64(AmpRef amp, int64_t amp_ld, const double *w,
     else
         k_ft_fp64<2><<<grid, 32 * WARPS, 0, s>>>(amp, amp_ld, tab, w, good, n_traj, K, n_blocks, n_E, part);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_reduce_parts<<<(n_E + 255) / 256, 256, 0, s>>>(part, (int)n_mt, n_E, ng, scale, I_out);
     *n_launch = 4;
-    return cudaGetLastError();
+    return launch_reduce_rows(part, (int)n_mt, n_E, ng, scale, I_out, s);
 }
 
 }  // namespace scivr

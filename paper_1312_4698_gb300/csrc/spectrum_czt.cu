@@ -32,6 +32,7 @@
 // Each CTA keeps its weighted |X|^2 sums in shared memory; a fixed-order reduction over CTAs
 // follows (deterministic).
 #include "scivr_internal.cuh"
+#include "spectrum_reduce.cuh"
 
 namespace scivr {
 namespace {
@@ -338,30 +339,6 @@ __global__ void __launch_bounds__((1 << LOGL) / 16, LOGL == 13 ? 1 : (LOGL == 12
     for (int k = threadIdx.x; k < n_E; k += NT) tb.part[(int64_t)blockIdx.x * n_E + k] = Ip[k];
 }
 
-// Partial rows summed in a fixed order: a thread of row y adds rows y, y + 8, ..., then the 8
-// sums are added in order of y.
-constexpr int kRedX = 32, kRedY = 8;
-
-__global__ void __launch_bounds__(kRedX *kRedY) k_czt_reduce(const double *__restrict__ part, int n_rows, int n_E,
-                                                   const int64_t *__restrict__ ng, double scale,
-                                                   double *__restrict__ I_out)
-{
-    __shared__ double sums[kRedY][kRedX];
-    const int k = blockIdx.x * kRedX + threadIdx.x;
-    double s = 0.0;
-    if (k < n_E) {
-#pragma unroll 8
-        for (int m = threadIdx.y; m < n_rows; m += kRedY) s += part[(int64_t)m * n_E + k];
-    }
-    sums[threadIdx.y][threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.y != 0 || k >= n_E) return;
-    s = 0.0;
-#pragma unroll
-    for (int y = 0; y < kRedY; ++y) s += sums[y][threadIdx.x];
-    I_out[k] = ng[0] > 0 ? s * (scale / (double)ng[0]) : 0.0;
-}
-
 inline size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct CztLayout {
@@ -466,9 +443,8 @@ cudaError_t launch_spectrum_czt(AmpRef amp, int64_t amp_ld, const double *w, con
     default: e = launch_czt<13>(Y, amp, amp_ld, w, good, n_traj, n_E, tb, s); break;
     }
     if (e != cudaSuccess) return e;
-    k_czt_reduce<<<(n_E + kRedX - 1) / kRedX, dim3(kRedX, kRedY), 0, s>>>(tb.part, Y.n_cta, n_E, tb.ng, scale, I_out);
     *n_launch = 4;
-    return cudaGetLastError();
+    return launch_reduce_rows(tb.part, Y.n_cta, n_E, tb.ng, scale, I_out, s);
 }
 
 }  // namespace scivr

@@ -22,6 +22,7 @@
 
 #include <cstdint>
 
+#include "spectrum_reduce.cuh"
 #include "tc_common.cuh"
 
 namespace scivr {
@@ -331,30 +332,6 @@ __global__ void k_tc_count_good(const uint8_t *__restrict__ good, int64_t n, int
     }
 }
 
-// Partial rows summed in a fixed order: a thread of row y adds rows y, y + 8, ..., then the 8
-// sums are added in order of y.
-constexpr int kRedX = 32, kRedY = 8;
-
-__global__ void __launch_bounds__(kRedX *kRedY) k_tc_reduce(const double *__restrict__ part, int n_rows, int n_E,
-                                                   const int64_t *__restrict__ ng, double scale,
-                                                   double *__restrict__ I_out)
-{
-    __shared__ double sums[kRedY][kRedX];
-    const int k = blockIdx.x * kRedX + threadIdx.x;
-    double s = 0.0;
-    if (k < n_E) {
-#pragma unroll 8
-        for (int m = threadIdx.y; m < n_rows; m += kRedY) s += part[(int64_t)m * n_E + k];
-    }
-    sums[threadIdx.y][threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.y != 0 || k >= n_E) return;
-    s = 0.0;
-#pragma unroll
-    for (int y = 0; y < kRedY; ++y) s += sums[y][threadIdx.x];
-    I_out[k] = ng[0] > 0 ? s * (scale / (double)ng[0]) : 0.0;
-}
-
 // Waits on an mbarrier that nothing completes, with a short limit: the
 // bounded-wait path must set SCIVR_ETIMEOUT and return.
 __global__ void k_wait_selftest(long long limit)
@@ -422,9 +399,8 @@ cudaError_t run(AmpRef amp, int64_t amp_ld, const double *w, const uint8_t *good
     dim3 grid((unsigned)L.n_nt, (unsigned)L.n_mt);
     k_ft_tc<ND><<<grid, 128, CF::SMEM, s>>>(At, Bt, w, good, n_traj, L.n_kt, n_E, part);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_tc_reduce<<<(n_E + kRedX - 1) / kRedX, dim3(kRedX, kRedY), 0, s>>>(part, (int)L.n_mt, n_E, ng, scale, I_out);
     *n_launch = 5;
-    return cudaGetLastError();
+    return launch_reduce_rows(part, (int)L.n_mt, n_E, ng, scale, I_out, s);
 }
 
 }  // namespace tc
