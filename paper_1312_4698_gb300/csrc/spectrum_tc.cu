@@ -44,18 +44,23 @@ __device__ __forceinline__ void split_digits(float x, __nv_bfloat16 (&d)[ND])
 // [cos(E c dt), -sin(E c dt)], rows 128..255 Im rows, [sin(E c dt), cos(E c dt)].
 //
 // A block of either operand takes 8 rows (trajectories, energies: one 8-row group of core
-// matrices) and SP_C samples, plus SP_HALO before them, as (re, im) pairs in shared memory, and
+// matrices) and C samples, plus SP_HALO before them, as (re, im) pairs in shared memory, and
 // writes all places they have: an amplitude is read from HBM once (a thread per output chunk read
 // every row twice, half of each sector at a time), a twiddle's phase -- five FP64 instructions on
 // a pipe that takes 64 cycles for each -- is formed once instead of four times.  The halo lets a
 // block own whole 16-byte chunks of the second half, whose samples start K mod 8 off a chunk
 // boundary.  16384 trajectories x 5001 samples, 4000 energies, two digits: amplitudes 288 ->
-// 243 us, twiddles 1066 -> 228 us.
-constexpr int SP_ROWS = 8, SP_C = 248, SP_HALO = 8, SP_W = SP_C + SP_HALO, SP_THREADS = SP_W;
-static_assert(SP_C % 8 == 0, "whole chunks");
+// 243 us, twiddles 1066 -> 228 us.  C = 248, but 56 for the amplitudes of up to 224 samples, whose blocks
+// of 256 threads had few of them at work or a second block that was nearly empty: the whole step for
+// 65536 trajectories and 100 energies, 248 / 56: 50 samples 158 / 107 us, 113 172 / 148, 168 159 / 143,
+// 224 166 / 164, 248 174 / 183.
+constexpr int SP_ROWS = 8, SP_C = 248, SP_FEW = 56, SP_HALO = 8;
+static_assert(SP_C % 8 == 0 && SP_FEW % 8 == 0, "whole chunks");
 
+template <int C>
 struct SplitTile {
-    float2 v[SP_ROWS][SP_W + 1];   // odd row length: the 8 rows of a chunk in different banks
+    static constexpr int W = C + SP_HALO;   // samples, and threads of a block
+    float2 v[SP_ROWS][W + 1];               // odd row length: the 8 rows of a chunk in different banks
 };
 
 template <int ND>
@@ -77,17 +82,17 @@ __device__ __forceinline__ void put_chunk(uint8_t *dst, int64_t digit_stride, co
 // (kp = K + c); the last block also has the zero columns past 2 K and the chunk that holds the end
 // of one half and the start of the other.  put(row, kp0, x, second): the 8 samples of one chunk;
 // edge(row, c): sample c from memory, for that last chunk.
-template <typename Put, typename Edge>
-__device__ __forceinline__ void split_chunks(const SplitTile &t, int cb, int n_c, int K, int n_kt, Put &&put, Edge &&edge)
+template <int C, typename Put, typename Edge>
+__device__ __forceinline__ void split_chunks(const SplitTile<C> &t, int cb, int n_c, int K, int n_kt, Put &&put, Edge &&edge)
 {
     const bool last = cb == n_c - 1;
-    const int c0 = cb * SP_C;                                         // first owned sample
-    const int lo1 = c0, hi1 = min(c0 + SP_C, K / 8 * 8);              // whole chunks of the first half
+    const int c0 = cb * C;                                         // first owned sample
+    const int lo1 = c0, hi1 = min(c0 + C, K / 8 * 8);              // whole chunks of the first half
     const int up = (K + 7) / 8 * 8;                                   // first whole chunk of the second
-    const int lo2 = max(up, (K + c0) / 8 * 8), hi2 = last ? n_kt * BK : (K + c0 + SP_C) / 8 * 8;
+    const int lo2 = max(up, (K + c0) / 8 * 8), hi2 = last ? n_kt * BK : (K + c0 + C) / 8 * 8;
     const int n1 = hi1 > lo1 ? (hi1 - lo1) / 8 : 0, n2 = hi2 > lo2 ? (hi2 - lo2) / 8 : 0;
     const int n3 = last && K % 8 ? 1 : 0;
-    for (int i = threadIdx.x; i < (n1 + n2 + n3) * SP_ROWS; i += SP_THREADS) {
+    for (int i = threadIdx.x; i < (n1 + n2 + n3) * SP_ROWS; i += SplitTile<C>::W) {
         const int row = i % SP_ROWS, ch = i / SP_ROWS;
         float2 x[8];
         if (ch < n1 + n2) {
@@ -95,7 +100,7 @@ __device__ __forceinline__ void split_chunks(const SplitTile &t, int cb, int n_c
             const int kp0 = second ? lo2 + 8 * (ch - n1) : lo1 + 8 * ch;
             const int at = kp0 - (second ? K : 0) - c0 + SP_HALO;
 #pragma unroll
-            for (int u = 0; u < 8; ++u) x[u] = at + u < SP_W ? t.v[row][at + u] : make_float2(0.0f, 0.0f);
+            for (int u = 0; u < 8; ++u) x[u] = at + u < SplitTile<C>::W ? t.v[row][at + u] : make_float2(0.0f, 0.0f);
             put(row, kp0, x, second ? 0 : 8);
         } else {
             const int kp0 = K / 8 * 8, first = K - kp0;   // first columns of the chunk are of the first half
@@ -109,15 +114,15 @@ __device__ __forceinline__ void split_chunks(const SplitTile &t, int cb, int n_c
     }
 }
 
-template <int ND>
-__global__ void __launch_bounds__(SP_THREADS)
+template <int ND, int C>
+__global__ void __launch_bounds__(SplitTile<C>::W)
     k_split_amp(const AmpRef amp, int64_t amp_ld, const uint8_t *__restrict__ good, int64_t n_traj, int K, int n_kt,
                 int n_c, uint8_t *__restrict__ At)
 {
-    __shared__ SplitTile t;
+    __shared__ SplitTile<C> t;
     const int cb = (int)(blockIdx.x % n_c);
     const int64_t row0 = (int64_t)(blockIdx.x / n_c) * SP_ROWS;
-    const int ci = threadIdx.x, c = cb * SP_C - SP_HALO + ci;
+    const int ci = threadIdx.x, c = cb * C - SP_HALO + ci;
     // a thread's eight loads go out together: bad rows are read too, their flags only select
     float2 v[SP_ROWS];
     bool ok[SP_ROWS];
@@ -156,10 +161,10 @@ __device__ __forceinline__ float2 twiddle(double E, double cdt)   // (cos, sin) 
 }
 
 template <int ND>
-__global__ void __launch_bounds__(SP_THREADS)
+__global__ void __launch_bounds__(SplitTile<SP_C>::W)
     k_split_tw(int K, int n_kt, int n_E, int n_c, double E_min, double dE, double dt, uint8_t *__restrict__ Bt)
 {
-    __shared__ SplitTile t;
+    __shared__ SplitTile<SP_C> t;
     __shared__ double Es[SP_ROWS];
     const int cb = blockIdx.x % n_c, e0 = blockIdx.x / n_c * SP_ROWS;
     if (threadIdx.x < SP_ROWS) Es[threadIdx.x] = E_min + (e0 + (int)threadIdx.x) * dE;
@@ -388,10 +393,17 @@ cudaError_t run(AmpRef amp, int64_t amp_ld, const double *w, const uint8_t *good
     k_tc_count_good<<<1, 1024, 0, s>>>(good, n_traj, ng, n_good_out);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     const int n_c = (L.K + SP_C - 1) / SP_C;
-    k_split_amp<ND><<<(unsigned)(L.rows_pad / SP_ROWS * n_c), SP_THREADS, 0, s>>>(amp, amp_ld, good, n_traj, L.K, L.n_kt,
-                                                                                  n_c, At);
+    const int64_t row_groups = L.rows_pad / SP_ROWS;
+    if (L.K <= 4 * SP_FEW) {
+        const int n_f = (L.K + SP_FEW - 1) / SP_FEW;
+        k_split_amp<ND, SP_FEW><<<(unsigned)(row_groups * n_f), SplitTile<SP_FEW>::W, 0, s>>>(amp, amp_ld, good, n_traj, L.K,
+                                                                                             L.n_kt, n_f, At);
+    } else {
+        k_split_amp<ND, SP_C><<<(unsigned)(row_groups * n_c), SplitTile<SP_C>::W, 0, s>>>(amp, amp_ld, good, n_traj, L.K,
+                                                                                         L.n_kt, n_c, At);
+    }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    k_split_tw<ND><<<(unsigned)(L.n_nt * (EPT / SP_ROWS) * n_c), SP_THREADS, 0, s>>>(L.K, L.n_kt, n_E, n_c, E_min, dE, dt,
+    k_split_tw<ND><<<(unsigned)(L.n_nt * (EPT / SP_ROWS) * n_c), SplitTile<SP_C>::W, 0, s>>>(L.K, L.n_kt, n_E, n_c, E_min, dE, dt,
                                                                                     Bt);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_ft_tc<ND>, cudaFuncAttributeMaxDynamicSharedMemorySize, CF::SMEM);
