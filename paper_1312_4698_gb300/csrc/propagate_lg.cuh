@@ -1375,9 +1375,13 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
         detA_last.y = __shfl_sync(FULL, detA.y, lastlane);
         if (!finite_bits(theta_last)) good = false;
         // ---------------- phase 4: amplitudes (job-parallel) ----------------
-        if (jvalid && active) {
-            const double S = sj_get(jb);
-            for (int x = 0; x < A.n_chi; ++x) {
+        // a chunk of one step has one job: the group's lanes take its reference states instead (eight of
+        // them, 40 steps of 4000 F = 24 trajectories: 16.9 -> 15.9 ms, uncoupled 10.1 -> 9.2)
+        constexpr bool kStates = C == 1;
+        const int jr = kStates ? t : jb;
+        if ((kStates ? g < A.n_chi : jvalid) && active) {
+            const double S = sj_get(jr), th = kStates ? theta_last : theta;
+            for (int x = kStates ? g : 0; x < A.n_chi; x += kStates ? G : 1) {
                 {
                     // the overlap's exponent and phase are O(1)-O(10) in size: FP32 from the FP32
                     // state copies; the action and the continuous phase join in FP64, and the
@@ -1385,25 +1389,25 @@ __device__ __forceinline__ void lg_body(const PropLaunch &L, int64_t cta, unsign
                     float rf = 0.0f, imf = 0.0f;
 #pragma unroll
                     for (int a = 0; a < F; ++a) {
-                        const float pa = sh.pj[a][jswz<JOBS>(a, jb)], qa = sh.qj[a][jswz<JOBS>(a, jb)];
+                        const float pa = sh.pj[a][jswz<JOBS>(a, jr)], qa = sh.qj[a][jswz<JOBS>(a, jr)];
                         const float dq = cc.q_eqf[x][a] - qa, dp = cc.p_eqf[x][a] - pa;
                         rf = fmaf(-cc.qwf[a] * dq, dq, rf);
                         rf = fmaf(-cc.pwf[a] * dp, dp, rf);
                         imf = fmaf(0.5f * (cc.p_eqf[x][a] + pa), dq, imf);
                     }
-                    double ph = fma(0.5, theta, widen_normal(imf) + S);
+                    double ph = fma(0.5, th, widen_normal(imf) + S);
                     if (A.amplitude == SCIVR_AMP_HK) {
                         // Herman-Kluk summand: |det A|^{1/2} and the division by the initial
                         // overlap times the sampling weight
                         const double2 o = sh.ov0[x][t];
-                        rf = (float)((double)rf - o.x + sh.lnA[jb]);
+                        rf = (float)((double)rf - o.x + sh.lnA[jr]);
                         ph -= o.y;
                     }
                     const double red = fma(-kTwoPi, rint(ph * kInvTwoPi), ph);   // FP64 reduction to [-pi, pi]
                     float sf, cf;
                     sincosf((float)red, &sf, &cf);
                     const float mag = expf(rf);
-                    const int64_t ia = x * L.chi_stride + jl * L.amp_ld + step0 + jc + 1;
+                    const int64_t ia = x * L.chi_stride + jl * L.amp_ld + step0 + (kStates ? 0 : jc) + 1;
                     if (L.amp_f32) reinterpret_cast<float2 *>(L.amp)[ia] = make_float2(mag * cf, mag * sf);
                     else L.amp[ia] = make_double2((double)(mag * cf), (double)(mag * sf));
                 }
