@@ -61,6 +61,8 @@ struct Geo {
     static constexpr int kRecordInstr =
         NC * (N2 * (N2 - 1) / 2) + N2 * (3 + NC) + NC + ilog2(G) + 4 * NM * F + 6 +
         (4 * (F * (F * F - 1)) / 3 + 11 * F + 4 * F * (F - 1) / 2 + 9 * F + 110) / C;
+    static constexpr int kStateInstr = (9 * F + 75) / C;   // of a record, for every reference state but the first (counted at
+                                                           // F = 1, where a step is little beside them)
     static constexpr int MAIL = NC * N2 + 2 * NM + 1;   // state of a step that its records need, per lane
 };
 
@@ -683,23 +685,25 @@ cudaError_t launch(const PropLaunch &L, int n_sm, cudaStream_t s)
 
 // The narrowest group a lane's registers allow (its columns and their copy for det M).
 constexpr int min_lanes(int F) { return F <= 1 ? 2 : F <= 6 ? 4 : 8; }
-// The widest that still saves instructions where a warp records.
-constexpr int max_lanes(int F) { return F <= 1 ? 2 : F == 2 ? 4 : F == 3 ? 8 : F <= 5 ? 16 : 32; }
+// The widest that still saves instructions where a warp records (at F = 1 beyond two lanes only those of
+// several reference states: eight states, 64 steps of 600 harmonic trajectories 0.61 -> 0.24 ms).
+constexpr int max_lanes(int F) { return F <= 1 ? 8 : F == 2 ? 4 : F == 3 ? 8 : F <= 5 ? 16 : 32; }
 
 }  // namespace g64
 
 // Group size: the fewest FP64 instructions over the rounds of four warps per SM that the
 // trajectories take; with a recording warp where two per SM suffice.
 template <int F, int G = g64::min_lanes(F)>
-void choose_g64_lanes(int64_t n_traj, int n_sm, double &best, int &lanes, bool &help)
+void choose_g64_lanes(int64_t n_traj, int n_chi, int n_sm, double &best, int &lanes, bool &help)
 {
     using E = g64::Geo<F, G>;
     const int64_t warps = (n_traj * G + 31) / 32, slots = (int64_t)g64::kMaxWarps * n_sm;
     const bool h = 2 * warps <= slots;
-    const int instr = !h ? E::kStepInstr + E::kRecordInstr : E::kStepInstr > E::kRecordInstr ? E::kStepInstr : E::kRecordInstr;
+    const int step = E::kStepInstr, record = E::kRecordInstr + (F == 1 ? (n_chi - 1) * E::kStateInstr : 0);
+    const int instr = !h ? step + record : step > record ? step : record;
     const double cost = (double)((warps + slots - 1) / slots) * instr;
     if (lanes == 0 || cost < best) { best = cost; lanes = G; help = h; }
-    if constexpr (G < g64::max_lanes(F)) choose_g64_lanes<F, 2 * G>(n_traj, n_sm, best, lanes, help);
+    if constexpr (G < g64::max_lanes(F)) choose_g64_lanes<F, 2 * G>(n_traj, n_chi, n_sm, best, lanes, help);
 }
 
 template <int F, int G = g64::min_lanes(F)>
@@ -719,7 +723,7 @@ template <int F> cudaError_t launch_group_fp64(const PropLaunch &L, cudaStream_t
     double cost = 0.0;
     int lanes = 0;
     bool help = false;
-    choose_g64_lanes<F>(L.n_traj, n_sm, cost, lanes, help);
+    choose_g64_lanes<F>(L.n_traj, L.args.n_chi, n_sm, cost, lanes, help);
     return launch_g64_lanes<F>(L, lanes, help, n_sm, s);
 }
 
