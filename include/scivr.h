@@ -247,8 +247,8 @@ int scivr_sample_initial(scivr_pes pes, const double *gamma, const double *p_eq,
  * path tests det M every 16 steps and at the last step (FP64: every step).
  * Built: SCIVR_FP64 for F <= 9 (both schedules), SCIVR_MIXED for F <= 24
  * (lane-group schedule; one trajectory per warp above F = 9, two column
- * groups per trajectory and tensors read from L2 above F = 16; at F = 14..23 surfaces
- * without quartic terms take a kernel of their own).  A surface of
+ * groups per trajectory and tensors read from L2 above F = 16; above F = 13 surfaces
+ * without quartic terms take kernels of their own).  A surface of
  * kind SCIVR_PES_CART3 (scivr_create_pes_cartesian) runs on SCIVR_FP64 with the
  * thread schedule only.
  * Errors: SCIVR_EINVAL (NULL pointers, n_traj < 1, n_steps < 1, dt <= 0,
@@ -333,7 +333,7 @@ typedef struct {
 typedef struct scivr_batch_s *scivr_batch;   /* opaque plan, library-owned */
 
 /* Build a plan for a batch (Sec. III.B: trajectories of all molecules are
- * independent).  Molecules are grouped by (F, precision), at F = 14..23 those
+ * independent).  Molecules are grouped by (F, precision), above F = 13 those
  * without quartic terms apart; each group runs as
  * one persistent lane-group launch whose CTAs pull (molecule, trajectory
  * tile) work items, largest cost first, so molecules of different sizes

@@ -1,7 +1,7 @@
 // Batched runs (scivr_batch_*): many molecules with different F, trajectory
 // counts and step counts.  Trajectories of all molecules are independent
 // (Sec. III.B of arXiv:1312.4698), so the plan groups molecules by
-// (F, precision; at F = 14..23 those without quartic terms apart) and runs each mixed-precision group as one persistent
+// (F, precision; above F = 13 those without quartic terms apart) and runs each mixed-precision group as one persistent
 // lane-group launch whose CTAs pull (molecule, tile) work items, the
 // longest first.  FP64 molecules are launched one by one.  Each molecule's
 // spectra follow.  The launch sequence allocates nothing and never

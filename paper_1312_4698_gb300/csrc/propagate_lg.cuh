@@ -241,7 +241,7 @@ constexpr int kDetMEvery = 16;
 
 template <int F, int G, bool CUBIC = false> __host__ __device__ constexpr int lg_chunk()
 {
-    if (CUBIC) return F > 16 ? 2 : 4;
+    if (CUBIC) return F > 23 ? 1 : (F > 16 ? 2 : 4);
     return G == 32 && F > 16 ? 1 : (G == 32 && F > 15 ? 2 : ((G == 32 && F > 12) || (G == 16 && F > 8) ? 4 : 8));
 }
 
@@ -1567,9 +1567,6 @@ template <int F> cudaError_t launch_group_mixed(const PropLaunch &L, cudaStream_
 {
     constexpr int G = mixed_group_lanes(F);
     constexpr int W = lg::lg_warps<F, G>();
-    if constexpr (cubic_schedule(F)) {
-        if (!L.pes.has4) return launch_lg<F, G, 4, 4, true>(L, s);
-    }
     if constexpr (F > 13) {
         // few trajectories: two or four per CTA, so that they spread over the SMs and the other
         // warps share their Hessians (F = 24: 50 steps of 64 trajectories take 3.6 ms two to a CTA,
@@ -1578,6 +1575,9 @@ template <int F> cudaError_t launch_group_mixed(const PropLaunch &L, cudaStream_
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
+        if constexpr (cubic_schedule(F)) {
+            if (!L.pes.has4 && (F < 24 || !L.pes.has3 || L.n_traj > 4 * (int64_t)n_sm)) return launch_lg<F, G, 4, 4, true>(L, s);
+        }
         if (L.n_traj <= 2 * (int64_t)n_sm) return launch_lg<F, G, W, 2>(L, s);
         if (L.n_traj <= 4 * (int64_t)n_sm) return launch_lg<F, G, W, 4>(L, s);
     }

@@ -199,13 +199,15 @@ cudaError_t launch_group_batch_multi(const PropLaunch *items, const int2 *work, 
 __host__ __device__ constexpr int mixed_group_lanes(int F) { return 2 * F <= 8 ? 8 : (F <= 9 ? 16 : 32); }
 
 // Mixed propagation of a surface without quartic terms at these F: four warps a CTA, each with its own
-// trajectory, cubic rows from L2, two steps a chunk above F = 16.  The Hessian that the other kernels
+// trajectory, cubic rows from L2, two steps a chunk above F = 16 (one at F = 24).  The Hessian that the other kernels
 // have a CTA's warps form together is small then, and its barriers and the one-step chunks that leave
 // room for its tensor rows cost more than it saves.  64 steps of 4096 uncoupled oscillators, shared / own:
 // F = 14 3.04 / 2.21 ms, 16 4.89 / 2.68, 17 7.19 / 4.48, 20 9.48 / 5.89, 23 12.57 / 8.62, with cubic
 // couplings 3.20 / 2.35, 5.06 / 2.97, 7.79 / 4.81, 10.28 / 6.26, 13.44 / 10.26; below, the kernels are that
-// already; at F = 24 the two-step chunks' matrices leave an SM too few warps: 13.27 / 13.83 and 14.20 / 17.37.
-__host__ __device__ constexpr bool cubic_schedule(int F) { return F > 13 && F < 24; }
+// already.  At F = 24 the Hessian with cubic terms is large enough to be shared by a CTA's warps while that
+// gives every trajectory an SM's: 40 steps of 300 1.83 / 1.96 ms, of 1000 2.34 / 2.30, of 4096 9.16 / 8.60,
+// uncoupled 8.58 / 7.52.
+__host__ __device__ constexpr bool cubic_schedule(int F) { return F > 13; }
 
 // log <chi_x|p0_j, q0_j> (Eq. coherent_state with unit-norm states).
 template <int F>
